@@ -83,10 +83,10 @@ typedef struct stab_term {
 
 /* ---------------------------------------------------------------- options */
 enum stab_kernel {
-    /* The library's choice.  n <= 6: vectors resident in shared memory; plans of
-     * 64 or more passes are cut in two and both parts run at once (the
-     * generators at n <= 4 through the second part's transfer matrix, <O> and
-     * gradients meeting at the cut).  n >= 7: vectors in HBM, passes grouped
+    /* The library's choice.  n <= 6: vectors resident in shared memory.  Plans of
+     * 64 or more passes: at n <= 4 everything is read off the 2^n x 2^n
+     * unitaries of the plan's segments, which run at once; at n = 5, 6 <O> and
+     * gradients run from both ends and meet at half the passes.  n >= 7: vectors in HBM, passes grouped
      * into shared-memory tiles where the vectors are small, else one fused pass
      * per launch (gradients again meet at the cut).  Batches pick their CTAs
      * per SM by timing a sample of their units. */
@@ -186,18 +186,16 @@ int stab_expect_async(stab_ctx *ctx, double *out_dev);
 
 /* Adjoint gradient of the loaded observable: expect_dev (device, may be NULL)
  * receives <O>, grads_dev (device) n_params doubles.  Queued like
- * stab_expect_async.  At n <= 4 (AUTO kernel, long circuits) the gradient is
- * cut into the parts of the generators' split sweep and takes its vectors at
- * the cuts from that sweep: when none was made for the current angles it is
- * queued first on the context stream (as by stab_run_generators, whose
- * results it leaves valid for reuse), then the gradient on the internal
+ * stab_expect_async.  At n <= 4 (AUTO kernel, long circuits) the gradient reads
+ * the unitaries of the plan's parts and segments: when they were not composed
+ * for the current angles that is queued first on the context stream (as by
+ * stab_run_generators, which reuses them), then the gradient on the internal
  * stream.  Same for stab_expect_async in that form. */
 int stab_grad_async(stab_ctx *ctx, double *expect_dev, double *grads_dev);
 
-/* How the last gradient's plan is cut: *parts receives K >= 2 when it is cut
- * into the K parts of the generators' split sweep (n <= 4; the pairs at the
- * cuts come from that sweep), 1 when it uses the meet-in-the-middle or a
- * streamed sweep, 0 before any gradient since the circuit was loaded.
+/* How the last gradient's plan is cut: *parts receives K >= 2 when it runs
+ * through the K parts of the generators' plan (n <= 4, their unitaries), 1 when
+ * it uses the meet-in-the-middle or a streamed sweep, 0 before any gradient since the circuit was loaded.
  * Errors: STAB_E_INVAL (ctx or parts NULL). */
 int stab_grad_parts(stab_ctx *ctx, int32_t *parts);
 
@@ -384,9 +382,9 @@ typedef struct stab_result {
 
 /* Admission footprint of a request: max(n 4^n 8, 4^n 8 x (4 for <O>, 12 for
  * a gradient: the vectors of the split sweeps)) bytes plus 96 bytes per gate,
- * plus at n <= 4 the split sweep's transfer matrices (8 x 16^n bytes each: two
- * at n = 4, up to min(49, 160 / (4^n - 1)) at n <= 3), its n + 1 first-part
- * vectors and the pairs at the cuts (two vectors per matrix),
+ * plus at n <= 4 room for the unitaries of the plan's segments and parts
+ * (8 x 16^n bytes twice at n = 4, min(49, 160 / (4^n - 1)) times at n <= 3, and
+ * n + 1 + 2 vectors of 4^n doubles each time),
  * plus, for a gradient, the adjoint's partial dot sums: per CTA of the
  * streamed sweep above n = 6, per thread of the resident sweep at n <= 5
  * (8 bytes x gates x 32, 32, 32, 64, 256 threads at n = 1..5, while that
@@ -508,21 +506,17 @@ int stab_sparse_order_history(stab_sparse *s, int64_t *orders, int64_t max, int6
 /* Number of qubits, loaded gates and fused passes of the current plan. */
 int stab_plan_info(stab_ctx *ctx, int64_t *n_gates, int64_t *n_passes, int32_t *kernel);
 
-/* The cut of the split resident sweeps of the current plan (n <= 6, AUTO
- * kernel, fused).  <O> = <lambda, r> for any cut of the circuit, since every
- * gate's map is orthogonal (Sec. II): r = rho_0 through passes [0, cut) and
- * lambda = O backward through [cut, n_passes) run at once; for n <= 4 the
- * generators are T a_k, a_k = Z_k through [0, cut) and T the transfer matrix
- * of [cut, n_passes).  Writes *cut (-1: no split; the plan runs as one
- * sweep), *gen_units (vectors of the generators' split sweep -- the n
- * generators and rho_0 through [0, cut), the 4^n - 1 columns of T; 0 when not
- * split; stab_density_matrix uses the same sweep, r = T r_1) and
- * *expect_units (of the expectation's own launch, 0 when not split).  At
- * n <= 3 a long plan is cut into K >= 3 parts of equal pass counts (cut = the
- * first cut): the sweep carries the K - 1 later parts' transfer matrices,
- * the generators are T_K ... T_2 a_k, and <O> = sum_P o_P (T_K ... T_2 r_1)_P
- * reuses the sweep made for the same angles (*expect_units = 0).
- * Any output pointer may be NULL.  Errors: STAB_E_INVAL (ctx NULL). */
+/* How the current plan is cut (n <= 6, AUTO kernel, fused, 64 or more passes).
+ * n <= 4: into K parts at *cut and (three parts) a second place; every part
+ * is carried by its 2^n x 2^n unitary, composed from segments that run at
+ * once.  *gen_units = n + 1 + (K - 1)(4^n - 1): the generators and rho_0, and
+ * per later part the nontrivial columns of the transfer matrix its unitary
+ * stands for; *expect_units = 0 (<O> reads the same unitaries).  n = 5, 6:
+ * <O> = <lambda, r> for any cut, since every gate's map is orthogonal
+ * (Sec. II): r = rho_0 through passes [0, cut) and lambda = O backward through
+ * [cut, n_passes) run at once; *gen_units = 0, *expect_units = 2.  *cut = -1:
+ * the plan runs as one sweep.  Any output pointer may be NULL.  Errors:
+ * STAB_E_INVAL (ctx NULL). */
 int stab_split_info(stab_ctx *ctx, int64_t *cut, int32_t *gen_units, int32_t *expect_units);
 
 /* Number of kernels this context launched since creation (all entry points). */
@@ -585,16 +579,14 @@ typedef struct stab_path_choice {
     int32_t resident;          /* n <= 6: 1 = each vector resident in shared memory on one CTA,
                                   0 = vectors streamed through HBM (grid-wide passes) */
     int32_t resident_adjoint;  /* n <= 6: 1 = gradients by the resident adjoint, 0 = streamed */
-    double gen_cut;            /* n <= 4: where the generators' split sweep cuts the plan, as a
-                                  fraction of its passes (0.3 .. 0.7): the end of the first part */
+    double gen_cut;            /* n <= 4: where a long plan is cut into parts, as a fraction of its
+                                  passes (0.3 .. 0.7): the end of the first part */
     int64_t tile_limit;        /* streamed plans: consecutive wire passes share one tile-fused
                                   launch while vectors x 4^n <= tile_limit, else one launch
                                   per pass (>= 0) */
     int32_t tuned;             /* 1: measured on this GPU model; 0: the built-in defaults */
-    int32_t gen_parts;         /* n = 4: 2 = the plan cut once at gen_cut (the generators through
-                                  one transfer matrix); 3 = a first part of gen_cut of the passes
-                                  and two equal parts after it (the generators through a chain of
-                                  two transfer matrices whose columns run four to an SM) */
+    int32_t gen_parts;         /* n = 4: 2 = the plan cut once at gen_cut; 3 = a first part of
+                                  gen_cut of the passes and two equal parts after it */
 } stab_path_choice;
 
 /* The built-in defaults for n qubits: resident and resident_adjoint 1,
@@ -627,14 +619,12 @@ int stab_path_load(const char *path);
 
 /* Measures the candidates for n qubits on CUDA device `device` now, stores
  * the result under that GPU's name and writes it to *out (may be NULL).
- * Candidates: n = 4: two parts with gen_cut in {0.50, 0.53, 0.56, 0.59, 0.62}
- * and three parts with gen_cut in {0.43, 0.45, 0.47, 0.49, 0.51} (time of the
- * generators of a 24,000-gate probe); n = 5, 6: resident against streamed for
+ * Candidates: n = 5, 6: resident against streamed for
  * <O> and, separately, for the gradient (2,000-gate probe); n = 7 .. 9: tiles
  * against one launch per pass, for one vector (<O>) and for n vectors (the
  * generators), giving tile_limit = the largest of those launch sizes where
- * tiles won (0 when neither); n <= 3 and n >= 10 have nothing measured and
- * keep the defaults (marked tuned).  Each candidate takes the best of five
+ * tiles won (0 when neither); n <= 4 (the parts' segments run at once wherever
+ * they are cut) and n >= 10 have nothing measured and keep the defaults (marked tuned).  Each candidate takes the best of five
  * timed calls; a candidate replaces the default only when it is more than 2 %
  * faster, so timing noise does not flip a choice.  Takes up to about a tenth
  * of a second.

@@ -50,17 +50,6 @@ struct StreamArgs {
     int32_t *status;         // set to a nonzero code when a bounded wait gives up
 };
 
-// One part of a many-part resident adjoint sweep (phase 1 of k_adjoint_split
-// with parts): the part's gradient stream, walked backward (the first part,
-// from its end) or forward (every later part, from its start), and the pair
-// (lambda, rho) where the walk starts.
-struct AdjPart {
-    const Rec *stream;
-    int32_t n_chunks;
-    int32_t forward;
-    const double *lam, *rho;
-};
-
 // Split resident adjoint (two CTAs, two launches; see k_adjoint_split).
 struct AdjointSplitArgs {
     const Rec *stream[2];    // phase 0: forward [0, cut), backward [cut, P); phase 1: backward
@@ -74,8 +63,6 @@ struct AdjointSplitArgs {
     double *partials;        // phase 1, optional: per-thread dots [rotation ordinal][threads]
                              // (summed afterwards by k_reduce_partials); null: each pass
                              // reduces its rotations' dots over the CTA into grad_rot
-    const AdjPart *parts;    // phase 1, optional (device array): one CTA per part, in place
-    int32_t n_parts;         // of stream[] and the pair (lmid, rmid); CTA 0 writes <O>
     double *expect_out;      // phase 1: <O>
     int32_t *status;
 };
@@ -95,12 +82,6 @@ struct AdjointStreamArgs {
 // Threads of the resident adjoint kernels' CTA at n qubits (the row length
 // of their per-thread partials).
 int resident_adjoint_threads(int n);
-// The pairs at the cuts of a K-part split at n <= 3, one CTA: rho_1 = r1,
-// rho_{k+1} = T_k rho_k, lambda_{K-1} = T_{K-1}^T o, lambda_k = T_k^T
-// lambda_{k+1}, with T_k (k = 1 .. K-1) at T + (k - 1) 16^n (by columns);
-// pairs = [lambda_1, rho_1, ..., lambda_{K-1}, rho_{K-1}], 4^n doubles each.
-cudaError_t launch_adjoint_pairs(const double *T, int K, int n, const double *r1,
-                                 const double *o, double *pairs, cudaStream_t st);
 // Bytes of the resident adjoint's per-thread dot shares for n_rot rotations
 // at n qubits, or 0 where the sweeps reduce each pass's dots themselves.
 size_t resident_partial_bytes(int n, int64_t n_rot);
@@ -198,10 +179,6 @@ namespace stab {
 // The context's main stream (work queued by the asynchronous entry points is
 // complete once this stream is).
 cudaStream_t ctx_stream(stab_ctx *ctx);
-// Marks the context's split generator sweep as not made for its current
-// angles, so the next call that needs it runs it again (timing probes that
-// call the same entry point repeatedly).
-void ctx_forget_sweep(stab_ctx *ctx);
 
 // Density matrix from the forward-evolved coefficients of 2^n |0><0|:
 // rho (device, 2 x 4^n doubles, interleaved complex, row-major).
@@ -235,43 +212,6 @@ cudaError_t launch_encode_stream(Rec *recs, const int32_t *enc, int n_enc, const
 
 // Shared-memory-resident propagation, one CTA per vector (n <= kMaxResidentQubits).
 cudaError_t launch_resident_stream(int n, const StreamArgs &a, cudaStream_t st);
-// out[k] = T a[k] (k < n_vec) for 4^n x 4^n T stored by columns; n <= 4.
-// Columns 1 .. 4^n - 1 of the transfer matrix of a stream (column j = basis
-// string j through its passes) into tmat (column j at tmat + j * 4^n), two
-// columns per CTA; n = 4 only.  transfer_cols_ctas(n): its grid (0: n unsupported).
-int transfer_cols_ctas(int n);
-// out_k = T_{n_mats-1} ... T_0 in_k for n <= 3 (matrices of 4^n x 4^n, column
-// j of matrix s at T + s 16^n + j 4^n); with dot_out (n_vec = 1) also
-// <O> = sum of terms' coeff x out[idx].  out may be null.
-cudaError_t launch_apply_chain(const double *T, int n_mats, const double *in, double *out,
-                               int n_vec, int n, const DevTerm *terms, int n_terms,
-                               double *dot_out, cudaStream_t st);
-// The columns of one or two transfer matrices (n_parts streams) at n = 4:
-// matrix p at tmat + p 16^n, column j at + j 4^n (column 0 is not written);
-// 128 CTAs of two (one matrix) or four (two matrices) columns each.
-struct ColArgs {
-    const Rec *stream[2];
-    int32_t n_chunks[2];
-    int32_t n_parts;
-    double *tmat;
-    int32_t *status;
-};
-cudaError_t launch_transfer_cols(const ColArgs &a, int n, cudaStream_t st);
-// Dynamic shared memory of a k_transfer_cols CTA (more than half an SM's).
-size_t transfer_cols_smem();
-// out = T^T in for one n = 4 transfer matrix (the backward step through its
-// part): 4^n outputs, each a column of T dotted with in.
-cudaError_t launch_apply_transfer_t(const double *T, const double *in, double *out, int n,
-                                    cudaStream_t st);
-// out_k = T_{n_mats-1} ... T_0 in_k at n = 4 (one k_apply_transfer per matrix,
-// tmp: 2 x n_vec x 4^n doubles between them); with dot_out (n_vec = 1) also
-// <O> = sum of terms' coeff x the result[idx], in term order.  out may be null.
-cudaError_t launch_apply_transfer_chain(const double *T, int n_mats, const double *in,
-                                        double *out, double *tmp, int n_vec, int n,
-                                        const DevTerm *terms, int n_terms, double *dot_out,
-                                        cudaStream_t st);
-cudaError_t launch_apply_transfer(const double *T, const double *a, double *out, int n_vec,
-                                  int n, cudaStream_t st);
 int resident_lanes_per_group(int n);
 
 // Streamed passes over n_vec vectors of 4^n doubles in global memory.
@@ -354,6 +294,53 @@ cudaError_t launch_reduce_partials(const double *partials, int n_rot, int n_bloc
 cudaError_t launch_gather_grads(const double *grad_rot, const int32_t *param_ptr,
                                 const int32_t *param_rot, int n_params, double *grads,
                                 cudaStream_t st);
+
+// ---------------------------------------------------------------- segment unitaries (k_unitary.cu)
+
+// 2 x 2 maps of the plan's wire runs from the angles: a thread per run, or a
+// warp per run when some run is longer than kSeqMapGates gates (max_count).
+cudaError_t launch_uni_maps(const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
+                            const double *thetas, UniMap *maps, cudaStream_t st);
+
+struct UniArgs {
+    const UniOp *ops;
+    const UniMap *maps;
+    const UniSeg *segs;
+    const UniPart *parts;
+    int32_t n_segs, n_parts;
+    double2 *nodes;          // node matrices, 4^n complex entries each, column-major
+    int32_t *node_parity;    // per node: U is kept times sqrt(2)^parity
+    int32_t *node_count;     // per node: arrivals of its children (zero between launches)
+};
+// Every segment's unitary and the trees' inner nodes up to each part's root,
+// one CTA per segment.
+cudaError_t launch_uni_segments(int n, const UniArgs &a, cudaStream_t st);
+// The parts' unitaries in plan order (at most kUniMaxParts).
+constexpr int kUniMaxParts = 3;
+struct UniRoots {
+    const double2 *nodes;
+    const int32_t *node_parity;
+    int32_t n;
+    int32_t root[kUniMaxParts];
+};
+// out[k] = the Pauli coefficients of U Z_k U^dagger, k < n, U the product of
+// the roots, one CTA per generator.
+cudaError_t launch_uni_images(int n, const UniRoots &r, double *out, cudaStream_t st);
+// out = roots 1 times 0.
+cudaError_t launch_uni_merge(int n, const UniRoots &r, double2 *out, int32_t *parity,
+                             cudaStream_t st);
+// psi = U |0>: *expect = <psi|O|psi> (may be null), r_out (may be null) = the
+// coefficients of 2^n |psi><psi|; psi and phi (may be null): the states and
+// the cotangents at the parts' boundaries, (r.n + 1) x 2^n entries each.
+cudaError_t launch_uni_states(int n, const UniRoots &r, const DevTerm *terms, int n_terms,
+                              double *expect, double2 *psi, double2 *phi, double *r_out,
+                              cudaStream_t st);
+// grad_gate[g] = d<O>/d(angle of gate g) for the rotations of the run-ordered
+// gate array; dots: 3 x 2^n doubles of scratch per run.
+cudaError_t launch_uni_grad(int n, const UniArgs &a, const double2 *psi, const double2 *phi,
+                            double *dots, const UniRun *runs, int n_runs, int max_count,
+                            const RawGate *gates, const double *thetas, double *grad_gate,
+                            cudaStream_t st);
 
 // ---------------------------------------------------------------- sparse term lists (k_sparse.cu)
 

@@ -980,9 +980,10 @@ void completer_main(stab_server *s) {
 
 extern "C" {
 
-// n <= 4: the split sweep's transfer matrices (at most two at n = 4, one
-// per later part of the chain at n <= 3: bounded by 160 SMs' worth of
-// columns), its first-part vectors and the pairs at the cuts.
+// n <= 4: with the 96 bytes per gate, a bound on the unitaries of the plan's
+// segments and parts (2 x 4^n complex entries per segment, at most one segment
+// per SM at n = 4 and two below, at least ten wire passes each) and its runs'
+// maps.
 static int64_t split_sweep_bytes(int n) {
     if (n > 4) return 0;
     const int64_t E = (int64_t)1 << (2 * n);

@@ -100,16 +100,22 @@ struct DevPlan {
     // split < 0: none
     DevStreamBuf h1, h2, h2b, h1b;
     int split = -1;
-    // n <= 3, long plans: K >= 3 forward parts, part k = passes [cuts[k], cuts[k+1])
-    // (the generators, rho_0 and <O> through the chain of the parts' transfer
-    // matrices); empty otherwise
-    std::vector<DevStreamBuf> parts;
+    // n <= 4, long plans (uni): K >= 2 parts, part k = passes [cuts[k],
+    // cuts[k+1]), each cut into segments whose unitaries are composed at once
+    // (see k_unitary.cu); no streams.
+    bool uni = false;
+    bool uni_identity = false;       // some wire run is the identity and holds no rotation
     std::vector<int> cuts;
-    std::vector<DevStreamBuf *> all_streams() {
-        std::vector<DevStreamBuf *> v = {&sf, &sb, &h1, &h2, &h2b, &h1b};
-        for (DevStreamBuf &p : parts) v.push_back(&p);
-        return v;
-    }
+    std::vector<UniOp> uops;
+    std::vector<UniRun> uruns;
+    std::vector<RawGate> ugates;
+    std::vector<UniSeg> usegs;
+    std::vector<UniPart> uparts;
+    int uni_max_run = 0, uni_nodes = 0;
+    UniArgs uargs{};
+    const UniRun *uruns_dev = nullptr;
+    const RawGate *ugates_dev = nullptr;
+    std::vector<DevStreamBuf *> all_streams() { return {&sf, &sb, &h1, &h2, &h2b, &h1b}; }
     DevBuf buf;
     Program prog{};
     const int32_t *map_gate_idx = nullptr;
@@ -169,24 +175,17 @@ struct stab_ctx {
     DevBuf lam2, tmp3;               // second-branch buffers of the split sweeps
     DevBuf dotbuf;                   // partial sums of the split expectation's inner product
     DevBuf gmid;                     // split resident adjoint: rho, then lambda, at the cut
-    DevBuf odense;                   // O as a dense vector, and a second vector for the
-                                     // transposed products of the aligned gradient
-    bool grad_aligned = false;       // the gradient plan's parts end where the generators' do
-    std::vector<int> grad_cuts;      // their pass boundaries in the gradient plan (K + 1)
-    DevBuf gpairs, gparts;           // the pairs at the cuts; the parts' descriptors
-    std::vector<AdjPart> gparts_host;
-    DevBuf chainbuf, chainbuf_e;     // n = 4 chain of transfer matrices: intermediate vectors
-                                     // of the context stream's products, of <O>'s (aux)
-    // split resident sweeps (n <= 6; see split_units): transfer matrix of the
-    // second part (n <= 4), first-part generators, meeting vectors, basis
-    // terms, batch units (generators; expectation), unit counters
-    DevBuf tmat, avec, rmid, lmid, bterms, units_g, units_e, cnt;
-    std::vector<const void *> key_g, key_e;
-    int n_units_g = 0;
+    bool grad_uni = false;           // the gradient runs through the segments' unitaries
+    DevBuf ustates, udots;           // its states at the parts' boundaries, runs' dot shares
+    // split sweeps of the small registers.  n <= 4: the wire runs' 2 x 2 maps,
+    // the segments' and parts' unitaries.  n = 5, 6: the two halves of <O>:
+    // meeting vectors, batch units, unit counter
+    DevBuf umaps, unodes, rmid, lmid, units_e, cnt;
+    std::vector<const void *> key_e;
     size_t split_smem = 0;
     int sms = 0;                     // SMs of the device
-    // the split sweep's launch (first-part vectors, columns of T) was made for
-    // these angles when tx_gen == param_gen; ev_tx marks its end on st
+    // the parts' unitaries were composed for these angles when tx_gen ==
+    // param_gen; ev_tx marks their end on st
     int64_t param_gen = 0, tx_gen = -1;
     cudaEvent_t ev_tx = nullptr;
     DevBuf status;                   // int32 set by kernels whose bounded waits gave up
@@ -269,11 +268,15 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     // resident plans read only their streams (plus maps and raw gates for encoding)
     const size_t n_pass = P.streams ? 0 : H.passes.size();
     const size_t n_ops = P.streams ? 0 : H.ops.size();
+    // plans applied through segment unitaries read their own op list and runs
+    const size_t n_maps = P.uni ? 0 : H.maps.size();
+    const size_t n_midx = P.uni ? 0 : H.map_gate_idx.size();
+    const size_t n_raw = P.uni ? 0 : H.raw.size();
     const size_t b_pass = align256(n_pass * sizeof(DevPass));
     const size_t b_ops = align256(n_ops * sizeof(DevOp));
-    const size_t b_maps = align256(H.maps.size() * sizeof(DevMap3));
-    const size_t b_midx = align256(H.map_gate_idx.size() * sizeof(int32_t));
-    const size_t b_raw = align256(H.raw.size() * sizeof(RawGate));
+    const size_t b_maps = align256(n_maps * sizeof(DevMap3));
+    const size_t b_midx = align256(n_midx * sizeof(int32_t));
+    const size_t b_raw = align256(n_raw * sizeof(RawGate));
     const size_t b_pptr = align256(H.param_ptr.size() * sizeof(int32_t));
     const size_t b_prot = align256(H.param_rot.size() * sizeof(int32_t));
     const size_t b_tabs = align256(H.tabs.size() * sizeof(DevTab));
@@ -282,8 +285,13 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     for (const DevStreamBuf *S : streams)
         b_streams += align256((S->host.size() + S->tail.size()) * sizeof(Rec)) +
                      align256((S->enc.size() + S->tail_enc.size()) * 4);
+    const size_t b_uops = align256(P.uops.size() * sizeof(UniOp));
+    const size_t b_uruns = align256(P.uruns.size() * sizeof(UniRun));
+    const size_t b_ugates = align256(P.ugates.size() * sizeof(RawGate));
+    const size_t b_usegs = align256(P.usegs.size() * sizeof(UniSeg));
+    const size_t b_uparts = align256(P.uparts.size() * sizeof(UniPart));
     const size_t total = b_pass + b_ops + b_maps + b_midx + b_raw + b_pptr + b_prot + b_tabs +
-                         b_streams;
+                         b_streams + b_uops + b_uruns + b_ugates + b_usegs + b_uparts;
     RC(c->dalloc(P.buf, total, c->st));
     CK(cudaEventSynchronize(c->ev_stage));
     RC(c->host_stage(c->stage, c->stage_bytes, total));
@@ -313,9 +321,9 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     };
     P.prog.passes = (const DevPass *)put(H.passes.data(), n_pass * sizeof(DevPass), b_pass);
     P.prog.ops = (const DevOp *)put(H.ops.data(), n_ops * sizeof(DevOp), b_ops);
-    P.prog.maps = (const DevMap3 *)put(H.maps.data(), H.maps.size() * sizeof(DevMap3), b_maps);
-    P.map_gate_idx = (const int32_t *)put(H.map_gate_idx.data(), H.map_gate_idx.size() * 4, b_midx);
-    P.raw = (const RawGate *)put(H.raw.data(), H.raw.size() * sizeof(RawGate), b_raw);
+    P.prog.maps = (const DevMap3 *)put(H.maps.data(), n_maps * sizeof(DevMap3), b_maps);
+    P.map_gate_idx = (const int32_t *)put(H.map_gate_idx.data(), n_midx * 4, b_midx);
+    P.raw = (const RawGate *)put(H.raw.data(), n_raw * sizeof(RawGate), b_raw);
     P.param_ptr = (const int32_t *)put(H.param_ptr.data(), H.param_ptr.size() * 4, b_pptr);
     P.param_rot = (const int32_t *)put(H.param_rot.data(), H.param_rot.size() * 4, b_prot);
     P.prog.tabs = (const DevTab *)put(H.tabs.data(), H.tabs.size() * sizeof(DevTab), b_tabs);
@@ -326,6 +334,16 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
         S->enc_dev = (const int32_t *)put(S->enc.data(), eb, align256(eb + teb),
                                           S->tail_enc.data(), teb);
     }
+    P.uargs = UniArgs{};
+    P.uargs.ops = (const UniOp *)put(P.uops.data(), P.uops.size() * sizeof(UniOp), b_uops);
+    P.uruns_dev = (const UniRun *)put(P.uruns.data(), P.uruns.size() * sizeof(UniRun), b_uruns);
+    P.ugates_dev = (const RawGate *)put(P.ugates.data(), P.ugates.size() * sizeof(RawGate),
+                                        b_ugates);
+    P.uargs.segs = (const UniSeg *)put(P.usegs.data(), P.usegs.size() * sizeof(UniSeg), b_usegs);
+    P.uargs.parts = (const UniPart *)put(P.uparts.data(), P.uparts.size() * sizeof(UniPart),
+                                         b_uparts);
+    P.uargs.n_segs = (int32_t)P.usegs.size();
+    P.uargs.n_parts = (int32_t)P.uparts.size();
     P.prog.n_passes = (int32_t)n_pass;
     P.prog.n_ops = (int32_t)n_ops;
     HostPool::run(copies);
@@ -339,6 +357,13 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
 
 int encode_plan(stab_ctx *c, DevPlan &P) {
     const double *th = (const double *)c->thetas.p;
+    if (P.uni) {
+        CK(launch_uni_maps(P.uruns_dev, (int)P.uruns.size(), P.uni_max_run, P.ugates_dev, th,
+                           (UniMap *)c->umaps.p, c->st));
+        c->launches += !P.uruns.empty();
+        P.encoded = true;
+        return STAB_OK;
+    }
     if (P.streams) {
         // resident plans: only the instruction streams are read by kernels;
         // each run's map is composed once and copied into every stream
@@ -421,41 +446,28 @@ void build_streams(const DevPlan &P, const std::vector<StreamSpec> &specs, bool 
     }
 }
 
+void clear_parts(DevPlan &P) {
+    P.uni = P.uni_identity = false;
+    P.cuts.clear();
+    P.uops.clear();
+    P.uruns.clear();
+    P.ugates.clear();
+    P.usegs.clear();
+    P.uparts.clear();
+}
+
 // Forward and backward streams, built concurrently on host threads; with
 // split_frac > 0 (and enough passes) also the split streams cut at that
 // fraction of the passes.  A split gradient plan (grad) needs only the four
 // half streams, not the whole-circuit ones.  Below kThreadedStreamPasses
 // passes the streams are built on the calling thread: handing them to the
 // pool would cost more than the work.
-void make_streams(DevPlan &P, double split_frac = 0.0, bool grad = false, int n_parts = 2,
-                  double first_frac = 0.0, int force_split = -1) {
+void make_streams(DevPlan &P, double split_frac = 0.0, bool grad = false) {
     P.streams = true;
     const int np = (int)P.host.passes.size();
     const bool threads = np >= kThreadedStreamPasses;
-    if (!grad && n_parts >= 3) {
-        // K forward parts of equal pass counts, or (first_frac > 0) a first
-        // part of that fraction of the passes and K - 1 equal parts after it
-        P.sf = P.sb = P.h1 = P.h2 = P.h2b = P.h1b = DevStreamBuf();
-        P.parts.resize((size_t)n_parts);
-        P.cuts.assign((size_t)n_parts + 1, 0);
-        if (first_frac > 0.0) {
-            const int c1 = (int)(np * first_frac);
-            for (int k = 1; k <= n_parts; ++k)
-                P.cuts[k] = c1 + (int)((int64_t)(np - c1) * (k - 1) / (n_parts - 1));
-        } else {
-            for (int k = 0; k <= n_parts; ++k) P.cuts[k] = (int)((int64_t)np * k / n_parts);
-        }
-        P.split = P.cuts[1];
-        std::vector<StreamSpec> specs;
-        for (int k = 0; k < n_parts; ++k)
-            specs.push_back({&P.parts[k], false, P.cuts[k], P.cuts[k + 1]});
-        build_streams(P, specs, threads);
-        return;
-    }
-    P.parts.clear();
-    P.cuts.clear();
+    clear_parts(P);
     P.split = (split_frac > 0.0 && np >= kSplitMinPasses) ? (int)(np * split_frac) : -1;
-    if (P.split >= 0 && force_split > 0 && force_split < np) P.split = force_split;
     // streams that are rebuilt keep their capacity; the others are released
     if (P.split < 0) P.h1 = P.h2 = P.h2b = DevStreamBuf();
     if (!(grad && P.split >= 0)) P.h1b = DevStreamBuf();
@@ -473,34 +485,13 @@ void make_streams(DevPlan &P, double split_frac = 0.0, bool grad = false, int n_
         build_streams(P, {{&P.sf, false, 0, np}, {&P.sb, true, 0, np}}, threads);
         return;
     }
-    // A split plan reads the halves: the generators (n <= 4) and the density
-    // matrix through h1 and h2, <O> through h1 and h2b.  Only n = 5, 6 still
-    // read the whole forward stream (their generators and density matrix are
-    // not split); nothing reads the whole backward stream.
-    P.sb = DevStreamBuf();
-    const bool whole_fwd = P.host_n > 4;
-    if (!whole_fwd) P.sf = DevStreamBuf();
-    std::vector<StreamSpec> specs = {
-        {&P.h1, false, 0, P.split}, {&P.h2, false, P.split, np}, {&P.h2b, true, P.split, np}};
-    if (whole_fwd) specs.push_back({&P.sf, false, 0, np});
-    build_streams(P, specs, threads);
-}
-
-// Gradient streams of a many-part split at the pass boundaries `cuts` (K + 1
-// of them, 0 and P included): part 0 backward over [0, cuts[1]) (walked from
-// its end), part k >= 1 forward over [cuts[k], cuts[k + 1]).
-void make_grad_part_streams(DevPlan &P, const std::vector<int> &cuts) {
-    P.streams = true;
-    const int np = (int)P.host.passes.size();
-    const size_t K = cuts.size() - 1;
-    P.sf = P.sb = P.h1 = P.h2 = P.h2b = P.h1b = DevStreamBuf();
-    P.parts.resize(K);
-    P.cuts = cuts;
-    P.split = cuts[1];
-    std::vector<StreamSpec> specs;
-    for (size_t k = 0; k < K; ++k)
-        specs.push_back({&P.parts[k], k == 0, cuts[k], cuts[k + 1]});
-    build_streams(P, specs, np >= kThreadedStreamPasses);
+    // A split plan (n = 5, 6) reads the whole forward stream (generators,
+    // density matrix) and the halves that <O> meets from, h1 and h2b; nothing
+    // reads the whole backward stream.
+    P.sb = P.h2 = DevStreamBuf();
+    build_streams(P,
+                  {{&P.h1, false, 0, P.split}, {&P.h2b, true, P.split, np}, {&P.sf, false, 0, np}},
+                  threads);
 }
 
 void no_streams(DevPlan &P) {
@@ -508,8 +499,7 @@ void no_streams(DevPlan &P) {
     P.sf = DevStreamBuf();
     P.sb = DevStreamBuf();
     P.h1 = P.h2 = P.h2b = P.h1b = DevStreamBuf();
-    P.parts.clear();
-    P.cuts.clear();
+    clear_parts(P);
     P.split = -1;
 }
 
@@ -617,207 +607,192 @@ void make_tile_group(int n, int n_vec, const std::vector<const DevPass *> &group
     bit_runs(rest, &tg->rest_runs);
 }
 
-// ---------------------------------------------------------------- split resident sweeps
+// ---------------------------------------------------------------- split sweeps of small registers
 //
 // A resident vector walks the circuit's passes one after another on one SM.
-// With the passes cut at `split` (DevPlan h1 = [0, split), h2 = [split, P)):
-//   generators (n <= 4): U Z_k U^dagger = T a_k with a_k = Z_k through h1 and
-//     T the transfer matrix of h2, whose 4^n - 1 nontrivial columns are the
-//     basis strings through h2 -- 4^n - 1 + n independent vectors, one batch
-//     launch, then one product;
-//   <O> = <lambda, r> with r = rho_0 through h1 and lambda = O backward through
-//     h2 -- two vectors at once, then one inner product.
-// Every part runs on its own CTA of the persistent batch kernel, except the
-// columns of T at n = 4 (255 of them, more than the SMs): k_transfer_cols
-// carries them two to a CTA.
+// n <= 4, plans of at least kSplitMinPasses passes: the plan is cut into parts
+// whose maps are carried by their unitaries, composed from segments that run
+// at once (k_unitary.cu); the generators, rho and <O> are read off the parts'
+// unitaries, the gradient off states carried through the segments.
+// n = 5, 6: <O> = <lambda, r> with r = rho_0 through the first half and
+// lambda = O backward through the second -- two vectors at once on two CTAs
+// of the persistent batch kernel, then one inner product.
 
-bool split_gens_ok(const stab_ctx *c) { return c->fwd.split >= 0 && c->n <= 4; }
+int later_parts(const stab_ctx *c) { return (int)c->fwd.uparts.size() - 1; }
 
-// n <= 3: parts of a long plan for the chain of transfer matrices -- as many
-// as the SMs hold one unit each (n generators and rho_0 through the first
-// part, 4^n - 1 columns per further part, two CTAs left for other work),
-// each part at least kChainMinPasses passes; < 3 means the two-part split.
+// Parts of a long plan: two cut at gen_cut of the passes, or three -- at n = 4
+// where the path choice says so (a first part of gen_cut, two equal ones), at
+// n <= 3 from kChainMinPasses passes a part (equal ones).  Where the cuts lie
+// costs nothing: every part's segments run at once.
 constexpr int kChainMinPasses = 32;
-int chain_parts(const stab_ctx *c) {
-    if (c->n > 3) return 2;
-    const int E = 1 << (2 * c->n);
+std::vector<int> part_cuts(const stab_ctx *c) {
     const int np = (int)c->fwd.host.passes.size();
-    const int by_sms = 1 + (c->sms - (c->n + 1) - 2) / (E - 1);
-    const int by_len = np / kChainMinPasses;
-    const int k = std::min(by_sms, by_len);
-    return k >= 3 ? k : 2;
+    if (c->n <= 3 && np >= 3 * kChainMinPasses)
+        return {0, (int)((int64_t)np / 3), (int)((int64_t)np * 2 / 3), np};
+    const int c1 = (int)(np * c->choice.gen_cut);
+    if (c->n == 4 && c->choice.gen_parts == 3 && np >= 3 * kSplitMinPasses)
+        return {0, c1, c1 + (np - c1) / 2, np};
+    return {0, c1, np};
 }
 
-bool chain_mode(const stab_ctx *c) { return !c->fwd.parts.empty(); }
-bool split_expect_ok(const stab_ctx *c) { return c->fwd.split >= 0; }
-
-int split_setup(stab_ctx *c, cudaStream_t s) {
-    if (c->split_smem == 0) {
-        // n = 4: as much shared memory as a k_transfer_cols CTA takes, so a
-        // first-part unit (the critical path) never shares an SM's FP64 pipe
-        // with a CTA of columns running beside it
-        c->split_smem = transfer_cols_ctas(c->n) > 0
-                            ? std::max(batch_smem_bytes(c->n), transfer_cols_smem())
-                            : batch_smem_bytes(c->n);
-        int occ = 0;
-        CK(batch_occupancy(c->split_smem, &occ));
-    }
-    const int E = 1 << (2 * c->n);
-    RC(c->dalloc(c->cnt, 256, s));
-    RC(c->dalloc(c->rmid, (size_t)E * 8, s));
-    RC(c->dalloc(c->lmid, (size_t)E * 8, s));
-    RC(c->dalloc(c->dotbuf, 256 * sizeof(double), s));
-    return STAB_OK;
+// Plans of one gate list in different modes hold the same sequence of units:
+// a P_CLIFF pass, or a maximal stretch of consecutive P_WIRE passes on one
+// wire (a gradient plan only cuts a wire's run into several passes).
+bool unit_start(const HostPlan &P, size_t i) {
+    if (i == 0) return true;
+    const DevPass &p = P.passes[i], &q = P.passes[i - 1];
+    return p.type != P_WIRE || q.type != P_WIRE || p.q != q.q;
 }
 
-// Units of the generators' split sweep (rebuilt when the plan changes):
-// the first part carries Z_0 .. Z_{n-1} and rho_0 into avec, the second part
-// the basis strings into the columns of T.
-int split_units_g(stab_ctx *c) {
-    const int n = c->n, E = 1 << (2 * n);
-    // one transfer matrix per part after the first
-    const int n_mats = chain_mode(c) ? (int)c->fwd.parts.size() - 1 : 1;
-    RC(split_setup(c, c->st));
-    RC(c->dalloc(c->tmat, (size_t)n_mats * E * E * 8, c->st));
-    RC(c->dalloc(c->avec, (size_t)(n + 1) * E * 8, c->st));
-    RC(c->dalloc(c->bterms, (size_t)E * sizeof(DevTerm), c->st));
-    RC(c->dalloc(c->units_g, (size_t)(n_mats * (E - 1) + n + 1) * sizeof(BatchUnit), c->st));
-    const DevStreamBuf &first = chain_mode(c) ? c->fwd.parts[0] : c->fwd.h1;
-    const std::vector<const void *> key = {(const void *)c->plan_gen, first.dev,
-                                           c->fwd.h2.dev, c->tmat.p, c->avec.p, c->bterms.p,
-                                           c->units_g.p, (const void *)(intptr_t)n_mats};
-    if (key == c->key_g) return STAB_OK;
-    std::vector<BatchUnit> U;
-    for (int k = 0; k < n; ++k) {
-        BatchUnit u{};
-        u.stream = first.dev;
-        u.n_chunks = first.n_chunks;
-        u.n = (int8_t)n;
-        u.init = INIT_GENERATOR;
-        u.gen = (int16_t)k;
-        u.out = (double *)c->avec.p + (size_t)k * E;
-        U.push_back(u);
-    }
-    {
-        // rho_0 through the first part, for the density matrix (r = T r_1)
-        BatchUnit u{};
-        u.stream = first.dev;
-        u.n_chunks = first.n_chunks;
-        u.n = (int8_t)n;
-        u.init = INIT_RHO0;
-        u.out = (double *)c->avec.p + (size_t)n * E;
-        U.push_back(u);
-    }
-    // the columns of T: units of the same launch, or (n = 4, where they would
-    // outnumber the SMs) the two-column CTAs of k_transfer_cols
-    const int n_basis = transfer_cols_ctas(n) > 0 ? 1 : E;
-    std::vector<DevTerm> basis((size_t)E);
-    for (int j = 1; j < E; ++j) basis[(size_t)j] = DevTerm{1.0, (uint64_t)j};
-    for (int mtx = 0; mtx < n_mats; ++mtx) {
-        const DevStreamBuf &part = chain_mode(c) ? c->fwd.parts[(size_t)mtx + 1] : c->fwd.h2;
-        for (int j = 1; j < n_basis; ++j) {
-            BatchUnit u{};
-            u.stream = part.dev;
-            u.n_chunks = part.n_chunks;
-            u.n = (int8_t)n;
-            u.init = INIT_TERMS;
-            u.terms = (const DevTerm *)c->bterms.p + j;
-            u.n_terms = 1;
-            u.out = (double *)c->tmat.p + (size_t)mtx * E * E + (size_t)j * E;
-            U.push_back(u);
-        }
-    }
-    // column 0 of every T: the identity string stays itself
-    std::vector<double> col0((size_t)E, 0.0);
-    col0[0] = 1.0;
-    for (int mtx = 0; mtx < n_mats; ++mtx)
-        CK(cudaMemcpyAsync((double *)c->tmat.p + (size_t)mtx * E * E, col0.data(), (size_t)E * 8,
-                           cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(c->bterms.p, basis.data(), basis.size() * sizeof(DevTerm),
-                       cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(c->units_g.p, U.data(), U.size() * sizeof(BatchUnit),
-                       cudaMemcpyHostToDevice, c->st));
-    CK(cudaStreamSynchronize(c->st));   // the host vectors above are temporaries
-    c->n_units_g = (int)U.size();
-    c->key_g = key;
-    return STAB_OK;
+// Segments of a plan with W wire passes.  A segment of W / K passes takes
+// 0.6 us a pass at n = 4 (0.3 below) and a level of the tree over the K
+// segments about 6 us (3), so the sum is least near ten passes a segment; it is
+// flat there (n = 4, 500 passes: 72, 69, 70, 71, 81 us a step at 6, 10, 15, 30,
+// 50; n = 2 and 3 alike).  At n = 4 a segment's eight warps fill an SM's FP64
+// pipe, so more segments than SMs only add levels.
+constexpr int kUniSegPasses = 10;
+int uni_segments(int n, int W, int sms) {
+    return std::max(1, std::min(n == 4 ? sms : 2 * sms, W / kUniSegPasses));
 }
 
-// The generators' split sweep on the context stream: the first-part vectors
-// into avec and the columns of T into tmat (the caller applies T).
-int split_run_g(stab_ctx *c) {
-    RC(split_units_g(c));
-    BatchArgs a{};
-    a.units = (const BatchUnit *)c->units_g.p;
-    a.n_units = c->n_units_g;
-    a.counter = (int32_t *)c->cnt.p;
-    a.status = (int32_t *)c->status.p;
-    CK(cudaMemsetAsync(c->cnt.p, 0, 4, c->st));
-    if (transfer_cols_ctas(c->n) > 0) {
-        // the first-part units and the columns of T (of both later parts in
-        // a three-part chain) at once, on two streams
-        CK(cudaEventRecord(c->ev_fork, c->st));
-        CK(cudaStreamWaitEvent(c->aux2, c->ev_fork, 0));
-        CK(launch_batch(a, c->n_units_g, c->split_smem, c->st));
-        ColArgs ca{};
-        if (chain_mode(c)) {
-            ca.n_parts = (int)c->fwd.parts.size() - 1;
-            if (ca.n_parts > 2) return STAB_E_STATE;
-            for (int k = 0; k < ca.n_parts; ++k) {
-                ca.stream[k] = c->fwd.parts[(size_t)k + 1].dev;
-                ca.n_chunks[k] = c->fwd.parts[(size_t)k + 1].n_chunks;
+// The forward plan as parts [cuts[k], cuts[k + 1]) cut into segments at unit
+// boundaries, each of about the same number of wire passes.
+void make_uni(DevPlan &P, const std::vector<int> &cuts, int sms) {
+    clear_parts(P);
+    P.streams = P.uni = true;
+    P.sf = P.sb = P.h1 = P.h2 = P.h2b = P.h1b = DevStreamBuf();
+    P.cuts = cuts;
+    P.split = cuts[1];
+    const HostPlan &H = P.host;
+    const int np = (int)H.passes.size(), K = (int)cuts.size() - 1;
+    std::vector<int> wires((size_t)np + 1, 0);   // wire passes before pass i
+    for (int i = 0; i < np; ++i)
+        wires[(size_t)i + 1] = wires[(size_t)i] + (H.passes[(size_t)i].type == P_WIRE);
+    const int W = wires[(size_t)np], want = uni_segments(P.host_n, W, sms);
+    P.uops.reserve((size_t)np + H.ops.size());
+    P.uruns.reserve((size_t)W);
+    P.ugates.reserve(H.map_gate_idx.size());
+    P.uni_max_run = 0;
+    int node = 0;
+    for (int k = 0; k < K; ++k) {
+        const int c0 = cuts[(size_t)k], c1 = cuts[(size_t)k + 1];
+        const int w0 = wires[(size_t)c0], wp = wires[(size_t)c1] - w0;
+        const int n_seg = std::max(1, (int)((int64_t)want * wp / std::max(1, W)));
+        UniPart part{};
+        part.seg_first = (int32_t)P.usegs.size();
+        part.node = node;
+        int at = c0;
+        for (int j = 1; j <= n_seg && at < c1; ++j) {
+            int end = c1;
+            if (j < n_seg) {
+                const int target = w0 + (int)((int64_t)wp * j / n_seg);
+                end = at + 1;
+                while (end < c1 && !(wires[(size_t)end] >= target && unit_start(H, (size_t)end)))
+                    ++end;
             }
-        } else {
-            ca.n_parts = 1;
-            ca.stream[0] = c->fwd.h2.dev;
-            ca.n_chunks[0] = c->fwd.h2.n_chunks;
+            UniSeg sg{};
+            sg.op_first = (int32_t)P.uops.size();
+            sg.map_first = (int32_t)P.uruns.size();
+            sg.part = k;
+            sg.index = (int32_t)P.usegs.size() - part.seg_first;
+            int parity = 0;
+            for (int i = at; i < end; ++i) {
+                const DevPass &p = H.passes[(size_t)i];
+                for (int o = 0; o < p.n_ops; ++o) {
+                    const DevOp &op = H.ops[p.first + (uint32_t)o];
+                    UniOp u{};
+                    u.q0 = op.q;
+                    if (p.type == P_CLIFF) {
+                        u.kind = op.kind == K_CX ? UK_CX : UK_CZ;
+                        u.q1 = op.q1;
+                    } else {
+                        u.kind = UK_WIRE;
+                        const DevMap3 &mp = H.maps[(size_t)op.param];
+                        UniRun r{(int32_t)P.ugates.size(), mp.count, parity};
+                        uint32_t perm = kPermIdentity;
+                        bool rotates = false;
+                        for (int g = 0; g < mp.count; ++g) {
+                            const RawGate rg =
+                                H.raw[(size_t)H.map_gate_idx[(size_t)(mp.first + g)]];
+                            parity ^= rg.op == STAB_H;
+                            if (rg.op >= STAB_RX) rotates = true;
+                            else if (!rotates) perm = perm_compose(perm, clifford_perm_code(rg.op));
+                            P.ugates.push_back(rg);
+                        }
+                        r.parity |= parity << 1;
+                        P.uruns.push_back(r);
+                        if (!rotates && perm == kPermIdentity) P.uni_identity = true;
+                        P.uni_max_run = std::max(P.uni_max_run, (int)mp.count);
+                    }
+                    P.uops.push_back(u);
+                }
+            }
+            sg.n_ops = (int32_t)P.uops.size() - sg.op_first;
+            sg.n_maps = (int32_t)P.uruns.size() - sg.map_first;
+            sg.parity = parity;
+            P.usegs.push_back(sg);
+            at = end;
         }
-        ca.tmat = (double *)c->tmat.p;
-        ca.status = (int32_t *)c->status.p;
-        CK(launch_transfer_cols(ca, c->n, c->aux2));
-        CK(cudaEventRecord(c->ev_join, c->aux2));
-        CK(cudaStreamWaitEvent(c->st, c->ev_join, 0));
-        c->launches++;
-    } else {
-        CK(launch_batch(a, c->n_units_g, c->split_smem, c->st));
+        part.n_seg = (int32_t)P.usegs.size() - part.seg_first;
+        int level = part.n_seg, root = node;
+        while (level > 1) {
+            root += level;
+            level = (level + 1) / 2;
+        }
+        part.root = root;
+        node = root + 1;
+        P.uparts.push_back(part);
     }
+    P.uni_nodes = node;
+}
+
+// Device buffers of the segments' maps and unitaries (the arrival counters
+// zeroed; every launch leaves them so).  One node more than the trees hold:
+// the first parts' product of a three-part plan.
+int uni_buffers(stab_ctx *c) {
+    DevPlan &P = c->fwd;
+    const size_t E = (size_t)1 << (2 * c->n), nn = (size_t)P.uni_nodes + 1;
+    RC(c->dalloc(c->umaps, std::max<size_t>(1, P.uruns.size()) * sizeof(UniMap), c->st));
+    RC(c->dalloc(c->unodes, nn * (E * sizeof(double2) + 2 * sizeof(int32_t)), c->st));
+    P.uargs.maps = (const UniMap *)c->umaps.p;
+    P.uargs.nodes = (double2 *)c->unodes.p;
+    P.uargs.node_parity = (int32_t *)(P.uargs.nodes + nn * E);
+    P.uargs.node_count = P.uargs.node_parity + nn;
+    CK(cudaMemsetAsync(P.uargs.node_count, 0, nn * sizeof(int32_t), c->st));
+    return STAB_OK;
+}
+
+// The parts' unitaries on the context stream.
+int uni_run(stab_ctx *c) {
+    CK(launch_uni_segments(c->n, c->fwd.uargs, c->st));
     c->launches++;
     CK(cudaEventRecord(c->ev_tx, c->st));
     c->tx_gen = c->param_gen;
     return STAB_OK;
 }
 
-// Applies the chain of the parts' transfer matrices (chain mode) or the one
-// transfer matrix to n_vec first-part vectors of avec starting at `first`.
-int split_apply(stab_ctx *c, int first, int n_vec, double *out, const DevTerm *terms, int n_terms,
-                double *dot_out, cudaStream_t s) {
-    const size_t E = (size_t)1 << (2 * c->n);
-    const double *in = (const double *)c->avec.p + (size_t)first * E;
-    if (chain_mode(c) && transfer_cols_ctas(c->n) > 0) {
-        // n = 4: one matrix-vector product per part, through a scratch pair
-        // of the calling stream's own (<O> on aux may overlap the generators)
-        DevBuf &scratch = s == c->st ? c->chainbuf : c->chainbuf_e;
-        RC(c->dalloc(scratch, 2 * (size_t)n_vec * E * 8, s));
-        const int n_mats = (int)c->fwd.parts.size() - 1;
-        CK(launch_apply_transfer_chain((const double *)c->tmat.p, n_mats, in, out,
-                                       (double *)scratch.p, n_vec, c->n, terms, n_terms, dot_out,
-                                       s));
-        c->launches += n_mats + (dot_out ? 1 : 0);   // a product per matrix, then the dot
-    } else if (chain_mode(c)) {
-        CK(launch_apply_chain((const double *)c->tmat.p, (int)c->fwd.parts.size() - 1, in, out,
-                              n_vec, c->n, terms, n_terms, dot_out, s));
-        c->launches++;
-    } else {
-        CK(launch_apply_transfer((const double *)c->tmat.p, in, out, n_vec, c->n, s));
-        c->launches++;
-    }
-    return STAB_OK;
+UniRoots uni_roots(const stab_ctx *c) {
+    UniRoots r{};
+    r.nodes = c->fwd.uargs.nodes;
+    r.node_parity = c->fwd.uargs.node_parity;
+    r.n = (int32_t)c->fwd.uparts.size();
+    for (int k = 0; k < r.n; ++k) r.root[k] = c->fwd.uparts[(size_t)k].root;
+    return r;
 }
 
 // Units of the expectation's split sweep on stream s (rebuilt when the plan
 // or the observable's device terms change).
 int split_units_e(stab_ctx *c, cudaStream_t s) {
-    RC(split_setup(c, s));
+    const size_t vb = c->vec_bytes();
+    if (c->split_smem == 0) {
+        c->split_smem = batch_smem_bytes(c->n);
+        int occ = 0;
+        CK(batch_occupancy(c->split_smem, &occ));
+    }
+    RC(c->dalloc(c->cnt, 256, s));
+    RC(c->dalloc(c->rmid, vb, s));
+    RC(c->dalloc(c->lmid, vb, s));
+    RC(c->dalloc(c->dotbuf, 256 * sizeof(double), s));
     RC(c->dalloc(c->units_e, 2 * sizeof(BatchUnit), s));
     const int32_t nt = c->n_obs_terms;
     const std::vector<const void *> key = {(const void *)c->plan_gen, c->fwd.h1.dev,
@@ -976,18 +951,10 @@ void reset_graphs(stab_ctx *c) {
     c->plan_gen++;
 }
 
-// Plans of one gate list in different modes hold the same sequence of units:
-// a P_CLIFF pass, or a maximal stretch of consecutive P_WIRE passes on one
-// wire (a gradient plan only cuts a wire's run into several passes).  Returns
-// the pass of plan B that starts the unit starting at pass k of plan A, or -1
+// The pass of plan B that starts the unit starting at pass k of plan A, or -1
 // when pass k starts no unit or the two plans' unit sequences differ (a run
 // that is the identity and holds no rotation makes no pass in some modes).
-bool unit_start(const HostPlan &P, size_t i) {
-    if (i == 0) return true;
-    const DevPass &p = P.passes[i], &q = P.passes[i - 1];
-    return p.type != P_WIRE || q.type != P_WIRE || p.q != q.q;
-}
-
+// (stab_selftest_align; the gradient's uni_identity is the same condition.)
 int aligned_pass(const HostPlan &A, int k, const HostPlan &B) {
     if (k <= 0 || k >= (int)A.passes.size() || !unit_start(A, (size_t)k)) return -1;
     // the units of both plans, as (type, wire), in order; the first pass of each in B
@@ -1008,67 +975,48 @@ int aligned_pass(const HostPlan &A, int k, const HostPlan &B) {
     return start_b[(size_t)unit_k];
 }
 
+// The gradient of a plan with segment unitaries: only the slot -> rotations
+// table (rotations by their place in the run-ordered gate array).  Circuits
+// with an identity run without rotations have no such run in their gradient
+// plan; they keep the two-part sweep (stab_grad_parts tells the two apart).
+bool uni_grad_ok(const stab_ctx *c) {
+    return c->use_resident() && c->use_resident_adjoint() && c->fwd.uni && !c->fwd.uni_identity;
+}
+
+int ensure_uni_grad(stab_ctx *c) {
+    if (c->grad.built) return STAB_OK;
+    HostPlan &H = c->grad.host;
+    const std::vector<RawGate> &g = c->fwd.ugates;
+    H = HostPlan();
+    H.param_ptr.assign((size_t)c->n_params + 1, 0);
+    for (const RawGate &r : g)
+        if (r.op >= STAB_RX) H.param_ptr[(size_t)r.param + 1]++;
+    for (int64_t j = 0; j < c->n_params; ++j) H.param_ptr[(size_t)j + 1] += H.param_ptr[(size_t)j];
+    H.param_rot.resize((size_t)H.param_ptr[(size_t)c->n_params]);
+    std::vector<int32_t> at(H.param_ptr.begin(), H.param_ptr.end() - 1);
+    for (size_t k = 0; k < g.size(); ++k)
+        if (g[k].op >= STAB_RX) H.param_rot[(size_t)at[(size_t)g[k].param]++] = (int32_t)k;
+    no_streams(c->grad);
+    RC(upload_plan(c, c->grad));
+    c->grad.encoded = true;
+    CK(cudaEventRecord(c->ev_ready, c->st));
+    return STAB_OK;
+}
+
 int ensure_grad_plan(stab_ctx *c) {
     if (!c->grad.built) {
         build_plan(c->n, c->gates.data(), (int64_t)c->gates.size(), c->n_params, PLAN_GRAD,
                    &c->grad.host, !c->use_resident_adjoint());
         // resident adjoint: split at half the passes (the AUTO kernel; the
-        // RESIDENT choice keeps the single-CTA forward-then-reverse sweep) --
-        // or, at n = 4 with the generators' split sweep, at the gate where the
-        // generators' first part ends, so the pair at the cut comes from that
-        // sweep (see stab_grad_async)
-        c->grad_aligned = false;
-        c->grad_cuts.clear();
+        // RESIDENT choice keeps the single-CTA forward-then-reverse sweep)
         if (c->use_resident_adjoint()) {
-            // the generators' part boundaries, as passes of the gradient plan
-            const int npg = (int)c->grad.host.passes.size();
-            if (c->kernel == STAB_KERNEL_AUTO && c->use_resident() && split_gens_ok(c) &&
-                npg >= kSplitMinPasses) {
-                std::vector<int> fc = chain_mode(c)
-                                          ? c->fwd.cuts
-                                          : std::vector<int>{0, c->fwd.split,
-                                                             (int)c->fwd.host.passes.size()};
-                std::vector<int> gc = {0};
-                for (size_t k = 1; k + 1 < fc.size(); ++k) {
-                    const int g = aligned_pass(c->fwd.host, fc[k], c->grad.host);
-                    if (g <= gc.back()) break;
-                    gc.push_back(g);
-                }
-                if (gc.size() + 1 == fc.size() && gc.back() < npg) {
-                    gc.push_back(npg);
-                    c->grad_cuts = gc;
-                }
-            }
-            if (!c->grad_cuts.empty()) make_grad_part_streams(c->grad, c->grad_cuts);
-            else make_streams(c->grad, c->kernel == STAB_KERNEL_AUTO ? 0.5 : 0.0, true);
-            c->grad_aligned = !c->grad_cuts.empty();
+            make_streams(c->grad, c->kernel == STAB_KERNEL_AUTO ? 0.5 : 0.0, true);
         } else {
             no_streams(c->grad);
         }
         c->g_grad.reset();
         c->plan_gen++;
         RC(upload_plan(c, c->grad));
-        if (c->grad_aligned) {
-            // the parts' descriptors: part 0 backward from the pair at the first
-            // cut, part k >= 1 forward from the pair at cut k
-            const int K = (int)c->grad_cuts.size() - 1;
-            const size_t E = (size_t)1 << (2 * c->n);
-            RC(c->dalloc(c->gpairs, (size_t)(K - 1) * 2 * E * sizeof(double), c->st));
-            RC(c->dalloc(c->gparts, (size_t)K * sizeof(AdjPart), c->st));
-            const double *pairs = (const double *)c->gpairs.p;
-            c->gparts_host.assign((size_t)K, AdjPart{});
-            for (int k = 0; k < K; ++k) {
-                AdjPart &q = c->gparts_host[(size_t)k];
-                const int at = k == 0 ? 1 : k;   // the pair this part starts from
-                q.stream = c->grad.parts[(size_t)k].dev;
-                q.n_chunks = c->grad.parts[(size_t)k].n_chunks;
-                q.forward = k > 0;
-                q.lam = pairs + (size_t)(at - 1) * 2 * E;
-                q.rho = q.lam + E;
-            }
-            CK(cudaMemcpyAsync(c->gparts.p, c->gparts_host.data(), (size_t)K * sizeof(AdjPart),
-                               cudaMemcpyHostToDevice, c->st));
-        }
     }
     if (!c->grad.encoded) RC(encode_plan(c, c->grad));
     CK(cudaEventRecord(c->ev_ready, c->st));
@@ -1078,9 +1026,6 @@ int ensure_grad_plan(stab_ctx *c) {
 }  // namespace
 
 cudaStream_t stab::ctx_stream(stab_ctx *c) { return c ? c->st : nullptr; }
-void stab::ctx_forget_sweep(stab_ctx *c) {
-    if (c) c->tx_gen = -1;
-}
 
 extern "C" {
 
@@ -1426,9 +1371,8 @@ int stab_destroy(stab_ctx *c) {
     DevBuf *bufs[] = {&c->fwd.buf, &c->grad.buf, &c->thetas, &c->gens, &c->gens_tmp, &c->lam,
                       &c->rho, &c->tmp, &c->tmp2, &c->terms, &c->scal, &c->grad_rot,
                       &c->partials, &c->grads, &c->status, &c->gbuf, &c->lam2, &c->tmp3,
-                      &c->dotbuf, &c->tmat, &c->avec, &c->rmid, &c->lmid, &c->bterms,
-                      &c->units_g, &c->units_e, &c->cnt, &c->gmid, &c->chainbuf,
-                      &c->chainbuf_e, &c->odense, &c->gpairs, &c->gparts};
+                      &c->dotbuf, &c->umaps, &c->unodes, &c->ustates, &c->udots, &c->rmid,
+                      &c->lmid, &c->units_e, &c->cnt, &c->gmid};
     for (DevBuf *b : bufs) c->dfree(*b, c->st);
     if (c->st) cudaStreamSynchronize(c->st);
     if (c->stage) cudaFreeHost(c->stage);
@@ -1464,30 +1408,19 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     reset_graphs(c);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
-        // split streams for the resident sweeps: generators through the
-        // transfer matrix of the second part (n <= 4), expectations meeting in
-        // the middle.  The cut balances the two parts' pass times; at n = 4,
-        // where k_transfer_cols carries two columns per CTA at a different
-        // pass rate than a first-part unit alone on its SM, the path tuner
-        // times candidate cuts (n <= 3: every unit has an SM to itself, half).
-        // At n = 4 the tuner may also cut the plan in three (a first part of
-        // gen_cut of the passes, then two equal parts whose transfer matrices
-        // share the SMs four columns to an SM).
+        // AUTO, long plans: at n <= 4 the parts' unitaries; at n = 5, 6 the two
+        // halves of <O>
         const bool split = c->kernel == STAB_KERNEL_AUTO && c->fuse;
-        const double cut = c->choice.gen_cut;
-        const int np = (int)c->fwd.host.passes.size();
-        int parts = split ? chain_parts(c) : 2;
-        double first = 0.0;
-        if (split && transfer_cols_ctas(c->n) > 0 && c->choice.gen_parts == 3 &&
-            np >= 3 * kSplitMinPasses) {
-            parts = 3;
-            first = cut;
+        if (split && c->n <= kUniMaxQubits && (int)c->fwd.host.passes.size() >= kSplitMinPasses) {
+            make_uni(c->fwd, part_cuts(c), c->sms);
+        } else {
+            make_streams(c->fwd, split ? c->choice.gen_cut : 0.0);
         }
-        make_streams(c->fwd, split ? cut : 0.0, false, parts, first);
     }
     else no_streams(c->fwd);
     RC(upload_thetas_host(c, thetas));
     RC(upload_plan(c, c->fwd));
+    if (c->fwd.uni) RC(uni_buffers(c));
     RC(encode_plan(c, c->fwd));
     CK(cudaEventRecord(c->ev_ready, c->st));
     c->param_gen++;
@@ -1524,11 +1457,24 @@ int stab_run_generators(stab_ctx *c) {
     const int n = c->n;
     const size_t bytes = c->vec_bytes() * (size_t)n;
     RC(c->dalloc(c->gens, bytes, c->st));
-    if (c->use_resident() && split_gens_ok(c)) {
-        // the split sweep for these angles may already have run (for <O> or
-        // the density matrix); then only the products with T remain
-        if (c->tx_gen != c->param_gen) RC(split_run_g(c));
-        RC(split_apply(c, 0, n, (double *)c->gens.p, nullptr, 0, nullptr, c->st));
+    if (c->use_resident() && c->fwd.uni) {
+        // the parts' unitaries for these angles may already be there (from
+        // <O>, a gradient or the density matrix); then only the read-out is left
+        if (c->tx_gen != c->param_gen) RC(uni_run(c));
+        UniRoots r = uni_roots(c);
+        if (n == 4 && r.n == 3) {
+            // the read-out multiplies two unitaries; a third joins the first here
+            const UniArgs &u = c->fwd.uargs;
+            const int32_t spare = c->fwd.uni_nodes;
+            CK(launch_uni_merge(n, r, u.nodes + (size_t)spare * ((size_t)1 << (2 * n)),
+                                u.node_parity + spare, c->st));
+            c->launches++;
+            r.n = 2;
+            r.root[0] = spare;
+            r.root[1] = r.root[2];
+        }
+        CK(launch_uni_images(n, r, (double *)c->gens.p, c->st));
+        c->launches++;
         c->gens_cur = (double *)c->gens.p;
     } else if (c->use_resident()) {
         StreamArgs a{};
@@ -1606,15 +1552,14 @@ int stab_expect_async(stab_ctx *c, double *out_dev) {
     cudaStream_t s = c->aux;
     CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
     const int32_t nt = c->n_obs_terms;
-    if (c->use_resident() && chain_mode(c)) {
-        // <O> = sum_P o_P r_P with r = T_K ... T_2 r_1 (Schroedinger picture;
-        // the orthogonal maps make it equal to the x-free sum of U^dagger O U):
-        // the generators' launch made for these angles carries rho_0 and the
-        // parts' transfer matrices; else it runs here first
-        if (c->tx_gen != c->param_gen) RC(split_run_g(c));
+    if (c->use_resident() && c->fwd.uni) {
+        // <O> = <psi|O|psi>, psi = U |0> through the parts' unitaries
+        if (c->tx_gen != c->param_gen) RC(uni_run(c));
         CK(cudaStreamWaitEvent(s, c->ev_tx, 0));
-        RC(split_apply(c, c->n, 1, nullptr, (const DevTerm *)c->terms.p, nt, out_dev, s));
-    } else if (c->use_resident() && split_expect_ok(c)) {
+        CK(launch_uni_states(c->n, uni_roots(c), (const DevTerm *)c->terms.p, nt, out_dev, nullptr,
+                             nullptr, nullptr, s));
+        c->launches++;
+    } else if (c->use_resident() && c->fwd.split >= 0) {
         RC(split_units_e(c, s));
         BatchArgs a{};
         a.units = (const BatchUnit *)c->units_e.p;
@@ -1713,11 +1658,40 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
     if (!c->loaded || !c->obs_loaded) return STAB_E_STATE;
     if (c->n_params > 0 && !grads_dev) return STAB_E_INVAL;
     CK(cudaSetDevice(c->device));
-    RC(ensure_grad_plan(c));
+    c->grad_uni = uni_grad_ok(c);
+    RC(c->grad_uni ? ensure_uni_grad(c) : ensure_grad_plan(c));
     cudaStream_t s = c->aux;
     CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
     const int32_t nt = c->n_obs_terms;
     const int n = c->n;
+    if (c->grad_uni) {
+        // the states at the parts' boundaries, then every segment at once
+        const DevPlan &P = c->fwd;
+        if (c->tx_gen != c->param_gen) RC(uni_run(c));
+        CK(cudaStreamWaitEvent(s, c->ev_tx, 0));
+        const size_t D = (size_t)1 << n, slots = P.uparts.size() + 1;
+        const size_t n_runs = P.uruns.size(), n_gates = P.ugates.size();
+        RC(c->dalloc(c->scal, 64 * sizeof(double), s));
+        RC(c->dalloc(c->ustates, 2 * slots * D * sizeof(double2), s));
+        RC(c->dalloc(c->udots, std::max<size_t>(1, n_runs) * 3 * D * sizeof(double), s));
+        RC(c->dalloc(c->grad_rot, std::max<size_t>(1, n_gates) * sizeof(double), s));
+        double2 *psi = (double2 *)c->ustates.p, *phi = psi + slots * D;
+        CK(launch_uni_states(n, uni_roots(c), (const DevTerm *)c->terms.p, nt,
+                             expect_dev ? expect_dev : (double *)c->scal.p + 1, psi, phi, nullptr,
+                             s));
+        c->launches++;
+        if (c->n_params > 0) {
+            CK(launch_uni_grad(n, P.uargs, psi, phi, (double *)c->udots.p, P.uruns_dev,
+                               (int)n_runs, P.uni_max_run, P.ugates_dev,
+                               (const double *)c->thetas.p, (double *)c->grad_rot.p, s));
+            CK(launch_gather_grads((const double *)c->grad_rot.p, c->grad.param_ptr,
+                                   c->grad.param_rot, (int)c->n_params, grads_dev, s));
+            c->launches += 2 + (n_runs > 0);
+        }
+        CK(cudaEventRecord(c->ev_aux, s));
+        CK(cudaStreamWaitEvent(c->st, c->ev_aux, 0));
+        return STAB_OK;
+    }
     const int n_rot = c->grad.host.n_rot;
     RC(c->dalloc(c->scal, 64 * sizeof(double), s));
     RC(c->dalloc(c->grad_rot, (size_t)(n_rot ? n_rot : 1) * sizeof(double), s));
@@ -1735,59 +1709,7 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
             partials = (double *)c->partials.p;
         }
     }
-    if (c->use_resident_adjoint() && c->grad_aligned) {
-        // the gradient plan's parts end where the generators' split sweep cuts
-        // the circuit, so the pair at every cut comes from that sweep: rho_0
-        // through the first part is its first-part vector, rho at a later cut
-        // the next parts' transfer matrices applied to it, and lambda at a cut
-        // is O carried backward through the parts after it, T_k^T (the maps
-        // being orthogonal) from the last part to the first; the sweep is
-        // reused when it was made for these angles.  Then every part is swept
-        // at once: the first backward from its end, the others forward.
-        if (c->tx_gen != c->param_gen) RC(split_run_g(c));
-        CK(cudaStreamWaitEvent(s, c->ev_tx, 0));
-        const int K = (int)c->grad_cuts.size() - 1;
-        const size_t E = (size_t)1 << (2 * n), EE = E * E;
-        RC(c->dalloc(c->odense, E * sizeof(double), s));
-        double *o = (double *)c->odense.p;
-        CK(launch_fill(o, n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, nt, s));
-        const double *T = (const double *)c->tmat.p;
-        const double *r1 = (const double *)c->avec.p + (size_t)n * E;
-        double *pairs = (double *)c->gpairs.p;
-        auto lam = [&](int k) { return pairs + (size_t)(k - 1) * 2 * E; };
-        if (n == 4) {
-            CK(cudaMemcpyAsync(lam(1) + E, r1, E * sizeof(double), cudaMemcpyDeviceToDevice, s));
-            for (int k = 1; k + 1 <= K - 1; ++k)
-                CK(launch_apply_transfer(T + (size_t)(k - 1) * EE, lam(k) + E, lam(k + 1) + E, 1,
-                                         n, s));
-            for (int k = K - 1; k >= 1; --k)
-                CK(launch_apply_transfer_t(T + (size_t)(k - 1) * EE, k == K - 1 ? o : lam(k + 1),
-                                           lam(k), n, s));
-            c->launches += 1 + 2 * (K - 1) - 1;
-        } else {
-            CK(launch_adjoint_pairs(T, K, n, r1, o, pairs, s));
-            c->launches += 2;
-        }
-        AdjointSplitArgs a{};
-        a.phase = 1;
-        a.parts = (const AdjPart *)c->gparts.p;
-        a.n_parts = K;
-        a.grad_rot = (double *)c->grad_rot.p;
-        a.partials = partials;
-        a.expect_out = e_out;
-        a.status = (int32_t *)c->status.p;
-        CK(launch_adjoint_split(n, a, s));
-        c->launches++;
-        if (partials) {
-            CK(launch_reduce_partials(partials, n_rot, part_threads, (double *)c->grad_rot.p, s));
-            c->launches++;
-        }
-        if (c->n_params > 0) {
-            CK(launch_gather_grads((const double *)c->grad_rot.p, c->grad.param_ptr,
-                                   c->grad.param_rot, (int)c->n_params, grads_dev, s));
-            c->launches++;
-        }
-    } else if (c->use_resident_adjoint() && c->grad.split >= 0) {
+    if (c->use_resident_adjoint() && c->grad.split >= 0) {
         // meet in the middle: rho_0 forward through the first part and O
         // backward through the second, then the pair at the cut backward
         // through the first part and forward through the second
@@ -2047,12 +1969,10 @@ int stab_density_matrix(stab_ctx *c, double *out, int out_is_device) {
     const size_t vb = c->vec_bytes();
     RC(c->dalloc(c->rho, vb, c->st));
     double *r = (double *)c->rho.p;
-    if (c->use_resident() && split_gens_ok(c)) {
-        // r = T r_1: rho_0 through the first part, then the later parts'
-        // transfer matrices (built alongside, as for the generators; reused
-        // when the sweep for these angles has run)
-        if (c->tx_gen != c->param_gen) RC(split_run_g(c));
-        RC(split_apply(c, n, 1, r, nullptr, 0, nullptr, c->st));
+    if (c->use_resident() && c->fwd.uni) {
+        if (c->tx_gen != c->param_gen) RC(uni_run(c));
+        CK(launch_uni_states(n, uni_roots(c), nullptr, 0, nullptr, nullptr, nullptr, r, c->st));
+        c->launches++;
     } else if (c->use_resident()) {
         StreamArgs a{};
         a.stream = c->fwd.sf.dev;
@@ -2107,9 +2027,8 @@ int stab_split_info(stab_ctx *c, int64_t *cut, int32_t *gen_units, int32_t *expe
     const bool on = c->loaded && c->use_resident() && c->fwd.split >= 0;
     const int E = 1 << (2 * c->n);
     if (cut) *cut = on ? c->fwd.split : -1;
-    const int n_mats = chain_mode(c) ? (int)c->fwd.parts.size() - 1 : 1;
-    if (gen_units) *gen_units = on && split_gens_ok(c) ? c->n + 1 + n_mats * (E - 1) : 0;
-    if (expect_units) *expect_units = on && !chain_mode(c) && split_expect_ok(c) ? 2 : 0;
+    if (gen_units) *gen_units = on && c->fwd.uni ? c->n + 1 + later_parts(c) * (E - 1) : 0;
+    if (expect_units) *expect_units = on && !c->fwd.uni ? 2 : 0;
     return STAB_OK;
 }
 
@@ -2117,7 +2036,7 @@ int64_t stab_launch_count(stab_ctx *c) { return c ? c->launches : 0; }
 
 int stab_grad_parts(stab_ctx *c, int32_t *parts) {
     if (!c || !parts) return STAB_E_INVAL;
-    *parts = !c->grad.built ? 0 : c->grad_aligned ? (int32_t)c->grad_cuts.size() - 1 : 1;
+    *parts = !c->grad.built ? 0 : c->grad_uni ? (int32_t)c->fwd.uparts.size() : 1;
     return STAB_OK;
 }
 

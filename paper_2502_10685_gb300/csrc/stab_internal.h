@@ -138,6 +138,54 @@ static_assert(sizeof(Rec) == 32, "Rec layout");
 // records as usual.
 constexpr uint16_t kPullRepeat = 1;
 
+// ---------------------------------------------------------------- segment unitaries
+//
+// n <= 4, long plans: the parts of the plan are carried by their 2^n x 2^n
+// unitaries, composed from segments (see k_unitary.cu), each an op list:
+constexpr int kUniMaxQubits = 4;
+
+enum UniKind : uint8_t { UK_WIRE = 0, UK_CX = 1, UK_CZ = 2 };
+
+struct UniOp {           // 4 bytes; the k-th UK_WIRE op of the plan uses map k
+    uint8_t kind;        // UniKind
+    uint8_t q0, q1;      // wire; control / first qubit, target / second qubit
+    uint8_t pad;
+};
+static_assert(sizeof(UniOp) == 4, "UniOp layout");
+
+// A wire run: gates [first, first + count) of the run-ordered gate array.
+// Matrices are kept times sqrt(2)^(H gates so far in the segment mod 2), H as
+// [[1, 1], [1, -1]], so Clifford circuits stay exact.
+struct UniRun {          // 12 bytes
+    int32_t first, count;
+    int32_t parity;      // H gates of the segment mod 2: bit 0 before the run, bit 1 after it
+};
+
+struct UniMap {          // 64 bytes, set on device: per row bit b, the factors of the
+    double f[8];         // entry itself and of its partner: (m00, m01), (m11, m10), complex
+};
+
+struct UniSeg {          // 32 bytes
+    int32_t op_first, n_ops;
+    int32_t map_first, n_maps;
+    int32_t part;        // part of the plan
+    int32_t index;       // segment within its part
+    int32_t parity;      // H gates of the segment mod 2 (U is kept times sqrt(2)^parity)
+    int32_t pad;
+};
+static_assert(sizeof(UniSeg) == 32, "UniSeg layout");
+
+// The segments' unitaries of a part are multiplied in a binary tree: level 0
+// holds the segments in order, node i of level l + 1 is node 2i + 1 times node
+// 2i of level l (or node 2i alone); all levels of a part are contiguous, level
+// after level.
+struct UniPart {         // 16 bytes
+    int32_t seg_first, n_seg;
+    int32_t node;        // first node (level 0)
+    int32_t root;        // the part's unitary
+};
+constexpr int kUniMaxLevels = 16;
+
 struct DevTerm {         // deduplicated observable term: index in the device layout
     double coeff;
     uint64_t idx;

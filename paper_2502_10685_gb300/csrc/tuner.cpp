@@ -4,12 +4,8 @@
 //
 // The choices are the ones a fixed threshold would otherwise make: whether
 // n = 5, 6 vectors stay resident in shared memory (one CTA each) or stream
-// through HBM, for <O> and for gradients; where the generators' split sweep
-// cuts the plan at n = 4 (the first part's vectors and the second part's
-// transfer-matrix columns run on different kernels at different speeds, and
-// the cut that makes them end together depends on both); and up to which
-// launch size consecutive wire passes of a streamed plan share one
-// tile-fused launch.  Each is timed on a probe circuit, candidate against
+// through HBM, for <O> and for gradients; and up to which launch size
+// consecutive wire passes of a streamed plan share one tile-fused launch.  Each is timed on a probe circuit, candidate against
 // candidate, through the public entry points of contexts created with the
 // candidate's choice.
 #include <cuda_runtime.h>
@@ -233,12 +229,7 @@ int time_op(int device, const stab_opts *like, const Probe &P, const stab_path_c
         rc = STAB_E_CUDA;
     }
     auto call = [&]() {
-        if (op == PR_GENS) {
-            // every timed call runs the whole sweep (a repeated call for the
-            // same angles would otherwise reuse the previous one)
-            ctx_forget_sweep(c);
-            return stab_run_generators(c);
-        }
+        if (op == PR_GENS) return stab_run_generators(c);
         if (op == PR_EXPECT) return stab_expect_async(c, dev);
         return stab_grad_async(c, dev, dev + 8);
     };
@@ -283,40 +274,9 @@ int measure(int device, const stab_opts *like, int n, stab_path_choice *out) {
     d.tuned = 1;
     Probe P;
     P.n = n;
-    if (n == 4) {
-        // long enough (about 7,500 passes) that a pass's cost, not the
-        // launch and staging overhead, decides between the cuts
-        P.m = 24000;
-        probe_circuit(n, P.m, &P.g, &P.th);
-        const double def = d.gen_cut;
-        float t_def = 0.0f, best = 1e30f;
-        double best_cut = def;
-        int best_parts = 2;
-        struct Cand {
-            int parts;
-            double cut;
-        };
-        const Cand cands[] = {{2, 0.50}, {2, 0.53}, {2, 0.56}, {2, 0.59}, {2, 0.62},
-                              {3, 0.43}, {3, 0.45}, {3, 0.47}, {3, 0.49}, {3, 0.51}};
-        for (const Cand &k : cands) {
-            stab_path_choice c = d;
-            c.gen_cut = k.cut;
-            c.gen_parts = k.parts;
-            float t = 0.0f;
-            int rc = time_op(device, like, P, c, PR_GENS, &t);
-            if (rc != STAB_OK) return rc;
-            if (k.parts == 2 && k.cut == def) t_def = t;
-            if (t < best) {
-                best = t;
-                best_cut = k.cut;
-                best_parts = k.parts;
-            }
-        }
-        if (clearly_faster(best, t_def)) {
-            d.gen_cut = best_cut;
-            d.gen_parts = best_parts;
-        }
-    } else if (n == 5 || n == 6) {
+    // n <= 4: the parts' maps come from their unitaries, whose segments run at
+    // once wherever the parts are cut, so there is nothing to choose
+    if (n == 5 || n == 6) {
         P.m = 2000;
         probe_circuit(n, P.m, &P.g, &P.th);
         P.obs = probe_observable(n);
