@@ -564,6 +564,12 @@ int stab_selftest_plan(int n, const stab_gate *gates, int64_t m, int64_t n_param
 int stab_selftest_align(int n, const stab_gate *gates, int64_t m, int64_t n_params,
                         int64_t *aligned);
 
+/* Host-only check of the streamed plans' Clifford gathers: the source index
+ * and sign of up to 2^16 strings through the gates as one run, forward and
+ * inverse, against the gates applied one at a time.  STAB_OK, or STAB_E_STATE
+ * when they differ.  Errors: as stab_load_circuit; a rotation is STAB_E_RANGE. */
+int stab_selftest_pull(int n, const stab_gate *gates, int64_t m);
+
 /* ---------------------------------------------------------------- path tuner */
 /* How a context of n qubits with the STAB_KERNEL_AUTO kernel runs, for one GPU
  * model.  The paper has no counterpart (its CPU pipeline has one form).  The
@@ -624,8 +630,8 @@ int stab_path_load(const char *path);
  * against one launch per pass, for one vector (<O>) and for n vectors (the
  * generators), giving tile_limit = the largest of those launch sizes where
  * tiles won (0 when neither); n <= 4 (the parts' segments run at once wherever
- * they are cut) and n >= 10 have nothing measured and keep the defaults (marked tuned).  Each candidate takes the best of five
- * timed calls; a candidate replaces the default only when it is more than 2 %
+ * they are cut) and n >= 10 have nothing measured and keep the defaults
+ * (marked tuned).  Each candidate takes the best of five timed calls; a candidate replaces the default only when it is more than 2 %
  * faster, so timing noise does not flip a choice.  Takes up to about a tenth
  * of a second.
  * Errors: STAB_E_RANGE (n), STAB_E_CUDA, STAB_E_NOMEM. */

@@ -14,6 +14,7 @@
 
 #include "device_ops.cuh"
 #include "launch.h"
+#include "pull.cuh"
 
 namespace stab {
 
@@ -27,13 +28,6 @@ __device__ __forceinline__ double pair_dot(int axis, double lx, double ly, doubl
     if (axis == AX_X) return fma(lz, ry, -ly * rz);
     if (axis == AX_Y) return fma(lx, rz, -lz * rx);
     return fma(ly, rx, -lx * ry);
-}
-
-__device__ __forceinline__ uint64_t deposit_runs(uint64_t v, const BitRuns &r) {
-    uint64_t out = 0;
-    for (int k = 0; k < r.n; ++k)
-        out |= ((v >> r.src[k]) & ((1ull << r.len[k]) - 1ull)) << r.dst[k];
-    return out;
 }
 
 __device__ __forceinline__ void add_slot(double (&part)[R], int slot, double d) {
@@ -203,21 +197,29 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_tile(const double *src,
     const uint64_t E = 1ull << (2 * n);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t tiles = 1ull << tg.rest_bits;
+    LanePull L{};
+    if (tg.pull) L = load_pull(tg.pull, n);
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const uint64_t base = deposit_runs(t, tg.rest_runs);
-        if (tg.pull_n == 0) {
+        if (tg.pull == nullptr) {
             for (uint32_t e = threadIdx.x; e < T; e += blockDim.x) {
                 tl[e] = src[base + offs[e]];
                 tr[e] = src[E + base + offs[e]];
             }
         } else {
             // the Clifford gather that precedes the group, on both vectors
-            for (uint32_t e = threadIdx.x; e < T; e += blockDim.x) {
-                uint32_t neg = 0;
-                const uint64_t j = pull_pass(base + offs[e], n, ops + tg.pull_first, tg.pull_n,
-                                             tg.pull_inverse, neg);
-                tl[e] = flip(src[j], neg);
-                tr[e] = flip(src[E + j], neg);
+            const BasePull B = base_pull(L, (uint32_t)base);
+            for (uint32_t e0 = 0; e0 < T; e0 += blockDim.x) {
+                const uint32_t e = e0 + threadIdx.x, off = offs[e < T ? e : 0];
+                uint32_t oj = 0, oq = 0, neg;
+                for (int r = 0; r < tg.tile_runs.n; ++r)
+                    for (int b = 0; b < tg.tile_runs.len[r]; ++b)
+                        off_bit(L, tg.tile_runs.dst[r] + b, off, oj, oq);
+                const uint32_t j = pull_entry(L, B, n, off, oj, oq, neg);
+                if (e < T) {
+                    tl[e] = flip(src[j], neg);
+                    tr[e] = flip(src[E + j], neg);
+                }
             }
         }
         __syncthreads();

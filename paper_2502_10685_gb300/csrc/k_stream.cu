@@ -9,6 +9,7 @@
 
 #include "device_ops.cuh"
 #include "launch.h"
+#include "pull.cuh"
 #include "tma.cuh"
 
 namespace stab {
@@ -226,123 +227,119 @@ __global__ void __launch_bounds__(kThreads) k_stream_cliff(const double *__restr
     }
 }
 
-// Exponent c (mod 4) of P(a) P(b) = i^c P(a xor b) for Hermitian Pauli strings
-// given by x / z masks: per qubit, with a = Y: z_b - x_b; a = X: z_b (2 x_b - 1);
-// a = Z: x_b (1 - 2 z_b) (the phase function of Aaronson and Gottesman's
-// tableau algorithm), summed with population counts.
-__device__ __forceinline__ uint32_t tab_mul_phase(uint32_t ax, uint32_t az, uint32_t bx,
-                                                  uint32_t bz) {
-    const uint32_t A = ax & az, B = ax & ~az, C = ~ax & az;
-    const uint32_t plus = (A & bz & ~bx) | (B & bz & bx) | (C & bx & ~bz);
-    const uint32_t minus = (A & bx & ~bz) | (B & bz & ~bx) | (C & bx & bz);
-    return (uint32_t)(__popc(plus) - __popc(minus)) & 3u;
-}
-
-// A Clifford run as one signed gather: dst[i] = sign * src[j] with
-// V P_i V^dagger = sign P_j for the map V whose tableau is given (the run's
-// inverse for a forward application).  V P(x, z) V^dagger is i^{|x & z|} times
-// the product of the generator images (X_q images for x, Z_q images for z, q
-// ascending, Y = i X Z), each factor adding its phase and sign.
-__global__ void __launch_bounds__(kThreads) k_stream_tab(const double *__restrict__ src,
-                                                         double *__restrict__ dst, int n,
-                                                         int n_vec, const DevTab *tab) {
-    // The tableau regrouped by chunks of 4 qubits: entry (c, t) is the ordered
-    // product of the generator images that subset t of chunk c selects (bit j:
-    // X of qubit 4c + j, bit 4 + j: its Z), built by every block in shared
-    // memory; an index then takes ceil(n / 4) lookups and string products
-    // instead of one product per set bit.
-    constexpr int kChunkQ = 4;
-    __shared__ uint32_t cx[3 * 256], cz[3 * 256], ce[3 * 256];
-    const int n_ch = (n + kChunkQ - 1) / kChunkQ;
-    for (int k = threadIdx.x; k < n_ch * 256; k += blockDim.x) {
-        const int c = k >> 8, t = k & 255;
-        uint32_t rx = 0, rz = 0, e = 0;
-        for (int j = 0; j < kChunkQ; ++j) {
-            const int q = kChunkQ * c + j;
-            if (q >= n) break;
-            for (int part = 0; part < 2; ++part) {   // X_q, then Z_q
-                if (!((t >> (part * kChunkQ + j)) & 1)) continue;
-                const int g = part ? n + q : q;
-                e += tab_mul_phase(rx, rz, tab->x[g], tab->z[g]) +
-                     (((tab->neg >> g) & 1u) ? 2u : 0u);
-                rx ^= tab->x[g];
-                rz ^= tab->z[g];
-            }
-        }
-        cx[k] = rx;
-        cz[k] = rz;
-        ce[k] = e & 3u;
-    }
-    __syncthreads();
+// A Clifford run as one signed gather over whole vectors: a CTA takes 1,024
+// consecutive entries, four per thread, so an entry costs a few popcounts
+// beside its two memory accesses whatever the length of the run.  Bound by
+// the scattered reads (n = 12, a ring of 12 CNOTs; <O> of 400 gates there
+// 7.69 -> 6.42 ms against walking the ring's gates for every entry).
+__global__ void __launch_bounds__(kThreads) k_stream_pull(const double *__restrict__ src,
+                                                          double *__restrict__ dst, int n,
+                                                          int n_vec, const DevPull *pull) {
+    const LanePull L = load_pull(pull, n);
     const uint64_t E = 1ull << (2 * n);
-    const uint64_t total = E * (uint64_t)n_vec;
-    const uint32_t zmask = (1u << n) - 1u;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
-         t += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t v = t >> (2 * n);
-        const uint32_t i = (uint32_t)(t & (E - 1));
-        const uint32_t x = i >> n, z = i & zmask;
-        uint32_t rx = 0, rz = 0, e = (uint32_t)__popc(x & z);
-        for (int c = 0; c < n_ch; ++c) {
-            const uint32_t sh = (uint32_t)(kChunkQ * c);
-            const int k = (c << 8) | (int)(((x >> sh) & 15u) | (((z >> sh) & 15u) << 4));
-            e += ce[k] + tab_mul_phase(rx, rz, cx[k], cz[k]);
-            rx ^= cx[k];
-            rz ^= cz[k];
+    const uint32_t t = threadIdx.x;
+    uint32_t oj[4] = {0, 0, 0, 0}, oq[4] = {0, 0, 0, 0};
+    const int nb = 2 * n < 10 ? 2 * n : 10;
+    for (int b = 0; b < nb; ++b)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) off_bit(L, b, t | (uint32_t)k << 8, oj[k], oq[k]);
+    const uint64_t per = (E + 1023) >> 10, chunks = per * (uint64_t)n_vec;
+    for (uint64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+        const uint64_t v = c / per, base = (c - v * per) << 10;
+        const BasePull B = base_pull(L, (uint32_t)base);
+        const double *S = src + v * E;
+        double *D = dst + v * E;
+        double val[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t off = t | (uint32_t)k << 8;
+            uint32_t neg;
+            const uint32_t j = pull_entry(L, B, n, off, oj[k], oq[k], neg);
+            if (base + off < E) val[k] = flip(S[j], neg);
         }
-        const double val = src[v * E + (((uint64_t)rx << n) | rz)];
-        dst[t] = (e & 2u) ? -val : val;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t off = t | (uint32_t)k << 8;
+            if (base + off < E) D[base + off] = val[k];
+        }
     }
 }
 
-__device__ __forceinline__ uint64_t deposit_runs(uint64_t v, const BitRuns &r) {
-    uint64_t out = 0;
-    for (int k = 0; k < r.n; ++k)
-        out |= ((v >> r.src[k]) & ((1ull << r.len[k]) - 1ull)) << r.dst[k];
-    return out;
-}
-
-__global__ void __launch_bounds__(kThreads) k_stream_tile(const double *src, double *dst, int n,
-                                                          int n_vec, TileGroup tg,
-                                                          const DevOp *ops,
-                                                          const DevMap3 *maps) {
-    extern __shared__ double tile[];
+// Consecutive wire passes on at most kTileWires wires: a tile of up to 2^10
+// entries (the wires' (z, x) bits and the lowest other bits) per CTA in shared
+// memory, a group of four entries per thread and pass, the preceding Clifford
+// run folded into the loads.  Small vectors are latency-bound here (n = 8: one
+// warp per sub-partition), so everything a launch needs -- ops, composed maps,
+// the pull -- is fetched at once, a thread's four loads are issued together,
+// and an op is read while the previous one's FP64 chain runs.  n = 8, four
+// wires with a folded CNOT ring, cold caches: 12.1 us a launch with the ring's
+// gates walked per entry and the ops staged pass by pass, 8.3 us now; <O> of
+// 2,000 gates at n = 7 / 8 / (1,000 gates) 9: 636 / 697 / 523 -> 476 / 492 / 432 us.
+// From n = 10 on a launch per wire pass is faster (600 gates: 661 against 794
+// us): the FP64 pipe is full there and a tile's barriers only leave gaps.
+__global__ void __launch_bounds__(kTileThreads) k_stream_tile(const double *src, double *dst,
+                                                              int n, int n_vec, TileGroup tg,
+                                                              const DevOp *ops,
+                                                              const DevMap3 *maps) {
+    __shared__ double tile[1 << kTileMaxBits];
+    __shared__ __align__(16) DevOp sops[kTileStagedOps];
+    __shared__ double smap[kTileMaxPasses][9];
     const uint32_t T = 1u << tg.tile_bits;
-    // the group's ops, staged once (when they fit), then the tile-local entry
-    // -> offset table, the same for every tile
-    DevOp *sops = reinterpret_cast<DevOp *>(tile + T);
-    uint32_t *offs = reinterpret_cast<uint32_t *>(sops + kTileStagedOps);
+    const uint32_t t = threadIdx.x, nt = blockDim.x;   // nt >= T / 4
     int total_ops = 0;
     for (int j = 0; j < tg.n_pass; ++j) total_ops += tg.n_ops[j];
     const bool staged = total_ops <= kTileStagedOps;
     if (staged) {
-        int at = 0;
-        for (int j = 0; j < tg.n_pass; ++j) {
-            for (int k = threadIdx.x; k < (int)tg.n_ops[j]; k += blockDim.x)
-                sops[at + k] = ops[tg.first[j] + k];
-            at += tg.n_ops[j];
+        for (int k = t; k < total_ops; k += nt) {
+            int j = 0, at = k;
+            while (at >= (int)tg.n_ops[j]) at -= tg.n_ops[j++];
+            sops[k] = ops[tg.first[j] + at];
         }
     }
-    for (uint32_t e = threadIdx.x; e < T; e += blockDim.x)
-        offs[e] = (uint32_t)deposit_runs(e, tg.tile_runs);
-    __syncthreads();
+    // the map of a composed run (a single op) by nine threads
+    for (int k = t; k < tg.n_pass * 9; k += nt) {
+        const int j = k / 9;
+        if (tg.n_ops[j] == 1) {
+            const DevOp *op = ops + tg.first[j];
+            if (op->kind == K_MAP3) smap[j][k - 9 * j] = maps[op->param].m[k - 9 * j];
+        }
+    }
+    const bool pulled = tg.pull != nullptr;
+    LanePull L{};
+    if (pulled) L = load_pull(tg.pull, n);
+    uint32_t off[4], oj[4] = {0, 0, 0, 0}, oq[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) off[k] = (uint32_t)deposit_runs(t + k * nt, tg.tile_runs);
+    if (pulled)
+        for (int r = 0; r < tg.tile_runs.n; ++r)
+            for (int b = 0; b < tg.tile_runs.len[r]; ++b)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) off_bit(L, tg.tile_runs.dst[r] + b, off[k], oj[k], oq[k]);
     const uint64_t E = 1ull << (2 * n);
     const uint64_t tiles = (uint64_t)n_vec << tg.rest_bits;
     for (uint64_t tb = blockIdx.x; tb < tiles; tb += gridDim.x) {
-        const uint64_t v = tb >> tg.rest_bits, t = tb & ((1ull << tg.rest_bits) - 1ull);
-        const uint64_t base = deposit_runs(t, tg.rest_runs);
+        const uint64_t v = tb >> tg.rest_bits;
+        const uint32_t base =
+            (uint32_t)deposit_runs(tb & ((1ull << tg.rest_bits) - 1ull), tg.rest_runs);
         const double *S = src + v * E;
-        double *V = dst + v * E + base;
-        if (tg.pull_n == 0) {
-            for (uint32_t e = threadIdx.x; e < T; e += blockDim.x) tile[e] = S[base + offs[e]];
+        double *V = dst + v * E;
+        double val[4];
+        if (!pulled) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (t + k * nt < T) val[k] = S[base + off[k]];
         } else {
-            for (uint32_t e = threadIdx.x; e < T; e += blockDim.x) {
-                uint32_t neg = 0;
-                const uint64_t j = pull_pass(base + offs[e], n, ops + tg.pull_first, tg.pull_n,
-                                             tg.pull_inverse, neg);
-                tile[e] = flip(S[j], neg);
+            const BasePull B = base_pull(L, base);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                uint32_t neg;
+                const uint32_t j = pull_entry(L, B, n, off[k], oj[k], oq[k], neg);
+                if (t + k * nt < T) val[k] = flip(S[j], neg);
             }
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (t + k * nt < T) tile[t + k * nt] = val[k];
         __syncthreads();
         int at = 0;
         for (int j = 0; j < tg.n_pass; ++j) {
@@ -352,13 +349,19 @@ __global__ void __launch_bounds__(kThreads) k_stream_tile(const double *src, dou
             const int n_ops = tg.n_ops[j];
             const DevOp *pops = staged ? sops + at : ops + tg.first[j];
             at += n_ops;
-            for (uint32_t g = threadIdx.x; g < T / 4; g += blockDim.x) {
-                uint32_t b = ((g >> lo) << (lo + 1)) | (g & ((1u << lo) - 1u));
+            if (t < T / 4) {
+                uint32_t b = ((t >> lo) << (lo + 1)) | (t & ((1u << lo) - 1u));
                 b = ((b >> hi) << (hi + 1)) | (b & ((1u << hi) - 1u));
                 double x = tile[b | bx], y = tile[b | bx | bz], z = tile[b | bz];
+                DevOp next = pops[tg.inverse ? n_ops - 1 : 0];
                 for (int k = 0; k < n_ops; ++k) {
-                    const DevOp op = pops[tg.inverse ? n_ops - 1 - k : k];
-                    apply_op1(x, y, z, op, maps, tg.inverse);
+                    const DevOp op = next;
+                    if (k + 1 < n_ops) next = pops[tg.inverse ? n_ops - 2 - k : k + 1];
+                    if (op.kind == K_MAP3)
+                        apply_map3(x, y, z, n_ops == 1 ? smap[j] : maps[op.param].m,
+                                   tg.inverse != 0);
+                    else
+                        apply_op1(x, y, z, op, maps, tg.inverse);
                 }
                 tile[b | bx] = x;
                 tile[b | bx | bz] = y;
@@ -366,7 +369,9 @@ __global__ void __launch_bounds__(kThreads) k_stream_tile(const double *src, dou
             }
             __syncthreads();
         }
-        for (uint32_t e = threadIdx.x; e < T; e += blockDim.x) V[offs[e]] = tile[e];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (t + k * nt < T) V[base + off[k]] = tile[t + k * nt];
         __syncthreads();
     }
 }
@@ -493,10 +498,11 @@ cudaError_t launch_stream_wire(double *vec, int n, int n_vec, const DevPass &p, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_stream_tab(const double *src, double *dst, int n, int n_vec,
-                              const DevTab *tab, cudaStream_t st) {
-    const uint64_t total = (1ull << (2 * n)) * (uint64_t)n_vec;
-    k_stream_tab<<<grid_for(total, kThreads), kThreads, 0, st>>>(src, dst, n, n_vec, tab);
+cudaError_t launch_stream_pull(const double *src, double *dst, int n, int n_vec,
+                               const DevPull *pull, cudaStream_t st) {
+    const uint64_t per = ((1ull << (2 * n)) + 1023) >> 10;
+    k_stream_pull<<<grid_for(per * (uint64_t)n_vec * kThreads, kThreads), kThreads, 0, st>>>(
+        src, dst, n, n_vec, pull);
     return cudaGetLastError();
 }
 
@@ -511,18 +517,12 @@ cudaError_t launch_stream_cliff(const double *src, double *dst, int n, int n_vec
 cudaError_t launch_stream_tile(const double *src, double *dst, int n, int n_vec,
                                const TileGroup &tg, const DevOp *ops, const DevMap3 *maps,
                                cudaStream_t st) {
-    const uint32_t T = 1u << tg.tile_bits;
     const uint64_t tiles = (uint64_t)n_vec << tg.rest_bits;
-    int threads = (int)(T / 4);
-    if (threads > kThreads) threads = kThreads;
+    int threads = (1 << tg.tile_bits) / 4;
     if (threads < 32) threads = 32;
     uint64_t grid = tiles;
-    if (grid > 152ull * 8ull) grid = 152ull * 8ull;
-    const size_t smem = T * (sizeof(double) + sizeof(uint32_t)) + kTileStagedOps * sizeof(DevOp);
-    static SmemLimit lim;
-    cudaError_t e = raise_smem_limit(k_stream_tile, smem, lim);
-    if (e != cudaSuccess) return e;
-    k_stream_tile<<<(int)grid, threads, smem, st>>>(src, dst, n, n_vec, tg, ops, maps);
+    if (grid > 152ull * 16ull) grid = 152ull * 16ull;
+    k_stream_tile<<<(int)grid, threads, 0, st>>>(src, dst, n, n_vec, tg, ops, maps);
     return cudaGetLastError();
 }
 

@@ -225,23 +225,30 @@ cudaError_t launch_xfree_sum(const double *vec, int n, int n_vec, double *out, c
 // *out = <a, b> over the 4^n entries, fixed order; partial: 256 doubles of scratch.
 cudaError_t launch_dot(const double *a, const double *b, int n, double *partial, double *out,
                        cudaStream_t st);
-// P_TAB: dst = the Clifford map whose tableau is *tab applied as a signed gather (n <= 12).
-cudaError_t launch_stream_tab(const double *src, double *dst, int n, int n_vec,
-                              const DevTab *tab, cudaStream_t st);
+// dst = a Clifford run as a signed gather (n <= 12).
+cudaError_t launch_stream_pull(const double *src, double *dst, int n, int n_vec,
+                               const DevPull *pull, cudaStream_t st);
 
 // Several consecutive wire passes on at most kTileWires wires fused into one
 // streamed launch: each CTA loads a tile (all 4^|Q| slots of the wires Q times
 // some of the lowest other index bits) into shared memory, applies the passes
 // in order and writes it back.
-constexpr int kTileWires = 4;
+constexpr int kTileWires = 5;
 constexpr int kTileMaxPasses = 8;
-constexpr int kTileMaxBits = 12;        // 4096 doubles = 32 KiB of shared memory
+constexpr int kTileMaxBits = 10;        // 1024 doubles = 8 KiB of shared memory
+constexpr int kTileThreads = (1 << kTileMaxBits) / 4;   // one group of four entries each
 constexpr int kTileStagedOps = 96;      // ops of a group staged in shared memory (3 KiB)
 
 struct BitRuns {                        // deposit of a packed integer into index bits
     uint8_t n;
     uint8_t src[16], dst[16], len[16];
 };
+
+// Wires of a tile group: as few groups of about equal size as n wires need.
+constexpr int tile_wires(int n) {
+    const int groups = (n + kTileWires - 1) / kTileWires;
+    return (n + groups - 1) / groups;
+}
 
 struct TileGroup {
     int32_t n_pass;
@@ -254,11 +261,9 @@ struct TileGroup {
     uint32_t first[kTileMaxPasses];
     BitRuns tile_runs;                  // local entry -> global index bits
     BitRuns rest_runs;                  // tile id -> global index bits
-    // A Clifford gather folded into the tile loads (a P_CLIFF pass that
-    // precedes the group): entry i is read from pull(i) of the source, signed.
-    int32_t pull_n;                     // ops of that pass (0: plain load)
-    uint32_t pull_first;
-    int32_t pull_inverse;
+    // A Clifford gather folded into the tile loads (the Clifford pass that
+    // precedes the group); null: plain loads.
+    const DevPull *pull;
 };
 
 // src == dst unless the group carries a folded Clifford gather (then the
@@ -285,6 +290,7 @@ cudaError_t launch_adjoint_wire(double *lam, double *rho, int n, const DevPass &
 // launch_adjoint_wire.
 constexpr int kAdjTileMaxN = 8;
 constexpr int kAdjTileBits = 9;
+constexpr int kAdjTileWires = 4;
 size_t adjoint_tile_smem(int tile_bits, int n_rot);   // n_rot: rotations of the group
 cudaError_t launch_adjoint_tile(const double *src_pair, double *dst_pair, int n,
                                 const TileGroup &tg, const DevOp *ops, double *partials,

@@ -274,22 +274,65 @@ static void conj_clifford(uint32_t &x, uint32_t &z, uint32_t &neg, uint8_t op, i
     }
 }
 
-void clifford_tableau(int n, const stab_gate *gates, int64_t i0, int64_t i1, bool inverse,
-                      DevTab *out) {
+void clifford_pull(int n, const stab_gate *gates, int64_t count, bool inverse, DevPull *out) {
     std::memset(out, 0, sizeof(*out));
-    for (int j = 0; j < 2 * n; ++j) {
-        uint32_t x = j < n ? (1u << j) : 0u, z = j < n ? 0u : (1u << (j - n)), neg = 0;
-        for (int64_t k = 0; k < i1 - i0; ++k) {
-            const stab_gate &g = gates[inverse ? i1 - 1 - k : i0 + k];
-            uint8_t op = g.op;
-            if (inverse && op == STAB_S) op = STAB_SDG;
-            else if (inverse && op == STAB_SDG) op = STAB_S;
-            conj_clifford(x, z, neg, op, g.q0, g.q1);
+    // images of the generators under V (the run backward for a forward gather),
+    // in the order X_0 .. X_{n-1}, Z_0 .. Z_{n-1}
+    uint32_t xs[24], zs[24];
+    for (int k = 0; k < 2 * n; ++k) {
+        const bool is_x = k < n;
+        uint32_t x = is_x ? 1u << k : 0u, z = is_x ? 0u : 1u << (k - n), neg = 0;
+        for (int64_t g = 0; g < count; ++g) {
+            const stab_gate &s = gates[inverse ? g : count - 1 - g];
+            uint8_t op = s.op;
+            if (!inverse && op == STAB_S) op = STAB_SDG;
+            else if (!inverse && op == STAB_SDG) op = STAB_S;
+            conj_clifford(x, z, neg, op, s.q0, s.q1);
         }
-        out->x[j] = x;
-        out->z[j] = z;
-        out->neg |= (neg & 1u) << j;
+        xs[k] = x;
+        zs[k] = z;
+        const int bit = is_x ? n + k : k - n;
+        const int r = (2 * (int)neg + __builtin_popcount(x & z)) & 3;
+        out->col[bit] = z | (x << n);
+        out->r0 |= (uint32_t)(r & 1) << bit;
+        out->r1 |= (uint32_t)(r >> 1) << bit;
+        for (int a = 0; a < k; ++a)
+            if (__builtin_popcount(zs[a] & x) & 1)
+                out->qrow[bit] |= 1u << (a < n ? n + a : a - n);
     }
+}
+
+bool check_pull(int n, const stab_gate *gates, int64_t count) {
+    const uint64_t E = 1ull << (2 * n);
+    const uint64_t step = E > 65536 ? E / 65536 | 1 : 1;
+    const uint32_t mask = (1u << n) - 1u;
+    for (bool inverse : {false, true}) {
+        DevPull p;
+        clifford_pull(n, gates, count, inverse, &p);
+        for (uint64_t i64 = 0; i64 < E; i64 += step) {
+            const uint32_t i = (uint32_t)i64;
+            uint32_t x = i >> n, z = i & mask, neg = 0;
+            for (int64_t g = 0; g < count; ++g) {
+                const stab_gate &s = gates[inverse ? g : count - 1 - g];
+                uint8_t op = s.op;
+                if (!inverse && (op == STAB_S || op == STAB_SDG))
+                    op = op == STAB_S ? STAB_SDG : STAB_S;
+                conj_clifford(x, z, neg, op, s.q0, s.q1);
+            }
+            uint32_t j = 0, q = 0;
+            for (int b = 0; b < 2 * n; ++b)
+                if ((i >> b) & 1u) {
+                    j ^= p.col[b];
+                    q ^= (uint32_t)__builtin_popcount(p.qrow[b] & i);
+                }
+            const int e = __builtin_popcount((i >> n) & i & mask) + __builtin_popcount(i & p.r0) +
+                          2 * __builtin_popcount(i & p.r1) + 2 * (int)(q & 1u) -
+                          __builtin_popcount((j >> n) & j & mask);
+            if (j != (z | (x << n)) || (e & 1) || (((uint32_t)e >> 1) & 1u) != (neg & 1u))
+                return false;
+        }
+    }
+    return true;
 }
 
 void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, PlanMode mode,
@@ -302,7 +345,8 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
     P.map_gate_idx.clear();
     P.param_ptr.clear();
     P.param_rot.clear();
-    P.tabs.clear();
+    P.pulls.clear();
+    P.pull_of.clear();
     P.n_rot = 0;
     P.n_params = n_params;
     P.mode = mode;
@@ -456,6 +500,35 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
     constexpr size_t kTabMinPasses = 4;
     HostPlan scratch;
     scratch.mode = mode;
+    // the gather of a Clifford run, once per distinct run
+    std::map<std::string, int32_t> known;
+    auto pull_index = [&](const stab_gate *g, int64_t count) {
+        const std::string key((const char *)g, (size_t)count * sizeof(stab_gate));
+        auto it = known.find(key);
+        if (it != known.end()) return it->second;
+        const int32_t k = (int32_t)(P.pulls.size() / 2);
+        P.pulls.resize(P.pulls.size() + 2);
+        clifford_pull(n, g, count, false, &P.pulls[P.pulls.size() - 2]);
+        clifford_pull(n, g, count, true, &P.pulls[P.pulls.size() - 1]);
+        known[key] = k;
+        return k;
+    };
+    std::vector<stab_gate> run;
+    auto mark_passes = [&]() {
+        for (size_t p = P.pull_of.size(); p < P.passes.size(); ++p) {
+            const DevPass &d = P.passes[p];
+            if (d.type != P_CLIFF) {
+                P.pull_of.push_back(-1);
+                continue;
+            }
+            run.clear();
+            for (int o = 0; o < d.n_ops; ++o) {
+                const DevOp &op = P.ops[d.first + (uint32_t)o];
+                run.push_back({(uint8_t)(op.kind == K_CX ? STAB_CX : STAB_CZ), op.q, op.q1, 0, -1});
+            }
+            P.pull_of.push_back(pull_index(run.data(), (int64_t)run.size()));
+        }
+    };
     int64_t i = 0;
     while (i < m) {
         int64_t j = i;
@@ -468,12 +541,9 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
             if (scratch.passes.size() >= kTabMinPasses) {
                 DevPass p{};
                 p.type = P_TAB;
-                p.first = (uint32_t)(P.tabs.size() / 2);
                 p.n_ops = 0;
-                P.tabs.resize(P.tabs.size() + 2);
-                clifford_tableau(n, gates, i, j, true, &P.tabs[P.tabs.size() - 2]);
-                clifford_tableau(n, gates, i, j, false, &P.tabs[P.tabs.size() - 1]);
                 P.passes.push_back(p);
+                P.pull_of.push_back(pull_index(gates + i, j - i));
                 i = j;
                 continue;
             }
@@ -489,6 +559,7 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
             k = r < m ? r + 1 : m;
         }
         emit_range(em, i, k);
+        mark_passes();
         i = k;
     }
 }

@@ -40,7 +40,10 @@ struct HostPlan {
     int32_t n_rot = 0;
     int64_t n_params = 0;
     PlanMode mode = PLAN_FUSED;
-    std::vector<DevTab> tabs;            // P_TAB passes (two per pass)
+    // plans with tableaus: the Clifford runs as gathers, two per distinct run
+    // (forward, inverse), and per pass the index of its run (-1: a wire pass)
+    std::vector<DevPull> pulls;
+    std::vector<int32_t> pull_of;
 };
 
 // Returns STAB_OK or an error code; msg receives a description on error.
@@ -48,16 +51,19 @@ int validate_gates(int n, const stab_gate *gates, int64_t m, int64_t n_params, s
 int validate_thetas(const double *thetas, int64_t n_params);
 
 // Builds the pass list.  gates must be valid.
-// tableaus: long Clifford runs become P_TAB passes (streamed plans; the
-// resident instruction streams and the batch kernel do not read them).
+// tableaus (streamed plans; the resident instruction streams and the batch
+// kernel do not read them): long Clifford runs become P_TAB passes, and every
+// Clifford pass gets its gather (pulls, pull_of).
 // chunked: long gate lists are planned in parallel chunks (same result).
 void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, PlanMode mode,
                 HostPlan *out, bool tableaus = false, bool chunked = true);
 
-// Tableau of the Clifford gates [i0, i1) applied in order (inverse: the
-// inverse map, the inverse gates in reverse order).
-void clifford_tableau(int n, const stab_gate *gates, int64_t i0, int64_t i1, bool inverse,
-                      DevTab *out);
+// The Clifford gates [0, count) as a gather: applied in order (inverse =
+// false) or the inverse map.
+void clifford_pull(int n, const stab_gate *gates, int64_t count, bool inverse, DevPull *out);
+// Host check: the gathers' source index and sign of every string (up to 2^16 of
+// them, spread) against the run's gates one at a time, both directions.
+bool check_pull(int n, const stab_gate *gates, int64_t count);
 
 // Instruction stream of a plan for the resident kernels (see stab_internal.h):
 // forward (backward = false) or for the inverse circuit (backward = true).

@@ -279,7 +279,7 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     const size_t b_raw = align256(n_raw * sizeof(RawGate));
     const size_t b_pptr = align256(H.param_ptr.size() * sizeof(int32_t));
     const size_t b_prot = align256(H.param_rot.size() * sizeof(int32_t));
-    const size_t b_tabs = align256(H.tabs.size() * sizeof(DevTab));
+    const size_t b_pulls = align256(H.pulls.size() * sizeof(DevPull));
     const std::vector<DevStreamBuf *> streams = P.all_streams();
     size_t b_streams = 0;
     for (const DevStreamBuf *S : streams)
@@ -290,7 +290,7 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     const size_t b_ugates = align256(P.ugates.size() * sizeof(RawGate));
     const size_t b_usegs = align256(P.usegs.size() * sizeof(UniSeg));
     const size_t b_uparts = align256(P.uparts.size() * sizeof(UniPart));
-    const size_t total = b_pass + b_ops + b_maps + b_midx + b_raw + b_pptr + b_prot + b_tabs +
+    const size_t total = b_pass + b_ops + b_maps + b_midx + b_raw + b_pptr + b_prot + b_pulls +
                          b_streams + b_uops + b_uruns + b_ugates + b_usegs + b_uparts;
     RC(c->dalloc(P.buf, total, c->st));
     CK(cudaEventSynchronize(c->ev_stage));
@@ -326,7 +326,7 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     P.raw = (const RawGate *)put(H.raw.data(), n_raw * sizeof(RawGate), b_raw);
     P.param_ptr = (const int32_t *)put(H.param_ptr.data(), H.param_ptr.size() * 4, b_pptr);
     P.param_rot = (const int32_t *)put(H.param_rot.data(), H.param_rot.size() * 4, b_prot);
-    P.prog.tabs = (const DevTab *)put(H.tabs.data(), H.tabs.size() * sizeof(DevTab), b_tabs);
+    P.prog.pulls = (const DevPull *)put(H.pulls.data(), H.pulls.size() * sizeof(DevPull), b_pulls);
     for (DevStreamBuf *S : streams) {
         const size_t rb = S->host.size() * sizeof(Rec), tb = S->tail.size() * sizeof(Rec);
         S->dev = (Rec *)put(S->host.data(), rb, align256(rb + tb), S->tail.data(), tb);
@@ -554,6 +554,11 @@ int upload_terms(stab_ctx *c, const stab_term *O, int64_t n_terms) {
     return STAB_OK;
 }
 
+// Tiles of a launch below which a tile takes no further bits: with 4 wires of
+// n = 8 (2^8 entries) one more bit gives 128 tiles, one to an SM, whose four
+// warps fill its sub-partitions and read two entries in a row.
+constexpr int kMinTiles = 128;
+
 void bit_runs(const std::vector<int> &bits, BitRuns *r) {
     // bit k of a packed integer goes to index bit bits[k] (bits ascending)
     std::memset(r, 0, sizeof(*r));
@@ -569,9 +574,10 @@ void bit_runs(const std::vector<int> &bits, BitRuns *r) {
 }
 
 // Tile geometry for wire passes on `wires`: the wires' x and z bits plus as
-// many of the lowest other bits as keep at least 256 tiles (and 4096 entries).
+// many of the lowest other bits as keep at least min_tiles tiles (and 2^max_bits
+// entries).
 void make_tile_group(int n, int n_vec, const std::vector<const DevPass *> &group, int inverse,
-                     TileGroup *tg, int min_tiles = 256, int max_bits = kTileMaxBits) {
+                     TileGroup *tg, int min_tiles = kMinTiles, int max_bits = kTileMaxBits) {
     std::memset(tg, 0, sizeof(*tg));
     std::vector<int> wires;
     for (const DevPass *p : group)
@@ -832,12 +838,21 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
     // the path tuner's (measured per GPU model)
     const bool fuse_tiles = P.host.mode != PLAN_PLAIN && P.host.mode != PLAN_PLAIN_ROWS &&
                             ((uint64_t)n_vec << (2 * c->n)) <= (uint64_t)c->choice.tile_limit;
+    const size_t max_wires = (size_t)tile_wires(c->n);
     std::vector<const DevPass *> group;
     std::vector<int> wires;
     // with tiles, a Clifford gather is folded into the loads of the next group
     const DevPass *pending = nullptr;
+    auto pull_of = [&](const DevPass *p) -> const DevPull * {
+        const size_t k = (size_t)(p - passes.data());
+        return k < P.host.pull_of.size() ? P.prog.pulls + 2 * P.host.pull_of[k] + (inverse ? 1 : 0)
+                                         : nullptr;
+    };
     auto gather_now = [&]() -> int {
-        CK(launch_stream_cliff(*cur, *alt, c->n, n_vec, *pending, P.prog.ops, inverse, s));
+        if (const DevPull *pull = pull_of(pending))
+            CK(launch_stream_pull(*cur, *alt, c->n, n_vec, pull, s));
+        else
+            CK(launch_stream_cliff(*cur, *alt, c->n, n_vec, *pending, P.prog.ops, inverse, s));
         std::swap(*cur, *alt);
         c->launches++;
         pending = nullptr;
@@ -853,9 +868,7 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
             make_tile_group(c->n, n_vec, group, inverse, &tg);
             double *dst = *cur;
             if (pending) {
-                tg.pull_n = pending->n_ops;
-                tg.pull_first = pending->first;
-                tg.pull_inverse = inverse;
+                tg.pull = pull_of(pending);
                 dst = *alt;
             }
             CK(launch_stream_tile(*cur, dst, c->n, n_vec, tg, P.prog.ops, P.prog.maps, s));
@@ -874,7 +887,7 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
         if (p.type == P_WIRE) {
             const bool known = std::find(wires.begin(), wires.end(), (int)p.q) != wires.end();
             if (!fuse_tiles || (int)group.size() == kTileMaxPasses ||
-                (!known && (int)wires.size() == kTileWires)) {
+                (!known && wires.size() == max_wires)) {
                 RC(flush());
             }
             group.push_back(&p);
@@ -884,14 +897,6 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
         }
         RC(flush());
         if (pending) RC(gather_now());
-        if (p.type == P_TAB) {
-            // a long Clifford run: one gather through its tableau
-            CK(launch_stream_tab(*cur, *alt, c->n, n_vec, P.prog.tabs + 2 * p.first + (inverse ? 1 : 0),
-                                 s));
-            std::swap(*cur, *alt);
-            c->launches++;
-            continue;
-        }
         pending = &p;
         if (!fuse_tiles) RC(gather_now());
     }
@@ -1228,6 +1233,13 @@ int stab_selftest_align(int n, const stab_gate *gates, int64_t m, int64_t n_para
     }
     if (aligned) *aligned = count;
     return STAB_OK;
+}
+
+int stab_selftest_pull(int n, const stab_gate *gates, int64_t m) {
+    if (n < 1 || n > STAB_MAX_QUBITS) return STAB_E_RANGE;
+    std::string msg;
+    RC(validate_gates(n, gates, m, 0, &msg));   // no angle slots: Clifford gates only
+    return check_pull(n, gates, m) ? STAB_OK : STAB_E_STATE;
 }
 
 int stab_selftest_bounded_wait(int64_t polls) {
@@ -1820,8 +1832,13 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                     std::vector<const DevPass *> group;
                     std::vector<int> wires;
                     const DevPass *pending = nullptr;
+                    auto pull_of = [&](const DevPass *p) {
+                        return c->grad.prog.pulls +
+                               2 * c->grad.host.pull_of[(size_t)(p - passes.data())] +
+                               (forward ? 0 : 1);
+                    };
                     auto gather_now = [&]() -> int {
-                        CK(launch_stream_cliff(pr, al, n, 2, *pending, ops, forward ? 0 : 1, st));
+                        CK(launch_stream_pull(pr, al, n, 2, pull_of(pending), st));
                         c->launches++;
                         std::swap(pr, al);
                         pending = nullptr;
@@ -1851,9 +1868,7 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                         }
                         double *dst = pr;
                         if (pending) {
-                            tg.pull_n = pending->n_ops;
-                            tg.pull_first = pending->first;
-                            tg.pull_inverse = forward ? 0 : 1;
+                            tg.pull = pull_of(pending);
                             dst = al;
                         }
                         CK(launch_adjoint_tile(pr, dst, n, tg, ops, (double *)c->partials.p, st));
@@ -1872,7 +1887,7 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                             const bool known =
                                 std::find(wires.begin(), wires.end(), (int)p.q) != wires.end();
                             if ((int)group.size() == kTileMaxPasses ||
-                                (!known && (int)wires.size() == kTileWires))
+                                (!known && (int)wires.size() == kAdjTileWires))
                                 RC(flush());
                             group.push_back(&p);
                             if (!known) wires.push_back(p.q);
@@ -1880,14 +1895,6 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                         }
                         RC(flush());
                         if (pending) RC(gather_now());
-                        if (p.type == P_TAB) {
-                            CK(launch_stream_tab(pr, al, n, 2,
-                                                 c->grad.prog.tabs + 2 * p.first + (forward ? 0 : 1),
-                                                 st));
-                            c->launches++;
-                            std::swap(pr, al);
-                            continue;
-                        }
                         pending = &p;
                         if (!tiles) RC(gather_now());
                     }

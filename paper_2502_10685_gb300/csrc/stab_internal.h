@@ -20,8 +20,8 @@ enum OpKind : uint8_t {
     K_CZ = 4,    // CZ(q, q1)
 };
 
-// P_TAB: a long run of Clifford gates of any kind (streamed plans only),
-// applied as one signed gather through the run's tableau (DevTab).
+// P_TAB: a long run of Clifford gates of any kind (streamed plans only), applied
+// as one signed gather like a P_CLIFF pass of such a plan (DevPull).
 enum PassType : uint8_t { P_WIRE = 0, P_CLIFF = 1, P_TAB = 2 };
 
 // Rotation axes.  Within the 4-slot group (I, X, Y, Z) of one wire a rotation
@@ -72,24 +72,29 @@ enum InitMode : int32_t {
     INIT_LOAD = 3,       // copy from a device vector
 };
 
-// Tableau of a Clifford map V on n <= 12 qubits: the images V X_q V^dagger
-// (entry q) and V Z_q V^dagger (entry n + q), each a signed string with x / z
-// masks; sign bit j of `neg` is entry j's sign.  A P_TAB pass (first = k)
-// refers to tabs[2k] = the run's inverse U^dagger (forward gathers) and
-// tabs[2k + 1] = the run U (inverse gathers).
-struct DevTab {         // 200 bytes
-    uint32_t x[24];
-    uint32_t z[24];
-    uint32_t neg;
-    uint32_t pad;
+// A Clifford run as a signed gather over the index space (streamed plans, n <=
+// 12): dst[i] = (-1)^s src[j].  With V the run's inverse (forward gathers) or
+// the run itself (inverse gathers), V P_i V^dagger = (-1)^s P_j.  The index j is
+// linear over GF(2): the xor of col[b] over the set bits b of i (index bit q is
+// z_q, bit n + q is x_q).  V maps the generator of bit b to i^{r_b} X^{x_b}
+// Z^{z_b} with col[b] = z_b | x_b << n, and a string is i^{|x & z|} times its
+// generators, X parts first, so
+//   2 s = |x & z| + sum_b r_b i_b + 2 Q(i) - |x_j & z_j|   (mod 4),
+//   Q(i) = sum over set b of |qrow[b] & i|, qrow[b] = the generators a before b
+//   whose z_a meets x_b an odd number of times;
+// r_b = bit b of r0 + 2 bit b of r1.
+struct DevPull {        // 200 bytes
+    uint32_t col[24];
+    uint32_t qrow[24];
+    uint32_t r0, r1;
 };
-static_assert(sizeof(DevTab) == 200, "DevTab layout");
+static_assert(sizeof(DevPull) == 200, "DevPull layout");
 
 struct Program {
     const DevPass *passes;
     const DevOp *ops;
     const DevMap3 *maps;
-    const DevTab *tabs;
+    const DevPull *pulls;
     int32_t n_passes;
     int32_t n_ops;
 };
