@@ -193,9 +193,10 @@ int stab_expect_async(stab_ctx *ctx, double *out_dev);
  * stream.  Same for stab_expect_async in that form. */
 int stab_grad_async(stab_ctx *ctx, double *expect_dev, double *grads_dev);
 
-/* How the last gradient's plan is cut: *parts receives K >= 2 when it runs
- * through the K parts of the generators' plan (n <= 4, their unitaries), 1 when
- * it uses the meet-in-the-middle or a streamed sweep, 0 before any gradient since the circuit was loaded.
+/* How the last gradient's plan is cut: *parts receives K >= 2 when its units
+ * are those of the generators' plan and both are cut into the same K parts (n
+ * <= 4), 1 when they are not (a wire run that is the identity and holds no
+ * rotation is a unit of the one but not of the other; plans of n >= 5), 0 before any gradient since the circuit was loaded.
  * Errors: STAB_E_INVAL (ctx or parts NULL). */
 int stab_grad_parts(stab_ctx *ctx, int32_t *parts);
 
@@ -625,8 +626,8 @@ int stab_path_load(const char *path);
 
 /* Measures the candidates for n qubits on CUDA device `device` now, stores
  * the result under that GPU's name and writes it to *out (may be NULL).
- * Candidates: n = 5, 6: resident against streamed for
- * <O> and, separately, for the gradient (2,000-gate probe); n = 7 .. 9: tiles
+ * Candidates: resident against streamed at n = 6 for <O> and, separately, at
+ * n = 5, 6 for the gradient (2,000-gate probe); n = 7 .. 9: tiles
  * against one launch per pass, for one vector (<O>) and for n vectors (the
  * generators), giving tile_limit = the largest of those launch sizes where
  * tiles won (0 when neither); n <= 4 (the parts' segments run at once wherever

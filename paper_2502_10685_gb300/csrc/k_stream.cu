@@ -116,6 +116,53 @@ __global__ void k_compose_maps(DevMap3 *maps, int n_maps, const int32_t *map_gat
         for (int j = 0; j < 9; ++j) maps[w].m[j] = M[j];
 }
 
+// The same with a CTA of 1,024 threads per map, for runs of thousands of gates
+// (n = 1, where a circuit is one run: 16,912 gates 1.24 ms with a warp, 0.31 so):
+// warp w composes chunks 32 w .. 32 w + 31, the first warp the warps' products.
+__global__ void __launch_bounds__(1024) k_compose_maps_cta(DevMap3 *maps,
+                                                           const int32_t *map_gate_idx,
+                                                           const RawGate *gates,
+                                                           const double *thetas) {
+    __shared__ double part[32][9];
+    const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
+    const DevMap3 &mp = maps[blockIdx.x];
+    const int first = mp.first, count = mp.count, per = (count + 1023) / 1024;
+    const int k0 = min((int)threadIdx.x * per, count), k1 = min(k0 + per, count);
+    double M[9] = {1.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0};
+    for (int k = k0; k < k1; ++k) {
+        double G[9], R[9];
+        gate_matrix3(gates[map_gate_idx[first + k]], thetas, G);
+        mul3(G, M, R);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) M[j] = R[j];
+    }
+    for (int round = 0; round < 2; ++round) {
+        if (round == 1) {
+            __syncthreads();
+            if (warp != 0) return;
+#pragma unroll
+            for (int j = 0; j < 9; ++j) M[j] = part[lane][j];
+        }
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            double O[9], R[9];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) O[j] = __shfl_down_sync(0xffffffffu, M[j], d);
+            if ((lane & (2 * d - 1)) == 0) {
+                mul3(O, M, R);
+#pragma unroll
+                for (int j = 0; j < 9; ++j) M[j] = R[j];
+            }
+        }
+        if (lane == 0)
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                if (round == 0) part[warp][j] = M[j];
+                else maps[blockIdx.x].m[j] = M[j];
+            }
+    }
+}
+
 // Composed map of every run, one thread per map walking its gates in order:
 // the form for plans of short runs (a warp per map would idle most lanes).
 __global__ void k_compose_maps_seq(DevMap3 *maps, int n_maps, const int32_t *map_gate_idx,
@@ -269,52 +316,60 @@ __global__ void __launch_bounds__(kThreads) k_stream_pull(const double *__restri
 // entries (the wires' (z, x) bits and the lowest other bits) per CTA in shared
 // memory, a group of four entries per thread and pass, the preceding Clifford
 // run folded into the loads.  Small vectors are latency-bound here (n = 8: one
-// warp per sub-partition), so everything a launch needs -- ops, composed maps,
-// the pull -- is fetched at once, a thread's four loads are issued together,
-// and an op is read while the previous one's FP64 chain runs.  n = 8, four
-// wires with a folded CNOT ring, cold caches: 12.1 us a launch with the ring's
-// gates walked per entry and the ops staged pass by pass, 8.3 us now; <O> of
-// 2,000 gates at n = 7 / 8 / (1,000 gates) 9: 636 / 697 / 523 -> 476 / 492 / 432 us.
-// From n = 10 on a launch per wire pass is faster (600 gates: 661 against 794
+// warp per sub-partition and 36 FP64 instructions a launch), so a launch
+// fetches everything it needs at once and a pass is the run's composed map:
+// three independent rows of three FMAs and no op decoding, where lifts would
+// be a chain of nine behind three decoded ops.  (n = 8, four wires with a
+// folded CNOT ring, two sequences on the GPU: 11 us a launch with the ring's
+// gates walked per entry, 7.3 with lifts, 6.9 so; k_stream_chain runs whole
+// sequences, this kernel the steps of plans outside them.)  From n = 10 on a launch per wire pass is faster (600 gates: 661 against 794
 // us): the FP64 pipe is full there and a tile's barriers only leave gaps.
+// MAPS = false: the runs' ops instead (lifts, three FMAs a rotation), for
+// vectors of 2^18 entries and more whose runs hold few rotations.
+template <bool MAPS>
 __global__ void __launch_bounds__(kTileThreads) k_stream_tile(const double *src, double *dst,
                                                               int n, int n_vec, TileGroup tg,
-                                                              const DevOp *ops,
-                                                              const DevMap3 *maps) {
+                                                              const DevMap3 *maps,
+                                                              const DevOp *ops) {
     __shared__ double tile[1 << kTileMaxBits];
-    __shared__ __align__(16) DevOp sops[kTileStagedOps];
-    __shared__ double smap[kTileMaxPasses][9];
+    __shared__ __align__(16) double smap[kTileMaxPasses][10];
+    __shared__ __align__(16) DevOp sops[MAPS ? 1 : kTileStagedOps];
     const uint32_t T = 1u << tg.tile_bits;
     const uint32_t t = threadIdx.x, nt = blockDim.x;   // nt >= T / 4
-    int total_ops = 0;
-    for (int j = 0; j < tg.n_pass; ++j) total_ops += tg.n_ops[j];
-    const bool staged = total_ops <= kTileStagedOps;
-    if (staged) {
-        for (int k = t; k < total_ops; k += nt) {
-            int j = 0, at = k;
-            while (at >= (int)tg.n_ops[j]) at -= tg.n_ops[j++];
-            sops[k] = ops[tg.first[j] + at];
+    bool staged = false;
+    if constexpr (MAPS) {
+        // the maps, transposed (the inverse) for backward sweeps
+        for (uint32_t k = t; k < (uint32_t)tg.n_pass * 9u; k += nt) {
+            const uint32_t j = k / 9u, e = k - 9u * j;
+            const uint32_t to = tg.inverse ? (e % 3u) * 3u + e / 3u : e;
+            smap[j][to] = maps[tg.map[j]].m[e];
         }
-    }
-    // the map of a composed run (a single op) by nine threads
-    for (int k = t; k < tg.n_pass * 9; k += nt) {
-        const int j = k / 9;
-        if (tg.n_ops[j] == 1) {
-            const DevOp *op = ops + tg.first[j];
-            if (op->kind == K_MAP3) smap[j][k - 9 * j] = maps[op->param].m[k - 9 * j];
-        }
+    } else {
+        int total = 0;
+        for (int j = 0; j < tg.n_pass; ++j) total += tg.n_ops[j];
+        staged = total <= kTileStagedOps;
+        if (staged)
+            for (int k = (int)t; k < total; k += (int)nt) {
+                int j = 0, at = k;
+                while (at >= (int)tg.n_ops[j]) at -= tg.n_ops[j++];
+                sops[k] = ops[tg.first[j] + at];
+            }
     }
     const bool pulled = tg.pull != nullptr;
     LanePull L{};
     if (pulled) L = load_pull(tg.pull, n);
-    uint32_t off[4], oj[4] = {0, 0, 0, 0}, oq[4] = {0, 0, 0, 0};
+    // entry t + k nt: this thread's offset, and one of the CTA for each k
+    const uint32_t off = (uint32_t)deposit_runs(t, tg.tile_runs);
+    uint32_t step[4], oj = 0, oq = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) off[k] = (uint32_t)deposit_runs(t + k * nt, tg.tile_runs);
-    if (pulled)
+    for (int k = 0; k < 4; ++k) step[k] = (uint32_t)deposit_runs(k * nt, tg.tile_runs);
+    if (pulled) {
+        const int bits = 31 - __clz((int)nt);
+        int at = 0;
         for (int r = 0; r < tg.tile_runs.n; ++r)
-            for (int b = 0; b < tg.tile_runs.len[r]; ++b)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) off_bit(L, tg.tile_runs.dst[r] + b, off[k], oj[k], oq[k]);
+            for (int b = 0; b < tg.tile_runs.len[r] && at < bits; ++b, ++at)
+                off_bit(L, tg.tile_runs.dst[r] + b, off, oj, oq);
+    }
     const uint64_t E = 1ull << (2 * n);
     const uint64_t tiles = (uint64_t)n_vec << tg.rest_bits;
     for (uint64_t tb = blockIdx.x; tb < tiles; tb += gridDim.x) {
@@ -324,18 +379,15 @@ __global__ void __launch_bounds__(kTileThreads) k_stream_tile(const double *src,
         const double *S = src + v * E;
         double *V = dst + v * E;
         double val[4];
-        if (!pulled) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (t + k * nt < T) val[k] = S[base + off[k]];
-        } else {
-            const BasePull B = base_pull(L, base);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                uint32_t neg;
-                const uint32_t j = pull_entry(L, B, n, off[k], oj[k], oq[k], neg);
-                if (t + k * nt < T) val[k] = flip(S[j], neg);
+        for (int k = 0; k < 4; ++k) {
+            const bool in = t + k * nt < T;
+            uint32_t neg = 0, j = base + step[k] + off;
+            if (pulled) {
+                const BasePull B = base_pull(L, base + step[k]);
+                j = pull_entry(L, B, n, off, oj, oq, neg);
             }
+            if (in) val[k] = flip(S[j], neg);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -353,15 +405,15 @@ __global__ void __launch_bounds__(kTileThreads) k_stream_tile(const double *src,
                 uint32_t b = ((t >> lo) << (lo + 1)) | (t & ((1u << lo) - 1u));
                 b = ((b >> hi) << (hi + 1)) | (b & ((1u << hi) - 1u));
                 double x = tile[b | bx], y = tile[b | bx | bz], z = tile[b | bz];
-                DevOp next = pops[tg.inverse ? n_ops - 1 : 0];
-                for (int k = 0; k < n_ops; ++k) {
-                    const DevOp op = next;
-                    if (k + 1 < n_ops) next = pops[tg.inverse ? n_ops - 2 - k : k + 1];
-                    if (op.kind == K_MAP3)
-                        apply_map3(x, y, z, n_ops == 1 ? smap[j] : maps[op.param].m,
-                                   tg.inverse != 0);
-                    else
+                if constexpr (MAPS) {
+                    apply_map3(x, y, z, smap[j], false);
+                } else {
+                    DevOp next = pops[tg.inverse ? n_ops - 1 : 0];
+                    for (int k = 0; k < n_ops; ++k) {
+                        const DevOp op = next;
+                        if (k + 1 < n_ops) next = pops[tg.inverse ? n_ops - 2 - k : k + 1];
                         apply_op1(x, y, z, op, maps, tg.inverse);
+                    }
                 }
                 tile[b | bx] = x;
                 tile[b | bx | bz] = y;
@@ -371,8 +423,251 @@ __global__ void __launch_bounds__(kTileThreads) k_stream_tile(const double *src,
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (t + k * nt < T) V[base + off[k]] = tile[t + k * nt];
+            if (t + k * nt < T) V[base + step[k] + off] = tile[t + k * nt];
         __syncthreads();
+    }
+}
+
+// Tables of one shape per CTA (see launch.h).
+__global__ void __launch_bounds__(128) k_chain_tables(const ChainShape *shapes, int n) {
+    __shared__ ChainShape S;
+    __shared__ DevPull P;
+    {
+        const uint32_t *from = reinterpret_cast<const uint32_t *>(shapes + blockIdx.x);
+        for (uint32_t k = threadIdx.x; k < sizeof(ChainShape) / 4; k += blockDim.x)
+            reinterpret_cast<uint32_t *>(&S)[k] = from[k];
+    }
+    __syncthreads();
+    if (S.pull) {
+        const uint32_t *from = reinterpret_cast<const uint32_t *>(S.pull);
+        for (uint32_t k = threadIdx.x; k < sizeof(DevPull) / 4; k += blockDim.x)
+            reinterpret_cast<uint32_t *>(&P)[k] = from[k];
+    }
+    __syncthreads();
+    const int lo = min(S.lz, S.lx), hi = max(S.lz, S.lx);
+    const uint32_t groups = 1u << (S.tile_bits - 2);
+    for (uint32_t t = threadIdx.x; t < groups; t += blockDim.x) {
+        uint32_t b = ((t >> lo) << (lo + 1)) | (t & ((1u << lo) - 1u));
+        b = ((b >> hi) << (hi + 1)) | (b & ((1u << hi) - 1u));
+        const uint32_t off = (uint32_t)deposit_runs(b, S.tile_runs);
+        uint32_t j = 0, q = 0;
+        if (S.pull)
+            for (int k = 0; k < 2 * n; ++k)
+                if ((off >> k) & 1u) {
+                    j ^= P.col[k];
+                    q ^= (uint32_t)__popc(P.qrow[k] & off);
+                }
+        S.threads[t] = make_uint2(off, j | (q & 1u) << 31);
+    }
+    const uint64_t entries = 4ull << S.rest_bits;
+    for (uint64_t m = threadIdx.x; m < entries; m += blockDim.x) {
+        const uint32_t k = (uint32_t)m & 3u;
+        const uint32_t i = (uint32_t)deposit_runs(m >> 2, S.rest_runs) |
+                           ((k & 1u) << S.wire) | ((k >> 1) << (n + S.wire));
+        uint32_t j = 0, q = 0, cross = 0;
+        if (S.pull)
+            for (int a = 0; a < 2 * n; ++a) {
+                const uint32_t par = (uint32_t)__popc(P.qrow[a] & i) & 1u;
+                cross ^= par << a;
+                if ((i >> a) & 1u) {
+                    j ^= P.col[a];
+                    cross ^= P.qrow[a];
+                    q ^= par;
+                }
+            }
+        S.tiles[m] = make_uint4(i, j | q << 31, cross, 0u);
+    }
+}
+
+// A chain of tile steps in one launch: the chain's CTAs stay and meet at a
+// counter in global memory after every step.  Nothing a step needs besides
+// its vector depends on the steps before it, so all of it (where the thread
+// reads and writes, the maps) is loaded during the step before, and a step is
+// its gather, its passes and the barrier's round trip.  The first pass's group
+// is gathered straight into registers and the last pass's stored from them;
+// shared memory carries the tile between passes.  The launch is cooperative
+// (all CTAs resident) and every wait is bounded: a CTA that gives up sets the
+// status word and leaves, and so do the others.
+// Per step at n = 8, four wires, two chains on the GPU: 6.9 us as launches
+// replayed from a graph, 6.3 in a chain that fetches after the barrier, 5.4
+// so; of it 1.9 are FP64 (two CTAs share most SMs), 0.5 the barrier's wait.
+// n = 7: 5.8 -> 4.2 us.
+constexpr uint32_t kChainPolls = 1u << 22;   // a second or two
+
+// ALONE: chains of one CTA each (n = 5) keep their vector in shared memory and
+// meet nobody (3,000 gates: <O> 515 -> 406 us, gradient 1048 -> 788).  Four CTAs of 256
+// threads fit an SM, so both chains of n = 9 (256 tiles each) have a CTA a tile.
+template <bool ALONE>
+__global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
+    __shared__ double tile[1 << kTileMaxBits];
+    __shared__ __align__(16) double smap[2][kTileMaxPasses * 9];
+    __shared__ double solo[2][ALONE ? 1 << kTileMaxBits : 1];
+    __shared__ ChainStep S[3];
+    __shared__ int s_ok;
+    const int ch = (int)blockIdx.x < a.ctas[0] ? 0 : 1;
+    const uint32_t rank = blockIdx.x - (ch ? (uint32_t)a.ctas[0] : 0u);
+    const uint32_t ctas = (uint32_t)(ch ? a.ctas[1] : a.ctas[0]);
+    const int n_steps = ch ? a.n_steps[1] : a.n_steps[0];
+    const ChainStep *steps = ch ? a.steps[1] : a.steps[0];
+    uint32_t *arrived = a.arrived + 32 * ch;
+    const uint32_t t = threadIdx.x;              // one group: blockDim.x = 2^tile_bits / 4
+    const int n = a.n;
+    const uint64_t E = 1ull << (2 * n);
+    const uint32_t zmask = (1u << n) - 1u;
+    constexpr uint32_t kWords = sizeof(ChainStep) / 4;   // <= blockDim.x
+    // registers loaded one step ahead
+    uint2 in_t{}, in_t1{};
+    uint32_t out_off = 0, out_off1 = 0, r0 = 0, r1 = 0, r01 = 0, r11 = 0;
+    uint4 tk[4], tk1[4];
+    double mval = 0.0;
+    uint32_t word = 0;
+    const uint32_t mj = t / 9u, me = t - 9u * mj;
+    // issues step s's loads (its description is in S[s % 3])
+    auto fetch = [&](int s) {
+        const ChainStep &d = S[s % 3];
+        in_t1 = d.in_threads[t];
+        out_off1 = d.out_threads[t].x;
+        if (d.pull) {
+            r01 = d.pull->r0;
+            r11 = d.pull->r1;
+        }
+        if ((rank >> d.rest_bits) < (uint32_t)a.n_vec) {
+            const uint4 *p = d.tiles + 4ull * (rank & ((1u << d.rest_bits) - 1u));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tk1[k] = p[k];
+        }
+        // thread (j, e) holds entry e of pass j's map, transposed (the inverse)
+        // for backward sweeps
+        if (mj < (uint32_t)d.n_pass)
+            mval = a.maps[d.map[mj]].m[d.inverse ? (me % 3u) * 3u + me / 3u : me];
+    };
+    auto land = [&](int s) {   // fetched values of step s become current
+        in_t = in_t1;
+        out_off = out_off1;
+        r0 = r01;
+        r1 = r11;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) tk[k] = tk1[k];
+        if (mj < (uint32_t)S[s % 3].n_pass) smap[s & 1][t] = mval;
+    };
+    for (int s = 0; s < 2 && s < n_steps; ++s)
+        if (t < kWords)
+            reinterpret_cast<uint32_t *>(&S[s])[t] =
+                reinterpret_cast<const uint32_t *>(steps + s)[t];
+    __syncthreads();
+    if (n_steps > 0) {
+        fetch(0);
+        land(0);
+    }
+    if (ALONE && n_steps > 0)
+        for (uint32_t i = t; i < (uint32_t)E; i += blockDim.x) solo[0][i] = S[0].src[i];
+    __syncthreads();
+    for (int s = 0; s < n_steps; ++s) {
+        const ChainStep &st = S[s % 3];
+        const int n_pass = st.n_pass;
+        const bool pulled = st.pull != nullptr;
+        const double *maps = smap[s & 1];
+        const uint64_t tiles = (uint64_t)a.n_vec << st.rest_bits;
+        bool first = true;
+        for (uint64_t tb = rank; tb < tiles; tb += ctas) {
+            const uint64_t v = tb >> st.rest_bits;
+            const double *src = st.src + v * E;
+            double *dst = st.dst + v * E;
+            if (!first) {
+                const uint4 *p = st.tiles + 4ull * (tb & ((1ull << st.rest_bits) - 1ull));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) tk[k] = p[k];
+            }
+            double val[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t i = tk[k].x + in_t.x;
+                uint32_t j = i, neg = 0;
+                if (pulled) {
+                    const uint32_t jq = tk[k].y ^ in_t.y;
+                    j = jq & 0x7fffffffu;
+                    const uint32_t q = (jq >> 31) ^ ((uint32_t)__popc(in_t.x & tk[k].z) & 1u);
+                    neg = ((uint32_t)(__popc((i >> n) & i & zmask) + __popc(i & r0) +
+                                      2 * __popc(i & r1) + 2 * (int)q -
+                                      __popc((j >> n) & j & zmask)) >> 1) & 1u;
+                }
+                // written by other SMs in this launch: through L2
+                val[k] = flip(ALONE ? solo[s & 1][j] : __ldcg(src + j), neg);
+            }
+            if (first) {
+                // the next step's loads, in flight during this one
+                if (s + 1 < n_steps) fetch(s + 1);
+                if (s + 2 < n_steps && t < kWords)
+                    word = reinterpret_cast<const uint32_t *>(steps + s + 2)[t];
+                first = false;
+            }
+            if (n_pass > 0) apply_map3(val[2], val[3], val[1], maps, false);
+            for (int j = 1; j < n_pass; ++j) {
+                // through shared memory from pass j - 1's groups to pass j's
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int lz = st.lz[j - 1 + h], lx = st.lx[j - 1 + h];
+                    const int lo = lz < lx ? lz : lx, hi = lz < lx ? lx : lz;
+                    const uint32_t bz = 1u << lz, bx = 1u << lx;
+                    uint32_t b = ((t >> lo) << (lo + 1)) | (t & ((1u << lo) - 1u));
+                    b = ((b >> hi) << (hi + 1)) | (b & ((1u << hi) - 1u));
+                    if (h == 0) {
+                        // (the last pass's reads of this buffer are behind a barrier)
+                        tile[b] = val[0];
+                        tile[b | bz] = val[1];
+                        tile[b | bx] = val[2];
+                        tile[b | bx | bz] = val[3];
+                        __syncthreads();
+                    } else {
+                        val[0] = tile[b];
+                        val[1] = tile[b | bz];
+                        val[2] = tile[b | bx];
+                        val[3] = tile[b | bx | bz];
+                        __syncthreads();
+                    }
+                }
+                apply_map3(val[2], val[3], val[1], maps + 9 * j, false);
+            }
+            const uint32_t base = n_pass > 0 ? tk[0].x + out_off : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t i = n_pass > 0 ? base + st.out_k[k] : tk[k].x + in_t.x;
+                dst[i] = val[k];
+                if (ALONE) solo[(s + 1) & 1][i] = val[k];
+            }
+        }
+        if (s + 1 == n_steps) return;
+        if (first) {   // a CTA without a tile in this step
+            fetch(s + 1);
+            if (s + 2 < n_steps && t < kWords)
+                word = reinterpret_cast<const uint32_t *>(steps + s + 2)[t];
+        }
+        __syncthreads();
+        if (t == 0 && !ALONE) {
+            __threadfence();
+            atomicAdd(arrived, 1u);
+        }
+        land(s + 1);
+        if (s + 2 < n_steps && t < kWords)
+            reinterpret_cast<uint32_t *>(&S[(s + 2) % 3])[t] = word;
+        if (ALONE) {
+            __syncthreads();
+            continue;
+        }
+        if (t == 0) {
+            const uint32_t want = ctas * (uint32_t)(s + 1);
+            bool ok = false;
+            for (uint32_t it = 0; it < kChainPolls && !ok; ++it) {
+                uint32_t seen;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                             : "=r"(seen) : "l"(arrived) : "memory");
+                ok = seen >= want;
+            }
+            if (!ok && a.status) atomicExch(a.status, STAB_KSTATUS_TIMEOUT);
+            s_ok = ok ? 1 : 0;
+        }
+        __syncthreads();
+        if (!s_ok) return;
     }
 }
 
@@ -455,7 +750,10 @@ cudaError_t launch_compose_maps(DevMap3 *maps, int n_maps, int max_count,
                                 const int32_t *map_gate_idx, const RawGate *gates,
                                 const double *thetas, cudaStream_t st) {
     if (n_maps == 0) return cudaSuccess;
-    if (max_count <= kSeqMapGates)
+    // a CTA per map while the CTAs are few and a warp's lanes would walk 32 gates and more
+    if (max_count >= 1024 && n_maps <= 1024)
+        k_compose_maps_cta<<<n_maps, 1024, 0, st>>>(maps, map_gate_idx, gates, thetas);
+    else if (!warp_per_run(n_maps, max_count))
         k_compose_maps_seq<<<(n_maps + 127) / 128, 128, 0, st>>>(maps, n_maps, map_gate_idx, gates,
                                                                  thetas);
     else
@@ -515,15 +813,53 @@ cudaError_t launch_stream_cliff(const double *src, double *dst, int n, int n_vec
 }
 
 cudaError_t launch_stream_tile(const double *src, double *dst, int n, int n_vec,
-                               const TileGroup &tg, const DevOp *ops, const DevMap3 *maps,
+                               const TileGroup &tg, const DevMap3 *maps, const DevOp *ops,
                                cudaStream_t st) {
     const uint64_t tiles = (uint64_t)n_vec << tg.rest_bits;
     int threads = (1 << tg.tile_bits) / 4;
     if (threads < 32) threads = 32;
     uint64_t grid = tiles;
     if (grid > 152ull * 16ull) grid = 152ull * 16ull;
-    k_stream_tile<<<(int)grid, threads, 0, st>>>(src, dst, n, n_vec, tg, ops, maps);
+    if (ops)
+        k_stream_tile<false><<<(int)grid, threads, 0, st>>>(src, dst, n, n_vec, tg, maps, ops);
+    else
+        k_stream_tile<true><<<(int)grid, threads, 0, st>>>(src, dst, n, n_vec, tg, maps, nullptr);
     return cudaGetLastError();
+}
+
+int chain_max_ctas(int threads) {
+    int dev = 0, sms = 0, per = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stream_chain<false>, threads, 0) !=
+            cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return coop ? per * sms : 0;
+}
+
+cudaError_t launch_chain_tables(const ChainShape *shapes, int n_shapes, int n, cudaStream_t st) {
+    if (n_shapes == 0) return cudaSuccess;
+    k_chain_tables<<<n_shapes, 128, 0, st>>>(shapes, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stream_chain(const ChainArgs &a, cudaStream_t st) {
+    const int threads = 1 << (a.tile_bits - 2);
+    if (a.n < kChainMinN || threads < (int)(sizeof(ChainStep) / 4) ||
+        threads < 9 * kTileMaxPasses || threads > kTileThreads)
+        return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(a.arrived, 0, 256, st);
+    if (e != cudaSuccess) return e;
+    ChainArgs args = a;
+    void *params[] = {&args};
+    const bool alone = a.n_vec == 1 && a.tile_bits == 2 * a.n && a.ctas[0] <= 1 && a.ctas[1] <= 1;
+    return cudaLaunchCooperativeKernel(alone ? (const void *)k_stream_chain<true>
+                                             : (const void *)k_stream_chain<false>,
+                                       dim3((unsigned)(a.ctas[0] + a.ctas[1])),
+                                       dim3((unsigned)threads), params, 0, st);
 }
 
 cudaError_t launch_dot(const double *a, const double *b, int n, double *partial, double *out,

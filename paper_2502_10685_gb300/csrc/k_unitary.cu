@@ -647,40 +647,39 @@ __device__ __forceinline__ void walk_run(double (&c)[3], const RawGate *gates, i
     }
 }
 
-// c of a run at its end: its rows' shares in row order, less the run's factor.
-template <int D>
-__device__ __forceinline__ void run_dots(const double *dots, int run, int parity, double (&c)[3]) {
+// c of a run at its end: its `rows` shares in order, less the run's factor.
+__device__ __forceinline__ void run_dots(const double *dots, int run, int rows, int parity,
+                                         double (&c)[3]) {
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const double *p = dots + ((size_t)run * 3 + j) * D;
+        const double *p = dots + ((size_t)run * 3 + j) * rows;
         double v = 0.0;
-#pragma unroll
-        for (int r = 0; r < D; ++r) v += p[r];
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) v += p[r];
         c[j] = parity ? 0.5 * v : v;
     }
 }
 
 // A thread per run.
-template <int N>
-__global__ void __launch_bounds__(64) k_uni_walk_seq(const UniRun *runs, int n_runs,
-                                                     const RawGate *gates, const double *thetas,
-                                                     const double *dots, double *grad_gate) {
+__global__ void __launch_bounds__(64) k_walk_seq(const UniRun *runs, int n_runs,
+                                                 const RawGate *gates, const double *thetas,
+                                                 const double *dots, int rows,
+                                                 double *grad_gate) {
     const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= n_runs) return;
     const UniRun r = runs[i];
     double c[3];
-    run_dots<UCfg<N>::D>(dots, i, r.parity >> 1, c);
+    run_dots(dots, i, rows, r.parity >> 1, c);
     walk_run(c, gates, r.first, r.first + r.count, thetas, grad_gate);
 }
 
 // A warp per run: every lane turns the three unit vectors back through its
 // chunk of the run, a suffix scan of these 3 x 3 maps gives c at the chunk's
 // end, and the chunk is walked again.
-template <int N>
-__global__ void __launch_bounds__(128) k_uni_walk_warp(const UniRun *runs, int n_runs,
-                                                       const RawGate *gates,
-                                                       const double *thetas, const double *dots,
-                                                       double *grad_gate) {
+__global__ void __launch_bounds__(128) k_walk_warp(const UniRun *runs, int n_runs,
+                                                   const RawGate *gates, const double *thetas,
+                                                   const double *dots, int rows,
+                                                   double *grad_gate) {
     const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = (int)(threadIdx.x & 31u);
     if (w >= n_runs) return;   // whole warps
@@ -717,7 +716,7 @@ __global__ void __launch_bounds__(128) k_uni_walk_warp(const UniRun *runs, int n
         }
     }
     double e[3], c[3];
-    run_dots<UCfg<N>::D>(dots, w, r.parity >> 1, e);
+    run_dots(dots, w, rows, r.parity >> 1, e);
     // the chunks after this lane's
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -756,17 +755,8 @@ cudaError_t states_n(const UniRoots &r, const DevTerm *terms, int n_terms, doubl
 
 template <int N>
 cudaError_t grad_n(const UniArgs &a, const double2 *psi, const double2 *phi, double *dots,
-                   const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
-                   const double *thetas, double *grad_gate, cudaStream_t st) {
+                   cudaStream_t st) {
     k_uni_grad<N><<<a.n_segs, 64, 0, st>>>(a, psi, phi, dots);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || n_runs == 0) return e;
-    if (max_count <= kSeqMapGates)
-        k_uni_walk_seq<N><<<(n_runs + 63) / 64, 64, 0, st>>>(runs, n_runs, gates, thetas, dots,
-                                                             grad_gate);
-    else
-        k_uni_walk_warp<N><<<(n_runs + 3) / 4, 128, 0, st>>>(runs, n_runs, gates, thetas, dots,
-                                                             grad_gate);
     return cudaGetLastError();
 }
 
@@ -775,7 +765,7 @@ cudaError_t grad_n(const UniArgs &a, const double2 *psi, const double2 *phi, dou
 cudaError_t launch_uni_maps(const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
                             const double *thetas, UniMap *maps, cudaStream_t st) {
     if (n_runs == 0) return cudaSuccess;
-    if (max_count <= kSeqMapGates)
+    if (!warp_per_run(n_runs, max_count))
         k_uni_maps_seq<<<(n_runs + 63) / 64, 64, 0, st>>>(runs, n_runs, gates, thetas, maps);
     else
         k_uni_maps_warp<<<(n_runs + 3) / 4, 128, 0, st>>>(runs, n_runs, gates, thetas, maps);
@@ -826,16 +816,27 @@ cudaError_t launch_uni_states(int n, const UniRoots &r, const DevTerm *terms, in
 }
 
 cudaError_t launch_uni_grad(int n, const UniArgs &a, const double2 *psi, const double2 *phi,
-                            double *dots, const UniRun *runs, int n_runs, int max_count,
-                            const RawGate *gates, const double *thetas, double *grad_gate,
-                            cudaStream_t st) {
+                            double *dots, cudaStream_t st) {
     switch (n) {
-    case 1: return grad_n<1>(a, psi, phi, dots, runs, n_runs, max_count, gates, thetas, grad_gate, st);
-    case 2: return grad_n<2>(a, psi, phi, dots, runs, n_runs, max_count, gates, thetas, grad_gate, st);
-    case 3: return grad_n<3>(a, psi, phi, dots, runs, n_runs, max_count, gates, thetas, grad_gate, st);
-    case 4: return grad_n<4>(a, psi, phi, dots, runs, n_runs, max_count, gates, thetas, grad_gate, st);
+    case 1: return grad_n<1>(a, psi, phi, dots, st);
+    case 2: return grad_n<2>(a, psi, phi, dots, st);
+    case 3: return grad_n<3>(a, psi, phi, dots, st);
+    case 4: return grad_n<4>(a, psi, phi, dots, st);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_run_grads(const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
+                             const double *thetas, const double *dots, int rows,
+                             double *grad_gate, cudaStream_t st) {
+    if (n_runs == 0) return cudaSuccess;
+    if (!warp_per_run(n_runs, max_count))
+        k_walk_seq<<<(n_runs + 63) / 64, 64, 0, st>>>(runs, n_runs, gates, thetas, dots, rows,
+                                                      grad_gate);
+    else
+        k_walk_warp<<<(n_runs + 3) / 4, 128, 0, st>>>(runs, n_runs, gates, thetas, dots, rows,
+                                                      grad_gate);
+    return cudaGetLastError();
 }
 
 }  // namespace stab

@@ -180,6 +180,10 @@ namespace stab {
 // complete once this stream is).
 cudaStream_t ctx_stream(stab_ctx *ctx);
 
+// The context's gradients keep within the vectors that the request footprint
+// counts (no stored sweeps).
+void ctx_no_checkpoints(stab_ctx *ctx);
+
 // Density matrix from the forward-evolved coefficients of 2^n |0><0|:
 // rho (device, 2 x 4^n doubles, interleaved complex, row-major).
 cudaError_t launch_decode_rho(const double *r, int n, double *rho, cudaStream_t st);
@@ -190,10 +194,15 @@ cudaError_t launch_bounded_wait(int64_t polls, int32_t *status, cudaStream_t st)
 // Records the CUDA error behind a STAB_E_CUDA status (stab_last_cuda_error).
 void record_cuda_error(cudaError_t e);
 
+// Whether runs of up to max_count gates are composed (or walked) by a warp each
+// instead of a thread each: a thread takes about 2.3 us a gate (a sincos and a
+// product, one after another), a warp about 6 us and, beyond the GPU's warps, 12
+// ns a run (five shuffled products).
+inline bool warp_per_run(int64_t n_runs, int max_count) {
+    return max_count > 32 || (max_count > 4 && 2.3 * max_count > 6.0 + 0.012 * (double)n_runs);
+}
 // Composed 3x3 map of every run (maps[i].m), from the angle array on the
-// device: one thread per map when no run is longer than kSeqMapGates gates
-// (max_count, the longest run), else one warp per map.
-constexpr int kSeqMapGates = 32;
+// device (max_count: the longest run).
 cudaError_t launch_compose_maps(DevMap3 *maps, int n_maps, int max_count,
                                 const int32_t *map_gate_idx, const RawGate *gates,
                                 const double *thetas, cudaStream_t st);
@@ -237,7 +246,6 @@ constexpr int kTileWires = 5;
 constexpr int kTileMaxPasses = 8;
 constexpr int kTileMaxBits = 10;        // 1024 doubles = 8 KiB of shared memory
 constexpr int kTileThreads = (1 << kTileMaxBits) / 4;   // one group of four entries each
-constexpr int kTileStagedOps = 96;      // ops of a group staged in shared memory (3 KiB)
 
 struct BitRuns {                        // deposit of a packed integer into index bits
     uint8_t n;
@@ -259,6 +267,7 @@ struct TileGroup {
     uint16_t n_ops[kTileMaxPasses];
     uint8_t n_rot[kTileMaxPasses];      // rotations of each pass (adjoint groups)
     uint32_t first[kTileMaxPasses];
+    uint32_t map[kTileMaxPasses];       // each pass's composed map (k_stream_tile)
     BitRuns tile_runs;                  // local entry -> global index bits
     BitRuns rest_runs;                  // tile id -> global index bits
     // A Clifford gather folded into the tile loads (the Clifford pass that
@@ -266,11 +275,73 @@ struct TileGroup {
     const DevPull *pull;
 };
 
-// src == dst unless the group carries a folded Clifford gather (then the
-// result goes to dst, a different buffer).
+// src == dst, or (always with a folded Clifford gather) a different buffer.  ops
+// null: the passes as composed maps (maps[tg.map[j]]); else as their ops (maps:
+// the plan's long runs).
+constexpr int kTileStagedOps = 96;      // ops of a group staged in shared memory (3 KiB)
 cudaError_t launch_stream_tile(const double *src, double *dst, int n, int n_vec,
-                               const TileGroup &tg, const DevOp *ops, const DevMap3 *maps,
+                               const TileGroup &tg, const DevMap3 *maps, const DevOp *ops,
                                cudaStream_t st);
+
+// Whole sequences of tile steps in one cooperative launch: up to two chains of
+// steps, each a number of CTAs that meet at a barrier after every step.  A
+// step gathers a tile, applies its passes and stores it.  Where each thread
+// reads and writes is tabulated per shape (tile geometry, the wire whose groups
+// the threads hold, the Clifford gather read through), so the chain only looks
+// it up: entry k = 0 .. 3 (I, Z, X, Y) of thread t's group in tile m is at index
+// tiles[4 m + k].x + threads[t].x, its source the xor of both tables' .y
+// (pulled shapes; see DevPull for the sign).
+struct ChainShape {
+    BitRuns tile_runs, rest_runs;
+    int32_t tile_bits, rest_bits;
+    int32_t lz, lx, wire;               // the wire: tile-local bits, qubit
+    int32_t pad;
+    const DevPull *pull;                // null: entries are read in place
+    uint2 *threads;                     // (offset, source | Q << 31) per thread
+    uint4 *tiles;                       // (index, source | Q << 31, cross bits, 0) per entry
+};
+cudaError_t launch_chain_tables(const ChainShape *shapes, int n_shapes, int n, cudaStream_t st);
+
+struct ChainStep {                      // 128 bytes
+    const double *src;
+    double *dst;
+    const uint2 *in_threads, *out_threads;   // shapes of the first and the last pass's wire
+    const uint4 *tiles;                 // of the first pass's shape
+    const DevPull *pull;                // of that shape
+    int32_t n_pass, inverse, rest_bits, pad;
+    uint32_t out_k[4];                  // index bits of the last pass's wire for I, Z, X, Y
+    uint8_t lz[kTileMaxPasses], lx[kTileMaxPasses];
+    uint32_t map[kTileMaxPasses];
+};
+static_assert(sizeof(ChainStep) == 128, "ChainStep layout");
+struct ChainArgs {
+    const ChainStep *steps[2];          // device
+    int32_t n_steps[2];
+    int32_t ctas[2];
+    int32_t n, n_vec, tile_bits;
+    const DevMap3 *maps;
+    uint32_t *arrived;                  // two counters 128 bytes apart, zeroed before the launch
+    int32_t *status;
+};
+constexpr int kChainMinN = 5;           // tiles of at least 2^9 entries
+// CTAs of `threads` threads that fit on the device at once (0 on an error).
+int chain_max_ctas(int threads);
+cudaError_t launch_stream_chain(const ChainArgs &a, cudaStream_t st);
+
+// The c of up to kTileWires wire runs of one block of wire passes, from rho and
+// lambda at the block's end (lambda read through `pull` unless null).
+struct DotJob {
+    const double *rho, *lam;
+    const DevPull *pull;
+    int32_t n_wires;
+    int32_t tile_bits, rest_bits;
+    int32_t run[kTileWires];
+    uint8_t lz[kTileWires], lx[kTileWires];   // tile-local bits of the wires
+    BitRuns tile_runs, rest_runs;
+};
+// dots[(3 run + s) chunks + chunk], a CTA per job and chunk of its tiles.
+cudaError_t launch_grad_dots(const DotJob *jobs, int n_jobs, int n, int chunks, double *dots,
+                             cudaStream_t st);
 
 // Adjoint gradient, shared-memory resident (n <= kMaxResidentAdjoint).
 cudaError_t launch_adjoint_split(int n, const AdjointSplitArgs &a, cudaStream_t s);
@@ -303,8 +374,7 @@ cudaError_t launch_gather_grads(const double *grad_rot, const int32_t *param_ptr
 
 // ---------------------------------------------------------------- segment unitaries (k_unitary.cu)
 
-// 2 x 2 maps of the plan's wire runs from the angles: a thread per run, or a
-// warp per run when some run is longer than kSeqMapGates gates (max_count).
+// 2 x 2 maps of the plan's wire runs from the angles (max_count: the longest run).
 cudaError_t launch_uni_maps(const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
                             const double *thetas, UniMap *maps, cudaStream_t st);
 
@@ -341,12 +411,15 @@ cudaError_t launch_uni_merge(int n, const UniRoots &r, double2 *out, int32_t *pa
 cudaError_t launch_uni_states(int n, const UniRoots &r, const DevTerm *terms, int n_terms,
                               double *expect, double2 *psi, double2 *phi, double *r_out,
                               cudaStream_t st);
-// grad_gate[g] = d<O>/d(angle of gate g) for the rotations of the run-ordered
-// gate array; dots: 3 x 2^n doubles of scratch per run.
+// The three numbers c of every wire run at its end, as 2^n shares:
+// dots[(3 run + s) 2^n + row] (see k_unitary.cu).
 cudaError_t launch_uni_grad(int n, const UniArgs &a, const double2 *psi, const double2 *phi,
-                            double *dots, const UniRun *runs, int n_runs, int max_count,
-                            const RawGate *gates, const double *thetas, double *grad_gate,
-                            cudaStream_t st);
+                            double *dots, cudaStream_t st);
+// grad_gate[g] = d<O>/d(angle of gate g) for the rotations of the run-ordered
+// gate array, from every run's c, given as `rows` shares each.
+cudaError_t launch_run_grads(const UniRun *runs, int n_runs, int max_count, const RawGate *gates,
+                             const double *thetas, const double *dots, int rows,
+                             double *grad_gate, cudaStream_t st);
 
 // ---------------------------------------------------------------- sparse term lists (k_sparse.cu)
 

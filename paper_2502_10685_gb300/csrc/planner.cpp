@@ -131,6 +131,15 @@ struct Emitter {
     HostPlan *P;
     PlanMode mode;
     const std::vector<int32_t> *rot_ordinal;
+    bool list_runs = false;    // record every wire pass's gates
+
+    // Gates run[k0, k1) belong to the pass just pushed (the passes since the
+    // last listed one are Clifford passes: empty ranges).
+    void list_run(const int64_t *run, size_t k0, size_t k1) {
+        if (!list_runs) return;
+        P->run_first.resize(P->passes.size(), (int32_t)P->run_gates.size());
+        for (size_t k = k0; k < k1; ++k) P->run_gates.push_back((int32_t)run[k]);
+    }
 
     void emit_cliff(const stab_gate *gates, int64_t i0, int64_t i1) {
         DevPass p{};
@@ -177,8 +186,10 @@ struct Emitter {
             p.n_ops = 1;
             P->ops.push_back(op);
             P->passes.push_back(p);
+            list_run(run, 0, run_len);
             return;
         }
+        size_t from = 0;   // first gate of the pass being filled
         DevPass p{};
         p.type = P_WIRE;
         p.q = (uint8_t)q;
@@ -198,9 +209,13 @@ struct Emitter {
             }
             pending = kPermIdentity;
         };
-        auto close_pass = [&]() {
+        auto close_pass = [&](size_t k) {   // the pass ends before gate k
             p.n_ops = (uint16_t)(P->ops.size() - p.first);
-            if (p.n_ops > 0) P->passes.push_back(p);
+            if (p.n_ops > 0) {
+                P->passes.push_back(p);
+                list_run(run, from, k);
+            }
+            from = k;
             p.first = (uint32_t)P->ops.size();
             rot_in_pass = 0;
         };
@@ -211,13 +226,13 @@ struct Emitter {
                 pending = perm_compose(pending, clifford_perm_code(op));
                 if (mode == PLAN_PLAIN) {
                     flush_perm();
-                    close_pass();
+                    close_pass(k + 1);
                 }
                 continue;
             }
             if (mode == PLAN_GRAD && rot_in_pass == kRotPerGradPass) {
                 flush_perm();
-                close_pass();
+                close_pass(k);
             }
             flush_perm();
             DevOp r{};
@@ -228,10 +243,10 @@ struct Emitter {
             r.gate = (*rot_ordinal)[i];
             P->ops.push_back(r);
             ++rot_in_pass;
-            if (mode == PLAN_PLAIN) close_pass();
+            if (mode == PLAN_PLAIN) close_pass(k + 1);
         }
         flush_perm();
-        close_pass();
+        close_pass(run_len);
     }
 };
 
@@ -347,6 +362,8 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
     P.param_rot.clear();
     P.pulls.clear();
     P.pull_of.clear();
+    P.run_gates.clear();
+    P.run_first.clear();
     P.n_rot = 0;
     P.n_params = n_params;
     P.mode = mode;
@@ -498,6 +515,7 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
     // A run of Clifford gates that would take kTabMinPasses or more passes
     // becomes one P_TAB pass: a signed gather through the run's tableau.
     constexpr size_t kTabMinPasses = 4;
+    em.list_runs = true;
     HostPlan scratch;
     scratch.mode = mode;
     // the gather of a Clifford run, once per distinct run
@@ -562,6 +580,7 @@ void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, Plan
         mark_passes();
         i = k;
     }
+    P.run_first.resize(P.passes.size() + 1, (int32_t)P.run_gates.size());
 }
 
 namespace {

@@ -44,6 +44,9 @@ struct HostPlan {
     // (forward, inverse), and per pass the index of its run (-1: a wire pass)
     std::vector<DevPull> pulls;
     std::vector<int32_t> pull_of;
+    // and the gates of every wire pass in order (indices into raw): pass p's are
+    // run_gates[run_first[p] .. run_first[p + 1])
+    std::vector<int32_t> run_gates, run_first;
 };
 
 // Returns STAB_OK or an error code; msg receives a description on error.
@@ -52,8 +55,9 @@ int validate_thetas(const double *thetas, int64_t n_params);
 
 // Builds the pass list.  gates must be valid.
 // tableaus (streamed plans; the resident instruction streams and the batch
-// kernel do not read them): long Clifford runs become P_TAB passes, and every
-// Clifford pass gets its gather (pulls, pull_of).
+// kernel do not read them): long Clifford runs become P_TAB passes, every
+// Clifford pass gets its gather (pulls, pull_of) and the gates of the wire
+// passes are listed (run_gates).
 // chunked: long gate lists are planned in parallel chunks (same result).
 void build_plan(int n, const stab_gate *gates, int64_t m, int64_t n_params, PlanMode mode,
                 HostPlan *out, bool tableaus = false, bool chunked = true);

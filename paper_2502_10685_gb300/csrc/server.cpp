@@ -257,6 +257,7 @@ Slot *make_slot(stab_server *s, int n) {
         delete sl;
         return nullptr;
     }
+    ctx_no_checkpoints(sl->ctx);   // requests are admitted by a fixed number of vectors
     cudaStream_t st = ctx_stream(sl->ctx);
     sl->d_res = (double *)s->hooks.get(256, st);
     if (!sl->d_res || cudaMallocHost(&sl->h_res, 64 * sizeof(double)) != cudaSuccess ||

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <new>
 #include <string>
 #include <thread>
@@ -73,6 +74,10 @@ namespace {
 // several host threads.
 constexpr int kThreadedStreamPasses = 2048;
 
+// Device memory a context may take for the stored sweeps of a gradient; above
+// it the pair sweep runs, which keeps a fixed number of vectors.
+constexpr size_t kCheckpointBytes = (size_t)4 << 30;
+
 // Instruction stream of a plan for the resident kernels, with the indices of
 // the records the encode kernel fills (rotations and maps).
 struct DevStreamBuf {
@@ -104,7 +109,8 @@ struct DevPlan {
     // cuts[k+1]), each cut into segments whose unitaries are composed at once
     // (see k_unitary.cu); no streams.
     bool uni = false;
-    bool uni_identity = false;       // some wire run is the identity and holds no rotation
+    bool uni_identity = false;       // some wire run is the identity and holds no rotation, so
+                                     // a gradient plan of its own would have other units
     std::vector<int> cuts;
     std::vector<UniOp> uops;
     std::vector<UniRun> uruns;
@@ -119,11 +125,15 @@ struct DevPlan {
     DevBuf buf;
     Program prog{};
     const int32_t *map_gate_idx = nullptr;
+    std::vector<DevMap3> pass_maps;  // of prog.pass_maps, before composition
+    int max_pass_gates = 0, wire_passes = 0;
+    const int32_t *run_gates = nullptr;
     const RawGate *raw = nullptr;
     const int32_t *param_ptr = nullptr;
     const int32_t *param_rot = nullptr;
     bool built = false;
     bool encoded = false;
+    bool ops_encoded = false, maps_encoded = false;   // streamed plans
 };
 
 // A captured sequence of streamed launches, valid while its key is unchanged.
@@ -141,6 +151,29 @@ struct GraphCache {
         launches = 0;
         result = nullptr;
     }
+};
+
+// Two chains of tile steps on the device (see k_stream_chain), valid while the
+// key (plan, buffers) is unchanged.
+struct ChainSet {
+    std::vector<const void *> key;
+    std::vector<ChainStep> host[2];
+    std::vector<ChainShape> shapes;           // tables, one per distinct shape
+    std::vector<int> in_shape[2], out_shape[2];   // per step
+    std::map<std::string, int> known;         // shape -> its index
+    void clear() {
+        key.clear();
+        shapes.clear();
+        known.clear();
+        for (int k = 0; k < 2; ++k) {
+            host[k].clear();
+            in_shape[k].clear();
+            out_shape[k].clear();
+        }
+    }
+    DevBuf dev, tables;
+    int ctas[2] = {0, 0};
+    double *result[2] = {nullptr, nullptr};   // where each chain's vectors end up
 };
 
 }  // namespace
@@ -170,12 +203,29 @@ struct stab_ctx {
     int64_t n_params = 0;
 
     DevPlan fwd, grad;
+    // gradients from stored sweeps (streamed; see ck_gradient): the fused plan
+    // when fwd is not one, the runs and their gates; blocks of wire passes
+    DevPlan ck;
+    struct CkBlock {
+        int p0, p1;                  // its wire passes
+        std::vector<int> before;     // Clifford passes between the previous block and this one
+    };
+    std::vector<CkBlock> ck_blocks;
+    std::vector<int> ck_after;       // Clifford passes after the last block
+    std::vector<DotJob> ck_jobs;     // pointers filled in once the slots exist
+    std::vector<int> ck_job_block;
+    int ck_chunks = 1;
+    bool ck_ready = false, ck_off = false;   // built for this plan; no room or not wanted
+    size_t ck_bytes_max = kCheckpointBytes;
+    DevBuf ckslots, ckjobs, ckdots;
+    std::vector<const void *> key_ck;
     DevBuf thetas, gens, gens_tmp, lam, rho, tmp, tmp2, terms, scal, grad_rot, partials, grads;
     DevBuf gbuf;                     // gradients written inside captured graphs
     DevBuf lam2, tmp3;               // second-branch buffers of the split sweeps
     DevBuf dotbuf;                   // partial sums of the split expectation's inner product
     DevBuf gmid;                     // split resident adjoint: rho, then lambda, at the cut
     bool grad_uni = false;           // the gradient runs through the segments' unitaries
+    bool grad_ran = false;           // a gradient was asked for since the circuit was loaded
     DevBuf ustates, udots;           // its states at the parts' boundaries, runs' dot shares
     // split sweeps of the small registers.  n <= 4: the wire runs' 2 x 2 maps,
     // the segments' and parts' unitaries.  n = 5, 6: the two halves of <O>:
@@ -184,12 +234,15 @@ struct stab_ctx {
     std::vector<const void *> key_e;
     size_t split_smem = 0;
     int sms = 0;                     // SMs of the device
+    int chain_ctas = 0;              // CTAs of a chain launch that fit on it at once
     // the parts' unitaries were composed for these angles when tx_gen ==
     // param_gen; ev_tx marks their end on st
     int64_t param_gen = 0, tx_gen = -1;
     cudaEvent_t ev_tx = nullptr;
     DevBuf status;                   // int32 set by kernels whose bounded waits gave up
     GraphCache g_gens, g_expect, g_grad; // streamed launch sequences (n > resident sizes)
+    ChainSet c_gens, c_expect, c_grad;   // the same as one launch, small vectors
+    DevBuf arrived;
     int64_t plan_gen = 0;            // bumped whenever a plan is rebuilt
     int32_t n_obs_terms = 0;
     bool obs_loaded = false;
@@ -268,6 +321,22 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     // resident plans read only their streams (plus maps and raw gates for encoding)
     const size_t n_pass = P.streams ? 0 : H.passes.size();
     const size_t n_ops = P.streams ? 0 : H.ops.size();
+    // streamed plans whose vectors are small enough for tile launches: every
+    // wire pass's run as a composed map
+    P.pass_maps.clear();
+    P.max_pass_gates = P.wire_passes = 0;
+    if (!P.streams && (uint64_t)c->vec_bytes() / sizeof(double) <= (uint64_t)c->choice.tile_limit &&
+        H.run_first.size() == n_pass + 1) {
+        P.pass_maps.resize(n_pass);
+        for (size_t p = 0; p < n_pass; ++p) {
+            DevMap3 &m = P.pass_maps[p];
+            m.first = H.run_first[p];
+            m.count = H.run_first[p + 1] - H.run_first[p];
+            P.max_pass_gates = std::max(P.max_pass_gates, (int)m.count);
+            P.wire_passes += H.passes[p].type == P_WIRE;
+        }
+    }
+    const size_t n_pmaps = P.pass_maps.size(), n_rg = n_pmaps ? H.run_gates.size() : 0;
     // plans applied through segment unitaries read their own op list and runs
     const size_t n_maps = P.uni ? 0 : H.maps.size();
     const size_t n_midx = P.uni ? 0 : H.map_gate_idx.size();
@@ -285,13 +354,14 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     for (const DevStreamBuf *S : streams)
         b_streams += align256((S->host.size() + S->tail.size()) * sizeof(Rec)) +
                      align256((S->enc.size() + S->tail_enc.size()) * 4);
+    const size_t b_pmaps = align256(n_pmaps * sizeof(DevMap3)), b_rg = align256(n_rg * 4);
     const size_t b_uops = align256(P.uops.size() * sizeof(UniOp));
     const size_t b_uruns = align256(P.uruns.size() * sizeof(UniRun));
     const size_t b_ugates = align256(P.ugates.size() * sizeof(RawGate));
     const size_t b_usegs = align256(P.usegs.size() * sizeof(UniSeg));
     const size_t b_uparts = align256(P.uparts.size() * sizeof(UniPart));
     const size_t total = b_pass + b_ops + b_maps + b_midx + b_raw + b_pptr + b_prot + b_pulls +
-                         b_streams + b_uops + b_uruns + b_ugates + b_usegs + b_uparts;
+                         b_streams + b_uops + b_uruns + b_ugates + b_usegs + b_uparts + b_pmaps + b_rg;
     RC(c->dalloc(P.buf, total, c->st));
     CK(cudaEventSynchronize(c->ev_stage));
     RC(c->host_stage(c->stage, c->stage_bytes, total));
@@ -333,6 +403,12 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
         const size_t eb = S->enc.size() * 4, teb = S->tail_enc.size() * 4;
         S->enc_dev = (const int32_t *)put(S->enc.data(), eb, align256(eb + teb),
                                           S->tail_enc.data(), teb);
+    }
+    P.prog.pass_maps = nullptr;
+    if (n_pmaps) {
+        P.prog.pass_maps =
+            (const DevMap3 *)put(P.pass_maps.data(), n_pmaps * sizeof(DevMap3), b_pmaps);
+        P.run_gates = (const int32_t *)put(H.run_gates.data(), n_rg * 4, b_rg);
     }
     P.uargs = UniArgs{};
     P.uargs.ops = (const UniOp *)put(P.uops.data(), P.uops.size() * sizeof(UniOp), b_uops);
@@ -384,17 +460,62 @@ int encode_plan(stab_ctx *c, DevPlan &P) {
         P.encoded = true;
         return STAB_OK;
     }
-    const int n_ops = P.prog.n_ops, n_maps = (int)P.host.maps.size();
-    if (n_ops == 0 && n_maps == 0) {
-        P.encoded = true;
-        return STAB_OK;
-    }
-    CK(launch_encode(const_cast<DevOp *>(P.prog.ops), n_ops, const_cast<DevMap3 *>(P.prog.maps),
-                     n_maps, max_map_count(P.host.maps.data(), P.host.maps.size()),
-                     P.map_gate_idx, P.raw, th, c->st));
-    c->launches += (n_maps > 0) + (n_ops > 0);
+    // streamed plans: what the next call reads (stream_ops, stream_maps)
+    P.ops_encoded = P.maps_encoded = false;
     P.encoded = true;
     return STAB_OK;
+}
+
+// The ops of a streamed plan for the current angles (a launch per pass reads
+// them), or its composed pass maps (tile launches), on the context stream;
+// ev_ready moves behind them.
+int stream_ops(stab_ctx *c, DevPlan &P) {
+    if (P.ops_encoded) return STAB_OK;
+    const int n_ops = P.prog.n_ops, n_maps = (int)P.host.maps.size();
+    if (n_ops > 0 || n_maps > 0)
+        CK(launch_encode(const_cast<DevOp *>(P.prog.ops), n_ops,
+                         const_cast<DevMap3 *>(P.prog.maps), n_maps,
+                         max_map_count(P.host.maps.data(), P.host.maps.size()), P.map_gate_idx,
+                         P.raw, (const double *)c->thetas.p, c->st));
+    c->launches += (n_maps > 0) + (n_ops > 0);
+    P.ops_encoded = true;
+    CK(cudaEventRecord(c->ev_ready, c->st));
+    return STAB_OK;
+}
+
+int stream_maps(stab_ctx *c, DevPlan &P) {
+    if (P.maps_encoded) return STAB_OK;
+    if (!P.pass_maps.empty()) {
+        CK(launch_compose_maps(const_cast<DevMap3 *>(P.prog.pass_maps), (int)P.pass_maps.size(),
+                               P.max_pass_gates, P.run_gates, P.raw,
+                               (const double *)c->thetas.p, c->st));
+        c->launches++;
+    }
+    P.maps_encoded = true;
+    CK(cudaEventRecord(c->ev_ready, c->st));
+    return STAB_OK;
+}
+
+// How wire passes on n_vec vectors run where the path choice allows tiles.
+// Small vectors: as composed maps, nine FMAs a group, because launches and
+// latency bound them.  From 2^18 entries on the FP64 pipe bounds a pass: maps
+// only where the runs hold two rotations and more (three FMAs each as lifts), one
+// vector's other plans as tiles of lifts, more vectors as a launch per pass.
+// (n = 9, <O> of 1,000 gates: 2.7 rotations a run 0.44 ms in tiles of maps, 0.55 a
+// launch per pass; 0.9 a run 0.90 in tiles of maps, 0.68 in tiles of lifts,
+// 0.82 a launch per pass.  Nine generators, 300 gates: 1.79 ms in tiles of maps,
+// 1.28 a launch per pass.)
+enum TileForm { kNoTiles, kTileMaps, kTileOps };
+TileForm tile_form(const stab_ctx *c, const DevPlan &P, int n_vec) {
+    const uint64_t size = (uint64_t)n_vec << (2 * c->n);
+    if (!P.prog.pass_maps || size > (uint64_t)c->choice.tile_limit) return kNoTiles;
+    if (size < ((uint64_t)1 << 18) || P.host.n_rot >= 2 * P.wire_passes) return kTileMaps;
+    return n_vec == 1 ? kTileOps : kNoTiles;
+}
+
+// What a sweep of n_vec vectors reads, for the current angles.
+int stream_encode(stab_ctx *c, DevPlan &P, int n_vec) {
+    return tile_form(c, P, n_vec) == kTileMaps ? stream_maps(c, P) : stream_ops(c, P);
 }
 
 // One instruction stream to build: passes [k0, k1) of the plan, forward or
@@ -573,15 +694,11 @@ void bit_runs(const std::vector<int> &bits, BitRuns *r) {
     }
 }
 
-// Tile geometry for wire passes on `wires`: the wires' x and z bits plus as
-// many of the lowest other bits as keep at least min_tiles tiles (and 2^max_bits
-// entries).
-void make_tile_group(int n, int n_vec, const std::vector<const DevPass *> &group, int inverse,
-                     TileGroup *tg, int min_tiles = kMinTiles, int max_bits = kTileMaxBits) {
-    std::memset(tg, 0, sizeof(*tg));
-    std::vector<int> wires;
-    for (const DevPass *p : group)
-        if (std::find(wires.begin(), wires.end(), (int)p->q) == wires.end()) wires.push_back(p->q);
+// Tile geometry for the wires: their x and z bits plus as many of the lowest
+// other bits as keep at least min_tiles tiles (and 2^max_bits entries).  tile
+// and rest receive the index bits of a tile's entries and of the tiles.
+void tile_bits_of(int n, int n_vec, const std::vector<int> &wires, int min_tiles, int max_bits,
+                  std::vector<int> *tile_out, std::vector<int> *rest_out) {
     std::vector<int> qbits;
     for (int q : wires) {
         qbits.push_back(q);
@@ -594,10 +711,21 @@ void make_tile_group(int n, int n_vec, const std::vector<const DevPass *> &group
     while (c < (int)others.size() && (int)qbits.size() + c + 1 <= max_bits &&
            ((int64_t)n_vec << (2 * n - ((int)qbits.size() + c + 1))) >= min_tiles)
         ++c;
-    std::vector<int> tile(qbits);
+    std::vector<int> &tile = *tile_out;
+    tile = qbits;
     tile.insert(tile.end(), others.begin(), others.begin() + c);
     std::sort(tile.begin(), tile.end());
-    std::vector<int> rest(others.begin() + c, others.end());
+    rest_out->assign(others.begin() + c, others.end());
+}
+
+void make_tile_group(int n, int n_vec, const std::vector<DevPass> &passes,
+                     const std::vector<const DevPass *> &group, int inverse, TileGroup *tg,
+                     int min_tiles = kMinTiles, int max_bits = kTileMaxBits) {
+    std::memset(tg, 0, sizeof(*tg));
+    std::vector<int> wires, tile, rest;
+    for (const DevPass *p : group)
+        if (std::find(wires.begin(), wires.end(), (int)p->q) == wires.end()) wires.push_back(p->q);
+    tile_bits_of(n, n_vec, wires, min_tiles, max_bits, &tile, &rest);
     tg->n_pass = (int32_t)group.size();
     tg->tile_bits = (int32_t)tile.size();
     tg->rest_bits = (int32_t)rest.size();
@@ -608,6 +736,7 @@ void make_tile_group(int n, int n_vec, const std::vector<const DevPass *> &group
         tg->lx[j] = (uint8_t)(std::find(tile.begin(), tile.end(), n + q) - tile.begin());
         tg->n_ops[j] = group[j]->n_ops;
         tg->first[j] = group[j]->first;
+        tg->map[j] = (uint32_t)(group[j] - passes.data());
     }
     bit_runs(tile, &tg->tile_runs);
     bit_runs(rest, &tg->rest_runs);
@@ -628,12 +757,12 @@ int later_parts(const stab_ctx *c) { return (int)c->fwd.uparts.size() - 1; }
 
 // Parts of a long plan: two cut at gen_cut of the passes, or three -- at n = 4
 // where the path choice says so (a first part of gen_cut, two equal ones), at
-// n <= 3 from kChainMinPasses passes a part (equal ones).  Where the cuts lie
+// n <= 3 from kPartMinPasses passes a part (equal ones).  Where the cuts lie
 // costs nothing: every part's segments run at once.
-constexpr int kChainMinPasses = 32;
+constexpr int kPartMinPasses = 32;
 std::vector<int> part_cuts(const stab_ctx *c) {
     const int np = (int)c->fwd.host.passes.size();
-    if (c->n <= 3 && np >= 3 * kChainMinPasses)
+    if (c->n <= 3 && np >= 3 * kPartMinPasses)
         return {0, (int)((int64_t)np / 3), (int)((int64_t)np * 2 / 3), np};
     const int c1 = (int)(np * c->choice.gen_cut);
     if (c->n == 4 && c->choice.gen_parts == 3 && np >= 3 * kSplitMinPasses)
@@ -824,6 +953,20 @@ int split_units_e(stab_ctx *c, cudaStream_t s) {
     return STAB_OK;
 }
 
+// A Clifford pass as one gather of its own.  One or two gates are walked per
+// entry (their few index operations hide behind the loads: n = 10, random
+// circuits of 107 gates 2.02 against 2.20 ms, n = 12 3.24 against 3.33), longer runs
+// read through their linear map.
+constexpr int kShortRun = 2;
+cudaError_t launch_gather(const stab_ctx *c, const DevPlan &P, const DevPass &p, int inverse,
+                          const double *src, double *dst, int n_vec, cudaStream_t s) {
+    const size_t k = (size_t)(&p - P.host.passes.data());
+    if (k >= P.host.pull_of.size() || (p.type == P_CLIFF && p.n_ops <= kShortRun))
+        return launch_stream_cliff(src, dst, c->n, n_vec, p, P.prog.ops, inverse, s);
+    return launch_stream_pull(src, dst, c->n, n_vec,
+                              P.prog.pulls + 2 * P.host.pull_of[k] + (inverse ? 1 : 0), s);
+}
+
 // Streamed propagation of n_vec vectors through a plan; *cur / *alt are the
 // ping-pong buffers (the result ends in *cur).  Consecutive wire passes on at
 // most kTileWires wires run as one tile-fused launch (fused plans only; the
@@ -836,8 +979,8 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
     // tiles pay where a launch is small (launch-bound: few vectors, n <= 8); larger
     // launches are FP64-bound and run faster one wire per launch; the limit is
     // the path tuner's (measured per GPU model)
-    const bool fuse_tiles = P.host.mode != PLAN_PLAIN && P.host.mode != PLAN_PLAIN_ROWS &&
-                            ((uint64_t)n_vec << (2 * c->n)) <= (uint64_t)c->choice.tile_limit;
+    const TileForm form = tile_form(c, P, n_vec);
+    const bool fuse_tiles = form != kNoTiles;
     const size_t max_wires = (size_t)tile_wires(c->n);
     std::vector<const DevPass *> group;
     std::vector<int> wires;
@@ -849,10 +992,7 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
                                          : nullptr;
     };
     auto gather_now = [&]() -> int {
-        if (const DevPull *pull = pull_of(pending))
-            CK(launch_stream_pull(*cur, *alt, c->n, n_vec, pull, s));
-        else
-            CK(launch_stream_cliff(*cur, *alt, c->n, n_vec, *pending, P.prog.ops, inverse, s));
+        CK(launch_gather(c, P, *pending, inverse, *cur, *alt, n_vec, s));
         std::swap(*cur, *alt);
         c->launches++;
         pending = nullptr;
@@ -860,18 +1000,21 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
     };
     auto flush = [&]() -> int {
         if (group.empty()) return STAB_OK;
-        if (group.size() == 1 && !pending) {
+        if (!fuse_tiles) {
             CK(launch_stream_wire(*cur, c->n, n_vec, *group[0], P.prog.ops, P.prog.maps, inverse,
                                   s));
         } else {
             TileGroup tg;
-            make_tile_group(c->n, n_vec, group, inverse, &tg);
+            make_tile_group(c->n, n_vec, passes, group, inverse, &tg);
             double *dst = *cur;
             if (pending) {
                 tg.pull = pull_of(pending);
                 dst = *alt;
             }
-            CK(launch_stream_tile(*cur, dst, c->n, n_vec, tg, P.prog.ops, P.prog.maps, s));
+            const bool maps = form == kTileMaps;
+            CK(launch_stream_tile(*cur, dst, c->n, n_vec, tg,
+                                  maps ? P.prog.pass_maps : P.prog.maps,
+                                  maps ? nullptr : P.prog.ops, s));
             if (pending) {
                 std::swap(*cur, *alt);
                 pending = nullptr;
@@ -902,6 +1045,208 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
     }
     RC(flush());
     if (pending) RC(gather_now());
+    return STAB_OK;
+}
+
+// ---------------------------------------------------------------- chains of tile steps
+//
+// Where a vector is small enough for tile launches (the path choice's
+// tile_limit), the whole sequence of them runs as one cooperative launch.
+
+int chain_tile_bits(int n) { return std::min(2 * n, std::max(9, 2 * tile_wires(n))); }
+
+bool use_chain(const stab_ctx *c, const DevPlan &P, int n_vec) {
+    return c->n >= kChainMinN && c->chain_ctas > 0 && tile_form(c, P, n_vec) == kTileMaps;
+}
+
+// Whether generators and <O> take the chain: a cooperative launch and its
+// tables cost about 7 us more than the first few launches of a graph (<O> of
+// 100 gates: n = 6 67 against 59, n = 8 69 against 62; 300 gates: 100 / 100, 104 /
+// 101; 1,000 gates: 210 / 244, 217 / 242), about the time of ten steps' gain;
+// at n = 9 every SM has work either way and launches spread it better (300 /
+// 1,000 / 3,000 gates: 178 / 465 / 1294 in a chain, 160 / 435 / 1204 launched).
+// (A gradient's two chains take twice the steps and always gain.)
+constexpr int kChainMinPasses = 40;
+constexpr int kChainMaxN = 8;
+bool use_chain_forward(const stab_ctx *c, const DevPlan &P, int n_vec) {
+    return c->n <= kChainMaxN && (int)P.host.passes.size() >= kChainMinPasses &&
+           use_chain(c, P, n_vec);
+}
+
+// One step of chain k: the wires' passes on src (through pull unless null) into
+// dst; no passes: the gather alone.  Every step's tile has the same size.
+void chain_step(const stab_ctx *c, const DevPlan &P, const std::vector<const DevPass *> &group,
+                bool inverse, const DevPull *pull, const double *src, double *dst, ChainSet *C,
+                int k) {
+    const int n = c->n;
+    std::vector<int> wires, tile, rest;
+    for (const DevPass *p : group)
+        if (std::find(wires.begin(), wires.end(), (int)p->q) == wires.end()) wires.push_back(p->q);
+    // a gather alone: any wire's groups
+    if (wires.empty()) wires.push_back(n - 1);
+    tile_bits_of(n, 1, wires, 1, chain_tile_bits(n), &tile, &rest);
+    auto local = [&](int bit) {
+        return (int)(std::find(tile.begin(), tile.end(), bit) - tile.begin());
+    };
+    auto shape = [&](int wire, const DevPull *through) {
+        ChainShape h{};
+        bit_runs(tile, &h.tile_runs);
+        bit_runs(rest, &h.rest_runs);
+        h.tile_bits = (int32_t)tile.size();
+        h.rest_bits = (int32_t)rest.size();
+        h.wire = wire;
+        h.lz = local(wire);
+        h.lx = local(n + wire);
+        h.pull = through;
+        const std::string id((const char *)&h, sizeof(h));
+        auto it = C->known.find(id);
+        if (it != C->known.end()) return it->second;
+        C->shapes.push_back(h);
+        const int at = (int)C->shapes.size() - 1;
+        C->known.emplace(id, at);
+        return at;
+    };
+    ChainStep s{};
+    s.src = src;
+    s.dst = dst;
+    s.pull = pull;
+    s.n_pass = (int32_t)group.size();
+    s.inverse = inverse;
+    s.rest_bits = (int32_t)rest.size();
+    for (size_t j = 0; j < group.size(); ++j) {
+        s.lz[j] = (uint8_t)local(group[j]->q);
+        s.lx[j] = (uint8_t)local(n + group[j]->q);
+        s.map[j] = (uint32_t)(group[j] - P.host.passes.data());
+    }
+    const int in = group.empty() ? wires[0] : group.front()->q;
+    const int out = group.empty() ? wires[0] : group.back()->q;
+    for (uint32_t e = 0; e < 4; ++e) s.out_k[e] = (e & 1u) << out | (e >> 1) << (n + out);
+    // the step's index comes from the unpulled wire bits of the first shape's
+    // entry I, so the last wire's bits are clear in it as well
+    C->host[k].push_back(s);
+    C->in_shape[k].push_back(shape(in, pull));
+    C->out_shape[k].push_back(shape(out, nullptr));
+}
+
+// Wire passes [p0, p1) of one block from src (through pull unless null) into dst.
+void chain_block(const stab_ctx *c, const DevPlan &P, int p0, int p1, bool inverse,
+                 const DevPull *pull, const double *src, double *dst, ChainSet *C, int ch) {
+    const auto &passes = P.host.passes;
+    std::vector<const DevPass *> group;
+    std::vector<int> wires;
+    for (int k = 0; k < p1 - p0; ++k) {
+        const DevPass *p = &passes[(size_t)(inverse ? p1 - 1 - k : p0 + k)];
+        const bool known = std::find(wires.begin(), wires.end(), (int)p->q) != wires.end();
+        if ((int)group.size() == kTileMaxPasses ||
+            (!known && (int)wires.size() == tile_wires(c->n))) {
+            chain_step(c, P, group, inverse, pull, src, dst, C, ch);
+            src = dst;
+            pull = nullptr;
+            group.clear();
+            wires.clear();
+            wires.push_back(p->q);
+        } else if (!known) {
+            wires.push_back(p->q);
+        }
+        group.push_back(p);
+    }
+    chain_step(c, P, group, inverse, pull, src, dst, C, ch);
+}
+
+// Passes [k0, k1) (walked backward when inverse) as steps between two buffers;
+// returns the one that holds the result.
+double *chain_passes(const stab_ctx *c, const DevPlan &P, double *cur, double *alt, bool inverse,
+                     int k0, int k1, ChainSet *C, int ch) {
+    const auto &passes = P.host.passes;
+    auto pull_of = [&](int p) {
+        return P.prog.pulls + 2 * P.host.pull_of[(size_t)p] + (inverse ? 1 : 0);
+    };
+    int pending = -1;
+    auto gather = [&]() {
+        chain_step(c, P, {}, inverse, pull_of(pending), cur, alt, C, ch);
+        std::swap(cur, alt);
+    };
+    for (int k = 0; k < k1 - k0;) {
+        const int p = inverse ? k1 - 1 - k : k0 + k;
+        if (passes[(size_t)p].type != P_WIRE) {
+            if (pending >= 0) gather();
+            pending = p;
+            ++k;
+            continue;
+        }
+        int m = 0;   // the block's wire passes
+        while (k + m < k1 - k0 && passes[(size_t)(inverse ? p - m : p + m)].type == P_WIRE) ++m;
+        double *dst = pending >= 0 ? alt : cur;
+        chain_block(c, P, inverse ? p - m + 1 : p, inverse ? p + 1 : p + m, inverse,
+                    pending >= 0 ? pull_of(pending) : nullptr, cur, dst, C, ch);
+        if (pending >= 0) std::swap(cur, alt);
+        pending = -1;
+        k += m;
+    }
+    if (pending >= 0) gather();
+    return cur;
+}
+
+// Builds the shapes' tables, uploads both chains' steps (on s) and sizes their
+// CTAs.
+int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key, int n_vec,
+                 cudaStream_t s) {
+    const size_t n0 = C.host[0].size(), n1 = C.host[1].size(), ns = C.shapes.size();
+    const size_t groups = (size_t)1 << (chain_tile_bits(c->n) - 2);
+    const size_t tiles = (size_t)1 << (2 * c->n - chain_tile_bits(c->n));
+    const size_t per = groups * sizeof(uint2) + 4 * tiles * sizeof(uint4);
+    const size_t b_shapes = align256(ns * sizeof(ChainShape));
+    RC(c->dalloc(C.tables, b_shapes + ns * per, s));
+    RC(c->dalloc(C.dev, std::max<size_t>(1, n0 + n1) * sizeof(ChainStep), s));
+    RC(c->dalloc(c->arrived, 256, s));
+    char *base = (char *)C.tables.p + b_shapes;
+    for (size_t k = 0; k < ns; ++k) {
+        C.shapes[k].tiles = (uint4 *)(base + k * per);
+        C.shapes[k].threads = (uint2 *)(base + k * per + 4 * tiles * sizeof(uint4));
+    }
+    ChainStep *d = (ChainStep *)C.dev.p;
+    for (int k = 0; k < 2; ++k) {
+        std::vector<ChainStep> &H = C.host[k];
+        for (size_t i = 0; i < H.size(); ++i) {
+            const ChainShape &in = C.shapes[(size_t)C.in_shape[k][i]];
+            H[i].in_threads = in.threads;
+            H[i].tiles = in.tiles;
+            H[i].out_threads = C.shapes[(size_t)C.out_shape[k][i]].threads;
+        }
+        C.ctas[k] = H.empty() ? 0
+                              : (int)std::min<int64_t>((int64_t)n_vec * (int64_t)tiles,
+                                                       c->chain_ctas / (n0 && n1 ? 2 : 1));
+        if (!H.empty())
+            CK(cudaMemcpyAsync(d + (k ? n0 : 0), H.data(), H.size() * sizeof(ChainStep),
+                               cudaMemcpyHostToDevice, s));
+    }
+    if (ns)
+        CK(cudaMemcpyAsync(C.tables.p, C.shapes.data(), ns * sizeof(ChainShape),
+                           cudaMemcpyHostToDevice, s));
+    CK(launch_chain_tables((const ChainShape *)C.tables.p, (int)ns, c->n, s));
+    CK(cudaStreamSynchronize(s));   // the host vectors may be rebuilt before the copies have run
+    c->launches += ns > 0;
+    C.key = key;
+    return STAB_OK;
+}
+
+int chain_run(stab_ctx *c, const ChainSet &C, const DevPlan &P, int n_vec, cudaStream_t s) {
+    ChainArgs a{};
+    a.steps[0] = (const ChainStep *)C.dev.p;
+    a.steps[1] = a.steps[0] + C.host[0].size();
+    for (int k = 0; k < 2; ++k) {
+        a.n_steps[k] = (int32_t)C.host[k].size();
+        a.ctas[k] = C.ctas[k];
+    }
+    if (a.ctas[0] + a.ctas[1] == 0) return STAB_OK;
+    a.n = c->n;
+    a.n_vec = n_vec;
+    a.tile_bits = chain_tile_bits(c->n);
+    a.maps = P.prog.pass_maps;
+    a.arrived = (uint32_t *)c->arrived.p;
+    a.status = (int32_t *)c->status.p;
+    CK(launch_stream_chain(a, s));
+    c->launches++;
     return STAB_OK;
 }
 
@@ -981,31 +1326,364 @@ int aligned_pass(const HostPlan &A, int k, const HostPlan &B) {
 }
 
 // The gradient of a plan with segment unitaries: only the slot -> rotations
-// table (rotations by their place in the run-ordered gate array).  Circuits
-// with an identity run without rotations have no such run in their gradient
-// plan; they keep the two-part sweep (stab_grad_parts tells the two apart).
+// table (rotations by their place in the run-ordered gate array).
 bool uni_grad_ok(const stab_ctx *c) {
-    return c->use_resident() && c->use_resident_adjoint() && c->fwd.uni && !c->fwd.uni_identity;
+    return c->use_resident() && c->use_resident_adjoint() && c->fwd.uni;
+}
+
+// Slot -> rotations, each by its place in the run-ordered gate array.
+void slot_table(const std::vector<RawGate> &g, int64_t n_params, HostPlan *H) {
+    H->param_ptr.assign((size_t)n_params + 1, 0);
+    for (const RawGate &r : g)
+        if (r.op >= STAB_RX) H->param_ptr[(size_t)r.param + 1]++;
+    for (int64_t j = 0; j < n_params; ++j)
+        H->param_ptr[(size_t)j + 1] += H->param_ptr[(size_t)j];
+    H->param_rot.resize((size_t)H->param_ptr[(size_t)n_params]);
+    std::vector<int32_t> at(H->param_ptr.begin(), H->param_ptr.end() - 1);
+    for (size_t k = 0; k < g.size(); ++k)
+        if (g[k].op >= STAB_RX) H->param_rot[(size_t)at[(size_t)g[k].param]++] = (int32_t)k;
 }
 
 int ensure_uni_grad(stab_ctx *c) {
     if (c->grad.built) return STAB_OK;
-    HostPlan &H = c->grad.host;
-    const std::vector<RawGate> &g = c->fwd.ugates;
-    H = HostPlan();
-    H.param_ptr.assign((size_t)c->n_params + 1, 0);
-    for (const RawGate &r : g)
-        if (r.op >= STAB_RX) H.param_ptr[(size_t)r.param + 1]++;
-    for (int64_t j = 0; j < c->n_params; ++j) H.param_ptr[(size_t)j + 1] += H.param_ptr[(size_t)j];
-    H.param_rot.resize((size_t)H.param_ptr[(size_t)c->n_params]);
-    std::vector<int32_t> at(H.param_ptr.begin(), H.param_ptr.end() - 1);
-    for (size_t k = 0; k < g.size(); ++k)
-        if (g[k].op >= STAB_RX) H.param_rot[(size_t)at[(size_t)g[k].param]++] = (int32_t)k;
+    c->grad.host = HostPlan();
+    slot_table(c->fwd.ugates, c->n_params, &c->grad.host);
     no_streams(c->grad);
     RC(upload_plan(c, c->grad));
     c->grad.encoded = true;
     CK(cudaEventRecord(c->ev_ready, c->st));
     return STAB_OK;
+}
+
+// ---------------------------------------------------------------- gradients from stored sweeps
+//
+// Streamed gradients (n >= 5).  rho goes forward through the whole plan and
+// lambda backward through it, each a chain of its own launches at once on two
+// streams, and every block of wire passes leaves its result in a slot of its
+// own; one launch then takes the three numbers c of every wire run from the
+// two vectors at its block's end (k_grad_dots), one turns them into the
+// rotations' derivatives.  Against carrying (lambda, rho) pairs from the
+// middle to both ends with every rotation's dot on the way: two sweeps of a
+// vector instead of three, six FMAs a group and run instead of three a
+// rotation, off the sequential chain, and runs of any length composed.
+
+const DevPlan &ck_plan(const stab_ctx *c) {
+    return !c->use_resident() && c->fwd.host.mode == PLAN_FUSED ? c->fwd : c->ck;
+}
+
+// The blocks, runs and jobs of the plan (host side, once per circuit).
+int ck_build(stab_ctx *c) {
+    const int n = c->n;
+    const bool own = &ck_plan(c) == &c->ck;
+    no_streams(c->ck);
+    if (own)
+        build_plan(n, c->gates.data(), (int64_t)c->gates.size(), c->n_params, PLAN_FUSED,
+                   &c->ck.host, true);
+    else
+        c->ck.host = HostPlan();
+    const HostPlan &H = ck_plan(c).host;
+    c->ck_blocks.clear();
+    c->ck_after.clear();
+    c->ck_jobs.clear();
+    c->ck_job_block.clear();
+    std::vector<RawGate> &gates = c->ck.ugates;
+    std::vector<int> between;
+    const int np = (int)H.passes.size();
+    c->ck.uni_max_run = 0;
+    for (int p = 0; p < np;) {
+        if (H.passes[(size_t)p].type != P_WIRE) {
+            between.push_back(p++);
+            continue;
+        }
+        stab_ctx::CkBlock b;
+        b.p0 = p;
+        b.before.swap(between);
+        std::vector<std::vector<int32_t>> wire((size_t)n);
+        for (; p < np && H.passes[(size_t)p].type == P_WIRE; ++p) {
+            std::vector<int32_t> &w = wire[H.passes[(size_t)p].q];
+            w.insert(w.end(), H.run_gates.begin() + H.run_first[(size_t)p],
+                     H.run_gates.begin() + H.run_first[(size_t)p + 1]);
+        }
+        b.p1 = p;
+        // a run per wire that holds a rotation, a job per tile_wires of them
+        std::vector<int> wires, runs;
+        auto flush = [&]() {
+            if (wires.empty()) return;
+            DotJob J{};
+            std::vector<int> tile, rest;
+            tile_bits_of(n, 1, wires, 1, std::min(kTileMaxBits, 2 * n), &tile, &rest);
+            J.n_wires = (int32_t)wires.size();
+            J.tile_bits = (int32_t)tile.size();
+            J.rest_bits = (int32_t)rest.size();
+            for (size_t w = 0; w < wires.size(); ++w) {
+                J.run[w] = runs[w];
+                J.lz[w] = (uint8_t)(std::find(tile.begin(), tile.end(), wires[w]) - tile.begin());
+                J.lx[w] =
+                    (uint8_t)(std::find(tile.begin(), tile.end(), n + wires[w]) - tile.begin());
+            }
+            bit_runs(tile, &J.tile_runs);
+            bit_runs(rest, &J.rest_runs);
+            c->ck_jobs.push_back(J);
+            c->ck_job_block.push_back((int)c->ck_blocks.size());
+            wires.clear();
+            runs.clear();
+        };
+        for (int q = 0; q < n; ++q) {
+            bool rotates = false;
+            for (int32_t g : wire[(size_t)q]) rotates |= c->gates[(size_t)g].op >= STAB_RX;
+            if (!rotates) continue;
+            UniRun r{(int32_t)gates.size(), (int32_t)wire[(size_t)q].size(), 0};
+            for (int32_t g : wire[(size_t)q]) {
+                const stab_gate &s = c->gates[(size_t)g];
+                gates.push_back({s.op, s.q0, s.q1, s.flags, s.param});
+            }
+            c->ck.uni_max_run = std::max(c->ck.uni_max_run, (int)r.count);
+            wires.push_back(q);
+            runs.push_back((int)c->ck.uruns.size());
+            c->ck.uruns.push_back(r);
+            if ((int)wires.size() == tile_wires(n)) flush();
+        }
+        flush();
+        c->ck_blocks.push_back(std::move(b));
+    }
+    c->ck_after = std::move(between);
+    const int64_t tiles = (int64_t)1 << std::max(0, 2 * n - kTileMaxBits);
+    const int64_t want = 16 * (int64_t)c->sms / std::max<int64_t>(1, (int64_t)c->ck_jobs.size()) + 1;
+    c->ck_chunks = (int)std::min<int64_t>(std::min<int64_t>(64, tiles), want);
+    HostPlan &K = c->ck.host;
+    if (!own) K.mode = PLAN_FUSED;
+    slot_table(gates, c->n_params, &K);
+    RC(upload_plan(c, c->ck));
+    c->ck.encoded = false;
+    c->ck_ready = true;
+    c->key_ck.clear();
+    c->g_grad.reset();
+    c->plan_gen++;
+    return STAB_OK;
+}
+
+// Slots of 4^n doubles: [0, B) rho at the end of each block, [B, 2 B) lambda at
+// its start, two spares of each chain, O, and one more wherever lambda passes
+// several Clifford passes in a row (the dots read it between them).
+constexpr size_t kCkSpares = 5;
+size_t ck_slots(const stab_ctx *c) {
+    size_t extra = kCkSpares;
+    for (const auto &b : c->ck_blocks) extra += b.before.size() > 1 ? b.before.size() - 1 : 0;
+    extra += c->ck_after.size() > 1 ? c->ck_after.size() - 1 : 0;
+    return 2 * c->ck_blocks.size() + extra;
+}
+
+// Whether the streamed gradient runs from stored sweeps: a circuit with
+// rotations whose slots fit (and could be allocated); else the pair sweep.
+bool ck_usable(stab_ctx *c, int *rc) {
+    *rc = STAB_OK;
+    if (c->ck_off || c->ck_bytes_max == 0 || c->n_params == 0) return false;
+    if (!c->ck_ready) *rc = ck_build(c);
+    if (*rc != STAB_OK) return false;
+    const size_t bytes = ck_slots(c) * c->vec_bytes();
+    if (c->ck_blocks.empty() || bytes > c->ck_bytes_max ||
+        c->dalloc(c->ckslots, bytes, c->aux) != STAB_OK) {
+        (void)cudaGetLastError();
+        c->ck_off = true;
+        return false;
+    }
+    return true;
+}
+
+// One block's wire passes from src (through Clifford pass `gather` unless
+// negative) into dst, a launch each.
+int ck_block(stab_ctx *c, const DevPlan &G, const stab_ctx::CkBlock &b, bool inverse,
+             const double *src, int gather, double *dst, cudaStream_t s) {
+    const int n = c->n, np = b.p1 - b.p0;
+    if (gather >= 0) {
+        CK(launch_gather(c, G, G.host.passes[(size_t)gather], inverse, src, dst, 1, s));
+        c->launches++;
+    } else if (src != dst) {
+        CK(cudaMemcpyAsync(dst, src, c->vec_bytes(), cudaMemcpyDeviceToDevice, s));
+    }
+    for (int k = 0; k < np; ++k)
+        CK(launch_stream_wire(dst, n, 1, G.host.passes[(size_t)(inverse ? b.p1 - 1 - k : b.p0 + k)],
+                              G.prog.ops, G.prog.maps, inverse, s));
+    c->launches += np;
+    return STAB_OK;
+}
+
+// Clifford passes between block b and the next one (or the end).
+const std::vector<int> &ck_between(const stab_ctx *c, int b) {
+    return b + 1 < (int)c->ck_blocks.size() ? c->ck_blocks[(size_t)b + 1].before : c->ck_after;
+}
+
+// The jobs' pointers into the slots, uploaded on s: block b's dots read lambda
+// through the first Clifford pass after the block.
+int ck_upload_jobs(stab_ctx *c, cudaStream_t s) {
+    const DevPlan &G = ck_plan(c);
+    const int B = (int)c->ck_blocks.size();
+    const double *slots = (const double *)c->ckslots.p;
+    const size_t E = (size_t)1 << (2 * c->n);
+    RC(c->dalloc(c->ckjobs, std::max<size_t>(1, c->ck_jobs.size()) * sizeof(DotJob), s));
+    const std::vector<const void *> key = {(const void *)c->plan_gen, slots, G.prog.pulls,
+                                           c->ckjobs.p};
+    if (key == c->key_ck || c->ck_jobs.empty()) return STAB_OK;
+    std::vector<size_t> src((size_t)B);
+    size_t extra = 2 * (size_t)B + kCkSpares;
+    for (int b = B - 1; b >= 0; --b) {
+        const size_t m = ck_between(c, b).size();
+        src[(size_t)b] = b == B - 1 ? 2 * (size_t)B + 4 : (size_t)(B + b + 1);
+        if (m > 1) {
+            extra += m - 1;
+            src[(size_t)b] = extra - 1;
+        }
+    }
+    for (size_t k = 0; k < c->ck_jobs.size(); ++k) {
+        const int b = c->ck_job_block[k];
+        const std::vector<int> &between = ck_between(c, b);
+        DotJob &J = c->ck_jobs[k];
+        J.rho = slots + (size_t)b * E;
+        J.lam = slots + src[(size_t)b] * E;
+        J.pull = between.empty() ? nullptr
+                                 : G.prog.pulls + 2 * G.host.pull_of[(size_t)between[0]] + 1;
+    }
+    CK(cudaMemcpyAsync(c->ckjobs.p, c->ck_jobs.data(), c->ck_jobs.size() * sizeof(DotJob),
+                       cudaMemcpyHostToDevice, s));
+    CK(cudaStreamSynchronize(s));   // ck_jobs may be rebuilt before the copy has run
+    c->key_ck = key;
+    return STAB_OK;
+}
+
+// The stored sweeps as two chains of steps: rho forward, lambda backward (the
+// slots as in ck_gradient).
+int ck_chains(stab_ctx *c, cudaStream_t s) {
+    const DevPlan &G = ck_plan(c);
+    const int B = (int)c->ck_blocks.size();
+    const size_t E = (size_t)1 << (2 * c->n), at = 2 * (size_t)B;
+    auto slot = [&](size_t k) { return (double *)c->ckslots.p + k * E; };
+    auto pull = [&](int p, bool inverse) {
+        return G.prog.pulls + 2 * G.host.pull_of[(size_t)p] + (inverse ? 1 : 0);
+    };
+    ChainSet &C = c->c_grad;
+    const std::vector<const void *> key = {(const void *)c->plan_gen, c->ckslots.p, G.buf.p};
+    if (C.key == key) return STAB_OK;
+    C.clear();
+    double *cur = c->ck_blocks[0].before.empty() ? slot(0) : slot(at);
+    for (int b = 0; b < B; ++b) {
+        const auto &blk = c->ck_blocks[(size_t)b];
+        for (size_t k = 0; k + 1 < blk.before.size(); ++k) {
+            double *to = cur == slot(at) ? slot(at + 1) : slot(at);
+            chain_step(c, G, {}, false, pull(blk.before[k], false), cur, to, &C, 0);
+            cur = to;
+        }
+        chain_block(c, G, blk.p0, blk.p1, false,
+                    blk.before.empty() ? nullptr : pull(blk.before.back(), false), cur,
+                    slot((size_t)b), &C, 0);
+        cur = slot((size_t)b);
+    }
+    cur = slot(at + 4);
+    size_t extra = at + kCkSpares;
+    for (int b = B - 1; b >= 0; --b) {
+        const auto &blk = c->ck_blocks[(size_t)b];
+        const std::vector<int> &between = ck_between(c, b);
+        for (size_t k = between.size(); k-- > 1;) {
+            chain_step(c, G, {}, true, pull(between[k], true), cur, slot(extra), &C, 1);
+            cur = slot(extra++);
+        }
+        chain_block(c, G, blk.p0, blk.p1, true, between.empty() ? nullptr : pull(between[0], true),
+                    cur, slot((size_t)(B + b)), &C, 1);
+        cur = slot((size_t)(B + b));
+    }
+    const std::vector<int> &lead = c->ck_blocks[0].before;
+    for (size_t k = lead.size(); k-- > 0;) {
+        double *to = cur == slot(at + 2) ? slot(at + 3) : slot(at + 2);
+        chain_step(c, G, {}, true, pull(lead[k], true), cur, to, &C, 1);
+        cur = to;
+    }
+    C.result[1] = cur;
+    return chain_upload(c, C, key, 1, s);
+}
+
+// The runs' numbers and the derivatives from the slots.
+int ck_finish(stab_ctx *c, cudaStream_t gs) {
+    CK(launch_grad_dots((const DotJob *)c->ckjobs.p, (int)c->ck_jobs.size(), c->n, c->ck_chunks,
+                        (double *)c->ckdots.p, gs));
+CK(launch_run_grads(c->ck.uruns_dev, (int)c->ck.uruns.size(), c->ck.uni_max_run,
+                        c->ck.ugates_dev, (const double *)c->thetas.p, (const double *)c->ckdots.p,
+                        c->ck_chunks, (double *)c->grad_rot.p, gs));
+    CK(launch_gather_grads((const double *)c->grad_rot.p, c->ck.param_ptr, c->ck.param_rot,
+                           (int)c->n_params, (double *)c->gbuf.p, gs));
+    c->launches += 2 + !c->ck_jobs.empty();
+    return STAB_OK;
+}
+
+// The launches of a gradient from stored sweeps, queued on gs (and aux2).
+int ck_gradient(stab_ctx *c, double *res, cudaStream_t gs) {
+    const DevPlan &G = ck_plan(c);
+    const int n = c->n, B = (int)c->ck_blocks.size();
+    const size_t E = (size_t)1 << (2 * n), at = 2 * (size_t)B;
+    auto slot = [&](size_t k) { return (double *)c->ckslots.p + k * E; };
+    auto gather = [&](const double *from, double *to, int p, bool inverse,
+                      cudaStream_t s) -> int {
+        CK(launch_gather(c, G, G.host.passes[(size_t)p], inverse, from, to, 1, s));
+        c->launches++;
+        return STAB_OK;
+    };
+    auto block = [&](int b, bool inverse, const double *from, int p, double *to,
+                     cudaStream_t s) -> int {
+        return ck_block(c, G, c->ck_blocks[(size_t)b], inverse, from, p, to, s);
+    };
+    if (use_chain(c, G, 1)) {
+        RC(ck_chains(c, gs));
+        const double *lam0 = c->c_grad.result[1];
+        CK(launch_fill(c->ck_blocks[0].before.empty() ? slot(0) : slot(at), n, 1, INIT_RHO0,
+                       nullptr, 0, gs));
+        CK(launch_fill(slot(at + 4), n, 1, INIT_TERMS, (const DevTerm *)c->terms.p,
+                       c->n_obs_terms, gs));
+        RC(chain_run(c, c->c_grad, G, 1, gs));
+        CK(launch_xfree_sum(lam0, n, 1, res, gs));
+        c->launches += (c->n_obs_terms ? 3 : 2) + 1;
+        return ck_finish(c, gs);
+    }
+    CK(cudaEventRecord(c->ev_fork, gs));
+    CK(cudaStreamWaitEvent(c->aux2, c->ev_fork, 0));
+    // rho forward
+    double *cur = c->ck_blocks[0].before.empty() ? slot(0) : slot(at);
+    CK(launch_fill(cur, n, 1, INIT_RHO0, nullptr, 0, gs));
+    c->launches++;
+    for (int b = 0; b < B; ++b) {
+        const std::vector<int> &before = c->ck_blocks[(size_t)b].before;
+        for (size_t k = 0; k + 1 < before.size(); ++k) {
+            double *to = cur == slot(at) ? slot(at + 1) : slot(at);
+            RC(gather(cur, to, before[k], false, gs));
+            cur = to;
+        }
+        RC(block(b, false, cur, before.empty() ? -1 : before.back(), slot((size_t)b), gs));
+        cur = slot((size_t)b);
+    }
+    // lambda backward
+    cudaStream_t s2 = c->aux2;
+    cur = slot(at + 4);
+    CK(launch_fill(cur, n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, c->n_obs_terms, s2));
+    c->launches += c->n_obs_terms ? 2 : 1;
+    size_t extra = at + kCkSpares;
+    for (int b = B - 1; b >= 0; --b) {
+        const std::vector<int> &between = ck_between(c, b);
+        for (size_t k = between.size(); k-- > 1;) {
+            RC(gather(cur, slot(extra), between[k], true, s2));
+            cur = slot(extra++);
+        }
+        RC(block(b, true, cur, between.empty() ? -1 : between[0], slot((size_t)(B + b)), s2));
+        cur = slot((size_t)(B + b));
+    }
+    // <O> = the x-free sum of lambda at the circuit's start
+    const std::vector<int> &lead = c->ck_blocks[0].before;
+    for (size_t k = lead.size(); k-- > 0;) {
+        double *to = cur == slot(at + 2) ? slot(at + 3) : slot(at + 2);
+        RC(gather(cur, to, lead[k], true, s2));
+        cur = to;
+    }
+    CK(launch_xfree_sum(cur, n, 1, res, s2));
+    c->launches++;
+    CK(cudaEventRecord(c->ev_join, c->aux2));
+    CK(cudaStreamWaitEvent(gs, c->ev_join, 0));
+    return ck_finish(c, gs);
 }
 
 int ensure_grad_plan(stab_ctx *c) {
@@ -1024,6 +1702,11 @@ int ensure_grad_plan(stab_ctx *c) {
         RC(upload_plan(c, c->grad));
     }
     if (!c->grad.encoded) RC(encode_plan(c, c->grad));
+    if (!c->grad.streams) {
+        // the pair sweep reads the ops, the first phase tiles where it may
+        RC(stream_ops(c, c->grad));
+        RC(stream_encode(c, c->grad, 1));
+    }
     CK(cudaEventRecord(c->ev_ready, c->st));
     return STAB_OK;
 }
@@ -1031,6 +1714,9 @@ int ensure_grad_plan(stab_ctx *c) {
 }  // namespace
 
 cudaStream_t stab::ctx_stream(stab_ctx *c) { return c ? c->st : nullptr; }
+void stab::ctx_no_checkpoints(stab_ctx *c) {
+    if (c) c->ck_bytes_max = 0;
+}
 
 extern "C" {
 
@@ -1314,6 +2000,8 @@ int create_ctx(int n, const stab_opts *opts, const stab_path_choice *forced, sta
     c->free = o.free;
     c->user = o.alloc_user;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && n >= kChainMinN)
+        c->chain_ctas = chain_max_ctas(1 << (chain_tile_bits(n) - 2));
     if (e == cudaSuccess) {
         c->device = dev;
         if (o.stream || o.stream_given) {
@@ -1384,7 +2072,9 @@ int stab_destroy(stab_ctx *c) {
                       &c->rho, &c->tmp, &c->tmp2, &c->terms, &c->scal, &c->grad_rot,
                       &c->partials, &c->grads, &c->status, &c->gbuf, &c->lam2, &c->tmp3,
                       &c->dotbuf, &c->umaps, &c->unodes, &c->ustates, &c->udots, &c->rmid,
-                      &c->lmid, &c->units_e, &c->cnt, &c->gmid};
+                      &c->lmid, &c->units_e, &c->cnt, &c->gmid, &c->ck.buf, &c->ckslots,
+                      &c->ckjobs, &c->ckdots, &c->c_gens.dev, &c->c_expect.dev, &c->c_grad.dev,
+                      &c->c_gens.tables, &c->c_expect.tables, &c->c_grad.tables, &c->arrived};
     for (DevBuf *b : bufs) c->dfree(*b, c->st);
     if (c->st) cudaStreamSynchronize(c->st);
     if (c->stage) cudaFreeHost(c->stage);
@@ -1417,6 +2107,7 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     c->n_params = n_params;
     c->grad.built = false;
     c->grad.encoded = false;
+    c->grad_ran = c->ck_ready = c->ck_off = false;
     reset_graphs(c);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
@@ -1456,6 +2147,7 @@ int stab_set_params(stab_ctx *c, const double *thetas, int is_device) {
     }
     RC(encode_plan(c, c->fwd));
     c->grad.encoded = false;
+    c->ck.encoded = false;
     c->gens_valid = false;
     c->param_gen++;
     CK(cudaEventRecord(c->ev_ready, c->st));
@@ -1501,11 +2193,24 @@ int stab_run_generators(stab_ctx *c) {
         c->gens_cur = (double *)c->gens.p;
     } else {
         RC(c->dalloc(c->gens_tmp, bytes, c->st));
+        RC(stream_encode(c, c->fwd, n));
         cudaStream_t s = c->aux;
         CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
         const std::vector<const void *> key = {(const void *)c->plan_gen, c->gens.p,
                                                c->gens_tmp.p};
-        RC(run_graph(c, c->g_gens, key, s, [&](cudaStream_t gs, void **result) {
+        if (use_chain_forward(c, c->fwd, n)) {
+            ChainSet &C = c->c_gens;
+            if (C.key != key) {
+                C.clear();
+                C.result[0] = chain_passes(c, c->fwd, (double *)c->gens.p, (double *)c->gens_tmp.p,
+                                           false, 0, (int)c->fwd.host.passes.size(), &C, 0);
+                RC(chain_upload(c, C, key, n, s));
+            }
+            CK(launch_fill((double *)c->gens.p, n, n, INIT_GENERATOR, nullptr, 0, s));
+            c->launches++;
+            RC(chain_run(c, C, c->fwd, n, s));
+            c->g_gens.result = C.result[0];
+        } else RC(run_graph(c, c->g_gens, key, s, [&](cudaStream_t gs, void **result) {
             double *cur = (double *)c->gens.p, *alt = (double *)c->gens_tmp.p;
             CK(launch_fill(cur, n, n, INIT_GENERATOR, nullptr, 0, gs));
             c->launches++;
@@ -1562,6 +2267,7 @@ int stab_expect_async(stab_ctx *c, double *out_dev) {
     if (!c->loaded || !c->obs_loaded) return STAB_E_STATE;
     CK(cudaSetDevice(c->device));
     cudaStream_t s = c->aux;
+    if (!c->use_resident()) RC(stream_encode(c, c->fwd, 1));
     CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
     const int32_t nt = c->n_obs_terms;
     if (c->use_resident() && c->fwd.uni) {
@@ -1616,7 +2322,24 @@ int stab_expect_async(stab_ctx *c, double *out_dev) {
                                                c->lam2.p, c->tmp3.p, c->dotbuf.p,
                                                c->terms.p, (const void *)(intptr_t)nt, res,
                                                (const void *)(intptr_t)split};
-        RC(run_graph(c, c->g_expect, key, s, [&](cudaStream_t gs, void **) {
+        if (split && use_chain_forward(c, c->fwd, 1)) {
+            ChainSet &C = c->c_expect;
+            double *lam = (double *)c->lam.p, *rho = (double *)c->lam2.p;
+            if (C.key != key) {
+                const int np = (int)c->fwd.host.passes.size(), mid = np / 2;
+                C.clear();
+                C.result[0] =
+                    chain_passes(c, c->fwd, lam, (double *)c->tmp.p, true, mid, np, &C, 0);
+                C.result[1] =
+                    chain_passes(c, c->fwd, rho, (double *)c->tmp3.p, false, 0, mid, &C, 1);
+                RC(chain_upload(c, C, key, 1, s));
+            }
+            CK(launch_fill(lam, c->n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, nt, s));
+            CK(launch_fill(rho, c->n, 1, INIT_RHO0, nullptr, 0, s));
+            RC(chain_run(c, C, c->fwd, 1, s));
+            CK(launch_dot(C.result[0], C.result[1], c->n, (double *)c->dotbuf.p, res, s));
+            c->launches += (nt ? 2 : 1) + 1 + 2;
+        } else RC(run_graph(c, c->g_expect, key, s, [&](cudaStream_t gs, void **) {
             double *cur = (double *)c->lam.p, *alt = (double *)c->tmp.p;
             if (!split) {
                 CK(launch_fill(cur, c->n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, nt, gs));
@@ -1671,11 +2394,45 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
     if (c->n_params > 0 && !grads_dev) return STAB_E_INVAL;
     CK(cudaSetDevice(c->device));
     c->grad_uni = uni_grad_ok(c);
-    RC(c->grad_uni ? ensure_uni_grad(c) : ensure_grad_plan(c));
+    int rc = STAB_OK;
+    const bool stored = !c->grad_uni && !c->use_resident_adjoint() && ck_usable(c, &rc);
+    RC(rc);
+    if (stored) {
+        DevPlan &G = &ck_plan(c) == &c->ck ? c->ck : c->fwd;
+        if (!G.encoded) RC(encode_plan(c, G));
+        RC(use_chain(c, G, 1) ? stream_maps(c, G) : stream_ops(c, G));
+        CK(cudaEventRecord(c->ev_ready, c->st));
+    } else {
+        RC(c->grad_uni ? ensure_uni_grad(c) : ensure_grad_plan(c));
+    }
+    c->grad_ran = true;
     cudaStream_t s = c->aux;
     CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
     const int32_t nt = c->n_obs_terms;
     const int n = c->n;
+    if (stored) {
+        RC(c->dalloc(c->scal, 64 * sizeof(double), s));
+        RC(c->dalloc(c->gbuf, (size_t)c->n_params * sizeof(double), s));
+        RC(c->dalloc(c->grad_rot, std::max<size_t>(1, c->ck.ugates.size()) * sizeof(double), s));
+        RC(c->dalloc(c->ckdots, std::max<size_t>(1, c->ck.uruns.size()) * 3 *
+                                    (size_t)c->ck_chunks * sizeof(double), s));
+        RC(ck_upload_jobs(c, s));
+        double *res = (double *)c->scal.p + 3;
+        const std::vector<const void *> key = {
+            (const void *)c->plan_gen, c->ckslots.p, c->ckjobs.p, c->ckdots.p, c->grad_rot.p,
+            c->gbuf.p, c->terms.p, (const void *)(intptr_t)nt, res, c->thetas.p, c->ck.buf.p};
+        // the chain is one launch; long vectors' launches are replayed from a graph
+        if (use_chain(c, ck_plan(c), 1)) RC(ck_gradient(c, res, s));
+        else RC(run_graph(c, c->g_grad, key, s,
+                          [&](cudaStream_t gs, void **) { return ck_gradient(c, res, gs); }));
+        CK(cudaMemcpyAsync(expect_dev ? expect_dev : (double *)c->scal.p + 1, res, sizeof(double),
+                           cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpyAsync(grads_dev, c->gbuf.p, (size_t)c->n_params * sizeof(double),
+                           cudaMemcpyDeviceToDevice, s));
+        CK(cudaEventRecord(c->ev_aux, s));
+        CK(cudaStreamWaitEvent(c->st, c->ev_aux, 0));
+        return STAB_OK;
+    }
     if (c->grad_uni) {
         // the states at the parts' boundaries, then every segment at once
         const DevPlan &P = c->fwd;
@@ -1693,9 +2450,10 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                              s));
         c->launches++;
         if (c->n_params > 0) {
-            CK(launch_uni_grad(n, P.uargs, psi, phi, (double *)c->udots.p, P.uruns_dev,
-                               (int)n_runs, P.uni_max_run, P.ugates_dev,
-                               (const double *)c->thetas.p, (double *)c->grad_rot.p, s));
+            CK(launch_uni_grad(n, P.uargs, psi, phi, (double *)c->udots.p, s));
+            CK(launch_run_grads(P.uruns_dev, (int)n_runs, P.uni_max_run, P.ugates_dev,
+                                (const double *)c->thetas.p, (const double *)c->udots.p, (int)D,
+                                (double *)c->grad_rot.p, s));
             CK(launch_gather_grads((const double *)c->grad_rot.p, c->grad.param_ptr,
                                    c->grad.param_rot, (int)c->n_params, grads_dev, s));
             c->launches += 2 + (n_runs > 0);
@@ -1799,7 +2557,8 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
             (const void *)c->plan_gen, c->lam.p, c->tmp.p, c->lam2.p, c->tmp3.p, c->partials.p,
             c->grad_rot.p, c->gbuf.p, c->terms.p, (const void *)(intptr_t)nt, res};
         {
-            // Split sweep.  The circuit's passes are cut in two halves at
+            // Pair sweep, for plans whose stored sweeps would not fit.  The
+            // circuit's passes are cut in two halves at
             // `mid`.  Phase 1, two branches at once: r forward through the
             // first half, lambda backward through the second; both meet at
             // `mid`.  Phase 2, two branches at once: the pair (lambda, r)
@@ -1838,7 +2597,7 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                                (forward ? 0 : 1);
                     };
                     auto gather_now = [&]() -> int {
-                        CK(launch_stream_pull(pr, al, n, 2, pull_of(pending), st));
+                        CK(launch_gather(c, c->grad, *pending, forward ? 0 : 1, pr, al, 2, st));
                         c->launches++;
                         std::swap(pr, al);
                         pending = nullptr;
@@ -1858,7 +2617,7 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
                             return STAB_OK;
                         }
                         TileGroup tg;
-                        make_tile_group(n, 1, group, forward ? 0 : 1, &tg, nb,
+                        make_tile_group(n, 1, passes, group, forward ? 0 : 1, &tg, nb,
                                         std::min(kAdjTileBits, 2 * n));
                         for (size_t j = 0; j < group.size(); ++j) {
                             int nr = 0;
@@ -1992,6 +2751,7 @@ int stab_density_matrix(stab_ctx *c, double *out, int out_is_device) {
         c->launches++;
     } else {
         RC(c->dalloc(c->tmp2, vb, c->st));
+        RC(stream_encode(c, c->fwd, 1));
         double *cur = r, *alt = (double *)c->tmp2.p;
         CK(launch_fill(cur, n, 1, INIT_RHO0, nullptr, 0, c->st));
         c->launches++;
@@ -2043,7 +2803,9 @@ int64_t stab_launch_count(stab_ctx *c) { return c ? c->launches : 0; }
 
 int stab_grad_parts(stab_ctx *c, int32_t *parts) {
     if (!c || !parts) return STAB_E_INVAL;
-    *parts = !c->grad.built ? 0 : c->grad_uni ? (int32_t)c->fwd.uparts.size() : 1;
+    *parts = !c->grad_ran                              ? 0
+             : c->grad_uni && !c->fwd.uni_identity ? (int32_t)c->fwd.uparts.size()
+                                                   : 1;
     return STAB_OK;
 }
 

@@ -95,6 +95,7 @@ struct Program {
     const DevOp *ops;
     const DevMap3 *maps;
     const DevPull *pulls;
+    const DevMap3 *pass_maps;   // per pass: a wire pass's run composed (tile launches)
     int32_t n_passes;
     int32_t n_ops;
 };

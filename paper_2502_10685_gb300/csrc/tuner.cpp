@@ -284,12 +284,15 @@ int measure(int device, const stab_opts *like, int n, stab_path_choice *out) {
         for (int r = 0; r < 2; ++r) {
             stab_path_choice c = d;
             c.resident = c.resident_adjoint = r;
-            int rc = time_op(device, like, P, c, PR_EXPECT, &t[0][r]);
+            int rc = n == 6 ? time_op(device, like, P, c, PR_EXPECT, &t[0][r]) : STAB_OK;
             if (rc == STAB_OK) rc = time_op(device, like, P, c, PR_GRAD, &t[1][r]);
             if (rc != STAB_OK) return rc;
         }
-        // the defaults are resident; streamed only when clearly faster
-        d.resident = clearly_faster(t[0][0], t[0][1]) ? 0 : 1;
+        // the defaults are resident; streamed only when clearly faster.  (n = 5:
+        // <O> of a layered circuit is a sixth faster streamed, but the generators
+        // and circuits of short runs up to twice slower, and the choice covers
+        // them all.)
+        if (n == 6) d.resident = clearly_faster(t[0][0], t[0][1]) ? 0 : 1;
         d.resident_adjoint = clearly_faster(t[1][0], t[1][1]) ? 0 : 1;
     } else if (n >= 7 && n <= 9) {
         P.m = n == 7 ? 400 : (n == 8 ? 300 : 200);

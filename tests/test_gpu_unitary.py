@@ -99,3 +99,20 @@ def test_long_clifford_circuits_stay_bit_exact(stab, n, m):
     obs = W.obs_chain(n)
     assert s.expect(obs) == oracle.expect(n, c.gates, c.thetas, obs)
     s.close()
+
+
+@pytest.mark.parametrize("n,m", [(1, 1023), (1, 1024), (1, 5000), (2, 40000)])
+def test_runs_of_thousands_of_gates(stab, n, m):
+    # one wire run of m gates per qubit, composed by a CTA
+    c = W.random_circuit(1, m, seed=920 + m)
+    gates = np.concatenate([c.gates] * n)
+    for q in range(n):
+        gates["q0"][q * m:(q + 1) * m] = q
+    obs = [(1.0, "Z" * n), (0.5, "X" + "I" * (n - 1)), (-0.25, "Y" * n)]
+    s = stab.Stab(n)
+    s.apply_circuit(gates, c.thetas)
+    tol = 1e-10 if m >= 40000 else 1e-12
+    assert np.abs(layout.lib_to_paper(n, s.generators())
+                  - oracle.generators(n, gates, c.thetas)).max() <= tol
+    assert abs(s.expect(obs) - oracle.expect(n, gates, c.thetas, obs)) <= 1.75 * tol
+    s.close()
