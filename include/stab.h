@@ -241,7 +241,9 @@ int stab_expect_static(int n, const stab_gate *gates, int64_t m, const double *t
 /* Many independent circuits of different sizes evaluated by one persistent
  * launch (replayed from a CUDA graph): every generator of a generator item
  * and the observable of an expectation item is one unit of work; CTAs take
- * units longest first.  The 2m parameter-shift copies of a circuit (Sec. I)
+ * units longest first.  (AUTO: items of n >= 6 so much longer than the rest that
+ * one CTA would still be at them when all others are done run on many SMs, in
+ * a second launch beside it.)  The 2m parameter-shift copies of a circuit (Sec. I)
  * are expectation items that differ only in their angles. */
 #define STAB_BATCH_MAX_QUBITS 8
 

@@ -5,7 +5,7 @@
 // host-to-device copy), encodes every rotation and map with one launch, and
 // builds the unit table (one unit per propagated vector) sorted longest
 // first.  Run replays a CUDA graph holding the counter reset and the
-// persistent launch.
+// persistent launch, beside a second one for the long items (pick_long).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,6 +20,7 @@
 #include "host_pool.h"
 #include "launch.h"
 #include "planner.h"
+#include "tuner.h"
 
 using namespace stab;
 
@@ -59,6 +60,20 @@ struct stab_batch {
     const BatchUnit *units_dev = nullptr;
     cudaGraphExec_t graph = nullptr;
     bool ran = false;
+
+    // long items: their contexts, chains and the chains' launch
+    struct LongItem {
+        int64_t item;
+        bool gens;
+        stab_ctx *ctx;
+    };
+    std::vector<LongItem> longs;
+    int n_long_units = 0, n_chains = 0, chain_grid = 0;
+    Buf chains;                       // descriptors, then 128 bytes of counter each
+    size_t chains_at = 0;             // of the counters
+    cudaStream_t st2 = nullptr;
+    cudaEvent_t ev_long = nullptr;
+    cudaGraphExec_t graph_long = nullptr;
 
     int dalloc(Buf &b, size_t bytes) {
         bytes = up256(bytes ? bytes : 256);
@@ -202,6 +217,143 @@ int autotune(stab_batch *b, int sms, const std::vector<Residency> &res) {
     return STAB_OK;
 }
 
+// Items whose vectors would outlast the rest of the batch on one CTA each: of
+// n = 6 .. 8, longest first, while one unit takes more than twice the time the
+// remaining work takes spread over the SMs (and half a millisecond, so that the
+// launches around its chains pay).  Such an item runs as chains of tile steps
+// on many SMs (k_stream_chain), all of them in one launch beside the persistent
+// kernel.  576 uneven circuits with 24 generator items, n = 2 .. 8, to 8,000 gates:
+// 123.6 -> 5.2 ms, the deepest n = 8 item alone 116 of them before; a batch of
+// thousands has no such item.  cost: a unit's chunks x 4^n, 16 ns each (n = 6: 66
+// us a chunk of 25 passes).
+constexpr double kCostNs = 16.0;
+std::vector<int64_t> pick_long(const stab_batch_item *items, const std::vector<int64_t> &cost,
+                               int sms, int max_chains) {
+    double left = 0.0;
+    std::vector<int64_t> order;
+    for (size_t k = 0; k < cost.size(); ++k) {
+        const int units = items[k].kind == STAB_ITEM_GENERATORS ? items[k].n : 1;
+        left += (double)cost[k] * units;
+        if (items[k].n >= 6 && (double)cost[k] * kCostNs >= 5e5) order.push_back((int64_t)k);
+    }
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int64_t x, int64_t y) { return cost[(size_t)x] > cost[(size_t)y]; });
+    std::vector<int64_t> out;
+    for (int64_t k : order) {
+        if ((double)cost[(size_t)k] * sms <= 2.0 * left || 2 * (int)out.size() + 2 > max_chains)
+            break;
+        const int units = items[k].kind == STAB_ITEM_GENERATORS ? items[k].n : 1;
+        left -= (double)cost[(size_t)k] * units;
+        out.push_back(k);
+    }
+    return out;
+}
+
+// Contexts, chains and descriptors of the long items.
+int build_long(stab_batch *b, const stab_batch_item *items, const std::vector<int64_t> &longs) {
+    const int budget = chain_max_ctas(128) / 2;   // the persistent kernel's CTAs fit beside them
+    std::vector<ChainDesc> chains;
+    std::vector<double> work;
+    for (int64_t it : longs) {
+        const stab_batch_item &I = items[it];
+        stab_opts o;
+        stab_default_opts(&o);
+        o.device = b->device;
+        o.kernel = STAB_KERNEL_AUTO;
+        o.stream = (void *)b->st;
+        o.stream_given = 1;
+        o.alloc = b->alloc;
+        o.free = b->free;
+        o.alloc_user = b->user;
+        stab_path_choice choice;
+        BRC(stab_path_defaults(I.n, &choice));
+        choice.resident = 0;
+        choice.tile_limit = (int64_t)I.n << (2 * I.n);
+        stab_batch::LongItem L{it, I.kind == STAB_ITEM_GENERATORS, nullptr};
+        BRC(create_with_choice(I.n, &o, &choice, &L.ctx));
+        b->longs.push_back(L);
+        BRC(stab_load_circuit(L.ctx, I.gates, I.m, I.thetas, I.n_params));
+        if (!L.gens) BRC(stab_set_observable(L.ctx, I.obs, I.n_terms));
+        const ChainDesc *c = nullptr;
+        int nc = 0;
+        BRC(long_item_prepare(L.ctx, L.gens, 1 << 20, &c, &nc));
+        for (int k = 0; k < nc; ++k) {   // ctas: one per tile and vector
+            chains.push_back(c[k]);
+            work.push_back((double)c[k].n_steps * c[k].ctas);
+        }
+        b->n_long_units += L.gens ? I.n : 1;
+    }
+    b->n_chains = (int)chains.size();
+    if (chains.empty()) return STAB_OK;
+    // CTAs in proportion to each chain's work, so that the chains end together,
+    // at least one and at most one per tile
+    double lo = 0.0, hi = 1e9;
+    auto ctas = [&](double f, size_t k) {
+        return std::max(1, (int)std::min<double>(chains[k].ctas, f * work[k]));
+    };
+    for (int r = 0; r < 80; ++r) {
+        const double f = 0.5 * (lo + hi);
+        int64_t sum = 0;
+        for (size_t k = 0; k < chains.size(); ++k) sum += ctas(f, k);
+        if (sum <= budget) lo = f;
+        else hi = f;
+    }
+    const size_t desc_bytes = up256(chains.size() * sizeof(ChainDesc));
+    BRC(b->dalloc(b->chains, desc_bytes + 128 * chains.size()));
+    b->chains_at = desc_bytes;
+    b->chain_grid = 0;
+    for (size_t k = 0; k < chains.size(); ++k) {
+        chains[k].ctas = ctas(lo, k);
+        chains[k].cta0 = b->chain_grid;
+        chains[k].arrived = (uint32_t *)((char *)b->chains.p + desc_bytes + 128 * k);
+        b->chain_grid += chains[k].ctas;
+    }
+    BCK(cudaMemcpyAsync(b->chains.p, chains.data(), chains.size() * sizeof(ChainDesc),
+                        cudaMemcpyHostToDevice, b->st));
+    BCK(cudaStreamSynchronize(b->st));
+    BCK(cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking));
+    BCK(cudaEventCreateWithFlags(&b->ev_long, cudaEventDisableTiming));
+    return STAB_OK;
+}
+
+// The long items' launches on st2.
+int queue_long(stab_batch *b) {
+    for (const auto &L : b->longs) BRC(long_item_fill(L.ctx, L.gens, b->st2));
+    BCK(cudaMemsetAsync((char *)b->chains.p + b->chains_at, 0, 128 * (size_t)b->n_chains, b->st2));
+    ChainArgs a{};
+    a.chains = (const ChainDesc *)b->chains.p;
+    a.n_chains = b->n_chains;
+    a.grid = b->chain_grid;
+    a.tile_bits = 9;
+    a.status = (int32_t *)b->counter.p + 32;
+    BCK(launch_stream_chain(a, b->st2));
+    for (const auto &L : b->longs) {
+        double *out = L.gens ? (double *)b->gens.p + b->gen_off[(size_t)L.item]
+                             : (double *)b->exps.p + L.item;
+        BRC(long_item_finish(L.ctx, L.gens, out, b->st2));
+    }
+    return STAB_OK;
+}
+
+int launch_long(stab_batch *b) {
+    if (!b->graph_long) {
+        cudaGraph_t g = nullptr;
+        BCK(cudaStreamBeginCapture(b->st2, cudaStreamCaptureModeThreadLocal));
+        const int rc = queue_long(b);
+        const cudaError_t e = cudaStreamEndCapture(b->st2, &g);
+        if (rc != STAB_OK || e != cudaSuccess) {
+            if (g) cudaGraphDestroy(g);
+            if (rc != STAB_OK) return rc;
+            BCK(e);
+        }
+        const cudaError_t e2 = cudaGraphInstantiate(&b->graph_long, g, 0);
+        cudaGraphDestroy(g);
+        BCK(e2);
+    }
+    BCK(cudaGraphLaunch(b->graph_long, b->st2));
+    return STAB_OK;
+}
+
 int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel) {
     std::vector<Rec> recs;
     std::vector<int32_t> enc;
@@ -261,6 +413,22 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
         for (auto &t : pool) t.join();
     }
     for (int64_t it = 0; it < count; ++it) BRC(plans[(size_t)it].rc);
+    int sms = 0;
+    BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
+    // long items leave the persistent kernel's tables
+    std::vector<int64_t> longs;
+    std::vector<char> is_long((size_t)count, 0);
+    if (kernel == STAB_KERNEL_AUTO && chain_max_ctas(128) > 0) {
+        std::vector<int64_t> cost((size_t)count);
+        for (int64_t it = 0; it < count; ++it)
+            cost[(size_t)it] = (int64_t)(plans[(size_t)it].S.size() / kChunkRecs)
+                               << (2 * items[it].n);
+        longs = pick_long(items, cost, sms, chain_max_ctas(128) / 4);
+        for (int64_t it : longs) {
+            is_long[(size_t)it] = 1;
+            plans[(size_t)it] = ItemPlan();
+        }
+    }
     // Concatenation in item order: offsets first, then every item's records,
     // maps and gate indices copied (references offset) on the host pool.
     struct Off {
@@ -276,7 +444,7 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
         tot.map += (int64_t)ip.P.maps.size();
         tot.midx += (int64_t)ip.P.map_gate_idx.size();
         tot.raw += (int64_t)ip.P.raw.size();
-        tot.th += items[it].n_params;
+        tot.th += is_long[(size_t)it] ? 0 : items[it].n_params;
         tot.term += (int64_t)ip.t.size();
     }
     if (tot.rec > (int64_t)INT32_MAX / 2) return STAB_E_RANGE;
@@ -322,7 +490,9 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
                         if (g.op >= STAB_RX) g.param += (int32_t)o.th;
                         raw[(size_t)o.raw + i] = g;
                     }
-                    std::copy(I.thetas, I.thetas + I.n_params, thetas.begin() + (ptrdiff_t)o.th);
+                    if (!is_long[(size_t)it])
+                        std::copy(I.thetas, I.thetas + I.n_params,
+                                  thetas.begin() + (ptrdiff_t)o.th);
                     std::copy(ip.t.begin(), ip.t.end(), terms.begin() + (ptrdiff_t)o.term);
                 }
             });
@@ -333,6 +503,13 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
         const stab_batch_item &I = items[it];
         b->item_n[it] = I.n;
         b->item_kind[it] = I.kind;
+        if (is_long[(size_t)it]) {
+            if (I.kind == STAB_ITEM_GENERATORS) {
+                b->gen_off[it] = gens_doubles;
+                gens_doubles += (int64_t)I.n << (2 * I.n);
+            }
+            continue;
+        }
         b->max_n = std::max(b->max_n, (int)I.n);
         const ItemPlan &ip = plans[(size_t)it];
         const Off &o = off[(size_t)it];
@@ -422,11 +599,9 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
     // 5 and 4 (less shared memory per CTA, so more CTAs per SM, at the cost of
     // n = 5, 6 vectors in L2-resident slabs); the autotuner times them.
     // RESIDENT keeps min(max n, 6); STREAMED takes 4 (every n >= 5 vector in a slab).
-    int sms = 0;
-    BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
     std::vector<Residency> res;
     const int top = std::min(b->max_n, kMaxResidentQubits);
-    const int lo = kernel == STAB_KERNEL_AUTO ? std::max(4, top - 2)
+    const int lo = kernel == STAB_KERNEL_AUTO ? std::min(top, std::max(4, top - 2))
                    : kernel == STAB_KERNEL_STREAMED ? std::min(4, top) : top;
     const int hi = kernel == STAB_KERNEL_STREAMED ? std::min(4, top) : top;
     for (int sn = hi; sn >= lo; --sn) {
@@ -448,10 +623,10 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
     b->smem_n = res[0].smem_n;
     b->smem = res[0].smem;
     b->ctas_per_sm = res[0].max_occ;
-    if (kernel == STAB_KERNEL_AUTO && (res.size() > 1 || res[0].max_occ > 1))
+    if (kernel == STAB_KERNEL_AUTO && b->n_units > 0 && (res.size() > 1 || res[0].max_occ > 1))
         BRC(autotune(b, sms, res));
     b->grid = sms * b->ctas_per_sm;
-    return STAB_OK;
+    return build_long(b, items, longs);
 }
 
 }  // namespace
@@ -512,7 +687,16 @@ int stab_batch_run(stab_batch *b) {
         BCK(cudaEventRecord(b->ev_in, b->user_st));
         BCK(cudaStreamWaitEvent(b->st, b->ev_in, 0));
     }
-    BRC(launch_graph_or_direct(b, a, b->grid, true));
+    if (b->n_chains > 0) {
+        // first, so that the chains' CTAs find room beside the persistent kernel's
+        // (and after everything queued so far that may read the results)
+        BCK(cudaEventRecord(b->ev_out, b->st));
+        BCK(cudaStreamWaitEvent(b->st2, b->ev_out, 0));
+        BRC(launch_long(b));
+        BCK(cudaEventRecord(b->ev_long, b->st2));
+    }
+    if (b->n_units > 0) BRC(launch_graph_or_direct(b, a, b->grid, true));
+    if (b->n_chains > 0) BCK(cudaStreamWaitEvent(b->st, b->ev_long, 0));
     if (b->has_user_st) {
         BCK(cudaEventRecord(b->ev_out, b->st));
         BCK(cudaStreamWaitEvent(b->user_st, b->ev_out, 0));
@@ -567,7 +751,7 @@ int stab_batch_generators(stab_batch *b, int64_t item, double *out, int out_is_d
 int stab_batch_info(stab_batch *b, int64_t *units, int32_t *grid, int32_t *ctas_per_sm,
                     int32_t *smem_max_n) {
     if (!b) return STAB_E_INVAL;
-    if (units) *units = b->n_units;
+    if (units) *units = b->n_units + b->n_long_units;
     if (grid) *grid = b->grid;
     if (ctas_per_sm) *ctas_per_sm = b->ctas_per_sm;
     if (smem_max_n) *smem_max_n = b->smem_n;
@@ -578,7 +762,13 @@ int stab_batch_destroy(stab_batch *b) {
     if (!b) return STAB_OK;
     cudaSetDevice(b->device);
     if (b->st) cudaStreamSynchronize(b->st);
+    if (b->st2) cudaStreamSynchronize(b->st2);
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    if (b->graph_long) cudaGraphExecDestroy(b->graph_long);
+    for (const auto &L : b->longs) stab_destroy(L.ctx);
+    if (b->ev_long) cudaEventDestroy(b->ev_long);
+    if (b->st2) cudaStreamDestroy(b->st2);
+    b->dfree(b->chains);
     b->dfree(b->data);
     b->dfree(b->gens);
     b->dfree(b->exps);

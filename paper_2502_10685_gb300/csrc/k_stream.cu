@@ -503,15 +503,19 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
     __shared__ __align__(16) double smap[2][kTileMaxPasses * 9];
     __shared__ double solo[2][ALONE ? 1 << kTileMaxBits : 1];
     __shared__ ChainStep S[3];
+    __shared__ ChainDesc C;
     __shared__ int s_ok;
-    const int ch = (int)blockIdx.x < a.ctas[0] ? 0 : 1;
-    const uint32_t rank = blockIdx.x - (ch ? (uint32_t)a.ctas[0] : 0u);
-    const uint32_t ctas = (uint32_t)(ch ? a.ctas[1] : a.ctas[0]);
-    const int n_steps = ch ? a.n_steps[1] : a.n_steps[0];
-    const ChainStep *steps = ch ? a.steps[1] : a.steps[0];
-    uint32_t *arrived = a.arrived + 32 * ch;
     const uint32_t t = threadIdx.x;              // one group: blockDim.x = 2^tile_bits / 4
-    const int n = a.n;
+    for (int k = (int)t; k < a.n_chains; k += (int)blockDim.x) {
+        const int c0 = a.chains[k].cta0;
+        if ((int)blockIdx.x >= c0 && (int)blockIdx.x < c0 + a.chains[k].ctas) C = a.chains[k];
+    }
+    __syncthreads();
+    const uint32_t rank = blockIdx.x - (uint32_t)C.cta0, ctas = (uint32_t)C.ctas;
+    const int n_steps = C.n_steps, n_vec = C.n_vec, n = C.n;
+    const ChainStep *steps = C.steps;
+    const DevMap3 *all_maps = C.maps;
+    uint32_t *arrived = C.arrived;
     const uint64_t E = 1ull << (2 * n);
     const uint32_t zmask = (1u << n) - 1u;
     constexpr uint32_t kWords = sizeof(ChainStep) / 4;   // <= blockDim.x
@@ -531,7 +535,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
             r01 = d.pull->r0;
             r11 = d.pull->r1;
         }
-        if ((rank >> d.rest_bits) < (uint32_t)a.n_vec) {
+        if ((rank >> d.rest_bits) < (uint32_t)n_vec) {
             const uint4 *p = d.tiles + 4ull * (rank & ((1u << d.rest_bits) - 1u));
 #pragma unroll
             for (int k = 0; k < 4; ++k) tk1[k] = p[k];
@@ -539,7 +543,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
         // thread (j, e) holds entry e of pass j's map, transposed (the inverse)
         // for backward sweeps
         if (mj < (uint32_t)d.n_pass)
-            mval = a.maps[d.map[mj]].m[d.inverse ? (me % 3u) * 3u + me / 3u : me];
+            mval = all_maps[d.map[mj]].m[d.inverse ? (me % 3u) * 3u + me / 3u : me];
     };
     auto land = [&](int s) {   // fetched values of step s become current
         in_t = in_t1;
@@ -567,7 +571,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
         const int n_pass = st.n_pass;
         const bool pulled = st.pull != nullptr;
         const double *maps = smap[s & 1];
-        const uint64_t tiles = (uint64_t)a.n_vec << st.rest_bits;
+        const uint64_t tiles = (uint64_t)n_vec << st.rest_bits;
         bool first = true;
         for (uint64_t tb = rank; tb < tiles; tb += ctas) {
             const uint64_t v = tb >> st.rest_bits;
@@ -848,18 +852,15 @@ cudaError_t launch_chain_tables(const ChainShape *shapes, int n_shapes, int n, c
 
 cudaError_t launch_stream_chain(const ChainArgs &a, cudaStream_t st) {
     const int threads = 1 << (a.tile_bits - 2);
-    if (a.n < kChainMinN || threads < (int)(sizeof(ChainStep) / 4) ||
+    if (a.n_chains < 1 || threads < (int)(sizeof(ChainStep) / 4) ||
         threads < 9 * kTileMaxPasses || threads > kTileThreads)
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(a.arrived, 0, 256, st);
-    if (e != cudaSuccess) return e;
     ChainArgs args = a;
     void *params[] = {&args};
-    const bool alone = a.n_vec == 1 && a.tile_bits == 2 * a.n && a.ctas[0] <= 1 && a.ctas[1] <= 1;
-    return cudaLaunchCooperativeKernel(alone ? (const void *)k_stream_chain<true>
-                                             : (const void *)k_stream_chain<false>,
-                                       dim3((unsigned)(a.ctas[0] + a.ctas[1])),
-                                       dim3((unsigned)threads), params, 0, st);
+    return cudaLaunchCooperativeKernel(a.alone ? (const void *)k_stream_chain<true>
+                                               : (const void *)k_stream_chain<false>,
+                                       dim3((unsigned)a.grid), dim3((unsigned)threads), params, 0,
+                                       st);
 }
 
 cudaError_t launch_dot(const double *a, const double *b, int n, double *partial, double *out,

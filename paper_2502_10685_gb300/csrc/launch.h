@@ -283,8 +283,8 @@ cudaError_t launch_stream_tile(const double *src, double *dst, int n, int n_vec,
                                const TileGroup &tg, const DevMap3 *maps, const DevOp *ops,
                                cudaStream_t st);
 
-// Whole sequences of tile steps in one cooperative launch: up to two chains of
-// steps, each a number of CTAs that meet at a barrier after every step.  A
+// Whole sequences of tile steps in one cooperative launch: independent chains
+// of steps, each a number of CTAs that meet at a barrier after every step.  A
 // step gathers a tile, applies its passes and stores it.  Where each thread
 // reads and writes is tabulated per shape (tile geometry, the wire whose groups
 // the threads hold, the Clifford gather read through), so the chain only looks
@@ -314,13 +314,19 @@ struct ChainStep {                      // 128 bytes
     uint32_t map[kTileMaxPasses];
 };
 static_assert(sizeof(ChainStep) == 128, "ChainStep layout");
-struct ChainArgs {
-    const ChainStep *steps[2];          // device
-    int32_t n_steps[2];
-    int32_t ctas[2];
-    int32_t n, n_vec, tile_bits;
+struct ChainDesc {                      // one chain, 64 bytes
+    const ChainStep *steps;             // device
     const DevMap3 *maps;
-    uint32_t *arrived;                  // two counters 128 bytes apart, zeroed before the launch
+    uint32_t *arrived;                  // its counter (128 bytes of its own), zero before the launch
+    int32_t n_steps, n, n_vec;
+    int32_t cta0, ctas;                 // its CTAs: [cta0, cta0 + ctas)
+    int32_t pad[5];
+};
+static_assert(sizeof(ChainDesc) == 64, "ChainDesc layout");
+struct ChainArgs {
+    const ChainDesc *chains;            // device
+    int32_t n_chains, grid, tile_bits;  // tiles of 2^tile_bits entries in every chain
+    bool alone;                         // every chain one CTA, one vector, one tile
     int32_t *status;
 };
 constexpr int kChainMinN = 5;           // tiles of at least 2^9 entries
@@ -499,4 +505,17 @@ namespace stab {
 // <0^n| U^dagger O U |0^n> for the loaded circuit, O given as nt deduplicated
 // device terms (stab_api.cpp); blocks until the value is on the host.
 int expect_device_terms(stab_ctx *c, const DevTerm *terms, int64_t nt, double *out);
+}  // namespace stab
+
+namespace stab {
+// Items of a batch whose vectors are too long for one CTA each: a context of
+// the streamed kernels (loaded, observable set) gives its chains of tile steps,
+// which the batch runs together with its other long items' in one launch.
+// gens: the n generators, else <O>.  prepare: buffers, maps, steps; *chains
+// (host, the context's) with cta0 and ctas for max_ctas CTAs alone.  Per run:
+// fill, the chains, finish (out: 8 bytes, or n 4^n doubles).
+int long_item_prepare(stab_ctx *c, bool gens, int max_ctas, const ChainDesc **chains,
+                      int *n_chains);
+int long_item_fill(stab_ctx *c, bool gens, cudaStream_t s);
+int long_item_finish(stab_ctx *c, bool gens, double *out, cudaStream_t s);
 }  // namespace stab

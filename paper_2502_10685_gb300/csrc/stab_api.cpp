@@ -172,7 +172,11 @@ struct ChainSet {
         }
     }
     DevBuf dev, tables;
-    int ctas[2] = {0, 0};
+    ChainDesc desc[2];                        // of the chains with steps, in order
+    int n_chains = 0, grid = 0;
+    const ChainDesc *desc_dev = nullptr;
+    uint32_t *arrived = nullptr;              // 32 words per chain
+    bool alone = false;
     double *result[2] = {nullptr, nullptr};   // where each chain's vectors end up
 };
 
@@ -242,7 +246,6 @@ struct stab_ctx {
     DevBuf status;                   // int32 set by kernels whose bounded waits gave up
     GraphCache g_gens, g_expect, g_grad; // streamed launch sequences (n > resident sizes)
     ChainSet c_gens, c_expect, c_grad;   // the same as one launch, small vectors
-    DevBuf arrived;
     int64_t plan_gen = 0;            // bumped whenever a plan is rebuilt
     int32_t n_obs_terms = 0;
     bool obs_loaded = false;
@@ -1188,38 +1191,53 @@ double *chain_passes(const stab_ctx *c, const DevPlan &P, double *cur, double *a
 }
 
 // Builds the shapes' tables, uploads both chains' steps (on s) and sizes their
-// CTAs.
-int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key, int n_vec,
-                 cudaStream_t s) {
+// CTAs: one per tile, as far as max_ctas allows for all chains together.
+int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
+                 const DevPlan &P, int n_vec, int max_ctas, cudaStream_t s) {
     const size_t n0 = C.host[0].size(), n1 = C.host[1].size(), ns = C.shapes.size();
     const size_t groups = (size_t)1 << (chain_tile_bits(c->n) - 2);
     const size_t tiles = (size_t)1 << (2 * c->n - chain_tile_bits(c->n));
     const size_t per = groups * sizeof(uint2) + 4 * tiles * sizeof(uint4);
     const size_t b_shapes = align256(ns * sizeof(ChainShape));
+    const size_t b_steps = align256((n0 + n1) * sizeof(ChainStep));
     RC(c->dalloc(C.tables, b_shapes + ns * per, s));
-    RC(c->dalloc(C.dev, std::max<size_t>(1, n0 + n1) * sizeof(ChainStep), s));
-    RC(c->dalloc(c->arrived, 256, s));
+    RC(c->dalloc(C.dev, b_steps + 256 + 2 * 128, s));
     char *base = (char *)C.tables.p + b_shapes;
     for (size_t k = 0; k < ns; ++k) {
         C.shapes[k].tiles = (uint4 *)(base + k * per);
         C.shapes[k].threads = (uint2 *)(base + k * per + 4 * tiles * sizeof(uint4));
     }
     ChainStep *d = (ChainStep *)C.dev.p;
+    C.desc_dev = (const ChainDesc *)((char *)C.dev.p + b_steps);
+    C.arrived = (uint32_t *)((char *)C.dev.p + b_steps + 256);
+    C.n_chains = C.grid = 0;
     for (int k = 0; k < 2; ++k) {
         std::vector<ChainStep> &H = C.host[k];
+        if (H.empty()) continue;
         for (size_t i = 0; i < H.size(); ++i) {
             const ChainShape &in = C.shapes[(size_t)C.in_shape[k][i]];
             H[i].in_threads = in.threads;
             H[i].tiles = in.tiles;
             H[i].out_threads = C.shapes[(size_t)C.out_shape[k][i]].threads;
         }
-        C.ctas[k] = H.empty() ? 0
-                              : (int)std::min<int64_t>((int64_t)n_vec * (int64_t)tiles,
-                                                       c->chain_ctas / (n0 && n1 ? 2 : 1));
-        if (!H.empty())
-            CK(cudaMemcpyAsync(d + (k ? n0 : 0), H.data(), H.size() * sizeof(ChainStep),
-                               cudaMemcpyHostToDevice, s));
+        ChainDesc e{};
+        e.steps = d + (k ? n0 : 0);
+        e.maps = P.prog.pass_maps;
+        e.arrived = C.arrived + 32 * C.n_chains;
+        e.n_steps = (int32_t)H.size();
+        e.n = c->n;
+        e.n_vec = n_vec;
+        e.cta0 = C.grid;
+        e.ctas = (int32_t)std::min<int64_t>((int64_t)n_vec * (int64_t)tiles,
+                                            std::max(1, max_ctas / (n0 && n1 ? 2 : 1)));
+        C.grid += e.ctas;
+        C.desc[C.n_chains++] = e;
+        CK(cudaMemcpyAsync(d + (k ? n0 : 0), H.data(), H.size() * sizeof(ChainStep),
+                           cudaMemcpyHostToDevice, s));
     }
+    C.alone = n_vec == 1 && tiles == 1;
+    if (C.n_chains)
+        CK(cudaMemcpyAsync((void *)C.desc_dev, C.desc, sizeof(C.desc), cudaMemcpyHostToDevice, s));
     if (ns)
         CK(cudaMemcpyAsync(C.tables.p, C.shapes.data(), ns * sizeof(ChainShape),
                            cudaMemcpyHostToDevice, s));
@@ -1230,23 +1248,40 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
     return STAB_OK;
 }
 
-int chain_run(stab_ctx *c, const ChainSet &C, const DevPlan &P, int n_vec, cudaStream_t s) {
+int chain_run(stab_ctx *c, const ChainSet &C, cudaStream_t s) {
+    if (C.n_chains == 0) return STAB_OK;
     ChainArgs a{};
-    a.steps[0] = (const ChainStep *)C.dev.p;
-    a.steps[1] = a.steps[0] + C.host[0].size();
-    for (int k = 0; k < 2; ++k) {
-        a.n_steps[k] = (int32_t)C.host[k].size();
-        a.ctas[k] = C.ctas[k];
-    }
-    if (a.ctas[0] + a.ctas[1] == 0) return STAB_OK;
-    a.n = c->n;
-    a.n_vec = n_vec;
+    a.chains = C.desc_dev;
+    a.n_chains = C.n_chains;
+    a.grid = C.grid;
     a.tile_bits = chain_tile_bits(c->n);
-    a.maps = P.prog.pass_maps;
-    a.arrived = (uint32_t *)c->arrived.p;
+    a.alone = C.alone;
     a.status = (int32_t *)c->status.p;
+    CK(cudaMemsetAsync(C.arrived, 0, 256, s));
     CK(launch_stream_chain(a, s));
     c->launches++;
+    return STAB_OK;
+}
+
+// <O> as two chains that meet at half the passes: O backward (from lam), rho_0
+// forward (from lam2).
+int expect_chains(stab_ctx *c, const std::vector<const void *> &key, int max_ctas,
+                  cudaStream_t s) {
+    ChainSet &C = c->c_expect;
+    const int np = (int)c->fwd.host.passes.size(), mid = np / 2;
+    C.clear();
+    C.result[0] = chain_passes(c, c->fwd, (double *)c->lam.p, (double *)c->tmp.p, true, mid, np,
+                               &C, 0);
+    C.result[1] = chain_passes(c, c->fwd, (double *)c->lam2.p, (double *)c->tmp3.p, false, 0, mid,
+                               &C, 1);
+    return chain_upload(c, C, key, c->fwd, 1, max_ctas, s);
+}
+
+int expect_fill(stab_ctx *c, cudaStream_t s) {
+    const int32_t nt = c->n_obs_terms;
+    CK(launch_fill((double *)c->lam.p, c->n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, nt, s));
+    CK(launch_fill((double *)c->lam2.p, c->n, 1, INIT_RHO0, nullptr, 0, s));
+    c->launches += (nt ? 2 : 1) + 1;
     return STAB_OK;
 }
 
@@ -1597,7 +1632,7 @@ int ck_chains(stab_ctx *c, cudaStream_t s) {
         cur = to;
     }
     C.result[1] = cur;
-    return chain_upload(c, C, key, 1, s);
+    return chain_upload(c, C, key, G, 1, c->chain_ctas, s);
 }
 
 // The runs' numbers and the derivatives from the slots.
@@ -1636,7 +1671,7 @@ int ck_gradient(stab_ctx *c, double *res, cudaStream_t gs) {
                        nullptr, 0, gs));
         CK(launch_fill(slot(at + 4), n, 1, INIT_TERMS, (const DevTerm *)c->terms.p,
                        c->n_obs_terms, gs));
-        RC(chain_run(c, c->c_grad, G, 1, gs));
+        RC(chain_run(c, c->c_grad, gs));
         CK(launch_xfree_sum(lam0, n, 1, res, gs));
         c->launches += (c->n_obs_terms ? 3 : 2) + 1;
         return ck_finish(c, gs);
@@ -2074,7 +2109,7 @@ int stab_destroy(stab_ctx *c) {
                       &c->dotbuf, &c->umaps, &c->unodes, &c->ustates, &c->udots, &c->rmid,
                       &c->lmid, &c->units_e, &c->cnt, &c->gmid, &c->ck.buf, &c->ckslots,
                       &c->ckjobs, &c->ckdots, &c->c_gens.dev, &c->c_expect.dev, &c->c_grad.dev,
-                      &c->c_gens.tables, &c->c_expect.tables, &c->c_grad.tables, &c->arrived};
+                      &c->c_gens.tables, &c->c_expect.tables, &c->c_grad.tables};
     for (DevBuf *b : bufs) c->dfree(*b, c->st);
     if (c->st) cudaStreamSynchronize(c->st);
     if (c->stage) cudaFreeHost(c->stage);
@@ -2204,11 +2239,11 @@ int stab_run_generators(stab_ctx *c) {
                 C.clear();
                 C.result[0] = chain_passes(c, c->fwd, (double *)c->gens.p, (double *)c->gens_tmp.p,
                                            false, 0, (int)c->fwd.host.passes.size(), &C, 0);
-                RC(chain_upload(c, C, key, n, s));
+                RC(chain_upload(c, C, key, c->fwd, n, c->chain_ctas, s));
             }
             CK(launch_fill((double *)c->gens.p, n, n, INIT_GENERATOR, nullptr, 0, s));
             c->launches++;
-            RC(chain_run(c, C, c->fwd, n, s));
+            RC(chain_run(c, C, s));
             c->g_gens.result = C.result[0];
         } else RC(run_graph(c, c->g_gens, key, s, [&](cudaStream_t gs, void **result) {
             double *cur = (double *)c->gens.p, *alt = (double *)c->gens_tmp.p;
@@ -2324,21 +2359,11 @@ int stab_expect_async(stab_ctx *c, double *out_dev) {
                                                (const void *)(intptr_t)split};
         if (split && use_chain_forward(c, c->fwd, 1)) {
             ChainSet &C = c->c_expect;
-            double *lam = (double *)c->lam.p, *rho = (double *)c->lam2.p;
-            if (C.key != key) {
-                const int np = (int)c->fwd.host.passes.size(), mid = np / 2;
-                C.clear();
-                C.result[0] =
-                    chain_passes(c, c->fwd, lam, (double *)c->tmp.p, true, mid, np, &C, 0);
-                C.result[1] =
-                    chain_passes(c, c->fwd, rho, (double *)c->tmp3.p, false, 0, mid, &C, 1);
-                RC(chain_upload(c, C, key, 1, s));
-            }
-            CK(launch_fill(lam, c->n, 1, INIT_TERMS, (const DevTerm *)c->terms.p, nt, s));
-            CK(launch_fill(rho, c->n, 1, INIT_RHO0, nullptr, 0, s));
-            RC(chain_run(c, C, c->fwd, 1, s));
+            if (C.key != key) RC(expect_chains(c, key, c->chain_ctas, s));
+            RC(expect_fill(c, s));
+            RC(chain_run(c, C, s));
             CK(launch_dot(C.result[0], C.result[1], c->n, (double *)c->dotbuf.p, res, s));
-            c->launches += (nt ? 2 : 1) + 1 + 2;
+            c->launches += 2;
         } else RC(run_graph(c, c->g_expect, key, s, [&](cudaStream_t gs, void **) {
             double *cur = (double *)c->lam.p, *alt = (double *)c->tmp.p;
             if (!split) {
@@ -2817,6 +2842,51 @@ int stab_transfer_bytes(stab_ctx *c, int64_t *h2d, int64_t *d2h) {
 }
 
 }  // extern "C"
+
+// ---------------------------------------------------------------- long items of a batch
+
+int stab::long_item_prepare(stab_ctx *c, bool gens, int max_ctas, const ChainDesc **chains,
+                            int *n_chains) {
+    if (!c || !c->loaded || c->use_resident() || (!gens && !c->obs_loaded)) return STAB_E_STATE;
+    const size_t vb = c->vec_bytes();
+    const std::vector<const void *> key = {(const void *)c->plan_gen};
+    ChainSet &C = gens ? c->c_gens : c->c_expect;
+    RC(stream_maps(c, c->fwd));
+    if (!c->fwd.prog.pass_maps) return STAB_E_STATE;
+    if (gens) {
+        const size_t bytes = vb * (size_t)c->n;
+        RC(c->dalloc(c->gens, bytes, c->st));
+        RC(c->dalloc(c->gens_tmp, bytes, c->st));
+        C.clear();
+        C.result[0] = chain_passes(c, c->fwd, (double *)c->gens.p, (double *)c->gens_tmp.p, false,
+                                   0, (int)c->fwd.host.passes.size(), &C, 0);
+        RC(chain_upload(c, C, key, c->fwd, c->n, max_ctas, c->st));
+    } else {
+        for (DevBuf *b : {&c->lam, &c->tmp, &c->lam2, &c->tmp3}) RC(c->dalloc(*b, vb, c->st));
+        RC(c->dalloc(c->dotbuf, 256 * sizeof(double), c->st));
+        RC(expect_chains(c, key, max_ctas, c->st));
+    }
+    *chains = C.desc;
+    *n_chains = C.n_chains;
+    return STAB_OK;
+}
+
+int stab::long_item_fill(stab_ctx *c, bool gens, cudaStream_t s) {
+    if (!gens) return expect_fill(c, s);
+    CK(launch_fill((double *)c->gens.p, c->n, c->n, INIT_GENERATOR, nullptr, 0, s));
+    return STAB_OK;
+}
+
+int stab::long_item_finish(stab_ctx *c, bool gens, double *out, cudaStream_t s) {
+    if (gens) {
+        CK(cudaMemcpyAsync(out, c->c_gens.result[0], c->vec_bytes() * (size_t)c->n,
+                           cudaMemcpyDeviceToDevice, s));
+        return STAB_OK;
+    }
+    CK(launch_dot(c->c_expect.result[0], c->c_expect.result[1], c->n, (double *)c->dotbuf.p, out,
+                  s));
+    return STAB_OK;
+}
 
 // Expectation of an observable already on the device as deduplicated terms
 // (the sparse path's list when it switches to the dense vector).

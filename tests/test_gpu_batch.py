@@ -147,3 +147,41 @@ def test_batch_c3_full_size_sampled(stab):
     kinds = np.array([it.kind == "expect" for it in items])
     assert np.all(np.isfinite(ex[kinds]))
     b.close()
+
+
+@pytest.mark.parametrize("n_light", [0, 40])
+def test_long_items_run_as_chains(stab, n_light):
+    """Items that would outlast the rest of the batch on one CTA (n = 6 .. 8, deep)
+    run as chains on many SMs, beside the others: <O> and generators of every
+    size against the oracle, twice (the second run replays the graphs), with
+    circuits that begin and end with Clifford runs."""
+    items = [W.BatchItem(W.layered_ansatz(8, 1301, seed=5), "expect", W.obs_chain(8)),
+             W.BatchItem(W.random_circuit(7, 2500, seed=6), "expect", W.obs_chain(7)),
+             W.BatchItem(W.layered_ansatz(7, 2000, seed=7), "generators"),
+             W.BatchItem(W.layered_ansatz(6, 6000, seed=8), "generators"),
+             W.BatchItem(W.clifford_plus_rotations(8, 4000, 300, seed=9), "expect",
+                         W.obs_chain(8))]
+    for k in range(n_light):
+        items.append(W.BatchItem(W.layered_ansatz(2 + k % 5, 60 + k, seed=20 + k), "expect",
+                                 W.obs_chain(2 + k % 5)))
+    b = stab.Batch(items)
+    assert b.info()["units"] == sum(1 if it.kind == "expect" else it.circuit.n for it in items)
+    runs = []
+    for _ in range(2):
+        b.run()
+        runs.append((b.expectations(), [b.generators(k) for k in (2, 3)]))
+    b.close()
+    np.testing.assert_array_equal(np.nan_to_num(runs[0][0]), np.nan_to_num(runs[1][0]))
+    for x, y in zip(runs[0][1], runs[1][1]):
+        np.testing.assert_array_equal(x, y)
+    ex, gens = runs[0]
+    for k, it in enumerate(items):
+        if it.kind == "expect":
+            c = it.circuit
+            ref = oracle.expect(c.n, c.gates, c.thetas, it.observable)
+            assert abs(ex[k] - ref) <= 1e-12 * l1(it.observable), k
+    for k, got in zip((2, 3), gens):
+        c = items[k].circuit
+        for q in (0, c.n - 1):
+            want = oracle.forward(c.n, c.gates, c.thetas, oracle.generator(c.n, q))
+            assert np.abs(layout.lib_to_paper(c.n, got[q]) - want).max() <= 1e-12
