@@ -173,6 +173,7 @@ cudaError_t launch_batch(const BatchArgs &a, int grid, size_t smem, cudaStream_t
 }  // namespace stab
 
 typedef struct stab_ctx stab_ctx;
+struct stab_gate;
 
 namespace stab {
 
@@ -180,9 +181,12 @@ namespace stab {
 // complete once this stream is).
 cudaStream_t ctx_stream(stab_ctx *ctx);
 
-// The context's gradients keep within the vectors that the request footprint
-// counts (no stored sweeps).
-void ctx_no_checkpoints(stab_ctx *ctx);
+// Device memory the context's gradients may take for stored sweeps (0: none, the
+// pair sweep's fixed number of vectors), and a bound on what a circuit's take.
+void ctx_checkpoint_limit(stab_ctx *ctx, size_t bytes);
+size_t checkpoint_bound(int n, const struct ::stab_gate *gates, int64_t m);
+// Hands the stored sweeps' memory back when it is more than `keep`.
+void ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);
 
 // Density matrix from the forward-evolved coefficients of 2^n |0><0|:
 // rho (device, 2 x 4^n doubles, interleaved complex, row-major).

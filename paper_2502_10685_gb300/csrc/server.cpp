@@ -257,7 +257,6 @@ Slot *make_slot(stab_server *s, int n) {
         delete sl;
         return nullptr;
     }
-    ctx_no_checkpoints(sl->ctx);   // requests are admitted by a fixed number of vectors
     cudaStream_t st = ctx_stream(sl->ctx);
     sl->d_res = (double *)s->hooks.get(256, st);
     if (!sl->d_res || cudaMallocHost(&sl->h_res, 64 * sizeof(double)) != cudaSuccess ||
@@ -344,9 +343,25 @@ size_t next_request_locked(const stab_server *s) {
     return best;
 }
 
+// The iteration engine advances a request's vector (or pair) on one CTA; a
+// request that would take it more than kLongUs runs on a context instead, whose
+// sweeps use many SMs (n <= 4: the segments' unitaries, n >= 5: chains of tile
+// steps).  48 requests at once, n = 4 .. 8, to 6,000 gates: 18.4 ms with all n <= 6 in
+// the engine (an n = 6 gradient of 3,585 gates finished last; alone on a context it
+// takes 1.2 ms), 7.9 with the line at 0.25, 0.6 or 2 ms, 8.6 at 0.1, where the many
+// small contexts' launches queue.  A new context costs half a millisecond once.
+// Estimate: 0.17 ns per gate and entry, four times that for a gradient's pair
+// (n = 6: 0.68 us a gate).
+constexpr double kLongUs = 600.0;
 bool use_iteration(const stab_server *s, const Req *r) {
-    return s->iterate && r->hdr.n <= s->opts.iter_max_n;
+    return s->iterate && r->hdr.n <= s->opts.iter_max_n &&
+           (double)r->hdr.m * (double)((int64_t)1 << (2 * r->hdr.n)) * 1.66e-4 *
+                   (r->hdr.kind == STAB_REQ_GRAD ? 4.0 : 1.0) <= kLongUs;
 }
+
+// A gradient's stored sweeps come on top of the footprint it was admitted with,
+// where the budget has room for them; they are handed back when they are large.
+constexpr size_t kKeepCheckpoints = (size_t)64 << 20;
 
 // ---------------------------------------------------------------- iteration requests: host side
 
@@ -919,6 +934,14 @@ void planner_main(stab_server *s) {
             r->slot = pool.back();
             pool.pop_back();
         }
+        int64_t stored = 0;
+        if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n > 4 && r->hdr.n <= STAB_MAX_QUBITS) {
+            stored = (int64_t)checkpoint_bound(r->hdr.n, r->gates.data(),
+                                               (int64_t)r->gates.size());
+            if (s->bytes_in_use + stored > s->opts.hbm_budget) stored = 0;
+            s->bytes_in_use += stored;
+            r->footprint += stored;
+        }
         lk.unlock();
         int rc = STAB_OK;
         if (!r->slot) {
@@ -929,7 +952,10 @@ void planner_main(stab_server *s) {
                 s->slots.push_back(r->slot);
             }
         }
-        if (rc == STAB_OK) rc = launch_on_context(s, r);
+        if (rc == STAB_OK) {
+            ctx_checkpoint_limit(r->slot->ctx, (size_t)stored);
+            rc = launch_on_context(s, r);
+        }
         lk.lock();
         if (rc != STAB_OK) {
             if (r->slot) stab_synchronize(r->slot->ctx);
@@ -957,6 +983,7 @@ void completer_main(stab_server *s) {
             }
             // status word of the context (bounded device waits)
             const int st = stab_synchronize(r->slot->ctx);
+            ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints);
             r->res.expect = r->slot->h_res[0];
             if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n_params > 0)
                 r->grads.assign(r->slot->h_grads, r->slot->h_grads + r->hdr.n_params);

@@ -1749,8 +1749,27 @@ int ensure_grad_plan(stab_ctx *c) {
 }  // namespace
 
 cudaStream_t stab::ctx_stream(stab_ctx *c) { return c ? c->st : nullptr; }
-void stab::ctx_no_checkpoints(stab_ctx *c) {
-    if (c) c->ck_bytes_max = 0;
+void stab::ctx_checkpoint_limit(stab_ctx *c, size_t bytes) {
+    if (c) c->ck_bytes_max = std::min(bytes, kCheckpointBytes);
+}
+size_t stab::checkpoint_bound(int n, const stab_gate *gates, int64_t m) {
+    size_t blocks = 0, cliffs = 0;   // a slot more than ck_slots per Clifford pass at most
+    bool two = true;
+    for (int64_t i = 0; i < m; ++i) {
+        const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
+        if (t && (!two || i == 0)) ++cliffs;
+        if (!t && two) ++blocks;
+        two = t;
+    }
+    return (2 * blocks + cliffs + kCkSpares) * (sizeof(double) << (2 * n));
+}
+void stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
+    if (c && c->ckslots.bytes > keep) {
+        c->dfree(c->ckslots, c->aux);
+        c->key_ck.clear();
+        c->c_grad.key.clear();
+        c->g_grad.reset();
+    }
 }
 
 extern "C" {
