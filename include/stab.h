@@ -314,7 +314,8 @@ int stab_batch_destroy(stab_batch *b);
  *    kind of unit; before a kind is measured, iter_chunks chunks at n = 4, a
  *    quarter of that per extra qubit, at least one), its vectors staying in
  *    its own device memory between launches.  New requests join at the next
- *    launch.  Larger requests run as in STAB_SERVE_CONTEXTS, beside them.
+ *    launch.  Larger requests, and those that would take one CTA more than
+ *    about half a millisecond, run as in STAB_SERVE_CONTEXTS, beside them.
  *  - STAB_SERVE_CONTEXTS: each admitted request runs on its own pooled
  *    context and streams, so the kernels of all admitted requests overlap on
  *    the device; contexts keep their device vectors between requests.
@@ -391,7 +392,9 @@ typedef struct stab_result {
  * plus, for a gradient, the adjoint's partial dot sums: per CTA of the
  * streamed sweep above n = 6, per thread of the resident sweep at n <= 5
  * (8 bytes x gates x 32, 32, 32, 64, 256 threads at n = 1..5, while that
- * stays within 256 MiB), as a bound on one per rotation. */
+ * stays within 256 MiB), as a bound on one per rotation.  A streamed gradient
+ * may keep its sweeps' vectors (two per block of single-qubit gates) where the
+ * budget has room for them when it starts; they are counted on top then. */
 int64_t stab_request_footprint(const stab_request *req);
 
 /* opts may be NULL (all defaults).  Errors: STAB_E_INVAL (unknown policy or
