@@ -3,23 +3,28 @@
 // order n' (the number of strings, Fig. 1) is small, so that n is limited by
 // the list, not by a 4^n vector (keys z | x << n in 64 bits, n <= 32).
 //
-// A run of Clifford gates maps every term in place: one signed string each
-// (Table I rows H and S, the map_CX list, and their compositions).  A rotation
-// R_sigma on wire q mixes the two strings of each anticommuting pair (u, v)
-// -- R_x: (Y, Z), R_y: (Z, X), R_z: (X, Y) -- as u' = c u - s v,
-// v' = s u + c v (Table I); a term whose partner is absent spawns it.  One
-// rotation is four launches:
-//   insert -- every anticommuting term claims a slot of an open-addressing
-//             table (keys are unique, so a claim never meets its own key);
-//   count  -- per term: the partner's position (or -1) and how many nonzero
-//             terms it emits; per block: the total;
-//   scan   -- one CTA: exclusive scan of the block totals, the new order,
-//             capacity and threshold checks;
-//   write  -- every term writes its images at their scanned positions (in
-//             input order, so the list order is deterministic and independent
-//             of the grid) and frees its table slot.
-// Exact zeros are never stored.  A step that finds the stop flag set by an
-// earlier step returns at once, so the host can launch several steps ahead.
+// Clifford gates do not touch the list.  A rotation behind a Clifford U acts on
+// U's images as the rotation about the string U^dagger sigma U acts on the
+// terms themselves, so every rotation is pulled back through the Clifford gates
+// before it (SpRot, made once per circuit load) and the gates' tableau is
+// applied to the last list alone.  (Mapping the whole list at each of 29
+// Clifford runs took a quarter of a 32-qubit call of 28 rotations.)
+//
+// A rotation about P mixes the two strings of each anticommuting pair (u, v),
+// v = u P up to a phase, as u' = c u - s v, v' = s u + c v (Table I); a term
+// whose partner is absent spawns it.  The images stand where the u term stood
+// (or the lone term), u first: the list order is the input order, independent
+// of the grid.  Exact zeros are never stored.  Two phases:
+//   pair  -- every anticommuting term puts its position at its pair's place in
+//            an open-addressing table (both strings of a pair hash alike, so the
+//            second one to come finds the first, and tells it);
+//   write -- images, their positions by a scan, and the table is cleared.
+// Short lists run in one CTA's shared memory, rotation after rotation
+// (k_sp_small); from there on the whole GPU takes the rest in one cooperative
+// launch (k_sp_run).  n = 32, 20,000 gates, 28 rotations, <O> up to 5.7 million
+// terms: 2.10 -> 0.73 ms; one generator, 96,000 terms: 1.19 -> 0.37 ms; n = 13, 12
+// rotations, 2,400 terms: 451 -> 90 us (before: five launches a rotation, the
+// list mapped at every Clifford run).
 #include <cuda_runtime.h>
 
 #include "../../include/stab.h"
@@ -30,115 +35,86 @@ namespace stab {
 namespace {
 
 constexpr int kSpThreads = 256;
+constexpr uint64_t kSpFree = ~0ull;
 
-// letter code 2x + z: I = 0, Z = 1, X = 2, Y = 3
-__device__ __forceinline__ uint32_t sp_letter(uint64_t key, int n, int q) {
-    return (uint32_t)(((key >> (n + q)) & 1u) << 1) | (uint32_t)((key >> q) & 1u);
+// one population count for both halves: they run at an eighth of the integer rate
+__device__ __forceinline__ uint32_t sp_parity(uint64_t x) {
+    return (uint32_t)__popc((uint32_t)(x >> 32) ^ (uint32_t)x) & 1u;
 }
 
-__device__ __forceinline__ uint64_t sp_with_letter(uint64_t key, int n, int q, uint32_t lc) {
-    key &= ~((1ull << q) | (1ull << (n + q)));
-    return key | ((uint64_t)(lc & 1u) << q) | ((uint64_t)(lc >> 1) << (n + q));
+__device__ __forceinline__ bool sp_nonzero(double x) {
+    return (__double_as_longlong(x) << 1) != 0;   // off the FP64 pipe
 }
 
-// the anticommuting pair (u, v) of each rotation axis
-__device__ __forceinline__ void sp_pair(int axis, uint32_t &u, uint32_t &v) {
-    if (axis == 0) { u = 3u; v = 1u; }        // R_x: (Y, Z)
-    else if (axis == 1) { u = 1u; v = 2u; }   // R_y: (Z, X)
-    else { u = 2u; v = 3u; }                  // R_z: (X, Y)
+__device__ __forceinline__ uint64_t sp_hash(uint64_t key) {
+    return (key ^ (key >> 31)) * 0x9E3779B97F4A7C15ull;
 }
 
-__device__ __forceinline__ uint32_t sp_hash(uint64_t key, int log_h) {
-    return (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> (64 - log_h));
+// Exponent c (mod 4) of P(a) P(b) = i^c P(a xor b) for Hermitian Pauli strings
+// given by x / z masks: per qubit, with a = Y: z_b - x_b; a = X: z_b (2 x_b - 1);
+// a = Z: x_b (1 - 2 z_b) (the phase function of the stabilizer tableau
+// algorithm of Aaronson and Gottesman), summed with one population count:
+// the complement of `minus` counts 32 - |minus|.
+__device__ __forceinline__ uint32_t sp_mul_phase(uint32_t ax, uint32_t az, uint32_t bx,
+                                                 uint32_t bz) {
+    const uint32_t A = ax & az, B = ax & ~az, C = ~ax & az;
+    const uint32_t plus = (A & bz & ~bx) | (B & bz & bx) | (C & bx & ~bz);
+    const uint32_t minus = (A & bx & ~bz) | (B & bz & ~bx) | (C & bx & bz);
+    return (uint32_t)__popcll(((uint64_t)~minus << 32) | plus) & 3u;
 }
 
-// Steps run until a stop: flags[0] != 0 at step flags[1].
-__device__ __forceinline__ bool sp_stopped_before(const int32_t *flags, int step) {
-    return flags[0] != 0 && flags[1] < step;
+__device__ __forceinline__ bool sp_anti(uint64_t key, const SpRot &d) {
+    return sp_parity(key & d.anti) != 0;
 }
 
-// Forward conjugation g P g^dagger of one Clifford gate on a key; sets the
-// sign bit in neg.  1q rules on (x, z) of the wire: H swaps x and z (Y -> -Y),
-// S: z ^= x (Y -> -X), S^dagger: z ^= x (X -> -Y), X: sign z, Y: sign x ^ z,
-// Z: sign x.  CX(c, t): x_t ^= x_c, z_c ^= z_t, minus iff x_c z_t (x_t == z_c);
-// CZ(a, b): z_a ^= x_b, z_b ^= x_a, minus iff x_a x_b (z_a != z_b).
-__device__ __forceinline__ uint64_t sp_clifford(uint64_t key, int n, const SpGate g,
-                                                uint32_t &neg) {
-    const int a = g.q0;
-    const uint32_t xa = (uint32_t)(key >> (n + a)) & 1u, za = (uint32_t)(key >> a) & 1u;
-    switch (g.op) {
-    case STAB_H:
-        neg ^= xa & za;
-        return sp_with_letter(key, n, a, (za << 1) | xa);
-    case STAB_S:
-        neg ^= xa & za;
-        return sp_with_letter(key, n, a, (xa << 1) | (za ^ xa));
-    case STAB_SDG:
-        neg ^= xa & (za ^ 1u);
-        return sp_with_letter(key, n, a, (xa << 1) | (za ^ xa));
-    case STAB_X: neg ^= za; return key;
-    case STAB_Y: neg ^= xa ^ za; return key;
-    case STAB_Z: neg ^= xa; return key;
-    case STAB_CX: {
-        const int t = g.q1;
-        const uint32_t xt = (uint32_t)(key >> (n + t)) & 1u, zt = (uint32_t)(key >> t) & 1u;
-        neg ^= xa & zt & ((xt ^ za) ^ 1u);
-        key = sp_with_letter(key, n, t, ((xt ^ xa) << 1) | zt);
-        return sp_with_letter(key, n, a, (xa << 1) | (za ^ zt));
+__device__ __forceinline__ bool sp_is_u(uint64_t key, const SpRot &d) {
+    return sp_parity(key & d.letter) == (d.flags & 1u);
+}
+
+__device__ __forceinline__ double sp_neg_if(double x, bool neg) {   // off the FP64 pipe, too
+    return __longlong_as_double(__double_as_longlong(x) ^ ((long long)neg << 63));
+}
+
+// The images of a term under the rotation: up to two (key, value) pairs in the
+// order u, v, their number returned.  i u P = +-v: with the minus, v enters and
+// leaves negated.  The FP64 pipe takes an instruction of a warp every 76 clocks
+// and is what this costs: a warp of lone terms issues the two products it
+// needs, a warp with a pair (any_paired: in the whole warp) four more.  With the
+// products by zero, the sign changes and the tests for zero there as well, a
+// tile took 2.5 times as long.  All lanes call this together.
+__device__ __forceinline__ int sp_images(bool in, bool any_paired, uint64_t key, double val,
+                                         bool paired, double pval, const SpRot &d, int n,
+                                         double c, double s, uint64_t &k0, double &v0,
+                                         uint64_t &k1, double &v1) {
+    const bool is_u = sp_is_u(key, d);
+    const uint64_t ku = is_u ? key : key ^ d.P;
+    const uint32_t zm = (uint32_t)((1ull << n) - 1ull);
+    const uint32_t e = 1u + (d.flags & 2u) +
+                       sp_mul_phase((uint32_t)(ku >> n), (uint32_t)ku & zm, (uint32_t)(d.P >> n),
+                                    (uint32_t)d.P & zm);
+    const bool minus = (e & 2u) != 0;
+    // u: (c u, +-s u); v = +-val: (-s v, c v), whose own sign comes back
+    const double cx = c * val, sx = s * val;
+    double ou = is_u ? cx : sp_neg_if(sx, !minus);
+    double ov = is_u ? sp_neg_if(sx, minus) : cx;
+    if (any_paired) {
+        const double vv = sp_neg_if(pval, minus);
+        const double pu = fma(c, val, -(s * vv));
+        const double pv = sp_neg_if(fma(s, val, c * vv), minus);
+        if (paired) {
+            ou = pu;
+            ov = pv;
+        }
     }
-    case STAB_CZ: {
-        const int b = g.q1;
-        const uint32_t xb = (uint32_t)(key >> (n + b)) & 1u, zb = (uint32_t)(key >> b) & 1u;
-        neg ^= xa & xb & (za ^ zb);
-        key = sp_with_letter(key, n, a, (xa << 1) | (za ^ xb));
-        return sp_with_letter(key, n, b, (xb << 1) | (zb ^ xa));
-    }
-    default: return key;
-    }
-}
-
-__device__ __forceinline__ void sp_block_range(int64_t count, int64_t &lo, int64_t &hi) {
-    const int64_t per = (count + gridDim.x - 1) / gridDim.x;
-    lo = (int64_t)blockIdx.x * per;
-    if (lo > count) lo = count;
-    hi = lo + per;
-    if (hi > count) hi = count;
-}
-
-// The images of term i under the rotation: up to two (key, value) pairs in the
-// order u, v.  partner = position of the other string of the pair, or -1.
-__device__ __forceinline__ int sp_images(uint64_t key, double val, int32_t partner,
-                                         const double *vals, int n, int q, int axis, double c,
-                                         double s, uint64_t &k0, double &v0, uint64_t &k1,
-                                         double &v1) {
-    uint32_t u, v;
-    sp_pair(axis, u, v);
-    const uint32_t L = sp_letter(key, n, q);
-    if (L != u && L != v) {
-        k0 = key;
-        v0 = val;
-        return 1;
-    }
-    double uu, vv;
-    if (L == u) {
-        uu = val;
-        vv = partner >= 0 ? vals[partner] : 0.0;
-    } else {
-        if (partner >= 0) return 0;   // the u term of the pair writes both
-        uu = 0.0;
-        vv = val;
-    }
-    const double ou = fma(c, uu, -(s * vv));
-    const double ov = fma(s, uu, c * vv);
-    const uint64_t ku = sp_with_letter(key, n, q, u), kv = sp_with_letter(key, n, q, v);
-    int e = 0;
-    if (ou != 0.0) { k0 = ku; v0 = ou; e = 1; }
-    if (ov != 0.0) {
-        if (e == 0) { k0 = kv; v0 = ov; }
-        else { k1 = kv; v1 = ov; }
-        ++e;
-    }
-    return e;
+    const bool anti = sp_anti(key, d);
+    // a commuting term stays; of a pair, the u term writes both
+    const bool mix = in && anti && (is_u || !paired);
+    const bool u_on = mix && sp_nonzero(ou), v_on = mix && sp_nonzero(ov);
+    k0 = mix ? (u_on ? ku : ku ^ d.P) : key;
+    v0 = mix ? (u_on ? ou : ov) : val;
+    k1 = ku ^ d.P;
+    v1 = ov;
+    return mix ? (u_on ? 1 : 0) + (v_on ? 1 : 0) : (in && !anti ? 1 : 0);
 }
 
 template <typename T>
@@ -164,76 +140,23 @@ __device__ T block_exclusive_scan(T x, T &total, T *sh) {
     __syncthreads();
     const T warp_before = warp > 0 ? sh[warp - 1] : (T)0;
     total = sh[(blockDim.x >> 5) - 1];
-    __syncthreads();
     return warp_before + incl - x;
 }
 
-// cos and sin of a slot's angle, from the table k_sp_cos_sin fills once per
-// circuit load (cs[2 p] = cos, cs[2 p + 1] = sin): every thread of every block
-// needs them, and evaluating sincos there cost the FP64 pipe more than the
-// rotation itself on short lists.
-__device__ __forceinline__ void sp_rot_cs(const double *cs, int param, int inverse, double &c,
-                                          double &s) {
-    c = cs[2 * param];
-    s = cs[2 * param + 1];
-    if (inverse) s = -s;
-}
-
+// Every term needs its slot's cos and sin; evaluating sincos for each cost the
+// FP64 pipe more than the rotation itself on short lists.
 __global__ void k_sp_cos_sin(const double *thetas, int64_t n_params, double *cs) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n_params) sincos(thetas[p], &cs[2 * p + 1], &cs[2 * p]);
 }
 
-__global__ void __launch_bounds__(kSpThreads) k_sp_cliff(uint64_t *keys, double *vals,
-                                                          int64_t *counts, const int32_t *flags,
-                                                          int step, int n, const SpGate *gates,
-                                                          int n_gates) {
-    if (sp_stopped_before(flags, step)) return;
-    const int64_t count = counts[step];
-    if (blockIdx.x == 0 && threadIdx.x == 0) counts[step + 1] = count;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = keys[i];
-        uint32_t neg = 0;
-        for (int g = 0; g < n_gates; ++g) k = sp_clifford(k, n, gates[g], neg);
-        keys[i] = k;
-        if (neg) vals[i] = -vals[i];
-    }
-}
-
-// A long Clifford run as its tableau: the images U X_q U^dagger and
-// U Z_q U^dagger of the 2n single-qubit generators (entry q: X_q, entry n + q:
-// Z_q), each a signed string.  One thread per generator, gate by gate.
-__global__ void k_sp_tableau(const SpGate *gates, const int32_t *run_first,
-                             const int32_t *run_count, int n, SpTab *tabs) {
-    const int r = blockIdx.x, j = threadIdx.x;
-    if (j >= 2 * n) return;
-    uint64_t k = j < n ? (1ull << (n + j)) : (1ull << (j - n));
-    uint32_t neg = 0;
-    const SpGate *g = gates + run_first[r];
-    for (int i = 0; i < run_count[r]; ++i) k = sp_clifford(k, n, g[i], neg);
-    tabs[(size_t)r * 64 + j] = SpTab{k, neg};
-}
-
-// Exponent c (mod 4) of P(a) P(b) = i^c P(a xor b) for Hermitian Pauli strings
-// given by x / z masks: per qubit, with a = Y: z_b - x_b; a = X: z_b (2 x_b - 1);
-// a = Z: x_b (1 - 2 z_b) (the phase function of the stabilizer tableau
-// algorithm of Aaronson and Gottesman), summed with population counts.
-__device__ __forceinline__ uint32_t sp_mul_phase(uint32_t ax, uint32_t az, uint32_t bx,
-                                                 uint32_t bz) {
-    const uint32_t A = ax & az, B = ax & ~az, C = ~ax & az;
-    const uint32_t plus = (A & bz & ~bx) | (B & bz & bx) | (C & bx & ~bz);
-    const uint32_t minus = (A & bx & ~bz) | (B & bz & ~bx) | (C & bx & bz);
-    return (uint32_t)(__popc(plus) - __popc(minus)) & 3u;
-}
-
-// The tableau regrouped by chunks of kSpChunkQubits qubits: entry
-// (chunk c, subset t) is the ordered product prod_{q in c} (U X_q U^dagger)^{x_q}
-// (U Z_q U^dagger)^{z_q} of the generator images the subset selects (bit j of
-// t: x of qubit 4c + j, bit 4 + j: its z), as a Hermitian string and a phase
-// i^e.  One block per (run, chunk), one thread per subset.
-__global__ void k_sp_tab_chunks(const SpTab *tabs, int n, SpChunk *chunks) {
-    const int r = blockIdx.x / kSpChunks, c = blockIdx.x % kSpChunks, t = threadIdx.x;
+// Entry (chunk c, subset t) of a tableau's chunk table is the ordered product
+// prod_{q in c} (U X_q U^dagger)^{x_q} (U Z_q U^dagger)^{z_q} of the generator
+// images the subset selects (bit j of t: x of qubit 4c + j, bit 4 + j: its z),
+// as a Hermitian string and a phase i^e.  One block per chunk, one thread per
+// subset.
+__global__ void k_sp_tab_chunks(const SpTab *tab, int n, SpChunk *chunks) {
+    const int c = blockIdx.x, t = threadIdx.x;
     const uint64_t zmask = (1ull << n) - 1;
     uint32_t rx = 0, rz = 0, e = 0;
     for (int j = 0; j < kSpChunkQubits; ++j) {
@@ -241,7 +164,7 @@ __global__ void k_sp_tab_chunks(const SpTab *tabs, int n, SpChunk *chunks) {
         if (q >= n) break;
         for (int part = 0; part < 2; ++part) {   // X_q, then Z_q
             if (!((t >> (part * kSpChunkQubits + j)) & 1)) continue;
-            const SpTab g = tabs[(size_t)r * 64 + (part ? n + q : q)];
+            const SpTab g = tab[part ? n + q : q];
             const uint32_t gx = (uint32_t)(g.key >> n), gz = (uint32_t)(g.key & zmask);
             e += sp_mul_phase(rx, rz, gx, gz) + (g.neg ? 2u : 0u);
             rx ^= gx;
@@ -253,207 +176,515 @@ __global__ void k_sp_tab_chunks(const SpTab *tabs, int n, SpChunk *chunks) {
 
 // U P U^dagger from the tableau: P(x, z) = i^{|x & z|} prod_q X_q^{x_q} Z_q^{z_q}
 // (Y = i X Z), so its image is i^{|x & z|} times the product of the generator
-// images in that order, each factor adding its phase and sign.  The product
-// is taken chunk by chunk from the run's chunk table (staged in shared
-// memory): ceil(n / 4) lookups and string products per term instead of one
-// product per set bit.
-__global__ void __launch_bounds__(kSpThreads) k_sp_cliff_tab(uint64_t *keys, double *vals,
-                                                              int64_t *counts,
-                                                              const int32_t *flags, int step,
-                                                              int n, const SpChunk *chunks) {
+// images in that order, taken chunk by chunk: ceil(n / 4) lookups and string
+// products.  A Hermitian image: e is 0 or 2 (mod 4).
+__device__ __forceinline__ uint64_t sp_image(uint64_t k, int n, const SpChunk *chunks, bool &neg) {
+    const uint32_t x = (uint32_t)(k >> n), z = (uint32_t)(k & ((1ull << n) - 1ull));
+    uint32_t rx = 0, rz = 0, e = (uint32_t)__popc(x & z);
+    for (int c = 0; c < (n + kSpChunkQubits - 1) / kSpChunkQubits; ++c) {
+        const uint32_t sh = (uint32_t)(kSpChunkQubits * c);
+        const SpChunk g = chunks[c * 256 + (((x >> sh) & 15u) | (((z >> sh) & 15u) << 4))];
+        e += g.e + sp_mul_phase(rx, rz, g.x, g.z);
+        rx ^= g.x;
+        rz ^= g.z;
+    }
+    neg = (e & 2u) != 0;
+    return ((uint64_t)rx << n) | rz;
+}
+
+__global__ void __launch_bounds__(kSpThreads) k_sp_images(const uint64_t *keys, const double *vals,
+                                                           int64_t count, int n,
+                                                           const SpChunk *chunks, DevTerm *out,
+                                                           stab_term *terms) {
     __shared__ SpChunk sc[kSpChunks * 256];
-    if (sp_stopped_before(flags, step)) return;
     const int n_ch = (n + kSpChunkQubits - 1) / kSpChunkQubits;
     for (int k = threadIdx.x; k < n_ch * 256; k += blockDim.x) sc[k] = chunks[k];
     __syncthreads();
-    const int64_t count = counts[step];
-    if (blockIdx.x == 0 && threadIdx.x == 0) counts[step + 1] = count;
-    const uint64_t zmask = (1ull << n) - 1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = keys[i];
-        const uint32_t x = (uint32_t)(k >> n), z = (uint32_t)(k & zmask);
-        uint32_t rx = 0, rz = 0, e = (uint32_t)__popc(x & z);
-        for (int c = 0; c < n_ch; ++c) {
-            const uint32_t sh = (uint32_t)(kSpChunkQubits * c);
-            const SpChunk g = sc[c * 256 + (((x >> sh) & 15u) | (((z >> sh) & 15u) << 4))];
-            e += g.e + sp_mul_phase(rx, rz, g.x, g.z);
-            rx ^= g.x;
-            rz ^= g.z;
+        bool neg;
+        const uint64_t k = sp_image(keys[i], n, sc, neg);
+        const double v = neg ? -vals[i] : vals[i];
+        if (out) out[i] = DevTerm{v, k};
+        if (terms) {
+            terms[i].coeff = v;
+            terms[i].x = k >> n;
+            terms[i].z = k & ((1ull << n) - 1ull);
         }
-        // a Hermitian image: e is 0 or 2 (mod 4)
-        keys[i] = ((uint64_t)rx << n) | rz;
-        if (e & 2u) vals[i] = -vals[i];
     }
 }
 
-__global__ void __launch_bounds__(kSpThreads) k_sp_insert(const uint64_t *keys,
-                                                           const int64_t *counts,
-                                                           const int32_t *flags, int step, int n,
-                                                           int q, int axis, SpSlot *table,
-                                                           int log_h,
-                                                           int32_t *slot_of, int32_t *err) {
-    if (sp_stopped_before(flags, step)) return;
-    const int64_t count = counts[step];
-    uint32_t u, v;
-    sp_pair(axis, u, v);
-    const uint32_t mask = (1u << log_h) - 1u;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = keys[i];
-        const uint32_t L = sp_letter(k, n, q);
-        if (L != u && L != v) continue;
-        uint32_t s = sp_hash(k, log_h);
-        // the table is at least twice the list, so a free slot is near; the
-        // bound only guards against a corrupted table
-        bool ok = false;
-        for (uint32_t probe = 0; probe <= mask; ++probe) {
-            if (atomicCAS(&table[s].pos, -1, (int32_t)i) == -1) {
-                table[s].key = k;
-                slot_of[i] = (int32_t)s;
-                ok = true;
-                break;
+// ---------------------------------------------------------------- one CTA
+
+// Lists of up to kSpSmallCap terms, in shared memory: two buffers of keys and
+// coefficients, a table of positions of twice that (the key is looked up by the
+// position), the partners.  A thread takes at most four neighbouring terms.  A
+// rotation is three barriers and their latency, 1 to 2 us; as four launches it
+// was about 20.  The rotation whose list would not fit is left to the grid kernel.
+constexpr int kSmallThreads = 1024, kSmallPer = kSpSmallCap / kSmallThreads;
+constexpr int kSmallLog = 13, kSmallRots = 64;
+struct SpSmall {
+    uint64_t key[2][kSpSmallCap];
+    double val[2][kSpSmallCap];
+    int32_t table[1 << kSmallLog];
+    int32_t partner[kSpSmallCap];
+    SpRot rot[kSmallRots];
+    double2 cs[kSmallRots];
+    int32_t sh[32];
+};
+static_assert((1 << kSmallLog) >= 2 * kSpSmallCap, "a free slot is always near");
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_sp_small(SpRunArgs a) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    SpSmall &S = *reinterpret_cast<SpSmall *>(raw);
+    const int t = threadIdx.x;
+    int count = (int)a.st->count, cur = 0, r = 0, stop = SP_RUNNING;
+    const int64_t lim = a.cap < kSpSmallCap ? a.cap : (int64_t)kSpSmallCap;
+    for (int i = t; i < count; i += kSmallThreads) {
+        S.key[0][i] = a.init[i];
+        S.val[0][i] = __longlong_as_double((long long)a.init[count + i]);
+    }
+    for (int i = t; i < (1 << kSmallLog); i += kSmallThreads) S.table[i] = -1;
+    for (int i = t; i < kSpSmallCap; i += kSmallThreads) S.partner[i] = -1;
+    __syncthreads();
+    for (; r < a.n_rot; ++r) {
+        if (r % kSmallRots == 0) {
+            if (t < kSmallRots && r + t < a.n_rot) {
+                const SpRot d = a.rots[r + t];
+                S.rot[t] = d;
+                S.cs[t] = double2{a.cs[2 * d.param],
+                                  a.inverse ? -a.cs[2 * d.param + 1] : a.cs[2 * d.param + 1]};
             }
-            s = (s + 1u) & mask;
+            __syncthreads();
         }
-        if (!ok) {
-            slot_of[i] = -1;
-            atomicExch(err, 1);
+        const SpRot d = S.rot[r % kSmallRots];
+        const double2 cs = S.cs[r % kSmallRots];
+        const int per = (count + kSmallThreads - 1) / kSmallThreads;
+        const int i0 = t * per;
+        int slot[kSmallPer];
+#pragma unroll
+        for (int j = 0; j < kSmallPer; ++j) {
+            const int i = i0 + j;
+            slot[j] = -1;
+            if (j >= per || i >= count) continue;
+            const uint64_t k = S.key[cur][i];
+            if (!sp_anti(k, d)) continue;
+            uint32_t s = (uint32_t)(sp_hash(sp_is_u(k, d) ? k : k ^ d.P) >> (64 - kSmallLog));
+            for (int probe = 0; probe < (1 << kSmallLog); ++probe) {
+                const int p = atomicCAS(&S.table[s], -1, i);
+                if (p == -1) {
+                    slot[j] = (int)s;
+                    break;
+                }
+                if ((S.key[cur][p] ^ k) == d.P) {
+                    S.partner[i] = p;
+                    S.partner[p] = i;
+                    break;
+                }
+                s = (s + 1u) & ((1u << kSmallLog) - 1u);
+            }
         }
+        __syncthreads();
+        uint64_t k0[kSmallPer], k1[kSmallPer];
+        double v0[kSmallPer], v1[kSmallPer];
+        int e[kSmallPer], mine = 0;
+#pragma unroll
+        for (int j = 0; j < kSmallPer; ++j) {
+            const int i = i0 + j;
+            const bool in = j < per && i < count;
+            e[j] = 0;
+            if (!__any_sync(0xffffffffu, in)) continue;
+            const int p = in ? S.partner[i] : -1;
+            e[j] = sp_images(in, __any_sync(0xffffffffu, p >= 0), in ? S.key[cur][i] : 0ull,
+                             in ? S.val[cur][i] : 0.0, p >= 0, p >= 0 ? S.val[cur][p] : 0.0, d,
+                             a.n, cs.x, cs.y, k0[j], v0[j], k1[j], v1[j]);
+            mine += e[j];
+            if (p >= 0) S.partner[i] = -1;
+            if (slot[j] >= 0) S.table[slot[j]] = -1;
+        }
+        int total;
+        int at = block_exclusive_scan<int>(mine, total, S.sh);
+        if (total > lim) break;
+#pragma unroll
+        for (int j = 0; j < kSmallPer; ++j) {
+            if (e[j] > 0) {
+                S.key[1 - cur][at] = k0[j];
+                S.val[1 - cur][at] = v0[j];
+                ++at;
+            }
+            if (e[j] > 1) {
+                S.key[1 - cur][at] = k1[j];
+                S.val[1 - cur][at] = v1[j];
+                ++at;
+            }
+        }
+        if (t == 0) a.counts[r + 1] = total;
+        count = total;
+        cur ^= 1;
+        __syncthreads();
+        if (a.threshold > 0 && total > a.threshold) {
+            stop = SP_THRESHOLD;
+            ++r;
+            break;
+        }
+    }
+    for (int i = t; i < count; i += kSmallThreads) {
+        a.keys[0][i] = S.key[cur][i];
+        a.vals[0][i] = S.val[cur][i];
+    }
+    if (t == 0) {
+        a.st->count = count;
+        a.st->rot = r;
+        a.st->buf = 0;
+        a.st->stop = stop;
     }
 }
 
-__device__ __forceinline__ int32_t sp_lookup(uint64_t k, const SpSlot *table, int log_h) {
-    const uint32_t mask = (1u << log_h) - 1u;
-    uint32_t s = sp_hash(k, log_h);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        // one 16-byte load: key and position of the slot
-        const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(table + s);
-        const int32_t p = (int32_t)(uint32_t)e.y;
-        if (p < 0) return -1;
-        if (e.x == k) return p;
-        s = (s + 1u) & mask;
-    }
-    return -1;
+// ---------------------------------------------------------------- whole GPU
+
+constexpr int kRunThreads = 512, kRunPer = 4;
+constexpr int kRunWarps = kRunThreads / 32, kRunRots = 64;
+constexpr uint32_t kRunPolls = 1u << 22;     // a second or two
+constexpr int kTileBits = 32;                // a tile word: step tag, emitted terms
+
+// Table slots (log2) for a list: four a term while that is no more than 8 MB
+// (a claim that meets another costs a round trip to L2, and the slowest chain
+// of a phase counts), one and a half beyond, where clearing counts.
+__host__ __device__ __forceinline__ int sp_table_bits(int64_t count) {
+    int l = 12;
+    while (l < 20 && (1ll << l) < 4 * count) ++l;
+    while ((1ll << l) < count + (count >> 1)) ++l;
+    return l;
 }
 
-__global__ void __launch_bounds__(kSpThreads) k_sp_count(const uint64_t *keys,
-                                                          const double *vals,
-                                                          const int64_t *counts,
-                                                          const int32_t *flags, int step, int n,
-                                                          int q, int axis, const double *cs,
-                                                          int param, int inverse,
-                                                          const SpSlot *table, int log_h,
-                                                          int32_t *partner, int64_t *blk) {
-    __shared__ int64_t sh[32];
-    if (sp_stopped_before(flags, step)) return;
-    const int64_t count = counts[step];
-    int64_t lo, hi;
-    sp_block_range(count, lo, hi);
-    double c, s;
-    sp_rot_cs(cs, param, inverse, c, s);
-    uint32_t u, v;
-    sp_pair(axis, u, v);
-    int64_t mine = 0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const uint64_t k = keys[i];
-        const uint32_t L = sp_letter(k, n, q);
-        int32_t p = -1;
-        if (L == u || L == v) {
-            p = sp_lookup(sp_with_letter(k, n, q, L == u ? v : u), table, log_h);
-            partner[i] = p;
-        }
-        uint64_t k0, k1;
-        double v0, v1;
-        mine += sp_images(k, vals[i], p, vals, n, q, axis, c, s, k0, v0, k1, v1);
-    }
-    int64_t total;
-    (void)block_exclusive_scan<int64_t>(mine, total, sh);
-    if (threadIdx.x == 0) blk[blockIdx.x] = total;
+// Tiles of a list of up to `cap` terms: G a round, kRunPer * kRunThreads terms at most.
+__host__ __device__ __forceinline__ int64_t sp_tile_words(int64_t cap, int64_t G) {
+    return cap / (kRunPer * kRunThreads) + G;
 }
 
-// One CTA of 1024 threads: exclusive scan of nblk <= 1024 block totals.
-__global__ void __launch_bounds__(1024) k_sp_scan(int64_t *blk, int nblk, int64_t *counts,
-                                                  int32_t *flags, int step, int64_t cap,
-                                                  int64_t threshold) {
-    __shared__ int64_t sh[32];
-    if (sp_stopped_before(flags, step)) return;
-    const int64_t x = (int)threadIdx.x < nblk ? blk[threadIdx.x] : 0;
-    int64_t total;
-    const int64_t ex = block_exclusive_scan<int64_t>(x, total, sh);
-    if ((int)threadIdx.x < nblk) blk[threadIdx.x] = ex;
+// All CTAs of the cooperative launch meet; false once a wait gave up.
+__device__ bool sp_grid_sync(SpState *st, uint32_t want, int *s_ok) {
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (total > cap) {
-            flags[0] = 1;          // overflow: the step is not applied
-            flags[1] = step;
-        } else {
-            counts[step + 1] = total;
-            if (threshold > 0 && total > threshold) {
-                flags[0] = 2;      // order above the threshold after this step
-                flags[1] = step;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" : : "l"(&st->arrived) : "memory");
+        bool ok = false;
+        for (uint32_t it = 0; it < kRunPolls && !ok; ++it) {
+            uint32_t seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                         : "=r"(seen) : "l"(&st->arrived) : "memory");
+            ok = (int32_t)(seen - want) >= 0;
+        }
+        if (!ok) atomicExch(&st->err, 2);
+        *s_ok = ok ? 1 : 0;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+// Rotations from the state's on, two grid barriers each.  The table takes the
+// list's size (1.5 slots a term at least, 8 bytes each: it stays in L2 up to
+// lists of ten million terms; one of the capacity's size did not).  Positions: a tile of
+// the write phase needs the emitted terms before it.  CTA b holds tiles b,
+// b + G, ...: between two of its tiles lie exactly G - 1 others, whose totals
+// it reads at once (a thread each, tagged with the step, so no clearing); the
+// tiles are all in flight on resident CTAs, which publish before they wait.
+// What other CTAs wrote is read past L1.
+struct SpTile {
+    uint64_t key[2 * kRunPer * kRunThreads];
+    double val[2 * kRunPer * kRunThreads];
+    SpRot rot[kRunRots];
+    double2 cs[kRunRots];
+    int64_t red[kRunWarps];
+    int32_t wt[kRunPer * kRunWarps];
+    int32_t own, ok;
+};
+
+__global__ void __launch_bounds__(kRunThreads, 2) k_sp_run(SpRunArgs a) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    SpTile &S = *reinterpret_cast<SpTile *>(raw);
+    SpState *st = a.st;
+    int64_t count = st->count;
+    int r = st->rot, cur = st->buf, stop = st->stop;
+    if (stop != SP_RUNNING || r >= a.n_rot) return;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t G = gridDim.x, b = blockIdx.x;
+    uint32_t meets = 0;
+    // tags of an earlier launch could match this one's
+    {
+        const int64_t words = sp_tile_words(a.cap, G);
+        for (int64_t i = b * kRunThreads + t; i < words; i += G * kRunThreads) a.tiles[i] = 0;
+    }
+    const int r0 = r;
+    for (; r < a.n_rot; ++r) {
+        if ((r - r0) % kRunRots == 0) {
+            if (t < kRunRots && r + t < a.n_rot) {
+                const SpRot f = a.rots[r + t];
+                S.rot[t] = f;
+                S.cs[t] = double2{a.cs[2 * f.param],
+                                  a.inverse ? -a.cs[2 * f.param + 1] : a.cs[2 * f.param + 1]};
+            }
+            __syncthreads();
+        }
+        const SpRot d = S.rot[(r - r0) % kRunRots];
+        const double c = S.cs[(r - r0) % kRunRots].x, s = S.cs[(r - r0) % kRunRots].y;
+        const uint64_t *keys = cur ? a.keys[1] : a.keys[0];
+        const double *vals = cur ? a.vals[1] : a.vals[0];
+        const int log_h = sp_table_bits(count);
+        const uint32_t mask = (1u << log_h) - 1u;
+        // as many rounds as full tiles would take, of equal tiles (whole warps: a
+        // full tile in a last round that few CTAs have took as long as one that
+        // all have, and so did a short list in few full tiles)
+        const int64_t full = G * kRunPer * kRunThreads, rounds = count > full ? (count + full - 1) / full : 1;
+        const int64_t even = (count + G * rounds - 1) / (G * rounds);
+        const int tile_terms = count > 0 ? (int)((even + 31) / 32 * 32) : 32;
+        // pair
+        uint64_t next[kRunPer];
+        auto look = [&](int64_t base) {
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                const int64_t i = base + j * kRunThreads + t;
+                next[j] = j * kRunThreads + t < tile_terms && i < count ? __ldcg((const unsigned long long *)keys + i) : 0ull;
+            }
+        };
+        look(b * tile_terms);
+        for (int64_t base = b * tile_terms; base < count; base += G * tile_terms) {
+            uint64_t k[kRunPer], old[kRunPer], mine[kRunPer];
+            uint32_t slot[kRunPer];
+            bool anti[kRunPer];
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) k[j] = next[j];
+            look(base + G * tile_terms);
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                // no key (zero, or past the end) is one that commutes with all
+                anti[j] = sp_anti(k[j], d);
+                const uint64_t h = sp_hash(sp_is_u(k[j], d) ? k[j] : k[j] ^ d.P);
+                slot[j] = (uint32_t)(h >> (64 - log_h));
+                mine[j] = ((uint64_t)(uint32_t)(h >> (32 - log_h)) << 32) |
+                          (uint32_t)(base + j * kRunThreads + t);
+                old[j] = kSpFree;
+                if (anti[j])
+                    old[j] = atomicCAS((unsigned long long *)a.table + slot[j], kSpFree, mine[j]);
+            }
+            // the terms that met an occupied slot look on together (one after the
+            // other they made this phase three times as long), each at its own odd
+            // step: neighbouring slots grow chains of 18 round trips among 250,000
+            // terms, which the whole GPU waited for
+            for (uint32_t probe = 0;; ++probe) {
+                bool more = false;
+#pragma unroll
+                for (int j = 0; j < kRunPer; ++j) {
+                    if (old[j] == kSpFree) continue;
+                    if ((uint32_t)(old[j] >> 32) == (uint32_t)(mine[j] >> 32)) {
+                        const uint32_t p = (uint32_t)old[j];
+                        if ((__ldcg((const unsigned long long *)keys + p) ^ k[j]) == d.P) {
+                            const uint32_t i = (uint32_t)mine[j];
+                            a.partner[i] = (int32_t)p;
+                            a.partner[p] = (int32_t)i;
+                            old[j] = kSpFree;
+                            continue;
+                        }
+                    }
+                    slot[j] = (slot[j] + ((uint32_t)(mine[j] >> 32) | 1u)) & mask;
+                    more = true;
+                }
+                if (!more) break;
+                if (probe > mask) {          // only guards against a corrupted table
+                    atomicExch(&st->err, 1);
+                    break;
+                }
+#pragma unroll
+                for (int j = 0; j < kRunPer; ++j)
+                    if (old[j] != kSpFree)
+                        old[j] = atomicCAS((unsigned long long *)a.table + slot[j], kSpFree,
+                                           mine[j]);
             }
         }
+        if (!sp_grid_sync(st, (uint32_t)G * ++meets, &S.ok)) return;
+        // write
+        const int64_t n_tiles = count > 0 ? (count + tile_terms - 1) / tile_terms : 1;
+        uint64_t *keys_out = cur ? a.keys[0] : a.keys[1];
+        double *vals_out = cur ? a.vals[0] : a.vals[1];
+        const uint64_t tag = (uint64_t)(uint32_t)(r + 1) << kTileBits;
+        {
+            const uint4 free4{~0u, ~0u, ~0u, ~0u};
+            const int64_t quads = (int64_t)1 << (log_h - 1);
+            for (int64_t i = b * kRunThreads + t; i < quads; i += G * kRunThreads)
+                reinterpret_cast<uint4 *>(a.table)[i] = free4;
+        }
+        int64_t before = 0;                  // emitted by this CTA's last tile and all before it
+        uint64_t k[kRunPer];
+        double v[kRunPer];
+        int32_t p[kRunPer];
+        auto fetch = [&](int64_t tile) {
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                const int64_t i = tile * tile_terms + j * kRunThreads + t;
+                const bool in = j * kRunThreads + t < tile_terms && i < count;
+                k[j] = in ? __ldcg((const unsigned long long *)keys + i) : 0ull;
+                v[j] = in ? __ldcg(vals + i) : 0.0;
+                p[j] = in ? __ldcg(a.partner + i) : -1;
+            }
+        };
+        fetch(b);
+        for (int64_t tile = b; tile < n_tiles; tile += G) {
+            uint64_t k1[kRunPer];
+            double v1[kRunPer], pv[kRunPer];
+            int32_t at[kRunPer];
+            int e[kRunPer];
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                const int64_t i = tile * tile_terms + j * kRunThreads + t;
+                pv[j] = 0.0;
+                if (p[j] >= 0) {
+                    pv[j] = __ldcg(vals + p[j]);
+                    a.partner[i] = -1;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                const bool in = j * kRunThreads + t < tile_terms &&
+                                tile * tile_terms + j * kRunThreads + t < count;
+                e[j] = 0;
+                if (__any_sync(0xffffffffu, in)) {
+                    const uint64_t key = k[j];
+                    const double val = v[j];
+                    e[j] = sp_images(in, __any_sync(0xffffffffu, p[j] >= 0), key, val, p[j] >= 0,
+                                     pv[j], d, a.n, c, s, k[j], v[j], k1[j], v1[j]);
+                }
+                const uint32_t one = __ballot_sync(0xffffffffu, e[j] > 0);
+                const uint32_t two = __ballot_sync(0xffffffffu, e[j] > 1);
+                const uint32_t lt = (1u << lane) - 1u;
+                at[j] = __popc(one & lt) + __popc(two & lt);
+                if (lane == 0) S.wt[j * kRunWarps + warp] = __popc(one) + __popc(two);
+            }
+            __syncthreads();
+            if (warp == 0) {                 // exclusive scan of the warp totals
+                constexpr int kTot = kRunPer * kRunWarps / 32;
+                int x[kTot], incl = 0;
+#pragma unroll
+                for (int k2 = 0; k2 < kTot; ++k2) {
+                    x[k2] = incl;
+                    incl += S.wt[kTot * lane + k2];
+                }
+                const int mine = incl;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+#pragma unroll
+                for (int k2 = 0; k2 < kTot; ++k2) S.wt[kTot * lane + k2] = incl - mine + x[k2];
+                if (lane == 31) {
+                    *(volatile unsigned long long *)(a.tiles + tile) = tag | (uint32_t)incl;
+                    S.own = incl;
+                }
+            }
+            __syncthreads();
+            const int own = S.own;
+#pragma unroll
+            for (int j = 0; j < kRunPer; ++j) {
+                const int o = S.wt[j * kRunWarps + warp] + at[j];
+                if (e[j] > 0) {
+                    S.key[o] = k[j];
+                    S.val[o] = v[j];
+                }
+                if (e[j] > 1) {
+                    S.key[o + 1] = k1[j];
+                    S.val[o + 1] = v1[j];
+                }
+            }
+            if (tile + G < n_tiles) fetch(tile + G);
+            // the tiles between this CTA's last one and this one
+            int64_t sum = 0;
+            bool ok = true;
+            for (int64_t u = tile - G + 1 + t; u < tile; u += kRunThreads) {
+                if (u < 0) continue;
+                uint64_t w = 0;
+                uint32_t it = 0;
+                do {
+                    w = *(volatile unsigned long long *)(a.tiles + u);
+                } while ((w >> kTileBits) != (tag >> kTileBits) && ++it < kRunPolls);
+                if ((w >> kTileBits) != (tag >> kTileBits)) ok = false;
+                sum += (int64_t)(uint32_t)w;
+            }
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0) S.red[warp] = sum;
+            if (!__syncthreads_and(ok)) {
+                if (t == 0) atomicExch(&st->err, 2);
+                return;
+            }
+            for (int w = 0; w < kRunWarps; ++w) before += S.red[w];
+            for (int i = t; i < own; i += kRunThreads) {
+                if (before + i < a.cap) {
+                    keys_out[before + i] = S.key[i];
+                    vals_out[before + i] = S.val[i];
+                }
+            }
+            before += own;
+            if (tile == n_tiles - 1 && t == 0) a.counts[r + 1] = before;
+            __syncthreads();                 // the tile's arrays are used again
+        }
+        if (!sp_grid_sync(st, (uint32_t)G * ++meets, &S.ok)) return;
+        const int64_t total = __ldcg((const long long *)a.counts + r + 1);
+        if (total > a.cap) {
+            stop = SP_OVERFLOW;
+            break;
+        }
+        count = total;
+        cur ^= 1;
+        if (a.threshold > 0 && total > a.threshold) {
+            stop = SP_THRESHOLD;
+            ++r;
+            break;
+        }
+    }
+    if (b == 0 && t == 0) {
+        st->count = count;
+        st->rot = r;
+        st->buf = cur;
+        st->stop = stop;
     }
 }
 
-__global__ void __launch_bounds__(kSpThreads) k_sp_write(
-    const uint64_t *keys, const double *vals, const int64_t *counts, const int32_t *flags,
-    int step, int n, int q, int axis, const double *cs, int param, int inverse,
-    SpSlot *table, const int32_t *slot_of, const int32_t *partner, const int64_t *blk,
-    uint64_t *keys_out, double *vals_out) {
-    __shared__ int64_t sh[32];
-    if (sp_stopped_before(flags, step)) return;
-    if (flags[0] == 1 && flags[1] == step) return;
-    const int64_t count = counts[step];
-    int64_t lo, hi;
-    sp_block_range(count, lo, hi);
-    double c, s;
-    sp_rot_cs(cs, param, inverse, c, s);
-    uint32_t u, v;
-    sp_pair(axis, u, v);
-    int64_t base = blk[blockIdx.x];
-    for (int64_t t0 = lo; t0 < hi; t0 += blockDim.x) {
-        const int64_t i = t0 + threadIdx.x;
-        uint64_t k0 = 0, k1 = 0;
-        double v0 = 0.0, v1 = 0.0;
-        int e = 0;
-        if (i < hi) {
-            const uint64_t k = keys[i];
-            const uint32_t L = sp_letter(k, n, q);
-            int32_t p = -1;
-            if (L == u || L == v) {
-                p = partner[i];
-                const int32_t slot = slot_of[i];
-                if (slot >= 0) table[slot].pos = -1;
-            }
-            e = sp_images(k, vals[i], p, vals, n, q, axis, c, s, k0, v0, k1, v1);
-        }
-        int64_t tile_total;
-        const int64_t at = base + block_exclusive_scan<int64_t>(e, tile_total, sh);
-        if (e > 0) {
-            keys_out[at] = k0;
-            vals_out[at] = v0;
-        }
-        if (e > 1) {
-            keys_out[at + 1] = k1;
-            vals_out[at + 1] = v1;
-        }
-        base += tile_total;
-    }
-}
-
-// Fixed-order sum of the coefficients of the x-free strings (x = key >> n == 0).
-__global__ void __launch_bounds__(kSpThreads) k_sp_xfree(const uint64_t *keys,
-                                                          const double *vals,
-                                                          const int64_t *counts, int step,
-                                                          int n, double *partial) {
+// Fixed-order sum of the coefficients whose images are x-free, in one launch:
+// block sums over contiguous ranges, then one warp of the last block to finish
+// (lane l a contiguous slice of the partials, then a shuffle tree).  The bits
+// of an image's x mask are tried one by one: of lists that are all but random,
+// a term takes two.
+__global__ void __launch_bounds__(kSpThreads) k_sp_xfree(SpRunArgs a, const uint64_t *xcol,
+                                                          const SpChunk *chunks,
+                                                          double *partial) {
     __shared__ double red[kSpThreads / 32];
-    const int64_t count = counts[step];
-    int64_t lo, hi;
-    sp_block_range(count, lo, hi);
+    __shared__ uint64_t col[32];
+    __shared__ int last;
+    const int n = a.n;
+    if ((int)threadIdx.x < n) col[threadIdx.x] = xcol[threadIdx.x];
+    __syncthreads();
+    const int64_t count = a.st->count;
+    const uint64_t *keys = a.keys[a.st->buf];
+    const double *vals = a.vals[a.st->buf];
+    const int64_t per = (count + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = min((int64_t)blockIdx.x * per, count), hi = min(lo + per, count);
     double acc = 0.0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        if ((keys[i] >> n) == 0) acc += vals[i];
+    constexpr int kAhead = 8;
+    for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += kAhead * kSpThreads) {
+        uint64_t k[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j)
+            k[j] = i0 + j * kSpThreads < hi ? keys[i0 + j * kSpThreads] : 0ull;
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int64_t i = i0 + j * kSpThreads;
+            int q = i < hi ? 0 : -1;
+            while (q >= 0 && q < n && !sp_parity(k[j] & col[q])) ++q;
+            if (q == n) {
+                bool neg;
+                (void)sp_image(k[j], n, chunks, neg);
+                acc += neg ? -vals[i] : vals[i];
+            }
+        }
+    }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -461,33 +692,24 @@ __global__ void __launch_bounds__(kSpThreads) k_sp_xfree(const uint64_t *keys,
         double t = 0.0;
         for (int w = 0; w < kSpThreads / 32; ++w) t += red[w];
         partial[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(&a.st->blocks, 1u) == gridDim.x - 1;
     }
-}
-
-// One warp: lane l sums a contiguous slice of the partials, then a fixed
-// shuffle tree; the order depends only on nblk.
-__global__ void k_sp_sum_partials(const double *partial, int nblk, double *out) {
-    const int lane = threadIdx.x;
-    const int per = (nblk + 31) / 32;
-    double t = 0.0;
-    for (int b = lane * per; b < nblk && b < (lane + 1) * per; ++b) t += partial[b];
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    constexpr int kPer = kSpMaxBlocks / 32;
+    static_assert(kPer * 32 == kSpMaxBlocks, "whole slices");
+    double p[kPer], t = 0.0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) p[j] = __ldcg(partial + threadIdx.x * kPer + j);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) t += p[j];
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) *out = t;
-}
-
-__global__ void k_sp_to_terms(const uint64_t *keys, const double *vals, const int64_t *counts,
-                              int step, DevTerm *out) {
-    const int64_t count = counts[step];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = DevTerm{vals[i], keys[i]};
-}
-
-int sp_grid(int64_t bound) {
-    int64_t b = (bound + 2047) / 2048;
-    if (b < 1) b = 1;
-    if (b > kSpMaxBlocks) b = kSpMaxBlocks;
-    return (int)b;
+    if (threadIdx.x == 0) {
+        a.st->value = t;
+        a.st->blocks = 0;
+    }
 }
 
 }  // namespace
@@ -499,59 +721,58 @@ cudaError_t launch_sp_cos_sin(const double *thetas, int64_t n_params, double *cs
     return cudaGetLastError();
 }
 
-cudaError_t launch_sp_cliff(uint64_t *keys, double *vals, int64_t *counts, const int32_t *flags,
-                            int step, int n, const SpGate *gates, int n_gates, int64_t bound,
-                            cudaStream_t st) {
-    k_sp_cliff<<<sp_grid(bound), kSpThreads, 0, st>>>(keys, vals, counts, flags, step, n, gates,
-                                                        n_gates);
+cudaError_t launch_sp_chunks(const SpTab *tab, int n, SpChunk *chunks, cudaStream_t st) {
+    k_sp_tab_chunks<<<kSpChunks, 256, 0, st>>>(tab, n, chunks);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sp_tableau(const SpGate *gates, const int32_t *run_first,
-                              const int32_t *run_count, int n_runs, int n, SpTab *tabs,
-                              SpChunk *chunks, cudaStream_t st) {
-    if (n_runs == 0) return cudaSuccess;
-    k_sp_tableau<<<n_runs, 64, 0, st>>>(gates, run_first, run_count, n, tabs);
-    cudaError_t e = cudaGetLastError();
+int sp_table_log(int64_t count) { return sp_table_bits(count); }
+
+int64_t sp_tiles(int64_t cap, int grid) { return sp_tile_words(cap, grid); }
+
+cudaError_t sp_run_grid(int device, int *grid) {
+    int sms = 0, per = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sp_run, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(SpTile));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sp_run, kRunThreads,
+                                                          sizeof(SpTile));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sp_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(SpSmall));
     if (e != cudaSuccess) return e;
-    k_sp_tab_chunks<<<n_runs * kSpChunks, 256, 0, st>>>(tabs, n, chunks);
+    *grid = sms * (per < 2 ? per : 2);
+    return *grid > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
+}
+
+cudaError_t launch_sp_small(const SpRunArgs &a, cudaStream_t st) {
+    k_sp_small<<<1, kSmallThreads, sizeof(SpSmall), st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sp_cliff_tab(uint64_t *keys, double *vals, int64_t *counts,
-                                const int32_t *flags, int step, int n, const SpChunk *chunks,
-                                int64_t bound, cudaStream_t st) {
-    k_sp_cliff_tab<<<sp_grid(bound), kSpThreads, 0, st>>>(keys, vals, counts, flags, step, n,
-                                                           chunks);
+cudaError_t launch_sp_run(const SpRunArgs &a, cudaStream_t st) {
+    SpRunArgs args = a;
+    void *params[] = {&args};
+    return cudaLaunchCooperativeKernel((const void *)k_sp_run, dim3((unsigned)a.grid),
+                                       dim3(kRunThreads), params, sizeof(SpTile), st);
+}
+
+cudaError_t launch_sp_xfree(const SpRunArgs &a, const uint64_t *xcol, const SpChunk *chunks,
+                            double *partial, cudaStream_t st) {
+    k_sp_xfree<<<kSpMaxBlocks, kSpThreads, 0, st>>>(a, xcol, chunks, partial);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sp_rotation(const SpRotArgs &a, cudaStream_t st) {
-    const int grid = sp_grid(a.bound);
-    k_sp_insert<<<grid, kSpThreads, 0, st>>>(a.keys, a.counts, a.flags, a.step, a.n, a.q,
-                                              a.axis, a.table, a.log_h, a.slot_of,
-                                              a.err);
-    k_sp_count<<<grid, kSpThreads, 0, st>>>(a.keys, a.vals, a.counts, a.flags, a.step, a.n, a.q,
-                                             a.axis, a.cs, a.param, a.inverse, a.table,
-                                             a.log_h, a.partner, a.blk);
-    k_sp_scan<<<1, 1024, 0, st>>>(a.blk, grid, a.counts, a.flags, a.step, a.cap, a.threshold);
-    k_sp_write<<<grid, kSpThreads, 0, st>>>(a.keys, a.vals, a.counts, a.flags, a.step, a.n, a.q,
-                                             a.axis, a.cs, a.param, a.inverse, a.table,
-                                             a.slot_of, a.partner, a.blk, a.keys_out,
-                                             a.vals_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sp_xfree(const uint64_t *keys, const double *vals, const int64_t *counts,
-                            int step, int n, double *partial, double *out, cudaStream_t st) {
-    k_sp_xfree<<<kSpMaxBlocks, kSpThreads, 0, st>>>(keys, vals, counts, step, n, partial);
-    k_sp_sum_partials<<<1, 32, 0, st>>>(partial, kSpMaxBlocks, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sp_to_terms(const uint64_t *keys, const double *vals, const int64_t *counts,
-                               int step, DevTerm *out, int64_t bound, cudaStream_t st) {
-    k_sp_to_terms<<<sp_grid(bound), kSpThreads, 0, st>>>(keys, vals, counts, step, out);
+cudaError_t launch_sp_images(const uint64_t *keys, const double *vals, int64_t count, int n,
+                             const SpChunk *chunks, DevTerm *out, stab_term *terms,
+                             cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    int64_t blocks = (count + 511) / 512;
+    if (blocks > kSpMaxBlocks) blocks = kSpMaxBlocks;
+    k_sp_images<<<(unsigned)blocks, kSpThreads, 0, st>>>(keys, vals, count, n, chunks, out,
+                                                         terms);
     return cudaGetLastError();
 }
 

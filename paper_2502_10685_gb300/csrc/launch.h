@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "../../include/stab.h"
 #include "stab_internal.h"
 
 namespace stab {
@@ -433,10 +434,18 @@ cudaError_t launch_run_grads(const UniRun *runs, int n_runs, int max_count, cons
 
 // ---------------------------------------------------------------- sparse term lists (k_sparse.cu)
 
-constexpr int kSpMaxBlocks = 608;        // 4 CTAs per SM on 152 SMs
+// A key is z | x << n.
+constexpr int kSpMaxBlocks = 608;        // partial sums of the x-free coefficients
+constexpr int kSpSmallCap = 4096;        // list entries one CTA keeps in shared memory
 
-struct SpGate {                          // one Clifford gate of a run, already inverted for
-    uint8_t op, q0, q1, pad;             // backward runs (S <-> S^dagger)
+// A rotation pulled back through the Clifford gates before it: about the Pauli
+// string P instead of a wire's letter, so those gates need not touch the list.
+struct SpRot {
+    uint64_t P;                          // key of the string
+    uint64_t anti;                       // parity(key & anti): the term anticommutes with P
+    uint64_t letter;                     // parity(key & letter) == (flags & 1): it is the u term
+    int32_t param;
+    uint32_t flags;                      // bit 0 see above, bit 1: the string's sign is minus
 };
 
 struct SpTab {                           // tableau entry: image of X_q or Z_q, its sign
@@ -445,8 +454,8 @@ struct SpTab {                           // tableau entry: image of X_q or Z_q, 
     uint32_t pad;
 };
 
-// A run's tableau regrouped by chunks of 4 qubits (8 generators): per chunk
-// the ordered products of all 256 subsets of its generator images.
+// The tableau regrouped by chunks of 4 qubits (8 generators): per chunk the
+// ordered products of all 256 subsets of its generator images.
 constexpr int kSpChunkQubits = 4;
 constexpr int kSpChunks = 8;             // 32 qubits
 constexpr int kSpChunkEntries = kSpChunks * 256;
@@ -454,53 +463,56 @@ struct SpChunk {                         // x, z of the product string, phase ex
     uint32_t x, z, e, pad;
 };
 
-struct SpSlot {                          // a table slot: key and list position (-1 free)
-    uint64_t key;
-    int32_t pos;
-    int32_t pad;
+enum { SP_RUNNING = 0, SP_OVERFLOW = 1, SP_THRESHOLD = 2 };
+
+// Where a run stands: the list is the one before rotation `rot`, in buffer `buf`.
+struct SpState {
+    int64_t count;
+    int32_t rot, buf;
+    int32_t stop;                        // SP_OVERFLOW: rotation `rot` would not fit (not applied)
+    int32_t err;                         // 1: a table probe ran out, 2: a wait (never expected)
+    uint32_t arrived;                    // the grid barrier
+    uint32_t blocks;                     // blocks of the x-free sum that are done
+    double value;                        // the x-free sum
+    int64_t pad[3];
 };
 
-struct SpRotArgs {
-    const uint64_t *keys;                // input list (keys z | x << n, coefficients)
-    const double *vals;
-    uint64_t *keys_out;                  // output list (the other buffer)
-    double *vals_out;
-    int64_t *counts;                     // counts[step] = order before step
-    int32_t *flags;                      // [0] stop code (1 overflow, 2 threshold), [1] step
-    int32_t step, n, q, axis;            // axis 0/1/2 = R_x/R_y/R_z
-    const double *cs;
-    int32_t param, inverse;
-    SpSlot *table;                       // open-addressing table (one 16-byte slot per probe)
-    int32_t log_h;
-    int32_t *slot_of;                    // per term: its table slot
-    int32_t *partner;                    // per term: position of its partner, -1 absent
-    int64_t *blk;                        // per block: emitted terms, then their offsets
-    int32_t *err;                        // set when a table probe runs out (never expected)
-    int64_t cap;                         // list capacity
-    int64_t threshold;                   // stop above this order (0: never)
-    int64_t bound;                       // host bound on counts[step] (sizes the grid)
+struct SpRunArgs {
+    SpState *st;
+    int64_t *counts;                     // counts[r + 1] = order after rotation r
+    const SpRot *rots;
+    const double *cs;                    // cos, sin per slot
+    int32_t n_rot, n, inverse;
+    int32_t grid;                        // CTAs of the grid kernel, all resident
+    int64_t cap, threshold;              // list capacity; stop above this order (0: never)
+    const uint64_t *init;                // the initial list: keys, then coefficients
+    uint64_t *keys[2];
+    double *vals[2];
+    uint64_t *table;                     // open-addressing table, all slots free between rotations
+    int32_t *partner;                    // per term: position of its partner, -1 absent (and idle)
+    uint64_t *tiles;                     // per tile: step tag and emitted terms
 };
 
-cudaError_t launch_sp_cliff(uint64_t *keys, double *vals, int64_t *counts, const int32_t *flags,
-                            int step, int n, const SpGate *gates, int n_gates, int64_t bound,
-                            cudaStream_t st);
-cudaError_t launch_sp_rotation(const SpRotArgs &a, cudaStream_t st);
 // cs[2 p] = cos(thetas[p]), cs[2 p + 1] = sin(thetas[p]) for every slot
 cudaError_t launch_sp_cos_sin(const double *thetas, int64_t n_params, double *cs,
                               cudaStream_t st);
-// tabs: 64 entries per run (2n used); runs [r] = gates [run_first[r], + run_count[r]);
-// chunks: kSpChunkEntries per run, built from tabs
-cudaError_t launch_sp_tableau(const SpGate *gates, const int32_t *run_first,
-                              const int32_t *run_count, int n_runs, int n, SpTab *tabs,
-                              SpChunk *chunks, cudaStream_t st);
-// chunks: the run's kSpChunkEntries entries
-cudaError_t launch_sp_cliff_tab(uint64_t *keys, double *vals, int64_t *counts,
-                                const int32_t *flags, int step, int n, const SpChunk *chunks,
-                                int64_t bound, cudaStream_t st);
-cudaError_t launch_sp_xfree(const uint64_t *keys, const double *vals, const int64_t *counts,
-                            int step, int n, double *partial, double *out, cudaStream_t st);
-cudaError_t launch_sp_to_terms(const uint64_t *keys, const double *vals, const int64_t *counts,
-                               int step, DevTerm *out, int64_t bound, cudaStream_t st);
+// chunks: kSpChunkEntries, from the tableau's 64 entries (2n used)
+cudaError_t launch_sp_chunks(const SpTab *tab, int n, SpChunk *chunks, cudaStream_t st);
+int sp_table_log(int64_t count);         // table slots (log2) for a list of `count` terms
+int64_t sp_tiles(int64_t cap, int grid); // tile words for lists of up to `cap` terms
+cudaError_t sp_run_grid(int device, int *grid);
+// the rotations while the list fits one CTA's shared memory, from a.init
+cudaError_t launch_sp_small(const SpRunArgs &a, cudaStream_t st);
+// the rest, from the state, on the whole GPU (cooperative launch)
+cudaError_t launch_sp_run(const SpRunArgs &a, cudaStream_t st);
+// st->value: fixed-order sum of the coefficients whose images are x-free;
+// parity(key & xcol[q]) is bit q of an image's x mask
+cudaError_t launch_sp_xfree(const SpRunArgs &a, const uint64_t *xcol, const SpChunk *chunks,
+                            double *partial, cudaStream_t st);
+// the final list's images, in the order of the list: into `out` or `terms`
+cudaError_t launch_sp_images(const uint64_t *keys, const double *vals, int64_t count, int n,
+                             const SpChunk *chunks, DevTerm *out, stab_term *terms,
+                             cudaStream_t st);
 
 }  // namespace stab
 

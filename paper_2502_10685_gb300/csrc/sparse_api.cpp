@@ -1,26 +1,28 @@
 // sparse_api.cpp -- the sparse term-list entry points (include/stab.h): step
-// plans, the launch loop with capacity growth, and the switch to the dense
-// path once the stabilizer order n' passes a threshold (Sec. II-B, Fig. 1).
+// plans, the run with capacity growth, and the switch to the dense path once
+// the stabilizer order n' passes a threshold (Sec. II-B, Fig. 1).
 //
 // A plan is the gate list in application order (backward: reversed, inverse
-// gates) cut into steps: maximal runs of Clifford gates (one launch, every
-// term mapped in place) and single rotations (four launches, k_sparse.cu).
-// The host launches steps ahead without reading the order back: a rotation at
-// most doubles n', so from the last order read it knows how many steps cannot
-// overflow the buffers or cross the threshold; it then reads the orders and
-// the stop flag once.  A step that would overflow is not applied; the buffers
-// grow 8x (the list is copied over) and the loop resumes at that step.
+// gates) cut into steps: maximal runs of Clifford gates and single rotations.
+// On the device only rotations run, each about its string pulled back through
+// the Clifford gates before it (k_sparse.cu); the images of the last list under
+// all of those gates are the result.  A run is one launch while the list is
+// short and one for the rest; its outcome and the orders are read once.  A
+// rotation that would overflow is not applied; the buffers grow 8x (the list is
+// copied over) and the run resumes at it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <new>
 #include <string>
 #include <vector>
 
 #include "../../include/stab.h"
+#include "host_pool.h"
 #include "launch.h"
 #include "planner.h"
 
@@ -45,7 +47,6 @@ namespace {
 
 constexpr int64_t kSpMinCap = 4096;
 constexpr int64_t kSpMaxCap = 1ll << 30;
-constexpr int kSpMinSegment = 16;   // steps launched ahead even when they might stop
 
 struct SpBuf {
     void *p = nullptr;
@@ -54,23 +55,22 @@ struct SpBuf {
 
 enum { SP_CLIFF = 0, SP_ROT = 1 };
 
+struct SpGate {               // one Clifford gate, already inverted for
+    uint8_t op, q0, q1, pad;  // backward plans (S <-> S^dagger)
+};
+
 struct SpStep {
     int kind;
-    int q, axis, param;       // rotation
-    int first, count;         // Clifford run: gates [first, first + count) of the run array
-    int tab;                  // Clifford run applied through its tableau (index), or -1
+    int first, count;         // Clifford run: gates [first, first + count)
     int64_t gate_lo, gate_hi; // circuit gates [gate_lo, gate_hi) the step covers
 };
 
 struct SpPlan {
     std::vector<SpStep> steps;
     std::vector<SpGate> gates;
-    std::vector<int32_t> tab_first, tab_count;   // runs that get a tableau
+    std::vector<SpRot> rots;
+    std::vector<int64_t> rot_step;   // the rotations' steps
 };
-
-// A run of at least this many gates is applied through its tableau (about
-// 2n phase products per term) instead of gate by gate.
-int tableau_min_gates(int n) { return 2 * n + 8; }
 
 // The outcome of one propagation.
 struct SpRun {
@@ -80,9 +80,108 @@ struct SpRun {
     bool stopped = false;     // threshold reached, or capacity exhausted
 };
 
-void build_sp_plan(const std::vector<stab_gate> &gates, bool backward, SpPlan *P) {
+// The strings U^dagger X_q U and U^dagger Z_q U, kept while gates are appended
+// to U: a gate g maps its wires' letters to products of at most two (g^dagger
+// sigma g), so it rewrites at most two rows.  What U does to a string follows
+// from the rows alone: bit x_q of the image of P is whether P anticommutes with
+// U^dagger Z_q U, bit z_q whether it does with U^dagger X_q U.
+struct SpPull {
+    struct Row {
+        uint64_t key;
+        uint32_t e;           // i^e times the Hermitian string `key`
+    };
+    int n;
+    uint64_t zm;
+    Row x[32], z[32];
+
+    explicit SpPull(int n_) : n(n_), zm((1ull << n_) - 1) {
+        for (int q = 0; q < n; ++q) {
+            x[q] = Row{1ull << (n + q), 0};
+            z[q] = Row{1ull << q, 0};
+        }
+    }
+    uint64_t flip(uint64_t k) const { return (k >> n) | ((k & zm) << n); }
+    // see sp_mul_phase of k_sparse.cu
+    Row mul(const Row &a, const Row &b) const {
+        const uint32_t ax = (uint32_t)(a.key >> n), az = (uint32_t)(a.key & zm);
+        const uint32_t bx = (uint32_t)(b.key >> n), bz = (uint32_t)(b.key & zm);
+        const uint32_t A = ax & az, B = ax & ~az, C = ~ax & az;
+        const uint32_t plus = (A & bz & ~bx) | (B & bz & bx) | (C & bx & ~bz);
+        const uint32_t minus = (A & bx & ~bz) | (B & bz & ~bx) | (C & bx & bz);
+        const uint32_t c = (uint32_t)__builtin_popcountll(((uint64_t)~minus << 32) | plus);
+        return Row{a.key ^ b.key, (a.e + b.e + c) & 3u};
+    }
+    Row y(int q) const {      // Y = i X Z
+        Row r = mul(x[q], z[q]);
+        r.e = (r.e + 1u) & 3u;
+        return r;
+    }
+    void apply(const SpGate &g) {
+        const int a = g.q0, b = g.q1;
+        switch (g.op) {
+        case STAB_H: std::swap(x[a], z[a]); break;
+        case STAB_S:          // S^dagger X S = -Y
+            x[a] = y(a);
+            x[a].e ^= 2u;
+            break;
+        case STAB_SDG: x[a] = y(a); break;
+        case STAB_X: z[a].e ^= 2u; break;
+        case STAB_Y:
+            x[a].e ^= 2u;
+            z[a].e ^= 2u;
+            break;
+        case STAB_Z: x[a].e ^= 2u; break;
+        case STAB_CX:         // X_c -> X_c X_t, Z_t -> Z_c Z_t
+            x[a] = mul(x[a], x[b]);
+            z[b] = mul(z[a], z[b]);
+            break;
+        case STAB_CZ: {       // X_a -> X_a Z_b, X_b -> Z_a X_b
+            x[a] = mul(x[a], z[b]);
+            x[b] = mul(z[a], x[b]);
+            break;
+        }
+        default: break;
+        }
+    }
+    SpRot rotation(int q, int axis, int param) const {
+        const Row P = axis == 0 ? x[q] : axis == 1 ? y(q) : z[q];
+        // pairs (u, v): R_x: (Y, Z), R_y: (Z, X), R_z: (X, Y); u is the one with
+        // x (Y of Y, Z), with z (Z of Z, X), without z (X of X, Y)
+        SpRot r{};
+        r.P = P.key;
+        r.anti = flip(P.key);
+        r.letter = flip(axis == 0 ? z[q].key : x[q].key);
+        r.param = param;
+        r.flags = (axis == 2 ? 0u : 1u) | P.e;
+        return r;
+    }
+    uint64_t xcol(int q) const { return flip(z[q].key); }
+    // U X_q U^dagger (entry q) and U Z_q U^dagger (entry n + q): the bits as
+    // above; the sign is that of the rows' product over the bits, which gives
+    // the generator back
+    void tableau(SpTab *tab) const {
+        for (int g = 0; g < 2 * n; ++g) {
+            const uint64_t k = g < n ? 1ull << (n + g) : 1ull << (g - n);
+            Row t{0, 0};
+            uint64_t w = 0;
+            for (int q = 0; q < n; ++q) {
+                const bool wx = __builtin_parityll(k & flip(z[q].key));
+                const bool wz = __builtin_parityll(k & flip(x[q].key));
+                if (wx) t = mul(t, x[q]);
+                if (wz) t = mul(t, z[q]);
+                if (wx && wz) t.e = (t.e + 1u) & 3u;
+                w |= ((uint64_t)wx << (n + q)) | ((uint64_t)wz << q);
+            }
+            tab[g] = SpTab{w, t.e >> 1, 0};
+        }
+    }
+};
+
+void build_sp_plan(const std::vector<stab_gate> &gates, bool backward, SpPlan *P, SpPull *U) {
     P->steps.clear();
     P->gates.clear();
+    P->rots.clear();
+    P->rot_step.clear();
     const int64_t m = (int64_t)gates.size();
     bool in_run = false;
     for (int64_t k = 0; k < m; ++k) {
@@ -91,11 +190,10 @@ void build_sp_plan(const std::vector<stab_gate> &gates, bool backward, SpPlan *P
         if (g.op >= STAB_RX) {
             SpStep s{};
             s.kind = SP_ROT;
-            s.q = g.q0;
-            s.axis = g.op - STAB_RX;
-            s.param = g.param;
             s.gate_lo = i;
             s.gate_hi = i + 1;
+            P->rots.push_back(U->rotation(g.q0, g.op - STAB_RX, g.param));
+            P->rot_step.push_back((int64_t)P->steps.size());
             P->steps.push_back(s);
             in_run = false;
             continue;
@@ -115,23 +213,31 @@ void build_sp_plan(const std::vector<stab_gate> &gates, bool backward, SpPlan *P
         }
         SpStep &s = P->steps.back();
         P->gates.push_back(SpGate{op, g.q0, g.q1, 0});
+        U->apply(P->gates.back());
         s.count++;
         s.gate_lo = std::min(s.gate_lo, i);
         s.gate_hi = std::max(s.gate_hi, i + 1);
     }
 }
 
-void assign_tableaus(int n, SpPlan *P) {
-    P->tab_first.clear();
-    P->tab_count.clear();
-    for (SpStep &s : P->steps) {
-        s.tab = -1;
-        if (s.kind != SP_CLIFF || s.count < tableau_min_gates(n)) continue;
-        s.tab = (int)P->tab_first.size();
-        P->tab_first.push_back(s.first);
-        P->tab_count.push_back(s.count);
-    }
+// What the device needs of a plan's whole Clifford part: the tableau, then the
+// masks of its x bits.
+struct SpFinal {
+    SpTab tab[64];
+    uint64_t xcol[32];
+};
+
+void fill_final(const SpPull &U, SpFinal *f) {
+    std::memset((void *)f, 0, sizeof *f);
+    U.tableau(f->tab);
+    for (int q = 0; q < U.n; ++q) f->xcol[q] = U.xcol(q);
 }
+
+// One direction of a loaded circuit.
+struct SpDir {
+    SpPlan plan;
+    SpBuf rots, fin, chunks;
+};
 
 }  // namespace
 
@@ -146,16 +252,16 @@ struct stab_sparse {
     std::vector<stab_gate> gates;
     std::vector<double> thetas_h;
     int64_t n_params = 0;
-    SpPlan fwd, bwd;
-    SpBuf thetas, cs, g_fwd, g_bwd, keys[2], vals[2], table, slot_of, partner, blk, counts,
-        flags, partial, scal, dterms, t_fwd, t_bwd, c_fwd, c_bwd, runs;
-    int log_h = 0;
+    SpDir fwd, bwd;
+    SpBuf thetas, cs, keys[2], vals[2], table, partner, tiles, init, run, partial, dterms, fin,
+        chunks;
+    int grid = 0;
     void *pinned = nullptr;
     size_t pinned_bytes = 0;
     std::vector<int64_t> history;
     stab_ctx *dense = nullptr;
     int32_t regrows = 0;
-    bool table_dirty = false;   // a run stopped on overflow with slots still claimed
+    bool table_dirty = false;   // a run that failed left slots claimed
 
     int dalloc(SpBuf &b, size_t bytes) {
         if (b.p && b.bytes >= bytes) return STAB_OK;
@@ -197,43 +303,56 @@ struct stab_sparse {
         return STAB_OK;
     }
 
+    int clear(int64_t c) {
+        SCK(cudaMemsetAsync(table.p, 0xff, (size_t)8 << sp_table_log(c), st));
+        SCK(cudaMemsetAsync(partner.p, 0xff, (size_t)c * 4, st));
+        return STAB_OK;
+    }
+
     // Capacity `c` for the list; the live list (count terms in buffer `from`)
-    // moves to buffer 0.  The table is twice the capacity, all slots free.
+    // moves to buffer 0.  The table's slots are all free, the partners all absent.
     int reserve(int64_t c, int from, int64_t count) {
         if (c <= cap && from == 0) return STAB_OK;
         c = std::max(c, cap);
+        const bool grow = c > cap;
+        cap = 0;   // until all buffers are there: after a failure the next run starts over
         SpBuf nk, nv;
         std::swap(nk, keys[0]);
         std::swap(nv, vals[0]);
-        SRC(dalloc(keys[0], (size_t)c * 8));
-        SRC(dalloc(vals[0], (size_t)c * 8));
-        const SpBuf &ok = from == 0 ? nk : keys[1], &ov = from == 0 ? nv : vals[1];
-        if (count > 0) {
-            SCK(cudaMemcpyAsync(keys[0].p, ok.p, (size_t)count * 8, cudaMemcpyDeviceToDevice, st));
-            SCK(cudaMemcpyAsync(vals[0].p, ov.p, (size_t)count * 8, cudaMemcpyDeviceToDevice, st));
+        int r = dalloc(keys[0], (size_t)c * 8);
+        if (r == STAB_OK) r = dalloc(vals[0], (size_t)c * 8);
+        if (r == STAB_OK && count > 0) {
+            const SpBuf &ok = from == 0 ? nk : keys[1], &ov = from == 0 ? nv : vals[1];
+            cudaError_t e = cudaMemcpyAsync(keys[0].p, ok.p, (size_t)count * 8,
+                                            cudaMemcpyDeviceToDevice, st);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(vals[0].p, ov.p, (size_t)count * 8, cudaMemcpyDeviceToDevice,
+                                    st);
+            if (e != cudaSuccess) {
+                record_cuda_error(e);
+                r = STAB_E_CUDA;
+            }
         }
         dfree(nk);
         dfree(nv);
-        if (c > cap) {
+        SRC(r);
+        if (grow) {
             SRC(dalloc(keys[1], (size_t)c * 8));
             SRC(dalloc(vals[1], (size_t)c * 8));
-            SRC(dalloc(slot_of, (size_t)c * 4));
             SRC(dalloc(partner, (size_t)c * 4));
-            int lh = 1;
-            while ((1ll << lh) < 2 * c) ++lh;
-            SRC(dalloc(table, ((size_t)1 << lh) * sizeof(SpSlot)));
-            SCK(cudaMemsetAsync(table.p, 0xff, ((size_t)1 << lh) * sizeof(SpSlot), st));
-            log_h = lh;
-            cap = c;
+            SRC(dalloc(tiles, (size_t)sp_tiles(c, grid) * 8));
+            SRC(dalloc(table, (size_t)8 << sp_table_log(c)));
+            SRC(clear(c));
         }
+        cap = c;
         return STAB_OK;
     }
 
     ~stab_sparse() {
         if (st) cudaStreamSynchronize(st);
-        for (SpBuf *b : {&thetas, &cs, &g_fwd, &g_bwd, &keys[0], &keys[1], &vals[0], &vals[1], &table,
-                         &slot_of, &partner, &blk, &counts, &flags, &partial, &scal,
-                         &dterms, &t_fwd, &t_bwd, &c_fwd, &c_bwd, &runs})
+        for (SpBuf *b : {&thetas, &cs, &keys[0], &keys[1], &vals[0], &vals[1], &table, &partner,
+                         &tiles, &init, &run, &partial, &dterms, &fin, &chunks, &fwd.rots,
+                         &fwd.fin, &fwd.chunks, &bwd.rots, &bwd.fin, &bwd.chunks})
             dfree(*b);
         if (pinned) cudaFreeHost(pinned);
         if (dense) stab_destroy(dense);
@@ -243,141 +362,131 @@ struct stab_sparse {
 
 namespace {
 
-// Uploads the initial list to buffer 0 and runs the plan.
-int sp_run(stab_sparse *s, const SpPlan &P, const SpBuf &run_gates, const SpBuf &chunks,
-           bool backward,
-           const std::vector<uint64_t> &k0, const std::vector<double> &v0, SpRun *R,
-           int64_t *order_max) {
-    const int64_t S = (int64_t)P.steps.size();
+// Runs the plan on a list.  With `sum`, the x-free sum of the last list's images
+// is queued behind it and returned there (of no use when the run stopped).
+int sp_run(stab_sparse *s, const SpDir &D, bool backward, const std::vector<uint64_t> &k0,
+           const std::vector<double> &v0, SpRun *R, int64_t *order_max, double *sum) {
+    const int64_t S = (int64_t)D.plan.steps.size(), rots = (int64_t)D.plan.rots.size();
     const int64_t n0 = (int64_t)k0.size();
     s->history.clear();
     s->regrows = 0;
     SRC(s->reserve(std::min(s->max_terms, std::max(kSpMinCap, 4 * n0)), 0, 0));
     if (n0 > s->cap) return STAB_E_RANGE;
     if (s->table_dirty) {
-        SCK(cudaMemsetAsync(s->table.p, 0xff, ((size_t)1 << s->log_h) * sizeof(SpSlot), s->st));
+        SRC(s->clear(s->cap));
         s->table_dirty = false;
     }
-    SRC(s->dalloc(s->counts, (size_t)(S + 1) * 8));
-    SRC(s->stage(std::max<size_t>((size_t)(S + 1) * 8 + 64, (size_t)n0 * 16 + 64)));
-    // initial list and order through pinned staging
+    // state and orders come back in one copy; initial list and first order go in one
+    const size_t back = sizeof(SpState) + (size_t)(rots + 1) * 8, there = (size_t)n0 * 16;
+    const size_t back_pad = (back + 63) & ~(size_t)63;
+    SRC(s->dalloc(s->run, back));
+    SRC(s->dalloc(s->init, std::max<size_t>(there, 16)));
+    SRC(s->stage(back_pad + there + sizeof(SpState) + 8));
     char *h = (char *)s->pinned;
-    if (n0) {
-        std::memcpy(h, k0.data(), (size_t)n0 * 8);
-        std::memcpy(h + (size_t)n0 * 8, v0.data(), (size_t)n0 * 8);
-        SCK(cudaMemcpyAsync(s->keys[0].p, h, (size_t)n0 * 8, cudaMemcpyHostToDevice, s->st));
-        SCK(cudaMemcpyAsync(s->vals[0].p, h + (size_t)n0 * 8, (size_t)n0 * 8,
-                            cudaMemcpyHostToDevice, s->st));
-    }
-    SCK(cudaMemcpyAsync(s->counts.p, &n0, 8, cudaMemcpyHostToDevice, s->st));
-    SCK(cudaMemsetAsync(s->flags.p, 0, 16, s->st));
-    SCK(cudaStreamSynchronize(s->st));   // the staging buffer is reused below
+    uint64_t *h_init = (uint64_t *)(h + back_pad);
+    char *h_state = h + back_pad + there;
+    std::copy(k0.begin(), k0.end(), h_init);
+    std::memcpy(h_init + n0, v0.data(), (size_t)n0 * 8);
+    SpState first{};
+    first.count = n0;
+    std::memcpy(h_state, &first, sizeof first);
+    std::memcpy(h_state + sizeof first, &n0, 8);
+    if (n0) SCK(cudaMemcpyAsync(s->init.p, h_init, there, cudaMemcpyHostToDevice, s->st));
+    SCK(cudaMemcpyAsync(s->run.p, h_state, sizeof first + 8, cudaMemcpyHostToDevice, s->st));
 
-    std::vector<int> buf_before((size_t)S + 1, 0);
-    *order_max = n0;
-    int64_t p = 0, known = n0;
-    int32_t *flags = (int32_t *)s->flags.p;
-    int64_t *counts = (int64_t *)s->counts.p;
-    const SpGate *gates = (const SpGate *)run_gates.p;
-    while (p < S) {
-        const int64_t lim = s->threshold > 0 ? std::min(s->cap, s->threshold) : s->cap;
-        // launch steps [p, e): all that cannot pass lim, at least kSpMinSegment
-        int64_t e = p, bound = known;
-        while (e < S) {
-            const SpStep &st = P.steps[e];
-            if (st.kind == SP_ROT && 2 * bound > lim && e >= p + kSpMinSegment) break;
-            const int cur = buf_before[e];
-            if (st.kind == SP_CLIFF && st.tab >= 0) {
-                SCK(launch_sp_cliff_tab((uint64_t *)s->keys[cur].p, (double *)s->vals[cur].p,
-                                        counts, flags, (int)e, s->n,
-                                        (const SpChunk *)chunks.p + (size_t)st.tab * kSpChunkEntries,
-                                        bound, s->st));
-                buf_before[e + 1] = cur;
-            } else if (st.kind == SP_CLIFF) {
-                SCK(launch_sp_cliff((uint64_t *)s->keys[cur].p, (double *)s->vals[cur].p,
-                                    counts, flags, (int)e, s->n, gates + st.first, st.count,
-                                    bound, s->st));
-                buf_before[e + 1] = cur;
-            } else {
-                SpRotArgs a{};
-                a.keys = (const uint64_t *)s->keys[cur].p;
-                a.vals = (const double *)s->vals[cur].p;
-                a.keys_out = (uint64_t *)s->keys[1 - cur].p;
-                a.vals_out = (double *)s->vals[1 - cur].p;
-                a.counts = counts;
-                a.flags = flags;
-                a.step = (int32_t)e;
-                a.n = s->n;
-                a.q = st.q;
-                a.axis = st.axis;
-                a.cs = (const double *)s->cs.p;
-                a.param = st.param;
-                a.inverse = backward ? 1 : 0;
-                a.table = (SpSlot *)s->table.p;
-                a.log_h = s->log_h;
-                a.slot_of = (int32_t *)s->slot_of.p;
-                a.partner = (int32_t *)s->partner.p;
-                a.blk = (int64_t *)s->blk.p;
-                a.err = flags + 2;
-                a.cap = s->cap;
-                a.threshold = s->threshold;
-                a.bound = bound;
-                SCK(launch_sp_rotation(a, s->st));
-                buf_before[e + 1] = 1 - cur;
-                bound = std::min(s->cap, 2 * bound);
-            }
-            ++e;
-        }
-        // read the orders of steps [p, e] and the flags
-        char *hp = (char *)s->pinned;
-        SCK(cudaMemcpyAsync(hp, counts + p, (size_t)(e - p + 1) * 8, cudaMemcpyDeviceToHost,
+    SpRunArgs a{};
+    a.st = (SpState *)s->run.p;
+    a.counts = (int64_t *)((char *)s->run.p + sizeof(SpState));
+    a.rots = (const SpRot *)D.rots.p;
+    a.cs = (const double *)s->cs.p;
+    a.n_rot = (int32_t)rots;
+    a.n = s->n;
+    a.inverse = backward ? 1 : 0;
+    a.grid = s->grid;
+    a.threshold = s->threshold;
+    a.init = (const uint64_t *)s->init.p;
+    // a list that can outgrow one CTA's memory needs the grid behind it
+    const int64_t small = std::min<int64_t>(s->cap, kSpSmallCap);
+    bool grid = n0 > small;
+    if (grid) {
+        SCK(cudaMemcpyAsync(s->keys[0].p, s->init.p, (size_t)n0 * 8, cudaMemcpyDeviceToDevice,
                             s->st));
-        SCK(cudaMemcpyAsync(hp + (size_t)(e - p + 1) * 8, flags, 16, cudaMemcpyDeviceToHost,
-                            s->st));
-        SCK(cudaStreamSynchronize(s->st));
-        const int64_t *hc = (const int64_t *)hp;
-        const int32_t *hf = (const int32_t *)(hp + (size_t)(e - p + 1) * 8);
-        if (hf[2] != 0) return STAB_E_NOMEM;   // a table probe ran out (never expected)
-        const int64_t done = hf[0] != 0 ? hf[1] + (hf[0] == 2 ? 1 : 0) : e;
-        for (int64_t j = p + 1; j <= done; ++j) {
-            s->history.push_back(hc[j - p]);
-            *order_max = std::max(*order_max, hc[j - p]);
-        }
-        if (hf[0] == 1) {
-            // step f would overflow: the list before it is intact
-            const int64_t f = hf[1];
-            const int64_t cnt = hc[f - p];
-            if (s->cap >= s->max_terms) {
-                s->table_dirty = true;
-                R->buf = buf_before[f];
-                R->step = f;
-                R->count = cnt;
-                R->stopped = true;
-                return STAB_OK;
-            }
-            SRC(s->reserve(std::min(s->max_terms, s->cap * 8), buf_before[f], cnt));
-            s->regrows++;
-            SCK(cudaMemsetAsync(s->flags.p, 0, 16, s->st));
-            buf_before[f] = 0;
-            p = f;
-            known = cnt;
-            continue;
-        }
-        if (hf[0] == 2) {
-            const int64_t f = hf[1];
-            R->buf = buf_before[f + 1];
-            R->step = f + 1;
-            R->count = hc[f + 1 - p];
-            R->stopped = f + 1 < S;
-            return STAB_OK;
-        }
-        known = hc[e - p];
-        p = e;
+        SCK(cudaMemcpyAsync(s->vals[0].p, (char *)s->init.p + (size_t)n0 * 8, (size_t)n0 * 8,
+                            cudaMemcpyDeviceToDevice, s->st));
     }
-    R->buf = buf_before[S];
+    int64_t bound = n0;
+    for (int64_t r = 0; r < rots && bound <= small; ++r) bound *= 2;
+    const bool one_cta = !grid;
+    grid = rots > 0 && (grid || bound > small);
+    SpState at{};
+    for (bool again = false;; again = true) {
+        a.cap = s->cap;
+        for (int b = 0; b < 2; ++b) {
+            a.keys[b] = (uint64_t *)s->keys[b].p;
+            a.vals[b] = (double *)s->vals[b].p;
+        }
+        a.table = (uint64_t *)s->table.p;
+        a.partner = (int32_t *)s->partner.p;
+        a.tiles = (uint64_t *)s->tiles.p;
+        if (one_cta && !again) SCK(launch_sp_small(a, s->st));
+        if (grid) SCK(launch_sp_run(a, s->st));
+        if (sum)
+            SCK(launch_sp_xfree(a, ((const SpFinal *)D.fin.p)->xcol, (const SpChunk *)D.chunks.p,
+                                (double *)s->partial.p, s->st));
+        SCK(cudaMemcpyAsync(h, s->run.p, back, cudaMemcpyDeviceToHost, s->st));
+        SCK(cudaStreamSynchronize(s->st));
+        std::memcpy(&at, h, sizeof at);
+        if (at.err != 0) {   // a table probe or a wait ran out (never expected)
+            s->table_dirty = true;
+            return at.err == 1 ? STAB_E_NOMEM : STAB_E_CUDA;
+        }
+        if (at.stop != SP_OVERFLOW || s->cap >= s->max_terms) break;
+        SRC(s->reserve(std::min(s->max_terms, s->cap * 8), at.buf, at.count));
+        s->regrows++;
+        at.buf = 0;
+        at.stop = SP_RUNNING;
+        at.arrived = 0;
+        std::memcpy(h_state, &at, sizeof at);
+        SCK(cudaMemcpyAsync(s->run.p, h_state, sizeof at, cudaMemcpyHostToDevice, s->st));
+    }
+    R->buf = at.buf;
+    R->count = at.count;
+    // stopped behind rotation rot - 1 (threshold) or before rotation rot (no room)
     R->step = S;
-    R->count = known;
-    R->stopped = false;
+    if (at.stop == SP_THRESHOLD) R->step = D.plan.rot_step[at.rot - 1] + 1;
+    if (at.stop == SP_OVERFLOW) R->step = D.plan.rot_step[at.rot];
+    R->stopped = at.stop == SP_OVERFLOW || R->step < S;
+    const int64_t *counts = (const int64_t *)(h + sizeof(SpState));
+    *order_max = n0;
+    int64_t order = n0;
+    for (int64_t j = 0, r = 0; j < R->step; ++j) {
+        if (D.plan.steps[(size_t)j].kind == SP_ROT) order = counts[++r];
+        s->history.push_back(order);
+        *order_max = std::max(*order_max, order);
+    }
+    if (sum) *sum = at.value;
+    return STAB_OK;
+}
+
+// The chunk table of the Clifford gates the list before step R.step has behind
+// it: the loaded one, or one of the first steps alone.
+int sp_chunks(stab_sparse *s, const SpDir &D, const SpRun &R, const SpChunk **out) {
+    *out = (const SpChunk *)D.chunks.p;
+    if (R.step == (int64_t)D.plan.steps.size()) return STAB_OK;
+    SpPull U(s->n);
+    for (int64_t j = 0; j < R.step; ++j) {
+        const SpStep &st = D.plan.steps[(size_t)j];
+        for (int g = 0; st.kind == SP_CLIFF && g < st.count; ++g)
+            U.apply(D.plan.gates[(size_t)(st.first + g)]);
+    }
+    SRC(s->dalloc(s->fin, sizeof(SpFinal)));
+    SRC(s->dalloc(s->chunks, kSpChunkEntries * sizeof(SpChunk)));
+    SRC(s->stage(sizeof(SpFinal)));
+    fill_final(U, (SpFinal *)s->pinned);
+    SCK(cudaMemcpyAsync(s->fin.p, s->pinned, sizeof(SpFinal), cudaMemcpyHostToDevice, s->st));
+    SCK(launch_sp_chunks(((const SpFinal *)s->fin.p)->tab, s->n, (SpChunk *)s->chunks.p, s->st));
+    SCK(cudaStreamSynchronize(s->st));   // the staging buffer may be reused
+    *out = (const SpChunk *)s->chunks.p;
     return STAB_OK;
 }
 
@@ -455,10 +564,14 @@ int stab_sparse_create(int n, int64_t max_terms, const stab_opts *opts, stab_spa
     o.stream = (void *)s->st;
     o.stream_given = 1;
     s->opts = o;
-    int r = s->dalloc(s->flags, 256);
-    if (r == STAB_OK) r = s->dalloc(s->blk, (size_t)kSpMaxBlocks * 8);
-    if (r == STAB_OK) r = s->dalloc(s->partial, (size_t)kSpMaxBlocks * 8);
-    if (r == STAB_OK) r = s->dalloc(s->scal, 64);
+    int r = s->dalloc(s->partial, (size_t)kSpMaxBlocks * 8);
+    if (r == STAB_OK) {
+        e = sp_run_grid(dev, &s->grid);
+        if (e != cudaSuccess) {
+            record_cuda_error(e);
+            r = STAB_E_CUDA;
+        }
+    }
     if (r != STAB_OK) {
         delete s;
         return r;
@@ -484,44 +597,40 @@ int stab_sparse_load_circuit(stab_sparse *s, const stab_gate *gates, int64_t m,
     s->gates.assign(gates, gates + m);
     s->thetas_h.assign(thetas, thetas + n_params);
     s->n_params = n_params;
-    build_sp_plan(s->gates, false, &s->fwd);
-    build_sp_plan(s->gates, true, &s->bwd);
-    assign_tableaus(s->n, &s->fwd);
-    assign_tableaus(s->n, &s->bwd);
-    const size_t bt = (size_t)std::max<int64_t>(n_params, 1) * 8;
-    const size_t bf = std::max<size_t>(s->fwd.gates.size(), 1) * sizeof(SpGate);
-    const size_t bb = std::max<size_t>(s->bwd.gates.size(), 1) * sizeof(SpGate);
-    const size_t nrf = s->fwd.tab_first.size(), nrb = s->bwd.tab_first.size();
-    const size_t br = std::max<size_t>(2 * (nrf + nrb), 1) * 4;
-    SRC(s->dalloc(s->thetas, bt));
-    SRC(s->dalloc(s->cs, 2 * bt));
-    SRC(s->dalloc(s->g_fwd, bf));
-    SRC(s->dalloc(s->g_bwd, bb));
-    SRC(s->dalloc(s->runs, br));
-    SRC(s->dalloc(s->t_fwd, std::max<size_t>(nrf, 1) * 64 * sizeof(SpTab)));
-    SRC(s->dalloc(s->t_bwd, std::max<size_t>(nrb, 1) * 64 * sizeof(SpTab)));
-    SRC(s->dalloc(s->c_fwd, std::max<size_t>(nrf, 1) * kSpChunkEntries * sizeof(SpChunk)));
-    SRC(s->dalloc(s->c_bwd, std::max<size_t>(nrb, 1) * kSpChunkEntries * sizeof(SpChunk)));
-    SRC(s->stage(bt + bf + bb + br));
+    const size_t bt = (size_t)n_params * 8;
+    SRC(s->dalloc(s->thetas, std::max<size_t>(bt, 8)));
+    SRC(s->dalloc(s->cs, std::max<size_t>(2 * bt, 8)));
+    SpDir *dirs[2] = {&s->fwd, &s->bwd};
+    size_t need = bt;
+    std::vector<SpFinal> fin(2);
+    for (int k = 0; k < 2; ++k) {
+        SpDir &D = *dirs[k];
+        SpPull U(s->n);
+        build_sp_plan(s->gates, k == 1, &D.plan, &U);
+        fill_final(U, &fin[k]);
+        const size_t br = D.plan.rots.size() * sizeof(SpRot);
+        SRC(s->dalloc(D.rots, std::max<size_t>(br, 8)));
+        SRC(s->dalloc(D.fin, sizeof(SpFinal)));
+        SRC(s->dalloc(D.chunks, kSpChunkEntries * sizeof(SpChunk)));
+        need += br + sizeof(SpFinal);
+    }
+    SRC(s->stage(need));
     char *h = (char *)s->pinned;
-    std::memcpy(h, s->thetas_h.data(), (size_t)n_params * 8);
-    std::memcpy(h + bt, s->fwd.gates.data(), s->fwd.gates.size() * sizeof(SpGate));
-    std::memcpy(h + bt + bf, s->bwd.gates.data(), s->bwd.gates.size() * sizeof(SpGate));
-    int32_t *hr = (int32_t *)(h + bt + bf + bb);
-    std::copy(s->fwd.tab_first.begin(), s->fwd.tab_first.end(), hr);
-    std::copy(s->fwd.tab_count.begin(), s->fwd.tab_count.end(), hr + nrf);
-    std::copy(s->bwd.tab_first.begin(), s->bwd.tab_first.end(), hr + 2 * nrf);
-    std::copy(s->bwd.tab_count.begin(), s->bwd.tab_count.end(), hr + 2 * nrf + nrb);
-    SCK(cudaMemcpyAsync(s->thetas.p, h, bt, cudaMemcpyHostToDevice, s->st));
+    auto put = [&](const SpBuf &d, const void *src, size_t bytes) {
+        if (bytes == 0) return cudaSuccess;
+        std::memcpy(h, src, bytes);
+        const cudaError_t e = cudaMemcpyAsync(d.p, h, bytes, cudaMemcpyHostToDevice, s->st);
+        h += bytes;
+        return e;
+    };
+    SCK(put(s->thetas, s->thetas_h.data(), bt));
     SCK(launch_sp_cos_sin((const double *)s->thetas.p, n_params, (double *)s->cs.p, s->st));
-    SCK(cudaMemcpyAsync(s->g_fwd.p, h + bt, bf, cudaMemcpyHostToDevice, s->st));
-    SCK(cudaMemcpyAsync(s->g_bwd.p, h + bt + bf, bb, cudaMemcpyHostToDevice, s->st));
-    SCK(cudaMemcpyAsync(s->runs.p, hr, br, cudaMemcpyHostToDevice, s->st));
-    const int32_t *dr = (const int32_t *)s->runs.p;
-    SCK(launch_sp_tableau((const SpGate *)s->g_fwd.p, dr, dr + nrf, (int)nrf, s->n,
-                          (SpTab *)s->t_fwd.p, (SpChunk *)s->c_fwd.p, s->st));
-    SCK(launch_sp_tableau((const SpGate *)s->g_bwd.p, dr + 2 * nrf, dr + 2 * nrf + nrb, (int)nrb,
-                          s->n, (SpTab *)s->t_bwd.p, (SpChunk *)s->c_bwd.p, s->st));
+    for (int k = 0; k < 2; ++k) {
+        SpDir &D = *dirs[k];
+        SCK(put(D.rots, D.plan.rots.data(), D.plan.rots.size() * sizeof(SpRot)));
+        SCK(put(D.fin, &fin[k], sizeof(SpFinal)));
+        SCK(launch_sp_chunks(((const SpFinal *)D.fin.p)->tab, s->n, (SpChunk *)D.chunks.p, s->st));
+    }
     SCK(cudaStreamSynchronize(s->st));
     s->loaded = true;
     return STAB_OK;
@@ -550,27 +659,24 @@ int stab_sparse_expect(stab_sparse *s, const stab_term *O, int64_t n_terms, doub
         fill_info(s, R, 0, -1, info);
         return STAB_OK;
     }
-    SRC(sp_run(s, s->bwd, s->g_bwd, s->c_bwd, true, k0, v0, &R, &order_max));
+    double value = 0.0;
+    SRC(sp_run(s, s->bwd, true, k0, v0, &R, &order_max, &value));
     int64_t dense_gates = -1;
     if (R.stopped) {
         // the rest of the circuit (backward: gates [0, g)) on the dense vector
         if (s->n > STAB_MAX_QUBITS) return STAB_E_RANGE;
-        const int64_t g = s->bwd.steps[R.step].gate_hi;
+        const int64_t g = s->bwd.plan.steps[R.step].gate_hi;
         if (!s->dense) SRC(stab_create(s->n, &s->opts, &s->dense));
         SRC(stab_load_circuit(s->dense, s->gates.data(), g, s->thetas_h.data(), s->n_params));
         SRC(s->dalloc(s->dterms, (size_t)std::max<int64_t>(R.count, 1) * sizeof(DevTerm)));
-        SCK(launch_sp_to_terms((const uint64_t *)s->keys[R.buf].p,
-                               (const double *)s->vals[R.buf].p, (const int64_t *)s->counts.p,
-                               (int)R.step, (DevTerm *)s->dterms.p, R.count, s->st));
+        const SpChunk *chunks;
+        SRC(sp_chunks(s, s->bwd, R, &chunks));
+        SCK(launch_sp_images((const uint64_t *)s->keys[R.buf].p, (const double *)s->vals[R.buf].p,
+                             R.count, s->n, chunks, (DevTerm *)s->dterms.p, nullptr, s->st));
         SRC(expect_device_terms(s->dense, (const DevTerm *)s->dterms.p, R.count, out));
         dense_gates = g;
     } else {
-        SCK(launch_sp_xfree((const uint64_t *)s->keys[R.buf].p, (const double *)s->vals[R.buf].p,
-                            (const int64_t *)s->counts.p, (int)R.step, s->n,
-                            (double *)s->partial.p, (double *)s->scal.p, s->st));
-        SCK(cudaMemcpyAsync(s->pinned, s->scal.p, 8, cudaMemcpyDeviceToHost, s->st));
-        SCK(cudaStreamSynchronize(s->st));
-        std::memcpy(out, s->pinned, 8);
+        *out = value;
     }
     fill_info(s, R, order_max, dense_gates, info);
     return STAB_OK;
@@ -588,7 +694,7 @@ int stab_sparse_generator(stab_sparse *s, int k, int64_t max_out, stab_term *out
     s->threshold = 0;   // generators stay on the list
     SpRun R;
     int64_t order_max = 0;
-    const int r = sp_run(s, s->fwd, s->g_fwd, s->c_fwd, false, k0, v0, &R, &order_max);
+    const int r = sp_run(s, s->fwd, false, k0, v0, &R, &order_max, nullptr);
     s->threshold = keep;
     SRC(r);
     if (R.stopped) return STAB_E_RANGE;
@@ -596,20 +702,24 @@ int stab_sparse_generator(stab_sparse *s, int k, int64_t max_out, stab_term *out
     fill_info(s, R, order_max, -1, info);
     if (R.count > max_out) return STAB_E_RANGE;
     if (R.count == 0) return STAB_OK;
-    SRC(s->stage((size_t)R.count * 16));
-    char *h = (char *)s->pinned;
-    SCK(cudaMemcpyAsync(h, s->keys[R.buf].p, (size_t)R.count * 8, cudaMemcpyDeviceToHost, s->st));
-    SCK(cudaMemcpyAsync(h + (size_t)R.count * 8, s->vals[R.buf].p, (size_t)R.count * 8,
-                        cudaMemcpyDeviceToHost, s->st));
+    const SpChunk *chunks;
+    SRC(sp_chunks(s, s->fwd, R, &chunks));
+    // the records are made there: 96,000 of them here took as long as the last rotations
+    const size_t bytes = (size_t)R.count * sizeof(stab_term);
+    SRC(s->dalloc(s->dterms, bytes));
+    SRC(s->stage(bytes));
+    SCK(launch_sp_images((const uint64_t *)s->keys[R.buf].p, (const double *)s->vals[R.buf].p,
+                         R.count, s->n, chunks, nullptr, (stab_term *)s->dterms.p, s->st));
+    SCK(cudaMemcpyAsync(s->pinned, s->dterms.p, bytes, cudaMemcpyDeviceToHost, s->st));
     SCK(cudaStreamSynchronize(s->st));
-    const uint64_t *hk = (const uint64_t *)h;
-    const double *hv = (const double *)(h + (size_t)R.count * 8);
-    const uint64_t zmask = (s->n >= 64) ? ~0ull : ((1ull << s->n) - 1);
-    for (int64_t i = 0; i < R.count; ++i) {
-        out[i].coeff = hv[i];
-        out[i].x = hk[i] >> s->n;
-        out[i].z = hk[i] & zmask;
-    }
+    // 2.3 MB (96,000 terms): 90 us on one core
+    constexpr size_t kPart = 256 << 10;
+    std::vector<std::function<void()>> jobs;
+    for (size_t at = 0; at < bytes; at += kPart)
+        jobs.push_back([=] {
+            std::memcpy((char *)out + at, (const char *)s->pinned + at, std::min(kPart, bytes - at));
+        });
+    HostPool::run(jobs);
     return STAB_OK;
 }
 

@@ -495,6 +495,7 @@ class Sparse:
                  torch_memory: bool = True):
         self.n = n
         self._keep = []
+        self._terms = np.empty(0, dtype=TERM_DTYPE)
         o = StabOpts()
         _lib.load().stab_default_opts(ctypes.byref(o))
         o.device = device
@@ -528,7 +529,10 @@ class Sparse:
         return out.value, _info_dict(info)
 
     def generator(self, k: int, max_out: int = 1 << 22):
-        out = np.zeros(max(1, max_out), dtype=TERM_DTYPE)
+        # kept between calls: mapping 100 MB afresh cost more than a short run
+        if len(self._terms) < max(1, max_out):
+            self._terms = np.empty(max(1, max_out), dtype=TERM_DTYPE)
+        out = self._terms
         cnt = ctypes.c_int64()
         info = StabSparseInfo()
         check(_lib.load().stab_sparse_generator(self.h, k, max_out, out.ctypes.data,
