@@ -196,7 +196,8 @@ int stab_grad_async(stab_ctx *ctx, double *expect_dev, double *grads_dev);
 /* How the last gradient's plan is cut: *parts receives K >= 2 when its units
  * are those of the generators' plan and both are cut into the same K parts (n
  * <= 4), 1 when they are not (a wire run that is the identity and holds no
- * rotation is a unit of the one but not of the other; plans of n >= 5), 0 before any gradient since the circuit was loaded.
+ * rotation is a unit of the one but not of the other; plans of n >= 5; plans
+ * of less than 64 passes), 0 before any gradient since the circuit was loaded.
  * Errors: STAB_E_INVAL (ctx or parts NULL). */
 int stab_grad_parts(stab_ctx *ctx, int32_t *parts);
 

@@ -54,6 +54,13 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Resident plans with at least this many passes also get split streams.
 constexpr int kSplitMinPasses = 64;
+// n = 2, 3: the unitaries' tree is two levels of 3 us and the read-outs are one
+// small launch, against a compose, two encodes and 0.1 us a pass and vector, so
+// almost any plan is better off there (angles in, generators, <O>: n = 2, 20 gates 32
+// -> 28 us, 100 gates 37 -> 31; n = 3 32 -> 30, 38 -> 33; gradients 60 -> 44 and 108
+// -> 57).  At n = 4 the levels take 6 us and the read-out 256 rows: 34 -> 37, 40 ->
+// 42 and even at 200 gates, about 64 passes; at n = 1 a plan is one run (37 -> 41).
+constexpr int kUniMinPasses = 8;
 // Resident adjoint: per-thread dot shares while the CTA has at most this many
 // threads (n <= 5) and the shares take at most this many bytes.
 constexpr int kPartialThreads = 256;
@@ -105,7 +112,7 @@ struct DevPlan {
     // split < 0: none
     DevStreamBuf h1, h2, h2b, h1b;
     int split = -1;
-    // n <= 4, long plans (uni): K >= 2 parts, part k = passes [cuts[k],
+    // n <= 4 (uni): K >= 2 parts, part k = passes [cuts[k],
     // cuts[k+1]), each cut into segments whose unitaries are composed at once
     // (see k_unitary.cu); no streams.
     bool uni = false;
@@ -748,7 +755,7 @@ void make_tile_group(int n, int n_vec, const std::vector<DevPass> &passes,
 // ---------------------------------------------------------------- split sweeps of small registers
 //
 // A resident vector walks the circuit's passes one after another on one SM.
-// n <= 4, plans of at least kSplitMinPasses passes: the plan is cut into parts
+// n <= 4 (from kUniMinPasses or kSplitMinPasses passes): the plan is cut into parts
 // whose maps are carried by their unitaries, composed from segments that run
 // at once (k_unitary.cu); the generators, rho and <O> are read off the parts'
 // unitaries, the gradient off states carried through the segments.
@@ -800,7 +807,7 @@ void make_uni(DevPlan &P, const std::vector<int> &cuts, int sms) {
     P.streams = P.uni = true;
     P.sf = P.sb = P.h1 = P.h2 = P.h2b = P.h1b = DevStreamBuf();
     P.cuts = cuts;
-    P.split = cuts[1];
+    P.split = (int)P.host.passes.size() >= kSplitMinPasses ? cuts[1] : -1;
     const HostPlan &H = P.host;
     const int np = (int)H.passes.size(), K = (int)cuts.size() - 1;
     std::vector<int> wires((size_t)np + 1, 0);   // wire passes before pass i
@@ -2165,10 +2172,10 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     reset_graphs(c);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
-        // AUTO, long plans: at n <= 4 the parts' unitaries; at n = 5, 6 the two
-        // halves of <O>
+        // AUTO: at n <= 4 the parts' unitaries, at n = 5, 6 the two halves of <O>
         const bool split = c->kernel == STAB_KERNEL_AUTO && c->fuse;
-        if (split && c->n <= kUniMaxQubits && (int)c->fwd.host.passes.size() >= kSplitMinPasses) {
+        const int least = c->n == 2 || c->n == 3 ? kUniMinPasses : kSplitMinPasses;
+        if (split && c->n <= kUniMaxQubits && (int)c->fwd.host.passes.size() >= least) {
             make_uni(c->fwd, part_cuts(c), c->sms);
         } else {
             make_streams(c->fwd, split ? c->choice.gen_cut : 0.0);
@@ -2848,8 +2855,9 @@ int64_t stab_launch_count(stab_ctx *c) { return c ? c->launches : 0; }
 int stab_grad_parts(stab_ctx *c, int32_t *parts) {
     if (!c || !parts) return STAB_E_INVAL;
     *parts = !c->grad_ran                              ? 0
-             : c->grad_uni && !c->fwd.uni_identity ? (int32_t)c->fwd.uparts.size()
-                                                   : 1;
+             : c->grad_uni && !c->fwd.uni_identity && c->fwd.split >= 0
+                 ? (int32_t)c->fwd.uparts.size()
+                 : 1;
     return STAB_OK;
 }
 

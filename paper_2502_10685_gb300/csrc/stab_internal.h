@@ -146,7 +146,7 @@ constexpr uint16_t kPullRepeat = 1;
 
 // ---------------------------------------------------------------- segment unitaries
 //
-// n <= 4, long plans: the parts of the plan are carried by their 2^n x 2^n
+// n <= 4: the parts of the plan are carried by their 2^n x 2^n
 // unitaries, composed from segments (see k_unitary.cu), each an op list:
 constexpr int kUniMaxQubits = 4;
 

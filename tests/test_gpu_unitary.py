@@ -116,3 +116,28 @@ def test_runs_of_thousands_of_gates(stab, n, m):
                   - oracle.generators(n, gates, c.thetas)).max() <= tol
     assert abs(s.expect(obs) - oracle.expect(n, gates, c.thetas, obs)) <= 1.75 * tol
     s.close()
+
+
+@pytest.mark.parametrize("n", [2, 3])
+@pytest.mark.parametrize("layers", [1, 2, 3, 4, 5, 12, 21, 22])
+def test_short_plans(stab, n, layers):
+    """From 8 passes on plans of two and three qubits run through the unitaries,
+    below through the coefficients; all read-outs, and Clifford circuits exactly."""
+    for c, exact in ((h_heavy(n, layers, 4, seed=940 + 10 * n + layers), False),
+                     (W.random_circuit(n, 6 * layers, seed=950 + layers, clifford_only=True), True)):
+        obs = W.obs_chain(n) + [(0.25, "Y" * n)]
+        tol = 0.0 if exact else 1e-12 * sum(abs(a) for a, _ in obs)
+        s = stab.Stab(n)
+        s.apply_circuit(c.gates, c.thetas)
+        gens = layout.lib_to_paper(n, s.generators())
+        assert np.abs(gens - oracle.generators(n, c.gates, c.thetas)).max() <= tol
+        assert abs(s.expect(obs) - oracle.expect(n, c.gates, c.thetas, obs)) <= tol
+        perm = bitrev(n)
+        rho = s.density_matrix()[np.ix_(perm, perm)]
+        assert np.abs(rho - oracle.density_matrix(n, c.gates, c.thetas)).max() <= max(tol, 1e-15)
+        e, g = s.grad(obs)
+        assert abs(e - oracle.expect(n, c.gates, c.thetas, obs)) <= tol
+        if c.n_params:
+            want = oracle.psr_grad(n, c.gates, c.thetas, obs)
+            assert np.abs(g - want).max() <= 1e-12 * sum(abs(a) for a, _ in obs)
+        s.close()
