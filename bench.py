@@ -68,10 +68,25 @@ def units_per_step(c):
     return (c.n + 1) * c.m * 4 ** c.n
 
 
-# DRAM bytes read + written by the generator phase's launches (k_batch first
-# part + k_transfer_cols), per step, from one ncu capture of the 60,200-gate
-# n = 4 workload: keyed by (n, gates, cut pass, transfer matrices)
-GEN_TRAFFIC = {(4, 60200, 10535, 1): 3393024.0, (4, 60200, 9218, 2): 3195136.0}
+# DRAM bytes read + written by the generator phase's launches (k_uni_segments,
+# k_uni_images) per step, from one ncu capture of the 60,200-gate n = 4
+# workload: keyed by (n, gates)
+GEN_TRAFFIC = {(4, 60200): 1135104.0}
+
+
+def wire_runs(c):
+    """Maximal stretches of single-qubit gates on one wire: the wire passes of
+    the fused plan."""
+    from paper_2502_10685_gb300 import workloads as W
+    open_run, runs = [False] * c.n, 0
+    for g in c.gates:
+        q0, q1 = int(g["q0"]), int(g["q1"])
+        if int(g["op"]) in (W.OPS["CX"], W.OPS["CZ"]):
+            open_run[q0] = open_run[q1] = False
+        elif not open_run[q0]:
+            open_run[q0] = True
+            runs += 1
+    return runs
 
 
 def algorithmic_flops_generators(c):
@@ -364,27 +379,21 @@ def run_ours(args):
     # ---- roofline of the dominant kernel (the generator launch)
     gen_avg_s = statistics.mean(gen_ms) / 1e3
     achieved = algorithmic_flops_generators(c) / gen_avg_s / 1e12
-    cut, gen_units, _ = s.split_info()
+    _, gen_units, _ = s.split_info()
     n_passes = s.plan_info()[1]
     if gen_units:
-        # the generators' persistent launch: n vectors through passes [0, cut)
-        # and the 4^n - 1 transfer-matrix columns through [cut, P), then one
-        # product; FP64 work executed per algorithmic flop, counted in passes
-        n_mats = (gen_units - (c.n + 1)) // (4 ** c.n - 1)
-        if c.n == 4:
-            kernel = ("k_transfer_cols (%d x 255 columns, %d per CTA) + k_batch (%d first-part "
-                      "units) + k_apply_transfer" % (n_mats, 2 * n_mats, c.n + 1))
-        else:
-            kernel = "k_batch (split: %d units) + k_apply_transfer" % gen_units
-        # every later part's columns together cover the passes after the cut once
-        executed = ((c.n + 1) * cut + (4 ** c.n - 1) * (n_passes - cut)) / (c.n * n_passes)
-        active_sms = min(sms, c.n + 1 + 128 if c.n == 4 else gen_units)
-        note = ("one circuit: the generators' first part ends at pass %d of %d, %d later "
-                "part(s) each through its transfer matrix; the n + 1 first-part vectors "
-                "and the basis columns run at once (%s); passes are sequential within a "
-                "vector" % (cut, n_passes, n_mats,
-                            "%d columns per CTA" % (2 * n_mats) if c.n == 4
-                            else "one CTA each"))
+        # the unitaries of the plan's segments and their tree, then the read-out:
+        # a wire pass is 8 FP64 instructions (16 flops) an entry of a 2^n x 2^n
+        # matrix, a tree product 4 FMA an entry and inner index
+        d = 2 ** c.n
+        segs = max(1, min(sms if c.n == 4 else 2 * sms, wire_runs(c) // 10))
+        flops = wire_runs(c) * d * d * 16.0 + (segs - 1) * d ** 3 * 8.0
+        kernel = "k_uni_segments (%d segments) + k_uni_images" % segs
+        executed = flops / algorithmic_flops_generators(c)
+        active_sms = min(sms, segs)
+        note = ("one circuit: %d passes cut into segments whose 2^n x 2^n unitaries are "
+                "composed at once and multiplied in a tree in the same launch; the "
+                "generators are read off the unitaries" % n_passes)
     else:
         kernel = "k_resident_stream (generators)"
         executed = 1.0
@@ -392,10 +401,9 @@ def run_ours(args):
         note = "one circuit: n independent vectors, one CTA each; passes are sequential"
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak_dfma, "unit": "TFLOP/s",
                 "frac": achieved / peak_dfma,
-                # DRAM bytes of the generator phase's two launches from one ncu
-                # capture of this workload with this split (the staged streams);
-                # another split stages other streams
-                "traffic": GEN_TRAFFIC.get((c.n, c.m, cut, n_mats if gen_units else 0)),
+                # DRAM bytes of the generator phase's launches from one ncu capture
+                # of this workload
+                "traffic": GEN_TRAFFIC.get((c.n, c.m)) if gen_units else None,
                 "kernel": kernel, "launch_ms": gen_avg_s * 1e3,
                 "peak_source": "of measured: FP64 DFMA chains on this GPU in this run "
                                "(stab_probe_fp64, best of 3; %d SMs)" % sms,
@@ -1143,15 +1151,17 @@ def _sparse_step_gates(c, backward=True):
 
 
 def _sparse_work(c, n0, history):
-    """(term-gate updates, algorithmic bytes) of one backward propagation:
-    every step reads its list (8 B key + 8 B coefficient per term) and writes
-    its output list; a Clifford run maps each term once per gate."""
+    """(term-gate updates, algorithmic bytes) of one backward propagation: a
+    Clifford run maps each term once per gate; a rotation reads its list (8 B
+    key + 8 B coefficient per term) and writes its output list.  (Clifford gates
+    need no pass over the list.)"""
     steps = _sparse_step_gates(c)
     assert len(steps) == len(history), (len(steps), len(history))
     upd, nbytes, before = 0, 0, n0
     for (kind, g), after in zip(steps, history):
         upd += before * g
-        nbytes += 16 * before + 16 * int(after)
+        if kind == "r":
+            nbytes += 16 * before + 16 * int(after)
         before = int(after)
     return upd, nbytes
 
@@ -1207,7 +1217,7 @@ def run_sparse(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_source": src,
                      "kernel": "whole call (all sparse kernels), algorithmic bytes = "
-                               "16 B per term read + 16 B per term written per step"},
+                               "16 B per term read + 16 B per term written per rotation"},
         "clocks": clk,
     }
     sp.close()
