@@ -316,7 +316,7 @@ int stab_batch_destroy(stab_batch *b);
  *    quarter of that per extra qubit, at least one), its vectors staying in
  *    its own device memory between launches.  New requests join at the next
  *    launch.  Larger requests, and those that would take one CTA more than
- *    about half a millisecond, run as in STAB_SERVE_CONTEXTS, beside them.
+ *    about two milliseconds, run as in STAB_SERVE_CONTEXTS, beside them.
  *  - STAB_SERVE_CONTEXTS: each admitted request runs on its own pooled
  *    context and streams, so the kernels of all admitted requests overlap on
  *    the device; contexts keep their device vectors between requests.

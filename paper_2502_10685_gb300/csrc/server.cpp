@@ -349,10 +349,13 @@ size_t next_request_locked(const stab_server *s) {
 // steps).  48 requests at once, n = 4 .. 8, to 6,000 gates: 18.4 ms with all n <= 6 in
 // the engine (an n = 6 gradient of 3,585 gates finished last; alone on a context it
 // takes 1.2 ms), 7.9 with the line at 0.25, 0.6 or 2 ms, 8.6 at 0.1, where the many
-// small contexts' launches queue.  A new context costs half a millisecond once.
+// small contexts' launches queue.  A new context costs half a millisecond once: 30
+// requests of n = 4 .. 7, to 2,000 gates, took a new server 16 ms with the line at 0.6
+// (4.6 later), 12 with it at 2 (5.6 later), as with all in the engine (5.6 later).  The
+// line does not look at the load: a result must not depend on what runs beside it.
 // Estimate: 0.17 ns per gate and entry, four times that for a gradient's pair
 // (n = 6: 0.68 us a gate).
-constexpr double kLongUs = 600.0;
+constexpr double kLongUs = 2000.0;
 bool use_iteration(const stab_server *s, const Req *r) {
     return s->iterate && r->hdr.n <= s->opts.iter_max_n &&
            (double)r->hdr.m * (double)((int64_t)1 << (2 * r->hdr.n)) * 1.66e-4 *
