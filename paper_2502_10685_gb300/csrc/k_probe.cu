@@ -9,8 +9,8 @@
 // rate shows whether the tensor path would beat plain DFMA for this work.
 //
 // The pass-latency probe times, on one CTA and with the SM's cycle counter,
-// the pieces of the n = 4 register pass loop that bounds a lone vector (the
-// first part of a split generator sweep): a wire pass on a wire whose group
+// the pieces of the n = 4 register pass loop that bounds a lone vector (short
+// plans, batch and serving units): a wire pass on a wire whose group
 // sits in a warp's lanes (three shuffles, then three dependent FP64
 // instructions per lane), a switch of the register layout through shared
 // memory, and a pull through a four-CNOT ring walked record by record.
