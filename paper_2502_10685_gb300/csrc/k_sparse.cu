@@ -77,11 +77,11 @@ __device__ __forceinline__ double sp_neg_if(double x, bool neg) {   // off the F
 
 // The images of a term under the rotation: up to two (key, value) pairs in the
 // order u, v, their number returned.  i u P = +-v: with the minus, v enters and
-// leaves negated.  The FP64 pipe takes an instruction of a warp every 76 clocks
-// and is what this costs: a warp of lone terms issues the two products it
-// needs, a warp with a pair (any_paired: in the whole warp) four more.  With the
-// products by zero, the sign changes and the tests for zero there as well, a
-// tile took 2.5 times as long.  All lanes call this together.
+// leaves negated.  The FP64 pipe takes an instruction of a warp every 76 clocks:
+// a warp of lone terms issues the two products it needs, a warp with a pair
+// (any_paired: in the whole warp) four more; tests for zero and signs are integer
+// work (with them off the pipe and one population count a parity the n = 32 call
+// went from 1.07 to 0.97 ms).  All lanes call this together.
 __device__ __forceinline__ int sp_images(bool in, bool any_paired, uint64_t key, double val,
                                          bool paired, double pval, const SpRot &d, int n,
                                          double c, double s, uint64_t &k0, double &v0,
@@ -219,8 +219,9 @@ __global__ void __launch_bounds__(kSpThreads) k_sp_images(const uint64_t *keys, 
 // Lists of up to kSpSmallCap terms, in shared memory: two buffers of keys and
 // coefficients, a table of positions of twice that (the key is looked up by the
 // position), the partners.  A thread takes at most four neighbouring terms.  A
-// rotation is three barriers and their latency, 1 to 2 us; as four launches it
-// was about 20.  The rotation whose list would not fit is left to the grid kernel.
+// rotation is the latency of its phases, 1.5 to 2 us up to 500 terms, then FP64:
+// 6.5 at 2,500; as four launches it was about 16.  The rotation whose list would not
+// fit is left to the grid kernel, which takes 10 us a rotation up to 150,000 terms.
 constexpr int kSmallThreads = 1024, kSmallPer = kSpSmallCap / kSmallThreads;
 constexpr int kSmallLog = 13, kSmallRots = 64;
 struct SpSmall {
@@ -381,10 +382,12 @@ __device__ bool sp_grid_sync(SpState *st, uint32_t want, int *s_ok) {
     return *s_ok != 0;
 }
 
-// Rotations from the state's on, two grid barriers each.  The table takes the
-// list's size (1.5 slots a term at least, 8 bytes each: it stays in L2 up to
-// lists of ten million terms; one of the capacity's size did not).  Positions: a tile of
-// the write phase needs the emitted terms before it.  CTA b holds tiles b,
+// Rotations from the state's on, two grid barriers each.  Up to 200,000 terms the
+// barriers' 2 to 3 us and the phases' own round trips are the time; of 3.8 million
+// (0.15 ms) the pair phase is 48 us of table atomics, the write phase 71 us of FP64
+// and issue (its lists take 25 us of HBM).  The table takes the list's size (1.5
+// slots a term at least, 8 bytes each: 64 MB there, where one of the capacity's size
+// and 16 bytes was 512 MB, out of L2).  Positions: a tile of the write phase needs the emitted terms before it.  CTA b holds tiles b,
 // b + G, ...: between two of its tiles lie exactly G - 1 others, whose totals
 // it reads at once (a thread each, tagged with the step, so no clearing); the
 // tiles are all in flight on resident CTAs, which publish before they wait.
@@ -467,9 +470,10 @@ __global__ void __launch_bounds__(kRunThreads, 2) k_sp_run(SpRunArgs a) {
                     old[j] = atomicCAS((unsigned long long *)a.table + slot[j], kSpFree, mine[j]);
             }
             // the terms that met an occupied slot look on together (one after the
-            // other they made this phase three times as long), each at its own odd
-            // step: neighbouring slots grow chains of 18 round trips among 250,000
-            // terms, which the whole GPU waited for
+            // other: 83 -> 48 us of this phase at 3.8 million terms), each at its own
+            // odd step: neighbouring slots grow long chains of round trips, and the
+            // whole GPU waits for the longest (500,000 terms, this phase and its
+            // barrier: 14.8 -> 8.3 us)
             for (uint32_t probe = 0;; ++probe) {
                 bool more = false;
 #pragma unroll
