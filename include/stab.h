@@ -577,6 +577,14 @@ int stab_selftest_align(int n, const stab_gate *gates, int64_t m, int64_t n_para
  * when they differ.  Errors: as stab_load_circuit; a rotation is STAB_E_RANGE. */
 int stab_selftest_pull(int n, const stab_gate *gates, int64_t m);
 
+/* Host-only check of the barrier that the CTAs of one launch meet at: with
+ * `ctas` CTAs at their meeting number `step` (from 0), the 32-bit counter's
+ * comparison lets a CTA pass exactly when all have arrived, for every number of
+ * arrivals the wait can see (wrapped counters included).  STAB_OK, or
+ * STAB_E_STATE when it does not.  Errors: STAB_E_RANGE (ctas outside [1, 2^20],
+ * step outside [0, 2^31)). */
+int stab_selftest_barrier(int64_t ctas, int64_t step);
+
 /* ---------------------------------------------------------------- path tuner */
 /* How a context of n qubits with the STAB_KERNEL_AUTO kernel runs, for one GPU
  * model.  The paper has no counterpart (its CPU pipeline has one form).  The

@@ -373,7 +373,7 @@ __device__ bool sp_grid_sync(SpState *st, uint32_t want, int *s_ok) {
             uint32_t seen;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
                          : "=r"(seen) : "l"(&st->arrived) : "memory");
-            ok = (int32_t)(seen - want) >= 0;
+            ok = arrivals_reached(seen, want);
         }
         if (!ok) atomicExch(&st->err, 2);
         *s_ok = ok ? 1 : 0;

@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_stream_chain(ChainArgs a) {
                 uint32_t seen;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
                              : "=r"(seen) : "l"(arrived) : "memory");
-                ok = seen >= want;
+                ok = arrivals_reached(seen, want);
             }
             if (!ok && a.status) atomicExch(a.status, STAB_KSTATUS_TIMEOUT);
             s_ok = ok ? 1 : 0;

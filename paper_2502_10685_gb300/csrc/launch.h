@@ -15,6 +15,14 @@ constexpr int kMaxResidentQubits = 6;   // two buffers of 4^6 doubles = 64 KiB o
 constexpr int kMaxResidentAdjoint = 6;  // four buffers of 4^6 doubles = 128 KiB
 constexpr int kRotPerGradPass = 8;      // rotations per P_WIRE pass in gradient plans
 
+// Whether a barrier's counter, which counts arrivals mod 2^32, has come to
+// `want`: the two are never 2^31 apart (a CTA is at most one meeting ahead), so
+// the sign of their difference tells, also where the count wraps (a chain of 600
+// CTAs: after 7 million steps, 14 million gates).
+__host__ __device__ inline bool arrivals_reached(uint32_t seen, uint32_t want) {
+    return (int32_t)(seen - want) >= 0;
+}
+
 // A kernel's dynamic shared-memory limit belongs to the function, not to a
 // launch: every thread and context of the process sees the same value.  It is
 // only ever raised here, under a lock, so that one thread lowering it cannot

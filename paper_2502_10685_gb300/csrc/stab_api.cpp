@@ -1989,6 +1989,15 @@ int stab_selftest_pull(int n, const stab_gate *gates, int64_t m) {
     return check_pull(n, gates, m) ? STAB_OK : STAB_E_STATE;
 }
 
+int stab_selftest_barrier(int64_t ctas, int64_t step) {
+    if (ctas < 1 || ctas > (1 << 20) || step < 0 || step > INT32_MAX) return STAB_E_RANGE;
+    const int64_t want = ctas * (step + 1);   // as k_stream_chain counts: mod 2^32
+    const uint32_t want32 = (uint32_t)ctas * (uint32_t)(step + 1);
+    for (int64_t arrived = ctas * step; arrived <= want + ctas; ++arrived)
+        if (arrivals_reached((uint32_t)arrived, want32) != (arrived >= want)) return STAB_E_STATE;
+    return STAB_OK;
+}
+
 int stab_selftest_bounded_wait(int64_t polls) {
     if (polls < 0) return STAB_E_RANGE;
     cudaStream_t s = nullptr;
