@@ -2901,6 +2901,9 @@ int stab::long_item_prepare(stab_ctx *c, bool gens, int max_ctas, const ChainDes
         for (DevBuf *b : {&c->lam, &c->tmp, &c->lam2, &c->tmp3}) RC(c->dalloc(*b, vb, c->st));
         RC(c->dalloc(c->dotbuf, 256 * sizeof(double), c->st));
         RC(expect_chains(c, key, max_ctas, c->st));
+        // the terms were allocated and copied on aux, and the batch reads them on
+        // a stream of its own that waits for c->st alone
+        CK(cudaStreamSynchronize(c->aux));
     }
     *chains = C.desc;
     *n_chains = C.n_chains;
