@@ -251,6 +251,9 @@ std::vector<int64_t> pick_long(const stab_batch_item *items, const std::vector<i
 
 // Contexts, chains and descriptors of the long items.
 int build_long(stab_batch *b, const stab_batch_item *items, const std::vector<int64_t> &longs) {
+    if (longs.empty()) return STAB_OK;
+    BCK(cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking));
+    BCK(cudaEventCreateWithFlags(&b->ev_long, cudaEventDisableTiming));
     const int budget = chain_max_ctas(128) / 2;   // the persistent kernel's CTAs fit beside them
     std::vector<ChainDesc> chains;
     std::vector<double> work;
@@ -284,7 +287,7 @@ int build_long(stab_batch *b, const stab_batch_item *items, const std::vector<in
         b->n_long_units += L.gens ? I.n : 1;
     }
     b->n_chains = (int)chains.size();
-    if (chains.empty()) return STAB_OK;
+    if (chains.empty()) return STAB_OK;   // identity circuits: nothing between fill and finish
     // CTAs in proportion to each chain's work, so that the chains end together,
     // at least one and at most one per tile
     double lo = 0.0, hi = 1e9;
@@ -311,22 +314,23 @@ int build_long(stab_batch *b, const stab_batch_item *items, const std::vector<in
     BCK(cudaMemcpyAsync(b->chains.p, chains.data(), chains.size() * sizeof(ChainDesc),
                         cudaMemcpyHostToDevice, b->st));
     BCK(cudaStreamSynchronize(b->st));
-    BCK(cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking));
-    BCK(cudaEventCreateWithFlags(&b->ev_long, cudaEventDisableTiming));
     return STAB_OK;
 }
 
 // The long items' launches on st2.
 int queue_long(stab_batch *b) {
     for (const auto &L : b->longs) BRC(long_item_fill(L.ctx, L.gens, b->st2));
-    BCK(cudaMemsetAsync((char *)b->chains.p + b->chains_at, 0, 128 * (size_t)b->n_chains, b->st2));
-    ChainArgs a{};
-    a.chains = (const ChainDesc *)b->chains.p;
-    a.n_chains = b->n_chains;
-    a.grid = b->chain_grid;
-    a.tile_bits = 9;
-    a.status = (int32_t *)b->counter.p + 32;
-    BCK(launch_stream_chain(a, b->st2));
+    if (b->n_chains > 0) {
+        BCK(cudaMemsetAsync((char *)b->chains.p + b->chains_at, 0, 128 * (size_t)b->n_chains,
+                            b->st2));
+        ChainArgs a{};
+        a.chains = (const ChainDesc *)b->chains.p;
+        a.n_chains = b->n_chains;
+        a.grid = b->chain_grid;
+        a.tile_bits = 9;
+        a.status = (int32_t *)b->counter.p + 32;
+        BCK(launch_stream_chain(a, b->st2));
+    }
     for (const auto &L : b->longs) {
         double *out = L.gens ? (double *)b->gens.p + b->gen_off[(size_t)L.item]
                              : (double *)b->exps.p + L.item;
@@ -687,7 +691,7 @@ int stab_batch_run(stab_batch *b) {
         BCK(cudaEventRecord(b->ev_in, b->user_st));
         BCK(cudaStreamWaitEvent(b->st, b->ev_in, 0));
     }
-    if (b->n_chains > 0) {
+    if (!b->longs.empty()) {
         // first, so that the chains' CTAs find room beside the persistent kernel's
         // (and after everything queued so far that may read the results)
         BCK(cudaEventRecord(b->ev_out, b->st));
@@ -696,7 +700,7 @@ int stab_batch_run(stab_batch *b) {
         BCK(cudaEventRecord(b->ev_long, b->st2));
     }
     if (b->n_units > 0) BRC(launch_graph_or_direct(b, a, b->grid, true));
-    if (b->n_chains > 0) BCK(cudaStreamWaitEvent(b->st, b->ev_long, 0));
+    if (!b->longs.empty()) BCK(cudaStreamWaitEvent(b->st, b->ev_long, 0));
     if (b->has_user_st) {
         BCK(cudaEventRecord(b->ev_out, b->st));
         BCK(cudaStreamWaitEvent(b->user_st, b->ev_out, 0));

@@ -2888,7 +2888,7 @@ int stab::long_item_prepare(stab_ctx *c, bool gens, int max_ctas, const ChainDes
     const std::vector<const void *> key = {(const void *)c->plan_gen};
     ChainSet &C = gens ? c->c_gens : c->c_expect;
     RC(stream_maps(c, c->fwd));
-    if (!c->fwd.prog.pass_maps) return STAB_E_STATE;
+    if (!c->fwd.prog.pass_maps && !c->fwd.host.passes.empty()) return STAB_E_STATE;
     if (gens) {
         const size_t bytes = vb * (size_t)c->n;
         RC(c->dalloc(c->gens, bytes, c->st));

@@ -111,3 +111,29 @@ def test_terms_are_there_before_the_first_run(stab):
         c = it.circuit
         want = oracle.expect(c.n, c.gates, c.thetas, it.observable)
         assert abs(e - want) <= 1e-12 * l1(it.observable)
+
+
+def test_identity_circuits_among_long_items(stab):
+    """An n = 8 circuit that does nothing (no gates, or pairs that cancel) counts
+    as long and has no chain step: its values come out all the same, alone and
+    beside a chain."""
+    empty = W.Circuit(8, np.zeros(0, dtype=W.GATE_DTYPE), np.zeros(0))
+    pairs = W.Circuit(8, W.gates_from_list([("X", 3), ("X", 3)]), np.zeros(0))
+    obs = [(0.75, "ZIIIIIIZ"), (0.5, "IIIIIIII"), (2.0, "XIIIIIII")]
+    still = [W.BatchItem(empty, "generators"), W.BatchItem(pairs, "expect", obs)]
+    deep = W.BatchItem(W.layered_ansatz(8, 1301, seed=5), "expect", W.obs_chain(8))
+    for items in (still[:1], still[1:], still, still + [deep]):
+        b = stab.Batch(items)
+        for _ in range(2):
+            b.run()
+            ex = b.expectations()
+            for k, it in enumerate(items):
+                c = it.circuit
+                if it.kind == "generators":
+                    assert math.isnan(ex[k])
+                    want = oracle.generators(8, c.gates, c.thetas)
+                    assert np.array_equal(layout.lib_to_paper(8, b.generators(k)), want)
+                else:
+                    want = oracle.expect(8, c.gates, c.thetas, it.observable)
+                    assert abs(ex[k] - want) <= 1e-12 * l1(it.observable)
+        b.close()
