@@ -68,6 +68,7 @@ struct stab_batch {
         stab_ctx *ctx;
     };
     std::vector<LongItem> longs;
+    bool picked_long = false;
     int n_long_units = 0, n_chains = 0, chain_grid = 0;
     Buf chains;                       // descriptors, then 128 bytes of counter each
     size_t chains_at = 0;             // of the counters
@@ -358,7 +359,8 @@ int launch_long(stab_batch *b) {
     return STAB_OK;
 }
 
-int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel) {
+int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel,
+          bool allow_long) {
     std::vector<Rec> recs;
     std::vector<int32_t> enc;
     std::vector<DevMap3> maps;
@@ -422,12 +424,13 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
     // long items leave the persistent kernel's tables
     std::vector<int64_t> longs;
     std::vector<char> is_long((size_t)count, 0);
-    if (kernel == STAB_KERNEL_AUTO && chain_max_ctas(128) > 0) {
+    if (allow_long && kernel == STAB_KERNEL_AUTO && chain_max_ctas(128) > 0) {
         std::vector<int64_t> cost((size_t)count);
         for (int64_t it = 0; it < count; ++it)
             cost[(size_t)it] = (int64_t)(plans[(size_t)it].S.size() / kChunkRecs)
                                << (2 * items[it].n);
         longs = pick_long(items, cost, sms, chain_max_ctas(128) / 4);
+        b->picked_long = !longs.empty();
         for (int64_t it : longs) {
             is_long[(size_t)it] = 1;
             plans[(size_t)it] = ItemPlan();
@@ -633,20 +636,8 @@ int build(stab_batch *b, const stab_batch_item *items, int64_t count, int kernel
     return build_long(b, items, longs);
 }
 
-}  // namespace
-
-extern "C" {
-
-int stab_batch_create(const stab_batch_item *items, int64_t count, const stab_opts *opts,
-                      stab_batch **out) {
-    if (!out) return STAB_E_INVAL;
-    *out = nullptr;
-    if (count < 1 || count > (int64_t)INT32_MAX / 16) return STAB_E_RANGE;
-    if (!items) return STAB_E_INVAL;
-    stab_opts o;
-    stab_default_opts(&o);
-    if (opts) o = *opts;
-    if ((o.alloc == nullptr) != (o.free == nullptr)) return STAB_E_INVAL;
+int create_batch(const stab_batch_item *items, int64_t count, const stab_opts &o, bool allow_long,
+                 stab_batch **out, bool *had_long) {
     stab_batch *b = new (std::nothrow) stab_batch();
     if (!b) return STAB_E_NOMEM;
     b->alloc = o.alloc;
@@ -674,13 +665,36 @@ int stab_batch_create(const stab_batch_item *items, int64_t count, const stab_op
         stab_batch_destroy(b);
         return STAB_E_CUDA;
     }
-    const int rc = build(b, items, count, o.kernel);
+    const int rc = build(b, items, count, o.kernel, allow_long);
+    *had_long = b->picked_long;
     if (rc != STAB_OK) {
         stab_batch_destroy(b);
         return rc;
     }
     *out = b;
     return STAB_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int stab_batch_create(const stab_batch_item *items, int64_t count, const stab_opts *opts,
+                      stab_batch **out) {
+    if (!out) return STAB_E_INVAL;
+    *out = nullptr;
+    if (count < 1 || count > (int64_t)INT32_MAX / 16) return STAB_E_RANGE;
+    if (!items) return STAB_E_INVAL;
+    stab_opts o;
+    stab_default_opts(&o);
+    if (opts) o = *opts;
+    if ((o.alloc == nullptr) != (o.free == nullptr)) return STAB_E_INVAL;
+    bool had_long = false;
+    int rc = create_batch(items, count, o, true, out, &had_long);
+    // no room for the long items' contexts: the persistent kernel takes them as
+    // any other item
+    if (rc == STAB_E_NOMEM && had_long) rc = create_batch(items, count, o, false, out, &had_long);
+    return rc;
 }
 
 int stab_batch_run(stab_batch *b) {

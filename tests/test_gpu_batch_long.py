@@ -137,3 +137,34 @@ def test_identity_circuits_among_long_items(stab):
                     want = oracle.expect(8, c.gates, c.thetas, it.observable)
                     assert abs(ex[k] - want) <= 1e-12 * l1(it.observable)
         b.close()
+
+
+def test_no_room_for_the_long_items_contexts(stab):
+    """An allocation that fails while the long items are set up (their terms, or
+    the last one of all) does not refuse the batch: they run as other items."""
+    items = [W.BatchItem(W.layered_ansatz(6, 3001, seed=5), "expect", W.obs_chain(6)),
+             W.BatchItem(W.layered_ansatz(6, 2000, seed=8), "generators")]
+    items += [W.BatchItem(W.layered_ansatz(3, 60 + k, seed=20 + k), "expect", W.obs_chain(3))
+              for k in range(5)]
+    calls = []
+    b = HookedBatch(stab, items, lambda nbytes, st: calls.append(st))
+    assert b.rc == 0
+    b.close()
+    terms = next(k for k, st in enumerate(calls) if st != calls[0])
+    for refuse in (terms, len(calls) - 1):
+        at = []
+
+        def on_alloc(nbytes, st):
+            at.append(st)
+            return len(at) - 1 != refuse
+
+        b = HookedBatch(stab, items, on_alloc)
+        assert b.rc == 0 and len(at) > len(calls) // 2
+        b.run()
+        ex = b.expectations()
+        b.close()
+        for e, it in zip(ex, items):
+            if it.kind == "expect":
+                c = it.circuit
+                want = oracle.expect(c.n, c.gates, c.thetas, it.observable)
+                assert abs(e - want) <= 1e-12 * l1(it.observable)
