@@ -1760,15 +1760,33 @@ void stab::ctx_checkpoint_limit(stab_ctx *c, size_t bytes) {
     if (c) c->ck_bytes_max = std::min(bytes, kCheckpointBytes);
 }
 size_t stab::checkpoint_bound(int n, const stab_gate *gates, int64_t m) {
-    size_t blocks = 0, cliffs = 0;   // a slot more than ck_slots per Clifford pass at most
-    bool two = true;
+    // a slot more than ck_slots per Clifford pass at most
+    size_t blocks = 0, cliffs = 0;
+    bool two = true, run_two = false;
+    int64_t run = 0, pairs = 0;
+    // a long run of single-qubit Clifford gates may become a gather inside its block
+    auto end_run = [&]() {
+        if (run >= 8 && !run_two) {
+            ++blocks;
+            ++cliffs;
+        }
+        run = 0;
+        run_two = false;
+    };
     for (int64_t i = 0; i < m; ++i) {
         const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
         if (t && (!two || i == 0)) ++cliffs;
         if (!t && two) ++blocks;
         two = t;
+        pairs += t;
+        if (gates[i].op >= STAB_RX) end_run();
+        else ++run;
+        run_two |= t;
     }
-    return (2 * blocks + cliffs + kCkSpares) * (sizeof(double) << (2 * n));
+    end_run();
+    cliffs += (size_t)(pairs / 65535);   // gates of a pass at most
+    const size_t bytes = (2 * blocks + cliffs + kCkSpares) * (sizeof(double) << (2 * n));
+    return bytes <= kCheckpointBytes ? bytes : 0;
 }
 void stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
     if (c && c->ckslots.bytes > keep) {
