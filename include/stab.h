@@ -393,9 +393,11 @@ typedef struct stab_result {
  * plus, for a gradient, the adjoint's partial dot sums: per CTA of the
  * streamed sweep above n = 6, per thread of the resident sweep at n <= 5
  * (8 bytes x gates x 32, 32, 32, 64, 256 threads at n = 1..5, while that
- * stays within 256 MiB), as a bound on one per rotation.  A streamed gradient
- * may keep its sweeps' vectors (two per block of single-qubit gates) where the
- * budget has room for them when it starts; they are counted on top then. */
+ * stays within 256 MiB), as a bound on one per rotation.  A gradient of n >= 5
+ * on a context keeps its sweeps' vectors (two per block of single-qubit gates)
+ * where they are at most 4 GiB and the whole budget has room for them beside
+ * this footprint; it is then admitted with both.  Else it carries a fixed number
+ * of vectors (the two forms agree to rounding). */
 int64_t stab_request_footprint(const stab_request *req);
 
 /* opts may be NULL (all defaults).  Errors: STAB_E_INVAL (unknown policy or

@@ -189,7 +189,8 @@ struct Req {
     std::vector<stab_gate> gates;
     std::vector<double> thetas;
     std::vector<stab_term> terms;
-    int64_t footprint = 0;
+    int64_t footprint = 0;      // with `sweeps`
+    int64_t sweeps = 0;         // a gradient's stored sweeps (0: the pair sweep runs)
     double work = 0.0;          // estimated work: gates x 4^n (x3 for a gradient)
     stab_result res{};
     std::vector<double> grads;
@@ -362,8 +363,16 @@ bool use_iteration(const stab_server *s, const Req *r) {
                    (r->hdr.kind == STAB_REQ_GRAD ? 4.0 : 1.0) <= kLongUs;
 }
 
-// A gradient's stored sweeps come on top of the footprint it was admitted with,
-// where the budget has room for them; they are handed back when they are large.
+// A gradient on a context runs from stored sweeps where these fit the budget
+// beside its footprint, and is admitted with both; else as the pair sweep.  The
+// two round differently, so what is in flight has no say in it.
+int64_t sweep_bytes(const stab_server *s, const Req *r) {
+    const stab_request &q = r->hdr;
+    if (q.kind != STAB_REQ_GRAD || q.n <= 4 || use_iteration(s, r)) return 0;
+    const int64_t b = (int64_t)checkpoint_bound(q.n, r->gates.data(), (int64_t)r->gates.size());
+    return r->footprint + b <= s->opts.hbm_budget ? b : 0;
+}
+// Stored sweeps are handed back when they are large.
 constexpr size_t kKeepCheckpoints = (size_t)64 << 20;
 
 // ---------------------------------------------------------------- iteration requests: host side
@@ -937,14 +946,6 @@ void planner_main(stab_server *s) {
             r->slot = pool.back();
             pool.pop_back();
         }
-        int64_t stored = 0;
-        if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n > 4 && r->hdr.n <= STAB_MAX_QUBITS) {
-            stored = (int64_t)checkpoint_bound(r->hdr.n, r->gates.data(),
-                                               (int64_t)r->gates.size());
-            if (s->bytes_in_use + stored > s->opts.hbm_budget) stored = 0;
-            s->bytes_in_use += stored;
-            r->footprint += stored;
-        }
         lk.unlock();
         int rc = STAB_OK;
         if (!r->slot) {
@@ -956,7 +957,7 @@ void planner_main(stab_server *s) {
             }
         }
         if (rc == STAB_OK) {
-            ctx_checkpoint_limit(r->slot->ctx, (size_t)stored);
+            ctx_checkpoint_limit(r->slot->ctx, (size_t)r->sweeps);
             rc = launch_on_context(s, r);
         }
         lk.lock();
@@ -1097,9 +1098,12 @@ int stab_server_submit(stab_server *s, const stab_request *req, int64_t *id) {
     r->hdr.thetas = r->thetas.empty() ? nullptr : r->thetas.data();
     r->hdr.obs = r->terms.empty() ? nullptr : r->terms.data();
     r->footprint = stab_request_footprint(req);
-    if (req->n >= 1 && req->n <= STAB_MAX_QUBITS)
+    if (req->n >= 1 && req->n <= STAB_MAX_QUBITS) {
         r->work = (double)(req->m > 0 ? req->m : 1) * (double)(1ull << (2 * req->n)) *
                   (req->kind == STAB_REQ_GRAD ? 3.0 : 1.0);
+        r->sweeps = sweep_bytes(s, r);
+        r->footprint += r->sweeps;
+    }
     r->res.n_params = (int32_t)req->n_params;
     std::lock_guard<std::mutex> lk(s->mu);
     r->id = s->next_id++;

@@ -47,3 +47,36 @@ def test_nothing_reserved_for_sweeps_that_are_too_large(stab):
     assert srv.wait(i, timeout_s=120)["status"] == 0
     srv.close()
     assert most == stab.Server.footprint(c, "grad", obs)
+
+
+# n = 8, 1,500 gates: 47 blocks, so at least 94 and at most 146 vectors of 512 KiB
+# of stored sweeps (47 to 77 MB) beside a footprint below 10 MB
+SWEEPS_FIT, SWEEPS_DO_NOT = 90 << 20, 40 << 20
+
+
+@pytest.mark.parametrize("budget", [SWEEPS_FIT, SWEEPS_DO_NOT])
+def test_gradient_alone_equals_in_mix_bit_for_bit(stab, budget):
+    """Six gradients at once, under a budget that holds several footprints but
+    the stored sweeps of one request alone (or of none): each result is that of
+    the request served alone, on both sides of the rule."""
+    obs = W.obs_chain(8)
+    reqs = [W.layered_ansatz(8, 1500, seed=70 + k) for k in range(6)]
+    fp = max(stab.Server.footprint(c, "grad", obs) for c in reqs)
+    assert 3 * fp < SWEEPS_DO_NOT < 94 << 19 and fp + (146 << 19) < SWEEPS_FIT < 188 << 19
+    srv = stab.Server(hbm_budget=budget)
+    ids = [srv.submit(c, "grad", obs) for c in reqs]
+    most = most_in_use(srv, ids)
+    mix = [srv.wait(i, timeout_s=120) for i in ids]
+    srv.close()
+    if budget == SWEEPS_FIT:
+        assert most >= 94 << 19            # a gradient was admitted with its sweeps
+    for c, r in zip(reqs, mix):
+        one = stab.Server(hbm_budget=budget)
+        a = one.wait(one.submit(c, "grad", obs), timeout_s=120)
+        one.close()
+        assert a["status"] == 0 and r["status"] == 0
+        assert a["expect"] == r["expect"]
+        np.testing.assert_array_equal(a["grads"], r["grads"])
+        rot = [i for i, g in enumerate(c.gates) if int(g["op"]) in W.ROTATIONS]
+        want = oracle.psr_grad_gate(8, c.gates, c.thetas, obs, rot[len(rot) // 2])
+        assert abs(r["grads"][int(c.gates[rot[len(rot) // 2]]["param"])] - want) <= 1e-12 * l1(obs)
