@@ -191,7 +191,8 @@ namespace stab {
 cudaStream_t ctx_stream(stab_ctx *ctx);
 
 // Device memory the context's gradients may take for stored sweeps (0: none, the
-// pair sweep's fixed number of vectors), and a bound on what a circuit's take (0:
+// pair sweep's fixed number of vectors; else a failed allocation of them is
+// STAB_E_NOMEM instead of the pair sweep), and a bound on what a circuit's take (0:
 // more than any context takes, so the pair sweep runs).
 void ctx_checkpoint_limit(stab_ctx *ctx, size_t bytes);
 size_t checkpoint_bound(int n, const struct ::stab_gate *gates, int64_t m);

@@ -218,6 +218,8 @@ struct stab_server {
     std::vector<IterReq *> ready;             // planned, waiting for the engine thread
     int64_t next_id = 0, submitted = 0, completed = 0, bytes_in_use = 0;
     int n_active = 0;
+    int waiting_alone = 0;                    // admitted requests that wait for all others
+    bool alone = false;                       // one of them is being launched
     bool stop = false;
     bool planners_done = false;
     std::vector<std::thread> planners;
@@ -324,6 +326,33 @@ int launch_on_context(stab_server *s, Req *r) {
         return STAB_E_CUDA;
     if (cudaEventRecord(sl->ev, st) != cudaSuccess) return STAB_E_CUDA;
     return STAB_OK;
+}
+
+// A gradient whose stored sweeps (or anything else) found no device memory beside
+// the other requests: nothing is admitted until all others are done and the idle
+// contexts' sweeps are handed back, then it is launched once more.  Only if there
+// is no room even then it runs as the pair sweep.  (Caller holds s->mu.)
+int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
+    s->waiting_alone++;
+    s->cv_queue.notify_all();
+    s->cv_queue.wait(lk, [&] { return s->n_active == s->waiting_alone && !s->alone; });
+    s->alone = true;
+    std::vector<Slot *> idle;
+    for (auto &kv : s->idle) idle.insert(idle.end(), kv.second.begin(), kv.second.end());
+    lk.unlock();
+    stab_synchronize(r->slot->ctx);
+    for (Slot *sl : idle) ctx_trim_checkpoints(sl->ctx, 0);
+    int rc = launch_on_context(s, r);
+    if (rc == STAB_E_NOMEM) {
+        stab_synchronize(r->slot->ctx);
+        ctx_checkpoint_limit(r->slot->ctx, 0);
+        rc = launch_on_context(s, r);
+    }
+    lk.lock();
+    s->alone = false;
+    s->waiting_alone--;
+    s->cv_queue.notify_all();
+    return rc;
 }
 
 double aging_bound(const stab_server *s) {
@@ -906,7 +935,7 @@ void planner_main(stab_server *s) {
             pick = next_request_locked(s);
             Req *h = s->queue[pick];
             if (h->footprint > s->opts.hbm_budget) return true;   // never fits
-            return s->n_active < s->opts.max_active &&
+            return s->waiting_alone == 0 && s->n_active < s->opts.max_active &&
                    s->bytes_in_use + h->footprint <= s->opts.hbm_budget;
         });
         if (s->queue.empty()) {
@@ -961,6 +990,7 @@ void planner_main(stab_server *s) {
             rc = launch_on_context(s, r);
         }
         lk.lock();
+        if (rc == STAB_E_NOMEM && r->slot && r->sweeps > 0) rc = launch_alone(s, r, lk);
         if (rc != STAB_OK) {
             if (r->slot) stab_synchronize(r->slot->ctx);
             release_locked(s, r);

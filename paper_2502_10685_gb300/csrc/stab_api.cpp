@@ -228,6 +228,8 @@ struct stab_ctx {
     int ck_chunks = 1;
     bool ck_ready = false, ck_off = false;   // built for this plan; no room or not wanted
     size_t ck_bytes_max = kCheckpointBytes;
+    bool ck_must = false;            // no room is an error (the caller tries again), not a reason
+                                     // for the pair sweep
     DevBuf ckslots, ckjobs, ckdots;
     std::vector<const void *> key_ck;
     DevBuf thetas, gens, gens_tmp, lam, rho, tmp, tmp2, terms, scal, grad_rot, partials, grads;
@@ -1523,13 +1525,14 @@ bool ck_usable(stab_ctx *c, int *rc) {
     if (!c->ck_ready) *rc = ck_build(c);
     if (*rc != STAB_OK) return false;
     const size_t bytes = ck_slots(c) * c->vec_bytes();
-    if (c->ck_blocks.empty() || bytes > c->ck_bytes_max ||
-        c->dalloc(c->ckslots, bytes, c->aux) != STAB_OK) {
-        (void)cudaGetLastError();
-        c->ck_off = true;
-        return false;
-    }
-    return true;
+    c->ck_off = c->ck_blocks.empty() || bytes > c->ck_bytes_max;
+    if (c->ck_off) return false;
+    const int room = c->dalloc(c->ckslots, bytes, c->aux);
+    if (room == STAB_OK) return true;
+    (void)cudaGetLastError();
+    if (c->ck_must) *rc = room;
+    else c->ck_off = true;
+    return false;
 }
 
 // One block's wire passes from src (through Clifford pass `gather` unless
@@ -1757,7 +1760,9 @@ int ensure_grad_plan(stab_ctx *c) {
 
 cudaStream_t stab::ctx_stream(stab_ctx *c) { return c ? c->st : nullptr; }
 void stab::ctx_checkpoint_limit(stab_ctx *c, size_t bytes) {
-    if (c) c->ck_bytes_max = std::min(bytes, kCheckpointBytes);
+    if (!c) return;
+    c->ck_bytes_max = std::min(bytes, kCheckpointBytes);
+    c->ck_must = bytes > 0;
 }
 size_t stab::checkpoint_bound(int n, const stab_gate *gates, int64_t m) {
     // a slot more than ck_slots per Clifford pass at most

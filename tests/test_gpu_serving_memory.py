@@ -1,6 +1,7 @@
 """What served gradients take beside their footprint (stored sweeps, tables) is
 decided by the request and the server's budget alone, counted while it is held,
 and given back."""
+import threading
 import time
 
 import numpy as np
@@ -80,3 +81,82 @@ def test_gradient_alone_equals_in_mix_bit_for_bit(stab, budget):
         rot = [i for i, g in enumerate(c.gates) if int(g["op"]) in W.ROTATIONS]
         want = oracle.psr_grad_gate(8, c.gates, c.thetas, obs, rot[len(rot) // 2])
         assert abs(r["grads"][int(c.gates[rot[len(rot) // 2]]["param"])] - want) <= 1e-12 * l1(obs)
+
+
+class HookedServer:
+    """A server on allocator hooks: ``refuse(nbytes, live)`` says which
+    allocations fail (live: the sizes of the blocks handed out)."""
+
+    def __init__(self, stab, refuse=lambda nbytes, live: False, **fields):
+        import ctypes
+
+        import torch
+        from paper_2502_10685_gb300 import _lib
+        self.stab, self.lib, self.live, self.most = stab, _lib.load(), {}, 0
+        self.lock = threading.Lock()
+
+        def _alloc(nbytes, st, user):
+            with self.lock:
+                if refuse(int(nbytes), self.live.values()):
+                    return None
+                p = int(torch.cuda.caching_allocator_alloc(int(nbytes), 0))
+                self.live[p] = int(nbytes)
+                self.most = max(self.most, sum(self.live.values()))
+                return p
+
+        def _free(ptr, nbytes, st, user):
+            with self.lock:
+                assert self.live.pop(int(ptr)) == int(nbytes)
+            torch.cuda.caching_allocator_delete(int(ptr))
+
+        self.hooks = (_lib.ALLOC_FN(_alloc), _lib.FREE_FN(_free))
+        o = _lib.StabServerOpts()
+        o.alloc, o.free = self.hooks
+        for k, v in fields.items():
+            setattr(o, k, v)
+        self.h = ctypes.c_void_p()
+        assert self.lib.stab_server_create(ctypes.byref(o), ctypes.byref(self.h)) == 0
+
+    def submit(self, c, kind, obs):
+        import ctypes
+        keep, i = [], ctypes.c_int64()
+        r = self.stab.Server._request(c, kind, obs, keep)
+        assert self.lib.stab_server_submit(self.h, ctypes.byref(r), ctypes.byref(i)) == 0
+        return i.value
+
+    def wait(self, i, n_params):
+        import ctypes
+        from paper_2502_10685_gb300 import _lib
+        res, grads = _lib.StabResult(), np.zeros(n_params)
+        assert self.lib.stab_server_wait(self.h, i, 120.0, ctypes.byref(res),
+                                         grads.ctypes.data) == 0
+        return res.status, res.expect, grads
+
+    def close(self):
+        assert self.lib.stab_server_destroy(self.h) == 0
+        assert not self.live
+
+
+@pytest.mark.parametrize("blocks_at_once", [1, 0])
+def test_no_memory_for_the_sweeps_beside_others(stab, blocks_at_once):
+    """The device has room for the stored sweeps of one request at a time (or of
+    none): requests wait for it, all are served, and every result is that of the
+    request alone on the same device."""
+    obs = W.obs_chain(8)
+    reqs = [W.layered_ansatz(8, 1500, seed=90 + k) for k in range(5)]
+    assert stab.Server.footprint(reqs[0], "grad", obs) < 40 << 20 < 94 << 19
+
+    def refuse(nbytes, live):
+        return nbytes > 40 << 20 and sum(b > 40 << 20 for b in live) >= blocks_at_once
+
+    srv = HookedServer(stab, refuse)
+    ids = [srv.submit(c, "grad", obs) for c in reqs]
+    mix = [srv.wait(i, c.n_params) for i, c in zip(ids, reqs)]
+    srv.close()
+    for c, (status, e, g) in zip(reqs, mix):
+        one = HookedServer(stab, refuse)
+        status1, e1, g1 = one.wait(one.submit(c, "grad", obs), c.n_params)
+        one.close()
+        assert status == 0 and status1 == 0
+        assert e == e1
+        np.testing.assert_array_equal(g, g1)
