@@ -196,6 +196,10 @@ cudaStream_t ctx_stream(stab_ctx *ctx);
 // more than any context takes, so the pair sweep runs).
 void ctx_checkpoint_limit(stab_ctx *ctx, size_t bytes);
 size_t checkpoint_bound(int n, const struct ::stab_gate *gates, int64_t m);
+// Whether streamed sweeps may run as chains of tile steps, and a bound on the
+// tables and steps that these take (<O>, or a gradient from stored sweeps).
+void ctx_allow_chains(stab_ctx *ctx, bool on);
+size_t chain_bound(int n, const struct ::stab_gate *gates, int64_t m, bool grad);
 // Hands the stored sweeps' memory back when it is more than `keep`.
 void ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);
 

@@ -189,8 +189,9 @@ struct Req {
     std::vector<stab_gate> gates;
     std::vector<double> thetas;
     std::vector<stab_term> terms;
-    int64_t footprint = 0;      // with `sweeps`
+    int64_t footprint = 0;      // with `sweeps` and the chains' tables
     int64_t sweeps = 0;         // a gradient's stored sweeps (0: the pair sweep runs)
+    bool chains = false;        // sweeps as chains of tile steps
     double work = 0.0;          // estimated work: gates x 4^n (x3 for a gradient)
     stab_result res{};
     std::vector<double> grads;
@@ -392,14 +393,25 @@ bool use_iteration(const stab_server *s, const Req *r) {
                    (r->hdr.kind == STAB_REQ_GRAD ? 4.0 : 1.0) <= kLongUs;
 }
 
-// A gradient on a context runs from stored sweeps where these fit the budget
-// beside its footprint, and is admitted with both; else as the pair sweep.  The
-// two round differently, so what is in flight has no say in it.
-int64_t sweep_bytes(const stab_server *s, const Req *r) {
+// What a request on a context takes beside its footprint: a gradient's stored
+// sweeps (else the pair sweep runs) and the tables of chains (else launches), each
+// where the whole budget has room for it, and it is admitted with them.  The forms
+// round differently, so what is in flight has no say in it.
+void add_context_bytes(const stab_server *s, Req *r) {
     const stab_request &q = r->hdr;
-    if (q.kind != STAB_REQ_GRAD || q.n <= 4 || use_iteration(s, r)) return 0;
-    const int64_t b = (int64_t)checkpoint_bound(q.n, r->gates.data(), (int64_t)r->gates.size());
-    return r->footprint + b <= s->opts.hbm_budget ? b : 0;
+    if (q.n <= 4 || use_iteration(s, r)) return;
+    const bool grad = q.kind == STAB_REQ_GRAD;
+    const int64_t m = (int64_t)r->gates.size();
+    if (grad) {
+        const int64_t b = (int64_t)checkpoint_bound(q.n, r->gates.data(), m);
+        if (b == 0 || r->footprint + b > s->opts.hbm_budget) return;   // pairs: no chains
+        r->sweeps = b;
+        r->footprint += b;
+    }
+    const int64_t t = (int64_t)chain_bound(q.n, r->gates.data(), m, grad);
+    if (r->footprint + t > s->opts.hbm_budget) return;
+    r->chains = true;
+    r->footprint += t;
 }
 // Stored sweeps are handed back when they are large.
 constexpr size_t kKeepCheckpoints = (size_t)64 << 20;
@@ -987,6 +999,7 @@ void planner_main(stab_server *s) {
         }
         if (rc == STAB_OK) {
             ctx_checkpoint_limit(r->slot->ctx, (size_t)r->sweeps);
+            ctx_allow_chains(r->slot->ctx, r->chains);
             rc = launch_on_context(s, r);
         }
         lk.lock();
@@ -1131,8 +1144,7 @@ int stab_server_submit(stab_server *s, const stab_request *req, int64_t *id) {
     if (req->n >= 1 && req->n <= STAB_MAX_QUBITS) {
         r->work = (double)(req->m > 0 ? req->m : 1) * (double)(1ull << (2 * req->n)) *
                   (req->kind == STAB_REQ_GRAD ? 3.0 : 1.0);
-        r->sweeps = sweep_bytes(s, r);
-        r->footprint += r->sweeps;
+        add_context_bytes(s, r);
     }
     r->res.n_params = (int32_t)req->n_params;
     std::lock_guard<std::mutex> lk(s->mu);

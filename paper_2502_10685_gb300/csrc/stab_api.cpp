@@ -248,6 +248,7 @@ struct stab_ctx {
     size_t split_smem = 0;
     int sms = 0;                     // SMs of the device
     int chain_ctas = 0;              // CTAs of a chain launch that fit on it at once
+    bool chains_off = false;         // no room for the chains' tables: launches instead
     // the parts' unitaries were composed for these angles when tx_gen ==
     // param_gen; ev_tx marks their end on st
     int64_t param_gen = 0, tx_gen = -1;
@@ -1068,7 +1069,8 @@ int run_streamed(stab_ctx *c, const DevPlan &P, double **cur, double **alt, int 
 int chain_tile_bits(int n) { return std::min(2 * n, std::max(9, 2 * tile_wires(n))); }
 
 bool use_chain(const stab_ctx *c, const DevPlan &P, int n_vec) {
-    return c->n >= kChainMinN && c->chain_ctas > 0 && tile_form(c, P, n_vec) == kTileMaps;
+    return c->n >= kChainMinN && c->chain_ctas > 0 && !c->chains_off &&
+           tile_form(c, P, n_vec) == kTileMaps;
 }
 
 // Whether generators and <O> take the chain: a cooperative launch and its
@@ -1764,34 +1766,70 @@ void stab::ctx_checkpoint_limit(stab_ctx *c, size_t bytes) {
     c->ck_bytes_max = std::min(bytes, kCheckpointBytes);
     c->ck_must = bytes > 0;
 }
+void stab::ctx_allow_chains(stab_ctx *c, bool on) {
+    if (c) c->chains_off = !on;
+}
+namespace {
+
+// Bounds on what a streamed plan of the gates has: blocks of wire passes, Clifford
+// passes, ranges that its wire passes are planned in.
+struct PlanCount {
+    size_t blocks = 0, cliffs = 0, ranges = 1;
+    PlanCount(const stab_gate *gates, int64_t m) {
+        bool two = true, run_two = false;
+        int64_t run = 0, pairs = 0;
+        // a long run of single-qubit Clifford gates may become a gather inside its block
+        auto end_run = [&]() {
+            if (run >= 8) {
+                ++ranges;
+                blocks += !run_two;
+                cliffs += !run_two;
+            }
+            run = 0;
+            run_two = false;
+        };
+        for (int64_t i = 0; i < m; ++i) {
+            const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
+            if (t && (!two || i == 0)) ++cliffs;
+            if (!t && two) ++blocks;
+            two = t;
+            pairs += t;
+            if (gates[i].op >= STAB_RX) end_run();
+            else ++run;
+            run_two |= t;
+        }
+        end_run();
+        cliffs += (size_t)(pairs / 65535);   // gates of a pass at most
+        ranges += (size_t)(m / 16384);
+    }
+};
+
+}  // namespace
+
 size_t stab::checkpoint_bound(int n, const stab_gate *gates, int64_t m) {
     // a slot more than ck_slots per Clifford pass at most
-    size_t blocks = 0, cliffs = 0;
-    bool two = true, run_two = false;
-    int64_t run = 0, pairs = 0;
-    // a long run of single-qubit Clifford gates may become a gather inside its block
-    auto end_run = [&]() {
-        if (run >= 8 && !run_two) {
-            ++blocks;
-            ++cliffs;
-        }
-        run = 0;
-        run_two = false;
-    };
-    for (int64_t i = 0; i < m; ++i) {
-        const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
-        if (t && (!two || i == 0)) ++cliffs;
-        if (!t && two) ++blocks;
-        two = t;
-        pairs += t;
-        if (gates[i].op >= STAB_RX) end_run();
-        else ++run;
-        run_two |= t;
-    }
-    end_run();
-    cliffs += (size_t)(pairs / 65535);   // gates of a pass at most
-    const size_t bytes = (2 * blocks + cliffs + kCkSpares) * (sizeof(double) << (2 * n));
+    const PlanCount k(gates, m);
+    const size_t bytes = (2 * k.blocks + k.cliffs + kCkSpares) * (sizeof(double) << (2 * n));
     return bytes <= kCheckpointBytes ? bytes : 0;
+}
+size_t stab::chain_bound(int n, const stab_gate *gates, int64_t m, bool grad) {
+    // the largest n whose vectors the path tuner gives to tiles
+    if (n < kChainMinN || n > 9) return 0;
+    const PlanCount k(gates, m);
+    const size_t per_block = (size_t)((n + tile_wires(n) - 1) / tile_wires(n));
+    const size_t dirs = grad ? 2 : 1;   // <O>: two chains of half the plan
+    const size_t steps = dirs * ((k.blocks + k.ranges) * per_block + k.cliffs + 2);
+    // shapes: one per wire set and first (or last) wire, and one per gather read through
+    size_t sets = 0, choose = 1;
+    for (int w = 1; w <= tile_wires(n); ++w) {
+        choose = choose * (size_t)(n - w + 1) / (size_t)w;
+        sets += choose * (size_t)w;
+    }
+    const size_t shapes = dirs * (k.blocks + k.cliffs + 2) + std::min(sets, 2 * steps);
+    const size_t groups = (size_t)1 << (chain_tile_bits(n) - 2);
+    const size_t tiles = (size_t)1 << (2 * n - chain_tile_bits(n));
+    return steps * sizeof(ChainStep) +
+           shapes * (sizeof(ChainShape) + groups * sizeof(uint2) + 4 * tiles * sizeof(uint4));
 }
 void stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
     if (c && c->ckslots.bytes > keep) {

@@ -117,6 +117,9 @@ class HookedServer:
         self.h = ctypes.c_void_p()
         assert self.lib.stab_server_create(ctypes.byref(o), ctypes.byref(self.h)) == 0
 
+    def stats(self):
+        return self.stab.Server.stats(self)
+
     def submit(self, c, kind, obs):
         import ctypes
         keep, i = [], ctypes.c_int64()
@@ -160,3 +163,35 @@ def test_no_memory_for_the_sweeps_beside_others(stab, blocks_at_once):
         assert status == 0 and status1 == 0
         assert e == e1
         np.testing.assert_array_equal(g, g1)
+
+
+@pytest.mark.parametrize("kind", ["expect", "grad"])
+@pytest.mark.parametrize("n,m", [(7, 5000), (8, 2500)])
+def test_tables_are_counted(stab, n, m, kind):
+    """Random circuits have a table per Clifford run: what a request has
+    allocated at any time (beside a megabyte of a context's and the server's own
+    small buffers) is covered by what it was admitted with."""
+    c, obs = W.random_circuit(n, m, seed=95 + n), W.obs_chain(n)
+    srv = HookedServer(stab)
+    i = srv.submit(c, kind, obs)
+    most = most_in_use(srv, [i])
+    status, e, g = srv.wait(i, c.n_params)
+    srv.close()
+    assert status == 0
+    assert abs(e - oracle.expect(n, c.gates, c.thetas, obs)) <= 1e-12 * l1(obs)
+    assert srv.most <= most + (1 << 20)
+
+
+def test_no_budget_for_the_tables(stab):
+    """A budget of the footprint alone: the same request runs without tables."""
+    c, obs = W.random_circuit(8, 2500, seed=97), W.obs_chain(8)
+    want = oracle.expect(8, c.gates, c.thetas, obs)
+    for kind in ("expect", "grad"):
+        fp = stab.Server.footprint(c, kind, obs)
+        srv = HookedServer(stab, hbm_budget=fp)
+        i = srv.submit(c, kind, obs)
+        most = most_in_use(srv, [i])
+        status, e, g = srv.wait(i, c.n_params)
+        srv.close()
+        assert status == 0 and most == fp and srv.most <= fp + (1 << 20)
+        assert abs(e - want) <= 1e-12 * l1(obs)
