@@ -200,8 +200,9 @@ size_t checkpoint_bound(int n, const struct ::stab_gate *gates, int64_t m);
 // tables and steps that these take (<O>, or a gradient from stored sweeps).
 void ctx_allow_chains(stab_ctx *ctx, bool on);
 size_t chain_bound(int n, const struct ::stab_gate *gates, int64_t m, bool grad);
-// Hands the stored sweeps' memory back when it is more than `keep`.
-void ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);
+// Hands the stored sweeps' memory back when it is more than `keep`; returns what
+// the context still holds.
+size_t ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);
 
 // Density matrix from the forward-evolved coefficients of 2^n |0><0|:
 // rho (device, 2 x 4^n doubles, interleaved complex, row-major).

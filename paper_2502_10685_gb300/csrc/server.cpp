@@ -32,6 +32,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <new>
@@ -137,6 +138,7 @@ struct Slot {
     double *h_res = nullptr;      // pinned host copies
     double *h_grads = nullptr;
     cudaEvent_t ev = nullptr;
+    int64_t kept = 0;             // stored sweeps' memory it holds while idle
 };
 
 // ---------------------------------------------------------------- iteration engine
@@ -218,6 +220,8 @@ struct stab_server {
     std::vector<Slot *> slots;
     std::vector<IterReq *> ready;             // planned, waiting for the engine thread
     int64_t next_id = 0, submitted = 0, completed = 0, bytes_in_use = 0;
+    int64_t kept = 0;                         // of the idle slots: inside the budget, too, but
+                                              // handed back for requests that need the room
     int n_active = 0;
     int waiting_alone = 0;                    // admitted requests that wait for all others
     bool alone = false;                       // one of them is being launched
@@ -238,7 +242,10 @@ void complete_locked(stab_server *s, Req *r, int status) {
 }
 
 void release_locked(stab_server *s, Req *r) {
-    if (r->slot) s->idle[r->slot->n].push_back(r->slot);
+    if (r->slot) {
+        s->kept += r->slot->kept;
+        s->idle[r->slot->n].push_back(r->slot);
+    }
     r->slot = nullptr;
     if (r->admitted) {
         s->n_active--;
@@ -338,11 +345,13 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     s->cv_queue.notify_all();
     s->cv_queue.wait(lk, [&] { return s->n_active == s->waiting_alone && !s->alone; });
     s->alone = true;
+    s->kept = 0;
     std::vector<Slot *> idle;
     for (auto &kv : s->idle) idle.insert(idle.end(), kv.second.begin(), kv.second.end());
     lk.unlock();
     stab_synchronize(r->slot->ctx);
     for (Slot *sl : idle) ctx_trim_checkpoints(sl->ctx, 0);
+    for (Slot *sl : idle) sl->kept = 0;   // (nothing is admitted meanwhile: they stay idle)
     int rc = launch_on_context(s, r);
     if (rc == STAB_E_NOMEM) {
         stab_synchronize(r->slot->ctx);
@@ -354,6 +363,24 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     s->waiting_alone--;
     s->cv_queue.notify_all();
     return rc;
+}
+
+// Hands the idle contexts' sweeps back when the admitted requests need their room
+// in the budget (the contexts are out of the pools meanwhile; caller holds s->mu).
+void make_room(stab_server *s, std::unique_lock<std::mutex> &lk) {
+    if (s->bytes_in_use + s->kept <= s->opts.hbm_budget) return;
+    std::vector<Slot *> trim;
+    for (auto &kv : s->idle) {
+        auto keeps = [](const Slot *sl) { return sl->kept > 0; };
+        std::copy_if(kv.second.begin(), kv.second.end(), std::back_inserter(trim), keeps);
+        kv.second.erase(std::remove_if(kv.second.begin(), kv.second.end(), keeps),
+                        kv.second.end());
+    }
+    for (const Slot *sl : trim) s->kept -= sl->kept;
+    lk.unlock();
+    for (Slot *sl : trim) sl->kept = (int64_t)ctx_trim_checkpoints(sl->ctx, 0);
+    lk.lock();
+    for (Slot *sl : trim) s->idle[sl->n].push_back(sl);
 }
 
 double aging_bound(const stab_server *s) {
@@ -413,7 +440,8 @@ void add_context_bytes(const stab_server *s, Req *r) {
     r->chains = true;
     r->footprint += t;
 }
-// Stored sweeps are handed back when they are large.
+// Stored sweeps are handed back when they are large, or when the budget has no
+// room for them beside the admitted requests.
 constexpr size_t kKeepCheckpoints = (size_t)64 << 20;
 
 // ---------------------------------------------------------------- iteration requests: host side
@@ -966,6 +994,7 @@ void planner_main(stab_server *s) {
         s->bytes_in_use += r->footprint;
         r->res.admit_s = now_s(s->t0);
         if (use_iteration(s, r)) {
+            make_room(s, lk);
             lk.unlock();
             IterReq *it = nullptr;
             const int rc = prepare_iter(s, r, &it);
@@ -986,8 +1015,11 @@ void planner_main(stab_server *s) {
         if (!pool.empty()) {
             r->slot = pool.back();
             pool.pop_back();
+            s->kept -= r->slot->kept;
         }
+        make_room(s, lk);
         lk.unlock();
+        if (r->slot) r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, (size_t)r->sweeps);
         int rc = STAB_OK;
         if (!r->slot) {
             r->slot = make_slot(s, r->hdr.n);
@@ -1005,7 +1037,10 @@ void planner_main(stab_server *s) {
         lk.lock();
         if (rc == STAB_E_NOMEM && r->slot && r->sweeps > 0) rc = launch_alone(s, r, lk);
         if (rc != STAB_OK) {
-            if (r->slot) stab_synchronize(r->slot->ctx);
+            if (r->slot) {
+                stab_synchronize(r->slot->ctx);
+                r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, 0);
+            }
             release_locked(s, r);
             complete_locked(s, r, rc);
             s->cv_done.notify_all();
@@ -1021,30 +1056,37 @@ void completer_main(stab_server *s) {
     std::unique_lock<std::mutex> lk(s->mu);
     while (true) {
         if (s->planners_done && s->active.empty()) break;
-        bool any = false;
+        std::vector<Req *> ended;
         for (size_t i = 0; i < s->active.size();) {
             Req *r = s->active[i];
             if (cudaEventQuery(r->slot->ev) != cudaSuccess) {
                 ++i;
                 continue;
             }
+            ended.push_back(r);
+            s->active[i] = s->active.back();
+            s->active.pop_back();
+        }
+        for (Req *r : ended) {
+            lk.unlock();
             // status word of the context (bounded device waits)
             const int st = stab_synchronize(r->slot->ctx);
-            ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints);
+            r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints);
             r->res.expect = r->slot->h_res[0];
             if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n_params > 0)
                 r->grads.assign(r->slot->h_grads, r->slot->h_grads + r->hdr.n_params);
+            lk.lock();
+            if (s->bytes_in_use - r->footprint + s->kept + r->slot->kept > s->opts.hbm_budget) {
+                lk.unlock();
+                r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, 0);
+                lk.lock();
+            }
             release_locked(s, r);
             complete_locked(s, r, st);
-            s->active[i] = s->active.back();
-            s->active.pop_back();
-            any = true;
-        }
-        if (any) {
             s->cv_done.notify_all();
             s->cv_queue.notify_all();
-            continue;
         }
+        if (!ended.empty()) continue;
         lk.unlock();
         std::this_thread::sleep_for(std::chrono::microseconds(50));
         lk.lock();

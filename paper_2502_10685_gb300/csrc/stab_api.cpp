@@ -1831,13 +1831,15 @@ size_t stab::chain_bound(int n, const stab_gate *gates, int64_t m, bool grad) {
     return steps * sizeof(ChainStep) +
            shapes * (sizeof(ChainShape) + groups * sizeof(uint2) + 4 * tiles * sizeof(uint4));
 }
-void stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
-    if (c && c->ckslots.bytes > keep) {
+size_t stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
+    if (!c) return 0;
+    if (c->ckslots.bytes > keep) {
         c->dfree(c->ckslots, c->aux);
         c->key_ck.clear();
         c->c_grad.key.clear();
         c->g_grad.reset();
     }
+    return c->ckslots.bytes;
 }
 
 extern "C" {

@@ -195,3 +195,25 @@ def test_no_budget_for_the_tables(stab):
         srv.close()
         assert status == 0 and most == fp and srv.most <= fp + (1 << 20)
         assert abs(e - want) <= 1e-12 * l1(obs)
+
+
+def test_idle_contexts_memory_stays_inside_the_budget(stab):
+    """Contexts keep up to 64 MiB of stored sweeps between requests; a request
+    that needs that room in the budget gets it first.  (Four requests at once
+    leave four contexts with 50 MiB each, then one of n = 9 needs 210.)"""
+    obs = W.obs_chain(8)
+    reqs = [W.layered_ansatz(8, 1500, seed=110 + k) for k in range(4)]
+    big = W.layered_ansatz(9, 1800, seed=120)
+    budget = 370 << 20
+    srv = HookedServer(stab, hbm_budget=budget, max_active=4)
+    ids = [srv.submit(c, "grad", obs) for c in reqs]
+    small = [srv.wait(i, c.n_params) for i, c in zip(ids, reqs)]
+    status, e, g = srv.wait(srv.submit(big, "grad", W.obs_chain(9)), big.n_params)
+    again = srv.wait(srv.submit(reqs[0], "grad", obs), reqs[0].n_params)
+    srv.close()
+    assert status == 0 and all(r[0] == 0 for r in small + [again])
+    assert srv.most <= budget + (1 << 20)
+    assert abs(e - oracle.expect(9, big.gates, big.thetas, W.obs_chain(9))) <= \
+        1e-12 * l1(W.obs_chain(9))
+    assert again[1] == small[0][1]
+    np.testing.assert_array_equal(again[2], small[0][2])
