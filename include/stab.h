@@ -315,8 +315,9 @@ int stab_batch_destroy(stab_batch *b);
  *    kind of unit; before a kind is measured, iter_chunks chunks at n = 4, a
  *    quarter of that per extra qubit, at least one), its vectors staying in
  *    its own device memory between launches.  New requests join at the next
- *    launch.  Larger requests, and those that would take one CTA more than
- *    about two milliseconds, run as in STAB_SERVE_CONTEXTS, beside them.
+ *    launch.  Larger requests, and (unless the caller sets iter_max_n) those
+ *    that would take one CTA more than about two milliseconds, run as in
+ *    STAB_SERVE_CONTEXTS, beside them.
  *  - STAB_SERVE_CONTEXTS: each admitted request runs on its own pooled
  *    context and streams, so the kernels of all admitted requests overlap on
  *    the device; contexts keep their device vectors between requests.
@@ -346,7 +347,8 @@ typedef struct stab_server_opts {
     int32_t iter_smem_kb;  /* ITERATE: KiB of shared memory per CTA for vectors (0 = 32, <= 200);
                               a request whose working vectors fit runs in shared memory,
                               others in their own device memory */
-    int32_t iter_max_n;    /* ITERATE: largest n the iteration engine takes (0 = 6, 1 .. 8);
+    int32_t iter_max_n;    /* ITERATE: largest n the iteration engine takes (0 = 6, without
+                              long requests; 1 .. 8: requests of any length);
                               larger requests run on contexts (one CTA per vector leaves a
                               4^7 or 4^8 vector latency-bound) */
     double aging_s;        /* SHORTEST: aging bound in seconds (0 = 4 s, < 0 = none) */

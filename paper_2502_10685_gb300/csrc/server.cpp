@@ -209,6 +209,7 @@ struct stab_server {
     stab_server_opts opts{};
     int device = 0;
     bool iterate = true;
+    bool take_long = false;                   // the caller has set iter_max_n
     Hooks hooks;
     std::chrono::steady_clock::time_point t0;
     std::mutex mu;
@@ -411,12 +412,13 @@ size_t next_request_locked(const stab_server *s) {
 // requests of n = 4 .. 7, to 2,000 gates, took a new server 16 ms with the line at 0.6
 // (4.6 later), 12 with it at 2 (5.6 later), as with all in the engine (5.6 later).  The
 // line does not look at the load: a result must not depend on what runs beside it.
+// A caller who sets iter_max_n gets every request of that size in the engine.
 // Estimate: 0.17 ns per gate and entry, four times that for a gradient's pair
 // (n = 6: 0.68 us a gate).
 constexpr double kLongUs = 2000.0;
 bool use_iteration(const stab_server *s, const Req *r) {
-    return s->iterate && r->hdr.n <= s->opts.iter_max_n &&
-           (double)r->hdr.m * (double)((int64_t)1 << (2 * r->hdr.n)) * 1.66e-4 *
+    if (!s->iterate || r->hdr.n > s->opts.iter_max_n) return false;
+    return s->take_long || (double)r->hdr.m * (double)((int64_t)1 << (2 * r->hdr.n)) * 1.66e-4 *
                    (r->hdr.kind == STAB_REQ_GRAD ? 4.0 : 1.0) <= kLongUs;
 }
 
@@ -1149,7 +1151,8 @@ int stab_server_create(const stab_server_opts *opts, stab_server **out) {
         return STAB_E_INVAL;
     }
     s->iterate = s->opts.engine == STAB_SERVE_ITERATE;
-    if (s->opts.iter_max_n == 0) s->opts.iter_max_n = kDefaultIterMaxN;
+    s->take_long = s->opts.iter_max_n > 0;
+    if (!s->take_long) s->opts.iter_max_n = kDefaultIterMaxN;
     s->hooks.alloc = s->opts.alloc;
     s->hooks.free = s->opts.free;
     s->hooks.user = s->opts.alloc_user;

@@ -93,6 +93,7 @@ class HookedServer:
         import torch
         from paper_2502_10685_gb300 import _lib
         self.stab, self.lib, self.live, self.most = stab, _lib.load(), {}, 0
+        self.allocs = 0
         self.lock = threading.Lock()
 
         def _alloc(nbytes, st, user):
@@ -101,6 +102,7 @@ class HookedServer:
                     return None
                 p = int(torch.cuda.caching_allocator_alloc(int(nbytes), 0))
                 self.live[p] = int(nbytes)
+                self.allocs += 1
                 self.most = max(self.most, sum(self.live.values()))
                 return p
 
@@ -217,3 +219,25 @@ def test_idle_contexts_memory_stays_inside_the_budget(stab):
         1e-12 * l1(W.obs_chain(9))
     assert again[1] == small[0][1]
     np.testing.assert_array_equal(again[2], small[0][2])
+
+
+@pytest.mark.parametrize("n,m,iter_max_n", [(8, 250, 8), (6, 3000, 6), (4, 60200, 4)])
+def test_iter_max_n_takes_long_requests(stab, n, m, iter_max_n):
+    """A caller's iter_max_n holds for requests of any length: a long gradient runs
+    in the iteration engine (many slices of both phases), which takes one block
+    of memory a request, also for the second of two equal ones (a pooled context
+    would have its buffers by then)."""
+    c, obs = W.layered_ansatz(n, m, seed=130 + n), W.obs_chain(n)
+    srv = HookedServer(stab, iter_max_n=iter_max_n, iter_chunks=8)
+    assert srv.wait(srv.submit(c, "grad", obs), c.n_params)[0] == 0
+    before = srv.allocs
+    status, e, g = srv.wait(srv.submit(c, "grad", obs), c.n_params)
+    assert srv.allocs - before == 1
+    srv.close()
+    tol = (1e-10 if m > 20000 else 1e-12) * l1(obs)
+    assert status == 0
+    assert abs(e - oracle.expect(n, c.gates, c.thetas, obs)) <= tol
+    rot = [i for i, gt in enumerate(c.gates) if int(gt["op"]) in W.ROTATIONS]
+    for gi in (rot[0], rot[len(rot) // 2], rot[-1]):
+        want = oracle.psr_grad_gate(n, c.gates, c.thetas, obs, gi)
+        assert abs(g[int(c.gates[gi]["param"])] - want) <= tol
