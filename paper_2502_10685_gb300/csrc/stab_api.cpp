@@ -143,6 +143,53 @@ struct DevPlan {
     bool ops_encoded = false, maps_encoded = false;   // streamed plans
 };
 
+// Pinned staging of uploads on the aux stream, so that the copies are queued and
+// the caller does not wait for what is queued before them: a block that is filled
+// from the front while copies are in flight and replaced when it is full (the old
+// one goes when they are done).  `copied` is behind the last copy.
+struct Staging {
+    char *p = nullptr;
+    size_t bytes = 0, at = 0;
+    std::vector<char *> full;
+    cudaEvent_t copied = nullptr;
+    int take(size_t want, char **out) {
+        want = align256(want);
+        if (!copied) CK(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
+        if (cudaEventQuery(copied) == cudaSuccess) {
+            for (char *b : full) cudaFreeHost(b);
+            full.clear();
+            at = 0;
+        } else {
+            (void)cudaGetLastError();   // not ready
+        }
+        if (at + want > bytes) {
+            if (p && at == 0) cudaFreeHost(p);
+            else if (p) full.push_back(p);
+            p = nullptr;
+            bytes = at = 0;
+            const size_t cap = std::max((size_t)128 << 10, 2 * want);
+            CK(cudaMallocHost((void **)&p, cap));
+            bytes = cap;
+        }
+        *out = p + at;
+        at += want;
+        return STAB_OK;
+    }
+    int queued(cudaStream_t s) {
+        CK(cudaEventRecord(copied, s));
+        return STAB_OK;
+    }
+    void release() {
+        full.push_back(p);
+        for (char *b : full)
+            if (b) cudaFreeHost(b);
+        full.clear();
+        p = nullptr;
+        if (copied) cudaEventDestroy(copied);
+        copied = nullptr;
+    }
+};
+
 // A captured sequence of streamed launches, valid while its key is unchanged.
 struct GraphCache {
     cudaGraphExec_t exec = nullptr;
@@ -266,6 +313,7 @@ struct stab_ctx {
     size_t stage_bytes = 0;
     void *aux_stage = nullptr;
     size_t aux_stage_bytes = 0;
+    Staging tables_stage;            // chains' steps and shapes, gradients' jobs
     int64_t launches = 0;
 
     int dalloc(DevBuf &b, size_t bytes, cudaStream_t s) {
@@ -1243,17 +1291,21 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
                                             std::max(1, max_ctas / (n0 && n1 ? 2 : 1)));
         C.grid += e.ctas;
         C.desc[C.n_chains++] = e;
-        CK(cudaMemcpyAsync(d + (k ? n0 : 0), H.data(), H.size() * sizeof(ChainStep),
-                           cudaMemcpyHostToDevice, s));
     }
     C.alone = n_vec == 1 && tiles == 1;
-    if (C.n_chains)
-        CK(cudaMemcpyAsync((void *)C.desc_dev, C.desc, sizeof(C.desc), cudaMemcpyHostToDevice, s));
+    // as on the device: steps, descriptors; then the shapes
+    char *h = nullptr;
+    RC(c->tables_stage.take(b_steps + 256 + b_shapes, &h));
+    std::copy(C.host[0].begin(), C.host[0].end(), (ChainStep *)h);
+    std::copy(C.host[1].begin(), C.host[1].end(), (ChainStep *)h + n0);
+    std::memcpy(h + b_steps, C.desc, sizeof(C.desc));
+    std::copy(C.shapes.begin(), C.shapes.end(), (ChainShape *)(h + b_steps + 256));
+    CK(cudaMemcpyAsync(C.dev.p, h, b_steps + 256, cudaMemcpyHostToDevice, s));
     if (ns)
-        CK(cudaMemcpyAsync(C.tables.p, C.shapes.data(), ns * sizeof(ChainShape),
+        CK(cudaMemcpyAsync(C.tables.p, h + b_steps + 256, ns * sizeof(ChainShape),
                            cudaMemcpyHostToDevice, s));
+    RC(c->tables_stage.queued(s));
     CK(launch_chain_tables((const ChainShape *)C.tables.p, (int)ns, c->n, s));
-    CK(cudaStreamSynchronize(s));   // the host vectors may be rebuilt before the copies have run
     c->launches += ns > 0;
     C.key = key;
     return STAB_OK;
@@ -1590,9 +1642,12 @@ int ck_upload_jobs(stab_ctx *c, cudaStream_t s) {
         J.pull = between.empty() ? nullptr
                                  : G.prog.pulls + 2 * G.host.pull_of[(size_t)between[0]] + 1;
     }
-    CK(cudaMemcpyAsync(c->ckjobs.p, c->ck_jobs.data(), c->ck_jobs.size() * sizeof(DotJob),
-                       cudaMemcpyHostToDevice, s));
-    CK(cudaStreamSynchronize(s));   // ck_jobs may be rebuilt before the copy has run
+    const size_t bytes = c->ck_jobs.size() * sizeof(DotJob);
+    char *h = nullptr;
+    RC(c->tables_stage.take(bytes, &h));
+    std::memcpy(h, c->ck_jobs.data(), bytes);
+    CK(cudaMemcpyAsync(c->ckjobs.p, h, bytes, cudaMemcpyHostToDevice, s));
+    RC(c->tables_stage.queued(s));
     c->key_ck = key;
     return STAB_OK;
 }
@@ -2210,6 +2265,7 @@ int stab_destroy(stab_ctx *c) {
                       &c->c_gens.tables, &c->c_expect.tables, &c->c_grad.tables};
     for (DevBuf *b : bufs) c->dfree(*b, c->st);
     if (c->st) cudaStreamSynchronize(c->st);
+    c->tables_stage.release();
     if (c->stage) cudaFreeHost(c->stage);
     if (c->aux_stage) cudaFreeHost(c->aux_stage);
     if (c->ev_ready) cudaEventDestroy(c->ev_ready);
