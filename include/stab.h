@@ -190,7 +190,12 @@ int stab_expect_async(stab_ctx *ctx, double *out_dev);
  * the unitaries of the plan's parts and segments: when they were not composed
  * for the current angles that is queued first on the context stream (as by
  * stab_run_generators, which reuses them), then the gradient on the internal
- * stream.  Same for stab_expect_async in that form. */
+ * stream.  Same for stab_expect_async in that form.
+ * A streamed gradient keeps both sweeps' vectors at every block of single-qubit
+ * gates (two of 4^n doubles a block) where they take at most 4 GiB and can be
+ * allocated; else it carries a fixed number of vectors.  The two agree to
+ * rounding.  The context holds that memory until stab_destroy, or until the load
+ * of a circuit that takes less than a quarter of it (above 64 MiB). */
 int stab_grad_async(stab_ctx *ctx, double *expect_dev, double *grads_dev);
 
 /* How the last gradient's plan is cut: *parts receives K >= 2 when its units

@@ -84,6 +84,9 @@ constexpr int kThreadedStreamPasses = 2048;
 // Device memory a context may take for the stored sweeps of a gradient; above
 // it the pair sweep runs, which keeps a fixed number of vectors.
 constexpr size_t kCheckpointBytes = (size_t)4 << 30;
+// More than this goes back at a load whose circuit takes less than a quarter of it
+// (a training loop's loads of like circuits keep theirs).
+constexpr size_t kCheckpointRelease = (size_t)64 << 20;
 
 // Instruction stream of a plan for the resident kernels, with the indices of
 // the records the encode kernel fills (rotations and maps).
@@ -2298,6 +2301,9 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     c->grad.encoded = false;
     c->grad_ran = c->ck_ready = c->ck_off = false;
     reset_graphs(c);
+    if (c->ckslots.bytes > kCheckpointRelease &&
+        checkpoint_bound(c->n, gates, m) < c->ckslots.bytes / 4)
+        ctx_trim_checkpoints(c, 0);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
         // AUTO: at n <= 4 the parts' unitaries, at n = 5, 6 the two halves of <O>
