@@ -195,8 +195,16 @@ int stab_expect_async(stab_ctx *ctx, double *out_dev);
  * gates (two of 4^n doubles a block) where they take at most 4 GiB and can be
  * allocated; else it carries a fixed number of vectors.  The two agree to
  * rounding.  The context holds that memory until stab_destroy, or until the load
- * of a circuit that takes less than a quarter of it (above 64 MiB). */
+ * of a circuit that takes less than a quarter of it (above 64 MiB).
+ * stab_set_grad_memory sets another limit than 4 GiB. */
 int stab_grad_async(stab_ctx *ctx, double *expect_dev, double *grads_dev);
+
+/* Device memory that the context's gradients may keep for their sweeps' vectors
+ * from now on: bytes, at most 4 GiB (the default); 0: none, every streamed
+ * gradient carries a fixed number of vectors.  Hands back what is held above it.
+ * For programs with many contexts.  Errors: STAB_E_INVAL (ctx NULL),
+ * STAB_E_RANGE (bytes < 0), STAB_E_CUDA. */
+int stab_set_grad_memory(stab_ctx *ctx, int64_t bytes);
 
 /* How the last gradient's plan is cut: *parts receives K >= 2 when its units
  * are those of the generators' plan and both are cut into the same K parts (n

@@ -2889,6 +2889,16 @@ int stab_grad_async(stab_ctx *c, double *expect_dev, double *grads_dev) {
     return STAB_OK;
 }
 
+int stab_set_grad_memory(stab_ctx *c, int64_t bytes) {
+    if (!c) return STAB_E_INVAL;
+    if (bytes < 0) return STAB_E_RANGE;
+    CK(cudaSetDevice(c->device));
+    c->ck_bytes_max = std::min((size_t)bytes, kCheckpointBytes);
+    c->ck_off = false;   // decided anew by the next gradient
+    ctx_trim_checkpoints(c, c->ck_bytes_max);
+    return STAB_OK;
+}
+
 int stab_grad(stab_ctx *c, const stab_term *O, int64_t n_terms, double *expect_out,
               double *grads_out) {
     if (!c) return STAB_E_INVAL;

@@ -357,6 +357,10 @@ class Stab:
     def launch_count(self) -> int:
         return stab_launch_count(self.h)
 
+    def set_grad_memory(self, nbytes: int) -> None:
+        """Device memory gradients may keep for their sweeps (default 4 GiB; 0: none)."""
+        check(_lib.load().stab_set_grad_memory(self.h, int(nbytes)), "stab_set_grad_memory")
+
     def grad_parts(self) -> int:
         """K >= 2: the last gradient was cut into the generators' K parts;
         1: meet-in-the-middle or streamed; 0: no gradient since the load."""

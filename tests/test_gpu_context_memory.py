@@ -1,5 +1,5 @@
 """What a context holds of a gradient's stored sweeps goes back when a circuit is
-loaded that needs much less."""
+loaded that needs much less, or when the caller says so."""
 import ctypes
 
 import numpy as np
@@ -59,3 +59,32 @@ def test_stored_sweeps_go_back_at_the_load_of_a_small_circuit(stab):
     assert held[1] >= 60 * 8 << 20          # the first gradient's sweeps
     assert held[2] <= held[1] - (60 * 8 << 20) and held[3] < held[1] // 2
     assert L.stab_destroy(h) == 0 and not live
+
+
+def test_the_caller_may_limit_the_memory(stab):
+    """With no memory for the sweeps' vectors a gradient carries a fixed number of
+    them; with a limit just below what it needs as well; with enough, and as
+    before, it keeps them."""
+    import torch
+    from paper_2502_10685_gb300._lib import StabError
+    c, obs = W.layered_ansatz(9, 360, seed=152), W.obs_chain(9)
+    e_want = oracle.expect(9, c.gates, c.thetas, obs)
+    tol = 1e-12 * sum(abs(a) for a, _ in obs)
+    s = stab.Stab(9)
+    s.load_circuit(c.gates, c.thetas)
+    e0, g0 = s.grad(obs)
+    kept = torch.cuda.memory_allocated()
+    values = []
+    # 10 blocks: 25 vectors of 2 MiB
+    for limit in (0, (25 * 2 << 20) - 1, 25 * 2 << 20):
+        s.set_grad_memory(limit)
+        e, g = s.grad(obs)
+        values.append((e, g))
+        assert abs(e - e_want) <= tol and np.abs(g - g0).max() <= tol
+    assert values[0][0] == values[1][0] and np.array_equal(values[0][1], values[1][1])
+    assert values[2][0] == e0 and np.array_equal(values[2][1], g0)
+    s.set_grad_memory(0)
+    assert torch.cuda.memory_allocated() < kept
+    with pytest.raises(StabError):
+        s.set_grad_memory(-1)
+    s.close()
