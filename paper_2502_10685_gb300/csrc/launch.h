@@ -195,11 +195,18 @@ cudaStream_t ctx_stream(stab_ctx *ctx);
 // STAB_E_NOMEM instead of the pair sweep), and a bound on what a circuit's take (0:
 // more than any context takes, so the pair sweep runs).
 void ctx_checkpoint_limit(stab_ctx *ctx, size_t bytes);
-size_t checkpoint_bound(int n, const struct ::stab_gate *gates, int64_t m);
+struct PlanCount;
+size_t checkpoint_bound(int n, const PlanCount &k);
 // Whether streamed sweeps may run as chains of tile steps, and a bound on the
 // tables and steps that these take (<O>, or a gradient from stored sweeps).
 void ctx_allow_chains(stab_ctx *ctx, bool on);
-size_t chain_bound(int n, const struct ::stab_gate *gates, int64_t m, bool grad);
+size_t chain_bound(int n, const PlanCount &k, bool grad);
+// Bounds on what a streamed plan of the gates has: blocks of wire passes, Clifford
+// passes, ranges that its wire passes are planned in.
+struct PlanCount {
+    size_t blocks = 0, cliffs = 0, ranges = 1;
+    PlanCount(const struct ::stab_gate *gates, int64_t m);
+};
 // Hands the stored sweeps' memory back when it is more than `keep`; returns what
 // the context still holds.
 size_t ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);

@@ -138,7 +138,7 @@ struct Slot {
     double *h_res = nullptr;      // pinned host copies
     double *h_grads = nullptr;
     cudaEvent_t ev = nullptr;
-    int64_t kept = 0;             // stored sweeps' memory it holds while idle
+    int64_t kept = 0;             // stored sweeps' memory it holds beyond its request's
 };
 
 // ---------------------------------------------------------------- iteration engine
@@ -221,8 +221,8 @@ struct stab_server {
     std::vector<Slot *> slots;
     std::vector<IterReq *> ready;             // planned, waiting for the engine thread
     int64_t next_id = 0, submitted = 0, completed = 0, bytes_in_use = 0;
-    int64_t kept = 0;                         // of the idle slots: inside the budget, too, but
-                                              // handed back for requests that need the room
+    int64_t kept = 0;                         // of all slots: inside the budget, too, but handed
+                                              // back for requests that need the room
     int n_active = 0;
     int waiting_alone = 0;                    // admitted requests that wait for all others
     bool alone = false;                       // one of them is being launched
@@ -243,10 +243,7 @@ void complete_locked(stab_server *s, Req *r, int status) {
 }
 
 void release_locked(stab_server *s, Req *r) {
-    if (r->slot) {
-        s->kept += r->slot->kept;
-        s->idle[r->slot->n].push_back(r->slot);
-    }
+    if (r->slot) s->idle[r->slot->n].push_back(r->slot);
     r->slot = nullptr;
     if (r->admitted) {
         s->n_active--;
@@ -337,6 +334,12 @@ int launch_on_context(stab_server *s, Req *r) {
     return STAB_OK;
 }
 
+// Sets what a slot holds beyond its request's sweeps (caller holds s->mu).
+void set_kept(stab_server *s, Slot *sl, int64_t kept) {
+    s->kept += kept - sl->kept;
+    sl->kept = kept;
+}
+
 // A gradient whose stored sweeps (or anything else) found no device memory beside
 // the other requests: nothing is admitted until all others are done and the idle
 // contexts' sweeps are handed back, then it is launched once more.  Only if there
@@ -346,13 +349,12 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     s->cv_queue.notify_all();
     s->cv_queue.wait(lk, [&] { return s->n_active == s->waiting_alone && !s->alone; });
     s->alone = true;
-    s->kept = 0;
-    std::vector<Slot *> idle;
+    std::vector<Slot *> idle;   // (nothing is admitted meanwhile: they stay so)
     for (auto &kv : s->idle) idle.insert(idle.end(), kv.second.begin(), kv.second.end());
+    for (Slot *sl : idle) set_kept(s, sl, 0);
     lk.unlock();
     stab_synchronize(r->slot->ctx);
     for (Slot *sl : idle) ctx_trim_checkpoints(sl->ctx, 0);
-    for (Slot *sl : idle) sl->kept = 0;   // (nothing is admitted meanwhile: they stay idle)
     int rc = launch_on_context(s, r);
     if (rc == STAB_E_NOMEM) {
         stab_synchronize(r->slot->ctx);
@@ -366,9 +368,10 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     return rc;
 }
 
-// Hands the idle contexts' sweeps back when the admitted requests need their room
-// in the budget (the contexts are out of the pools meanwhile; caller holds s->mu).
-void make_room(stab_server *s, std::unique_lock<std::mutex> &lk) {
+// Hands back what idle contexts, then r's own, hold beyond their requests' sweeps
+// when the admitted requests need that room in the budget (the idle ones are out
+// of the pools meanwhile; caller holds s->mu).
+void make_room(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     if (s->bytes_in_use + s->kept <= s->opts.hbm_budget) return;
     std::vector<Slot *> trim;
     for (auto &kv : s->idle) {
@@ -377,9 +380,12 @@ void make_room(stab_server *s, std::unique_lock<std::mutex> &lk) {
         kv.second.erase(std::remove_if(kv.second.begin(), kv.second.end(), keeps),
                         kv.second.end());
     }
-    for (const Slot *sl : trim) s->kept -= sl->kept;
+    for (Slot *sl : trim) set_kept(s, sl, 0);
+    const bool own = r->slot && r->slot->kept > 0;
+    if (own) set_kept(s, r->slot, 0);
     lk.unlock();
-    for (Slot *sl : trim) sl->kept = (int64_t)ctx_trim_checkpoints(sl->ctx, 0);
+    for (Slot *sl : trim) ctx_trim_checkpoints(sl->ctx, 0);
+    if (own) ctx_trim_checkpoints(r->slot->ctx, (size_t)r->sweeps);
     lk.lock();
     for (Slot *sl : trim) s->idle[sl->n].push_back(sl);
 }
@@ -430,14 +436,14 @@ void add_context_bytes(const stab_server *s, Req *r) {
     const stab_request &q = r->hdr;
     if (q.n <= 4 || use_iteration(s, r)) return;
     const bool grad = q.kind == STAB_REQ_GRAD;
-    const int64_t m = (int64_t)r->gates.size();
+    const PlanCount k(r->gates.data(), (int64_t)r->gates.size());
     if (grad) {
-        const int64_t b = (int64_t)checkpoint_bound(q.n, r->gates.data(), m);
+        const int64_t b = (int64_t)checkpoint_bound(q.n, k);
         if (b == 0 || r->footprint + b > s->opts.hbm_budget) return;   // pairs: no chains
         r->sweeps = b;
         r->footprint += b;
     }
-    const int64_t t = (int64_t)chain_bound(q.n, r->gates.data(), m, grad);
+    const int64_t t = (int64_t)chain_bound(q.n, k, grad);
     if (r->footprint + t > s->opts.hbm_budget) return;
     r->chains = true;
     r->footprint += t;
@@ -996,7 +1002,7 @@ void planner_main(stab_server *s) {
         s->bytes_in_use += r->footprint;
         r->res.admit_s = now_s(s->t0);
         if (use_iteration(s, r)) {
-            make_room(s, lk);
+            make_room(s, r, lk);
             lk.unlock();
             IterReq *it = nullptr;
             const int rc = prepare_iter(s, r, &it);
@@ -1017,11 +1023,10 @@ void planner_main(stab_server *s) {
         if (!pool.empty()) {
             r->slot = pool.back();
             pool.pop_back();
-            s->kept -= r->slot->kept;
+            set_kept(s, r->slot, std::max<int64_t>(0, r->slot->kept - r->sweeps));
         }
-        make_room(s, lk);
+        make_room(s, r, lk);
         lk.unlock();
-        if (r->slot) r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, (size_t)r->sweeps);
         int rc = STAB_OK;
         if (!r->slot) {
             r->slot = make_slot(s, r->hdr.n);
@@ -1041,7 +1046,8 @@ void planner_main(stab_server *s) {
         if (rc != STAB_OK) {
             if (r->slot) {
                 stab_synchronize(r->slot->ctx);
-                r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, 0);
+                ctx_trim_checkpoints(r->slot->ctx, 0);
+                set_kept(s, r->slot, 0);
             }
             release_locked(s, r);
             complete_locked(s, r, rc);
@@ -1069,26 +1075,42 @@ void completer_main(stab_server *s) {
             s->active[i] = s->active.back();
             s->active.pop_back();
         }
-        for (Req *r : ended) {
+        if (!ended.empty()) {
             lk.unlock();
-            // status word of the context (bounded device waits)
-            const int st = stab_synchronize(r->slot->ctx);
-            r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints);
-            r->res.expect = r->slot->h_res[0];
-            if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n_params > 0)
-                r->grads.assign(r->slot->h_grads, r->slot->h_grads + r->hdr.n_params);
+            std::vector<int> status;
+            std::vector<int64_t> kept;
+            int64_t freed = 0;
+            for (Req *r : ended) {
+                // status word of the context (bounded device waits)
+                status.push_back(stab_synchronize(r->slot->ctx));
+                kept.push_back((int64_t)ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints));
+                r->res.expect = r->slot->h_res[0];
+                if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n_params > 0)
+                    r->grads.assign(r->slot->h_grads, r->slot->h_grads + r->hdr.n_params);
+                freed += r->footprint;
+            }
             lk.lock();
-            if (s->bytes_in_use - r->footprint + s->kept + r->slot->kept > s->opts.hbm_budget) {
+            std::vector<Slot *> trim;
+            for (size_t i = 0; i < ended.size(); ++i) {
+                Slot *sl = ended[i]->slot;
+                set_kept(s, sl, kept[i]);
+                if (s->bytes_in_use - freed + s->kept <= s->opts.hbm_budget) continue;
+                set_kept(s, sl, 0);
+                trim.push_back(sl);
+            }
+            if (!trim.empty()) {
                 lk.unlock();
-                r->slot->kept = (int64_t)ctx_trim_checkpoints(r->slot->ctx, 0);
+                for (Slot *sl : trim) ctx_trim_checkpoints(sl->ctx, 0);
                 lk.lock();
             }
-            release_locked(s, r);
-            complete_locked(s, r, st);
+            for (size_t i = 0; i < ended.size(); ++i) {
+                release_locked(s, ended[i]);
+                complete_locked(s, ended[i], status[i]);
+            }
             s->cv_done.notify_all();
             s->cv_queue.notify_all();
+            continue;
         }
-        if (!ended.empty()) continue;
         lk.unlock();
         std::this_thread::sleep_for(std::chrono::microseconds(50));
         lk.lock();

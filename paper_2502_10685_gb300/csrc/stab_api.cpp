@@ -1827,53 +1827,42 @@ void stab::ctx_checkpoint_limit(stab_ctx *c, size_t bytes) {
 void stab::ctx_allow_chains(stab_ctx *c, bool on) {
     if (c) c->chains_off = !on;
 }
-namespace {
-
-// Bounds on what a streamed plan of the gates has: blocks of wire passes, Clifford
-// passes, ranges that its wire passes are planned in.
-struct PlanCount {
-    size_t blocks = 0, cliffs = 0, ranges = 1;
-    PlanCount(const stab_gate *gates, int64_t m) {
-        bool two = true, run_two = false;
-        int64_t run = 0, pairs = 0;
-        // a long run of single-qubit Clifford gates may become a gather inside its block
-        auto end_run = [&]() {
-            if (run >= 8) {
-                ++ranges;
-                blocks += !run_two;
-                cliffs += !run_two;
-            }
-            run = 0;
-            run_two = false;
-        };
-        for (int64_t i = 0; i < m; ++i) {
-            const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
-            if (t && (!two || i == 0)) ++cliffs;
-            if (!t && two) ++blocks;
-            two = t;
-            pairs += t;
-            if (gates[i].op >= STAB_RX) end_run();
-            else ++run;
-            run_two |= t;
+stab::PlanCount::PlanCount(const stab_gate *gates, int64_t m) {
+    bool two = true, run_two = false;
+    int64_t run = 0, pairs = 0;
+    // a long run of single-qubit Clifford gates may become a gather inside its block
+    auto end_run = [&]() {
+        if (run >= 8) {
+            ++ranges;
+            blocks += !run_two;
+            cliffs += !run_two;
         }
-        end_run();
-        cliffs += (size_t)(pairs / 65535);   // gates of a pass at most
-        ranges += (size_t)(m / 16384);
+        run = 0;
+        run_two = false;
+    };
+    for (int64_t i = 0; i < m; ++i) {
+        const bool t = gates[i].op == STAB_CX || gates[i].op == STAB_CZ;
+        if (t && (!two || i == 0)) ++cliffs;
+        if (!t && two) ++blocks;
+        two = t;
+        pairs += t;
+        if (gates[i].op >= STAB_RX) end_run();
+        else ++run;
+        run_two |= t;
     }
-};
+    end_run();
+    cliffs += (size_t)(pairs / 65535);   // gates of a pass at most
+    ranges += (size_t)(m / 16384);
+}
 
-}  // namespace
-
-size_t stab::checkpoint_bound(int n, const stab_gate *gates, int64_t m) {
+size_t stab::checkpoint_bound(int n, const PlanCount &k) {
     // a slot more than ck_slots per Clifford pass at most
-    const PlanCount k(gates, m);
     const size_t bytes = (2 * k.blocks + k.cliffs + kCkSpares) * (sizeof(double) << (2 * n));
     return bytes <= kCheckpointBytes ? bytes : 0;
 }
-size_t stab::chain_bound(int n, const stab_gate *gates, int64_t m, bool grad) {
+size_t stab::chain_bound(int n, const PlanCount &k, bool grad) {
     // the largest n whose vectors the path tuner gives to tiles
     if (n < kChainMinN || n > 9) return 0;
-    const PlanCount k(gates, m);
     const size_t per_block = (size_t)((n + tile_wires(n) - 1) / tile_wires(n));
     const size_t dirs = grad ? 2 : 1;   // <O>: two chains of half the plan
     const size_t steps = dirs * ((k.blocks + k.ranges) * per_block + k.cliffs + 2);
@@ -2302,7 +2291,7 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     c->grad_ran = c->ck_ready = c->ck_off = false;
     reset_graphs(c);
     if (c->ckslots.bytes > kCheckpointRelease &&
-        checkpoint_bound(c->n, gates, m) < c->ckslots.bytes / 4)
+        checkpoint_bound(c->n, PlanCount(gates, m)) < c->ckslots.bytes / 4)
         ctx_trim_checkpoints(c, 0);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
