@@ -150,6 +150,7 @@ struct DevPlan {
 // the caller does not wait for what is queued before them: a block that is filled
 // from the front while copies are in flight and replaced when it is full (the old
 // one goes when they are done).  `copied` is behind the last copy.
+constexpr size_t kStagingBytes = (size_t)512 << 10;   // what 10,000 gates' gradient takes
 struct Staging {
     char *p = nullptr;
     size_t bytes = 0, at = 0;
@@ -170,7 +171,7 @@ struct Staging {
             else if (p) full.push_back(p);
             p = nullptr;
             bytes = at = 0;
-            const size_t cap = std::max((size_t)128 << 10, 2 * want);
+            const size_t cap = std::max(kStagingBytes, 2 * want);
             CK(cudaMallocHost((void **)&p, cap));
             bytes = cap;
         }
@@ -314,9 +315,7 @@ struct stab_ctx {
 
     void *stage = nullptr;           // pinned host staging
     size_t stage_bytes = 0;
-    void *aux_stage = nullptr;
-    size_t aux_stage_bytes = 0;
-    Staging tables_stage;            // chains' steps and shapes, gradients' jobs
+    Staging aux_stage;               // terms, chains' steps and shapes, gradients' jobs
     int64_t launches = 0;
 
     int dalloc(DevBuf &b, size_t bytes, cudaStream_t s) {
@@ -723,16 +722,18 @@ int upload_terms(stab_ctx *c, const stab_term *O, int64_t n_terms) {
     RC(encode_terms(c->n, O, n_terms, &t));
     const size_t bytes = (t.size() ? t.size() : 1) * sizeof(DevTerm);
     // The terms are read on the aux stream (expectations, gradients), so they
-    // are uploaded there, from the aux staging buffer: the upload does not
-    // queue behind generator work on the main stream.  The aux stream may
-    // still read the previous terms and its staging buffer.
+    // are uploaded there, from the aux staging: the upload does not queue behind
+    // generator work on the main stream.  The aux stream may still read the
+    // previous terms.
     CK(cudaStreamSynchronize(c->aux));
     RC(c->dalloc(c->terms, bytes, c->aux));
     if (!t.empty()) {
-        RC(c->host_stage(c->aux_stage, c->aux_stage_bytes, bytes));
-        std::memcpy(c->aux_stage, t.data(), t.size() * sizeof(DevTerm));
-        CK(cudaMemcpyAsync(c->terms.p, c->aux_stage, t.size() * sizeof(DevTerm),
-                           cudaMemcpyHostToDevice, c->aux));
+        char *h = nullptr;
+        RC(c->aux_stage.take(bytes, &h));
+        std::memcpy(h, t.data(), t.size() * sizeof(DevTerm));
+        CK(cudaMemcpyAsync(c->terms.p, h, t.size() * sizeof(DevTerm), cudaMemcpyHostToDevice,
+                           c->aux));
+        RC(c->aux_stage.queued(c->aux));
         c->h2d_bytes += (int64_t)(t.size() * sizeof(DevTerm));
     }
     c->n_obs_terms = (int32_t)t.size();
@@ -1298,7 +1299,7 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
     C.alone = n_vec == 1 && tiles == 1;
     // as on the device: steps, descriptors; then the shapes
     char *h = nullptr;
-    RC(c->tables_stage.take(b_steps + 256 + b_shapes, &h));
+    RC(c->aux_stage.take(b_steps + 256 + b_shapes, &h));
     std::copy(C.host[0].begin(), C.host[0].end(), (ChainStep *)h);
     std::copy(C.host[1].begin(), C.host[1].end(), (ChainStep *)h + n0);
     std::memcpy(h + b_steps, C.desc, sizeof(C.desc));
@@ -1307,7 +1308,7 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
     if (ns)
         CK(cudaMemcpyAsync(C.tables.p, h + b_steps + 256, ns * sizeof(ChainShape),
                            cudaMemcpyHostToDevice, s));
-    RC(c->tables_stage.queued(s));
+    RC(c->aux_stage.queued(s));
     CK(launch_chain_tables((const ChainShape *)C.tables.p, (int)ns, c->n, s));
     c->launches += ns > 0;
     C.key = key;
@@ -1647,10 +1648,10 @@ int ck_upload_jobs(stab_ctx *c, cudaStream_t s) {
     }
     const size_t bytes = c->ck_jobs.size() * sizeof(DotJob);
     char *h = nullptr;
-    RC(c->tables_stage.take(bytes, &h));
+    RC(c->aux_stage.take(bytes, &h));
     std::memcpy(h, c->ck_jobs.data(), bytes);
     CK(cudaMemcpyAsync(c->ckjobs.p, h, bytes, cudaMemcpyHostToDevice, s));
-    RC(c->tables_stage.queued(s));
+    RC(c->aux_stage.queued(s));
     c->key_ck = key;
     return STAB_OK;
 }
@@ -2257,9 +2258,8 @@ int stab_destroy(stab_ctx *c) {
                       &c->c_gens.tables, &c->c_expect.tables, &c->c_grad.tables};
     for (DevBuf *b : bufs) c->dfree(*b, c->st);
     if (c->st) cudaStreamSynchronize(c->st);
-    c->tables_stage.release();
+    c->aux_stage.release();
     if (c->stage) cudaFreeHost(c->stage);
-    if (c->aux_stage) cudaFreeHost(c->aux_stage);
     if (c->ev_ready) cudaEventDestroy(c->ev_ready);
     if (c->ev_tx) cudaEventDestroy(c->ev_tx);
     if (c->ev_aux) cudaEventDestroy(c->ev_aux);
