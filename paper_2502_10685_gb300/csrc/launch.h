@@ -416,7 +416,7 @@ struct UniArgs {
     const UniMap *maps;
     const UniSeg *segs;
     const UniPart *parts;
-    int32_t n_segs, n_parts;
+    int32_t n_segs;
     double2 *nodes;          // node matrices, 4^n complex entries each, column-major
     int32_t *node_parity;    // per node: U is kept times sqrt(2)^parity
     int32_t *node_count;     // per node: arrivals of its children (zero between launches)

@@ -482,7 +482,6 @@ int upload_plan(stab_ctx *c, DevPlan &P) {
     P.uargs.parts = (const UniPart *)put(P.uparts.data(), P.uparts.size() * sizeof(UniPart),
                                          b_uparts);
     P.uargs.n_segs = (int32_t)P.usegs.size();
-    P.uargs.n_parts = (int32_t)P.uparts.size();
     P.prog.n_passes = (int32_t)n_pass;
     P.prog.n_ops = (int32_t)n_ops;
     HostPool::run(copies);
@@ -1710,7 +1709,7 @@ int ck_chains(stab_ctx *c, cudaStream_t s) {
 int ck_finish(stab_ctx *c, cudaStream_t gs) {
     CK(launch_grad_dots((const DotJob *)c->ckjobs.p, (int)c->ck_jobs.size(), c->n, c->ck_chunks,
                         (double *)c->ckdots.p, gs));
-CK(launch_run_grads(c->ck.uruns_dev, (int)c->ck.uruns.size(), c->ck.uni_max_run,
+    CK(launch_run_grads(c->ck.uruns_dev, (int)c->ck.uruns.size(), c->ck.uni_max_run,
                         c->ck.ugates_dev, (const double *)c->thetas.p, (const double *)c->ckdots.p,
                         c->ck_chunks, (double *)c->grad_rot.p, gs));
     CK(launch_gather_grads((const double *)c->grad_rot.p, c->ck.param_ptr, c->ck.param_rot,

@@ -190,7 +190,6 @@ struct UniPart {         // 16 bytes
     int32_t node;        // first node (level 0)
     int32_t root;        // the part's unitary
 };
-constexpr int kUniMaxLevels = 16;
 
 struct DevTerm {         // deduplicated observable term: index in the device layout
     double coeff;
