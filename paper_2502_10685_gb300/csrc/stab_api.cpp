@@ -254,6 +254,7 @@ struct stab_ctx {
     cudaEvent_t ev_ready = nullptr;    // plan uploaded and encoded (on st); the aux work waits
                                        // on it (the observable's terms are uploaded on aux)
     cudaEvent_t ev_aux = nullptr;      // aux work done
+    cudaEvent_t ev_gens = nullptr;     // readers of the generators queued so far (on st)
     cudaEvent_t ev_stage = nullptr;    // staging buffer free
     stab_alloc_fn alloc = nullptr;
     stab_free_fn free = nullptr;
@@ -2198,6 +2199,7 @@ int create_ctx(int n, const stab_opts *opts, const stab_path_choice *forced, sta
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_tx, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_aux, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_gens, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_stage, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_stage, c->st);
     if (e == cudaSuccess) {
@@ -2262,6 +2264,7 @@ int stab_destroy(stab_ctx *c) {
     if (c->ev_ready) cudaEventDestroy(c->ev_ready);
     if (c->ev_tx) cudaEventDestroy(c->ev_tx);
     if (c->ev_aux) cudaEventDestroy(c->ev_aux);
+    if (c->ev_gens) cudaEventDestroy(c->ev_gens);
     if (c->ev_stage) cudaEventDestroy(c->ev_stage);
     if (c->aux) cudaStreamDestroy(c->aux);
     if (c->aux2) cudaStreamDestroy(c->aux2);
@@ -2378,7 +2381,10 @@ int stab_run_generators(stab_ctx *c) {
         RC(c->dalloc(c->gens_tmp, bytes, c->st));
         RC(stream_encode(c, c->fwd, n));
         cudaStream_t s = c->aux;
-        CK(cudaStreamWaitEvent(s, c->ev_ready, 0));
+        // behind all that is queued on st: the encoding, and copies of the last run's
+        // generators that have not run yet
+        CK(cudaEventRecord(c->ev_gens, c->st));
+        CK(cudaStreamWaitEvent(s, c->ev_gens, 0));
         const std::vector<const void *> key = {(const void *)c->plan_gen, c->gens.p,
                                                c->gens_tmp.p};
         if (use_chain_forward(c, c->fwd, n)) {

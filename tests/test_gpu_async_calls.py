@@ -57,3 +57,29 @@ def test_first_calls_after_a_load_do_not_wait(stab, n, m):
         assert abs(got[1][int(c.gates[gi]["param"])] - want) <= tol
     want = oracle.forward(n, c.gates, c.thetas, oracle.generator(n, n - 1))
     assert np.abs(layout.lib_to_paper(n, got[2][n - 1]) - want).max() <= 1e-12
+
+
+@pytest.mark.parametrize("n,m", [(7, 2000), (9, 600)])
+def test_a_second_run_waits_for_the_copy_of_the_first(stab, n, m):
+    """Generators copied to device memory are those of the run before the copy,
+    also where the copy is still queued when the generators run again."""
+    import torch
+    c = W.layered_ansatz(n, m, seed=180 + n)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = stab.Stab(n)
+        s.load_circuit(c.gates, c.thetas)
+        out = torch.zeros(6, n, 4 ** n, dtype=torch.float64, device="cuda")
+        s.run_generators()
+        s.generators(out=out[0])
+        for k in range(1, 6):
+            s.run_generators()
+            torch.cuda._sleep(300_000 * k)
+            s.generators(out=out[k])
+        s.run_generators()
+        torch.cuda.synchronize()
+        s.close()
+    assert all(torch.equal(out[0], out[k]) for k in range(1, 6))
+    got = out[0].cpu().numpy()
+    want = oracle.forward(n, c.gates, c.thetas, oracle.generator(n, 0))
+    assert np.abs(layout.lib_to_paper(n, got[0]) - want).max() <= 1e-12
