@@ -83,13 +83,15 @@ typedef struct stab_term {
 
 /* ---------------------------------------------------------------- options */
 enum stab_kernel {
-    /* The library's choice.  n <= 6: vectors resident in shared memory.  Plans of
-     * 64 or more passes: at n <= 4 everything is read off the 2^n x 2^n
-     * unitaries of the plan's segments, which run at once; at n = 5, 6 <O> and
-     * gradients run from both ends and meet at half the passes.  n >= 7: vectors in HBM, passes grouped
-     * into shared-memory tiles where the vectors are small, else one fused pass
-     * per launch (gradients again meet at the cut).  Batches pick their CTAs
-     * per SM by timing a sample of their units. */
+    /* The library's choice.  n <= 6: vectors resident in shared memory (n = 5, 6:
+     * as far as the path tuner finds that faster).  Plans of 64 or more passes (n =
+     * 2, 3: 8): at n <= 4 everything is read off the 2^n x 2^n unitaries of the
+     * plan's segments, which run at once; at n = 5, 6 resident <O> and gradients
+     * run from both ends and meet at half the passes.  Else vectors in HBM, passes
+     * grouped into shared-memory tiles where the vectors are small, else one fused
+     * pass per launch; <O> runs from both ends, gradients keep both sweeps'
+     * vectors (stab_grad_async).  Batches pick their CTAs per SM by timing a sample
+     * of their units. */
     STAB_KERNEL_AUTO = 0,
     STAB_KERNEL_RESIDENT = 1,  /* n <= 6: one CTA per vector through the whole circuit, never cut */
     STAB_KERNEL_STREAMED = 2,  /* vector in HBM, fused passes (any n) */
@@ -257,7 +259,8 @@ int stab_expect_static(int n, const stab_gate *gates, int64_t m, const double *t
  * and the observable of an expectation item is one unit of work; CTAs take
  * units longest first.  (AUTO: items of n >= 6 so much longer than the rest that
  * one CTA would still be at them when all others are done run on many SMs, in
- * a second launch beside it.)  The 2m parameter-shift copies of a circuit (Sec. I)
+ * a second launch beside it, if there is memory for their tables.  Whether an item
+ * does depends on the rest of its batch; the two forms agree to rounding.)  The 2m parameter-shift copies of a circuit (Sec. I)
  * are expectation items that differ only in their angles. */
 #define STAB_BATCH_MAX_QUBITS 8
 

@@ -6,20 +6,23 @@
 // work unless the oldest has waited longer than the aging bound) whenever a
 // slot and enough HBM budget are free.  Two engines then run it:
 //
-//  * the iteration engine (STAB_SERVE_ITERATE, requests of n <= iter_max_n): the
+//  * the iteration engine (STAB_SERVE_ITERATE, requests of n <= iter_max_n, by
+//    default without those that would take one CTA more than two milliseconds): the
 //    planner thread plans the request on the host; the engine thread uploads
 //    it into one device block and, once per iteration, launches one
 //    persistent k_serve kernel that advances every admitted request by a
-//    slice of its instruction streams (a fixed number of chunks per n).  The
+//    slice of its instruction streams (sized by the measured cost of its kind).  The
 //    requests' vectors stay in their device blocks between iterations, new
 //    requests join at the next iteration, finished ones leave after the
 //    launch that finished them.  Two iterations are in flight at a time, so
 //    the host prepares the next launch while the GPU runs the current one.
-//  * the context engine (every request with STAB_SERVE_CONTEXTS, and larger
-//    requests with ITERATE): the request runs on a pooled context with its own
-//    streams (the vectors of a large request fill the GPU by themselves);
-//    its kernels overlap on the device with every other request's.  A
-//    completion thread polls each request's event.
+//  * the context engine (every request with STAB_SERVE_CONTEXTS, the others with
+//    ITERATE): the request runs on a pooled context with its own streams (the
+//    vectors of a large request fill the GPU by themselves, long ones run on many
+//    SMs); its kernels overlap on the device with every other request's.  A
+//    completion thread polls each request's event.  Stored sweeps and tables
+//    that a request uses there are part of what it is admitted with, and what
+//    idle contexts keep of them stays inside the budget.
 //
 // Device memory comes from the allocator hooks of the options (else
 // cudaMallocAsync / cudaFreeAsync on the engine's or context's stream) and is
