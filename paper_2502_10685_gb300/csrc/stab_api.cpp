@@ -167,11 +167,14 @@ struct Staging {
             (void)cudaGetLastError();   // not ready
         }
         if (at + want > bytes) {
+            const size_t last = at;
             if (p && at == 0) cudaFreeHost(p);
             else if (p) full.push_back(p);
             p = nullptr;
             bytes = at = 0;
-            const size_t cap = std::max(kStagingBytes, 2 * want);
+            // room for what was in the old one and this, so that calls which take
+            // turns settle in one block
+            const size_t cap = std::max(kStagingBytes, last + want);
             CK(cudaMallocHost((void **)&p, cap));
             bytes = cap;
         }
@@ -1862,8 +1865,8 @@ size_t stab::checkpoint_bound(int n, const PlanCount &k) {
     return bytes <= kCheckpointBytes ? bytes : 0;
 }
 size_t stab::chain_bound(int n, const PlanCount &k, bool grad) {
-    // the largest n whose vectors the path tuner gives to tiles
-    if (n < kChainMinN || n > 9) return 0;
+    // the largest n whose vectors the path tuner gives to tiles; <O> see use_chain_forward
+    if (n < kChainMinN || n > (grad ? 9 : kChainMaxN)) return 0;
     const size_t per_block = (size_t)((n + tile_wires(n) - 1) / tile_wires(n));
     const size_t dirs = grad ? 2 : 1;   // <O>: two chains of half the plan
     const size_t steps = dirs * ((k.blocks + k.ranges) * per_block + k.cliffs + 2);

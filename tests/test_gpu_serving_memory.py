@@ -38,6 +38,17 @@ def most_in_use(srv, ids):
     pytest.fail("requests not done")
 
 
+def test_nothing_reserved_for_tables_that_are_not_used(stab):
+    """<O> at n = 9 runs as launches, without the chains' tables."""
+    c, obs = W.layered_ansatz(9, 2000, seed=62), W.obs_chain(9)
+    srv = stab.Server()
+    i = srv.submit(c, "expect", obs)
+    most = most_in_use(srv, [i])
+    assert srv.wait(i, timeout_s=120)["status"] == 0
+    srv.close()
+    assert most == stab.Server.footprint(c, "expect", obs)
+
+
 def test_nothing_reserved_for_sweeps_that_are_too_large(stab):
     """69 blocks of wire runs at n = 11: their vectors are more than a context
     keeps, the pair sweep runs, and only the request's footprint is taken."""
