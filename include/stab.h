@@ -417,8 +417,8 @@ typedef struct stab_result {
  * this footprint; it is then admitted with both.  Else it carries a fixed number
  * of vectors (the two forms agree to rounding).  Likewise a request of 5 <= n <= 9
  * there is admitted with a bound on its sweeps' tables, or runs without them.  An
- * idle context keeps up to 64 MiB of sweeps' vectors while the budget has room for
- * them beside the admitted requests.  Where the device has no memory
+ * idle context keeps up to 64 MiB of both while the budget has room for them
+ * beside the admitted requests.  Where the device has no memory
  * for them beside the other requests, the request waits until it is alone; where
  * it has none even then, the fixed number of vectors. */
 int64_t stab_request_footprint(const stab_request *req);

@@ -207,9 +207,10 @@ struct PlanCount {
     size_t blocks = 0, cliffs = 0, ranges = 1;
     PlanCount(const struct ::stab_gate *gates, int64_t m);
 };
-// Hands the stored sweeps' memory back when it is more than `keep`; returns what
-// the context still holds.
-size_t ctx_trim_checkpoints(stab_ctx *ctx, size_t keep);
+// Hands back the memory of stored sweeps, then that of chains' tables, when the
+// context holds more than `keep` of it (no call in flight); returns what it still
+// holds.
+size_t ctx_trim(stab_ctx *ctx, size_t keep);
 
 // Density matrix from the forward-evolved coefficients of 2^n |0><0|:
 // rho (device, 2 x 4^n doubles, interleaved complex, row-major).

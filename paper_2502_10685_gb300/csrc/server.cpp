@@ -141,7 +141,7 @@ struct Slot {
     double *h_res = nullptr;      // pinned host copies
     double *h_grads = nullptr;
     cudaEvent_t ev = nullptr;
-    int64_t kept = 0;             // stored sweeps' memory it holds beyond its request's
+    int64_t kept = 0;             // memory of sweeps and tables it holds beyond its request's
 };
 
 // ---------------------------------------------------------------- iteration engine
@@ -194,8 +194,9 @@ struct Req {
     std::vector<stab_gate> gates;
     std::vector<double> thetas;
     std::vector<stab_term> terms;
-    int64_t footprint = 0;      // with `sweeps` and the chains' tables
+    int64_t footprint = 0;      // with `sweeps` and `tables`
     int64_t sweeps = 0;         // a gradient's stored sweeps (0: the pair sweep runs)
+    int64_t tables = 0;         // the chains'
     bool chains = false;        // sweeps as chains of tile steps
     double work = 0.0;          // estimated work: gates x 4^n (x3 for a gradient)
     stab_result res{};
@@ -337,7 +338,8 @@ int launch_on_context(stab_server *s, Req *r) {
     return STAB_OK;
 }
 
-// Sets what a slot holds beyond its request's sweeps (caller holds s->mu).
+// Sets what a slot holds of sweeps and tables beyond its request's (caller holds
+// s->mu).
 void set_kept(stab_server *s, Slot *sl, int64_t kept) {
     s->kept += kept - sl->kept;
     sl->kept = kept;
@@ -357,7 +359,7 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     for (Slot *sl : idle) set_kept(s, sl, 0);
     lk.unlock();
     stab_synchronize(r->slot->ctx);
-    for (Slot *sl : idle) ctx_trim_checkpoints(sl->ctx, 0);
+    for (Slot *sl : idle) ctx_trim(sl->ctx, 0);
     int rc = launch_on_context(s, r);
     if (rc == STAB_E_NOMEM) {
         stab_synchronize(r->slot->ctx);
@@ -371,7 +373,7 @@ int launch_alone(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     return rc;
 }
 
-// Hands back what idle contexts, then r's own, hold beyond their requests' sweeps
+// Hands back what idle contexts, then r's own, hold beyond their requests' needs
 // when the admitted requests need that room in the budget (the idle ones are out
 // of the pools meanwhile; caller holds s->mu).
 void make_room(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
@@ -387,8 +389,8 @@ void make_room(stab_server *s, Req *r, std::unique_lock<std::mutex> &lk) {
     const bool own = r->slot && r->slot->kept > 0;
     if (own) set_kept(s, r->slot, 0);
     lk.unlock();
-    for (Slot *sl : trim) ctx_trim_checkpoints(sl->ctx, 0);
-    if (own) ctx_trim_checkpoints(r->slot->ctx, (size_t)r->sweeps);
+    for (Slot *sl : trim) ctx_trim(sl->ctx, 0);
+    if (own) ctx_trim(r->slot->ctx, (size_t)(r->sweeps + r->tables));
     lk.lock();
     for (Slot *sl : trim) s->idle[sl->n].push_back(sl);
 }
@@ -449,11 +451,12 @@ void add_context_bytes(const stab_server *s, Req *r) {
     const int64_t t = (int64_t)chain_bound(q.n, k, grad);
     if (r->footprint + t > s->opts.hbm_budget) return;
     r->chains = true;
+    r->tables = t;
     r->footprint += t;
 }
-// Stored sweeps are handed back when they are large, or when the budget has no
-// room for them beside the admitted requests.
-constexpr size_t kKeepCheckpoints = (size_t)64 << 20;
+// Both are handed back when they are large, or when the budget has no room for
+// them beside the admitted requests.
+constexpr size_t kKeepIdle = (size_t)64 << 20;
 
 // ---------------------------------------------------------------- iteration requests: host side
 
@@ -1026,7 +1029,7 @@ void planner_main(stab_server *s) {
         if (!pool.empty()) {
             r->slot = pool.back();
             pool.pop_back();
-            set_kept(s, r->slot, std::max<int64_t>(0, r->slot->kept - r->sweeps));
+            set_kept(s, r->slot, std::max<int64_t>(0, r->slot->kept - r->sweeps - r->tables));
         }
         make_room(s, r, lk);
         lk.unlock();
@@ -1049,7 +1052,7 @@ void planner_main(stab_server *s) {
         if (rc != STAB_OK) {
             if (r->slot) {
                 stab_synchronize(r->slot->ctx);
-                ctx_trim_checkpoints(r->slot->ctx, 0);
+                ctx_trim(r->slot->ctx, 0);
                 set_kept(s, r->slot, 0);
             }
             release_locked(s, r);
@@ -1086,7 +1089,7 @@ void completer_main(stab_server *s) {
             for (Req *r : ended) {
                 // status word of the context (bounded device waits)
                 status.push_back(stab_synchronize(r->slot->ctx));
-                kept.push_back((int64_t)ctx_trim_checkpoints(r->slot->ctx, kKeepCheckpoints));
+                kept.push_back((int64_t)ctx_trim(r->slot->ctx, kKeepIdle));
                 r->res.expect = r->slot->h_res[0];
                 if (r->hdr.kind == STAB_REQ_GRAD && r->hdr.n_params > 0)
                     r->grads.assign(r->slot->h_grads, r->slot->h_grads + r->hdr.n_params);
@@ -1103,7 +1106,7 @@ void completer_main(stab_server *s) {
             }
             if (!trim.empty()) {
                 lk.unlock();
-                for (Slot *sl : trim) ctx_trim_checkpoints(sl->ctx, 0);
+                for (Slot *sl : trim) ctx_trim(sl->ctx, 0);
                 lk.lock();
             }
             for (size_t i = 0; i < ended.size(); ++i) {

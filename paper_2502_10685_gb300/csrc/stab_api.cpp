@@ -1882,15 +1882,27 @@ size_t stab::chain_bound(int n, const PlanCount &k, bool grad) {
     return steps * sizeof(ChainStep) +
            shapes * (sizeof(ChainShape) + groups * sizeof(uint2) + 4 * tiles * sizeof(uint4));
 }
-size_t stab::ctx_trim_checkpoints(stab_ctx *c, size_t keep) {
+size_t stab::ctx_trim(stab_ctx *c, size_t keep) {
     if (!c) return 0;
-    if (c->ckslots.bytes > keep) {
+    auto held = [&]() {
+        size_t sum = c->ckslots.bytes;
+        for (const ChainSet *C : {&c->c_gens, &c->c_expect, &c->c_grad})
+            sum += C->tables.bytes + C->dev.bytes;
+        return sum;
+    };
+    if (held() > keep) {
         c->dfree(c->ckslots, c->aux);
         c->key_ck.clear();
         c->c_grad.key.clear();
         c->g_grad.reset();
     }
-    return c->ckslots.bytes;
+    if (held() > keep)
+        for (ChainSet *C : {&c->c_gens, &c->c_expect, &c->c_grad}) {
+            c->dfree(C->tables, c->aux);
+            c->dfree(C->dev, c->aux);
+            C->clear();
+        }
+    return held();
 }
 
 extern "C" {
@@ -2297,7 +2309,7 @@ int stab_load_circuit(stab_ctx *c, const stab_gate *gates, int64_t m, const doub
     reset_graphs(c);
     if (c->ckslots.bytes > kCheckpointRelease &&
         checkpoint_bound(c->n, PlanCount(gates, m)) < c->ckslots.bytes / 4)
-        ctx_trim_checkpoints(c, 0);
+        ctx_trim(c, 0);
     build_plan(c->n, gates, m, n_params, c->fwd_mode(), &c->fwd.host, !c->use_resident());
     if (c->use_resident()) {
         // AUTO: at n <= 4 the parts' unitaries, at n = 5, 6 the two halves of <O>
@@ -2892,7 +2904,7 @@ int stab_set_grad_memory(stab_ctx *c, int64_t bytes) {
     CK(cudaSetDevice(c->device));
     c->ck_bytes_max = std::min((size_t)bytes, kCheckpointBytes);
     c->ck_off = false;   // decided anew by the next gradient
-    ctx_trim_checkpoints(c, c->ck_bytes_max);
+    if (c->ckslots.bytes > c->ck_bytes_max) ctx_trim(c, 0);
     return STAB_OK;
 }
 

@@ -252,3 +252,19 @@ def test_iter_max_n_takes_long_requests(stab, n, m, iter_max_n):
     for gi in (rot[0], rot[len(rot) // 2], rot[-1]):
         want = oracle.psr_grad_gate(n, c.gates, c.thetas, obs, gi)
         assert abs(g[int(c.gates[gi]["param"])] - want) <= tol
+
+
+def test_idle_contexts_hand_large_tables_back(stab):
+    """100,000 random gates at n = 8 have more than 64 MiB of tables: an idle context
+    keeps none of them."""
+    c, obs = W.random_circuit(8, 100000, seed=200), W.obs_chain(8)
+    srv = HookedServer(stab)
+    status, e, g = srv.wait(srv.submit(c, "expect", obs), c.n_params)
+    most, after = srv.most, sum(srv.live.values())
+    srv.close()
+    assert status == 0
+    s = stab.Stab(8)
+    s.load_circuit(c.gates, c.thetas)
+    assert abs(e - s.expect(obs)) <= 1e-10 * l1(obs)
+    s.close()
+    assert most > 80 << 20 and after < most - (60 << 20)
