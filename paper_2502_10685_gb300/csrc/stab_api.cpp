@@ -149,22 +149,25 @@ struct DevPlan {
 // Pinned staging of uploads on the aux stream, so that the copies are queued and
 // the caller does not wait for what is queued before them: a block that is filled
 // from the front while copies are in flight and replaced when it is full (the old
-// one goes when they are done).  `copied` is behind the last copy.
-constexpr size_t kStagingBytes = (size_t)512 << 10;   // what 10,000 gates' gradient takes
+// one goes when they are done).
 struct Staging {
+    size_t least = 4096;   // of a block
     char *p = nullptr;
     size_t bytes = 0, at = 0;
     std::vector<char *> full;
-    cudaEvent_t copied = nullptr;
-    int take(size_t want, char **out) {
+    cudaEvent_t copied = nullptr;   // behind the copies up to the last mark()
+    bool unmarked = false;          // a copy was queued after it
+    // idle: the caller knows that no copy is in flight.
+    int take(size_t want, bool idle, char **out) {
         want = align256(want);
-        if (!copied) CK(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
-        if (cudaEventQuery(copied) == cudaSuccess) {
+        if (!idle && !unmarked) {
+            idle = !copied || cudaEventQuery(copied) == cudaSuccess;
+            if (!idle) (void)cudaGetLastError();   // not ready
+        }
+        if (idle) {
             for (char *b : full) cudaFreeHost(b);
             full.clear();
             at = 0;
-        } else {
-            (void)cudaGetLastError();   // not ready
         }
         if (at + want > bytes) {
             const size_t last = at;
@@ -174,16 +177,19 @@ struct Staging {
             bytes = at = 0;
             // room for what was in the old one and this, so that calls which take
             // turns settle in one block
-            const size_t cap = std::max(kStagingBytes, last + want);
+            const size_t cap = std::max(least, last + want);
             CK(cudaMallocHost((void **)&p, cap));
             bytes = cap;
         }
         *out = p + at;
         at += want;
+        unmarked = true;
         return STAB_OK;
     }
-    int queued(cudaStream_t s) {
+    int mark(cudaStream_t s) {
+        if (!copied) CK(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
         CK(cudaEventRecord(copied, s));
+        unmarked = false;
         return STAB_OK;
     }
     void release() {
@@ -196,6 +202,11 @@ struct Staging {
         copied = nullptr;
     }
 };
+
+// Where tables and jobs follow the terms: what 10,000 gates' gradient takes.  (A
+// block of 4 KiB comes out of pinned memory that the driver holds already: the
+// first call at n = 2 takes 0.22 ms, 0.24 with 512 KiB.)
+constexpr size_t kStagingTables = (size_t)512 << 10;
 
 // A captured sequence of streamed launches, valid while its key is unchanged.
 struct GraphCache {
@@ -732,11 +743,10 @@ int upload_terms(stab_ctx *c, const stab_term *O, int64_t n_terms) {
     RC(c->dalloc(c->terms, bytes, c->aux));
     if (!t.empty()) {
         char *h = nullptr;
-        RC(c->aux_stage.take(bytes, &h));
+        RC(c->aux_stage.take(bytes, true, &h));
         std::memcpy(h, t.data(), t.size() * sizeof(DevTerm));
         CK(cudaMemcpyAsync(c->terms.p, h, t.size() * sizeof(DevTerm), cudaMemcpyHostToDevice,
                            c->aux));
-        RC(c->aux_stage.queued(c->aux));
         c->h2d_bytes += (int64_t)(t.size() * sizeof(DevTerm));
     }
     c->n_obs_terms = (int32_t)t.size();
@@ -1302,7 +1312,7 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
     C.alone = n_vec == 1 && tiles == 1;
     // as on the device: steps, descriptors; then the shapes
     char *h = nullptr;
-    RC(c->aux_stage.take(b_steps + 256 + b_shapes, &h));
+    RC(c->aux_stage.take(b_steps + 256 + b_shapes, false, &h));
     std::copy(C.host[0].begin(), C.host[0].end(), (ChainStep *)h);
     std::copy(C.host[1].begin(), C.host[1].end(), (ChainStep *)h + n0);
     std::memcpy(h + b_steps, C.desc, sizeof(C.desc));
@@ -1311,7 +1321,7 @@ int chain_upload(stab_ctx *c, ChainSet &C, const std::vector<const void *> &key,
     if (ns)
         CK(cudaMemcpyAsync(C.tables.p, h + b_steps + 256, ns * sizeof(ChainShape),
                            cudaMemcpyHostToDevice, s));
-    RC(c->aux_stage.queued(s));
+    RC(c->aux_stage.mark(s));
     CK(launch_chain_tables((const ChainShape *)C.tables.p, (int)ns, c->n, s));
     c->launches += ns > 0;
     C.key = key;
@@ -1651,10 +1661,10 @@ int ck_upload_jobs(stab_ctx *c, cudaStream_t s) {
     }
     const size_t bytes = c->ck_jobs.size() * sizeof(DotJob);
     char *h = nullptr;
-    RC(c->aux_stage.take(bytes, &h));
+    RC(c->aux_stage.take(bytes, false, &h));
     std::memcpy(h, c->ck_jobs.data(), bytes);
     CK(cudaMemcpyAsync(c->ckjobs.p, h, bytes, cudaMemcpyHostToDevice, s));
-    RC(c->aux_stage.queued(s));
+    RC(c->aux_stage.mark(s));
     c->key_ck = key;
     return STAB_OK;
 }
@@ -2198,6 +2208,7 @@ int create_ctx(int n, const stab_opts *opts, const stab_path_choice *forced, sta
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && n >= kChainMinN)
         c->chain_ctas = chain_max_ctas(1 << (chain_tile_bits(n) - 2));
+    if (n >= kChainMinN) c->aux_stage.least = kStagingTables;
     if (e == cudaSuccess) {
         c->device = dev;
         if (o.stream || o.stream_given) {
