@@ -29,17 +29,24 @@ __host__ __device__ inline bool arrivals_reached(uint32_t seen, uint32_t want) {
 // fail another thread's larger launch.  One SmemLimit per kernel.
 struct SmemLimit {
     std::mutex mu;
-    size_t set[64] = {};   // per device: the limit set so far
+    size_t set[64] = {};   // per device: the limit so far (0: not asked yet)
 };
 
 template <typename K>
 cudaError_t raise_smem_limit(K kernel, size_t smem, SmemLimit &lim) {
-    if (smem <= 48 * 1024) return cudaSuccess;   // the default limit
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> g(lim.mu);
     const bool tracked = dev >= 0 && dev < 64;
+    if (!tracked || lim.set[dev] == 0) {
+        // the default: what 48 KiB hold beside the kernel's static shared memory
+        cudaFuncAttributes fa{};
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return e;
+        if (tracked) lim.set[dev] = (size_t)fa.maxDynamicSharedSizeBytes;
+        if ((size_t)fa.maxDynamicSharedSizeBytes >= smem) return cudaSuccess;
+    }
     if (tracked && lim.set[dev] >= smem) return cudaSuccess;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess && tracked) lim.set[dev] = smem;

@@ -60,3 +60,26 @@ def test_both_forms_match_parameter_shift(stab, n, family, m, memory):
         for slot in (0, c.n_params // 2, c.n_params - 1):
             assert abs(g[slot] - slot_derivative(c, obs, slot)) <= tol, slot
     s.close()
+
+
+@pytest.mark.parametrize("rotations", range(33, 38))
+def test_groups_that_fill_the_default_shared_memory(stab, rotations):
+    """A tile group of the pair sweep keeps a row per rotation in shared memory:
+    35 rotations of one group take exactly 48 KiB, where the kernel's static
+    shared memory no longer fits beside them."""
+    n = 7
+    row = W.gates_from_list([("RX", q, k) for k, q in enumerate(range(1, n))])
+    row2 = W.gates_from_list([("RY", q, n + k) for k, q in enumerate(range(1, n))])
+    cx = W.gates_from_list([("CX", 0, 1)])
+    run = W.gates_from_list([(("RX", "RY", "RZ")[k % 3], 0, 2 * n + k) for k in range(rotations)])
+    gates = np.concatenate([row, cx, row2, cx, run])
+    c = W.Circuit(n, gates, np.random.default_rng(rotations).uniform(0, 6, 2 * n + rotations))
+    obs = W.obs_chain(n)
+    tol = 1e-12 * sum(abs(a) for a, _ in obs)
+    s = stab.Stab(n)
+    s.set_grad_memory(0)
+    s.load_circuit(c.gates, c.thetas)
+    e, g = s.grad(obs)
+    s.close()
+    assert abs(e - oracle.expect(n, c.gates, c.thetas, obs)) <= tol
+    assert np.abs(g - oracle.psr_grad(n, c.gates, c.thetas, obs)).max() <= tol
