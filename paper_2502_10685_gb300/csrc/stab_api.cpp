@@ -151,7 +151,7 @@ struct DevPlan {
 // from the front while copies are in flight and replaced when it is full (the old
 // one goes when they are done).
 struct Staging {
-    size_t least = 4096;   // of a block
+    size_t least = 0;      // bytes of a block
     char *p = nullptr;
     size_t bytes = 0, at = 0;
     std::vector<char *> full;
@@ -203,9 +203,10 @@ struct Staging {
     }
 };
 
-// Where tables and jobs follow the terms: what 10,000 gates' gradient takes.  (A
-// block of 4 KiB comes out of pinned memory that the driver holds already: the
-// first call at n = 2 takes 0.22 ms, 0.24 with 512 KiB.)
+// Where chains' tables follow the terms (kChainMinN to kChainMaxN): what 10,000
+// gates' gradient takes.  (A few bytes come out of pinned memory that the
+// driver holds already, one of 512 KiB takes 0.1 ms: the first call at n = 2 takes
+// 0.22 ms, 0.24 with 512 KiB.)
 constexpr size_t kStagingTables = (size_t)512 << 10;
 
 // A captured sequence of streamed launches, valid while its key is unchanged.
@@ -2208,7 +2209,7 @@ int create_ctx(int n, const stab_opts *opts, const stab_path_choice *forced, sta
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && n >= kChainMinN)
         c->chain_ctas = chain_max_ctas(1 << (chain_tile_bits(n) - 2));
-    if (n >= kChainMinN) c->aux_stage.least = kStagingTables;
+    if (n >= kChainMinN && n <= kChainMaxN) c->aux_stage.least = kStagingTables;
     if (e == cudaSuccess) {
         c->device = dev;
         if (o.stream || o.stream_given) {
